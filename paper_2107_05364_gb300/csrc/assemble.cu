@@ -21,85 +21,141 @@ namespace {
 // high faces.
 //   N_xx = -(1/4 pi) sum_corners s atan(dy dz / (dx R))
 //   N_xy = +(1/4 pi) sum_corners s log(dz + R)         (xz: dy, yz: dx)
-// dx == 0 (point in a face plane, outside the face): the arctan term is 0,
-// its +-pi/2 limits cancel between corners.  A log pair whose two offsets
-// are both negative is rewritten with log(R - d), exact and free of the
-// cancellation of d + R when the point lies far on the negative side.
-struct Corners {
-  double d[3][2];  // offsets r - face, [axis][face]
-  double R[8];     // corner distance, index fx | fy << 1 | fz << 2
+// The FP64 pipe bounds assembly (GB300 executes ~2 FP64 operations per clock
+// and SM), so the 24 arctangents and 24 logarithms of the sums are not taken
+// one by one: the arctangents of an entry are the arguments of complex
+// numbers dx R + i dy dz, which are multiplied, and the logarithms of an
+// entry are one logarithm of a ratio of products: 3 + 3 transcendental
+// functions per block instead of 48.  The rounding of the products is a few
+// ulps of the angle or of the ratio, as much as that of the sums it replaces
+// (whose logarithms of lengths in metres are of order 20); against 128-bit
+// arithmetic distant blocks come out 7 to 13 times closer, touching ones as
+// before.  n = 6,000 graded film, tensor and first field: 150.1 -> 39.3 ms.
+__device__ __forceinline__ double small_series(double t, double z) {
+  // t (1 + z/3 + z^2/5 + z^3/7 + z^4/9 + z^5/11): atan t with z = -t^2,
+  // atanh t with z = t^2; |t| < 2^-5 leaves z^6 / 13 < 7e-20
+  return t * fma(z, fma(z, fma(z, fma(z, fma(z, 1.0 / 11, 1.0 / 9), 1.0 / 7), 1.0 / 5), 1.0 / 3), 1.0);
+}
+constexpr double kSmallArg = 0.03125;
+
+// Arguments p of one face pair: theta_1 - theta_0 with theta = atan(b / a),
+// a > 0, as a complex number (its argument is in (-pi, pi)).
+struct Cplx {
+  double re, im;
 };
-
-__device__ __forceinline__ double atan_ratio(double num_a, double num_b, double den, double R) {
-  return den == 0.0 ? 0.0 : atan((num_a * num_b) / (den * R));
+__device__ __forceinline__ Cplx arg_diff(double a1, double b1, double a0, double b0) {
+  return {fma(a1, a0, b1 * b0), fma(b1, a0, -(a1 * b0))};
+}
+__device__ __forceinline__ Cplx cmul(Cplx p, Cplx q) {
+  return {fma(p.re, q.re, -(p.im * q.im)), fma(p.re, q.im, p.im * q.re)};
 }
 
-// log(dp + Rp) - log(dm + Rm) for the two faces (m = low face, p = high face)
-// of one axis, with the fixed other two corner coordinates.
-__device__ __forceinline__ double log_diff(double dm, double Rm, double dp, double Rp) {
-  if (dm < 0.0 && dp < 0.0) return log(Rm - dm) - log(Rp - dp);
-  return log(dp + Rp) - log(dm + Rm);
+// Sum over the corners of s atan(v w / (u R)) for the axis u: the faces
+// u[0], u[1]; vw[fv | fw << 1] the products of the other two offsets;
+// R(fu, fv, fw) the distances.  For a face u = 0 (the point in its plane,
+// outside the face) the arctangents count 0: their +-pi/2 limits cancel.
+template <typename RF>
+__device__ __forceinline__ double angle_sum(const double u[2], const double vw[4], RF R) {
+  Cplx pa[2], pb[2], f[2];
+  bool plain = true;  // every partial argument within (-pi/2, pi/2): the products keep the branch
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double a = fabs(u[k]);
+    if (a == 0.0) {
+      pa[k] = pb[k] = f[k] = {1.0, 0.0};
+      continue;
+    }
+    pa[k] = arg_diff(a * R(k, 1, 0), vw[1], a * R(k, 0, 0), vw[0]);
+    pb[k] = arg_diff(a * R(k, 0, 1), vw[2], a * R(k, 1, 1), vw[3]);
+    f[k] = cmul(pa[k], pb[k]);
+    if (u[k] < 0.0) {
+      pa[k].im = -pa[k].im;
+      pb[k].im = -pb[k].im;
+      f[k].im = -f[k].im;
+    }
+    plain = plain && pa[k].re > 0.0 && pb[k].re > 0.0 && f[k].re > 0.0;
+  }
+  if (plain) {
+    const Cplx t = cmul(f[0], {f[1].re, -f[1].im});
+    if (fabs(t.im) < kSmallArg * t.re) {
+      const double q = t.im / t.re;
+      return small_series(q, -q * q);
+    }
+    return atan2(t.im, t.re);
+  }
+  return (atan2(pa[0].im, pa[0].re) + atan2(pb[0].im, pb[0].re)) -
+         (atan2(pa[1].im, pa[1].re) + atan2(pb[1].im, pb[1].re));
 }
 
-__device__ void cuboid_tensor(const double *r, const double *c, const double *e, double out[6]) {
-  Corners K;
+// Sum over the corners of s log(w + R) for the log's axis w: w[0], w[1] its
+// offsets; R(f1, f2, fw).  Where both offsets are negative, log(R - w) of the
+// swapped faces takes its place: exact, and free of the cancellation of
+// w + R for a point far on the negative side.
+template <typename RF>
+__device__ __forceinline__ double log_sum(const double w[2], RF R) {
+  const bool neg = w[0] < 0.0 && w[1] < 0.0;
+  const double w0 = neg ? -w[0] : w[0], w1 = neg ? -w[1] : w[1];
+  const double n = ((R(0, 0, 1) + w1) * (R(1, 1, 1) + w1)) * ((R(1, 0, 0) + w0) * (R(0, 1, 0) + w0));
+  const double d = ((R(0, 0, 0) + w0) * (R(1, 1, 0) + w0)) * ((R(1, 0, 1) + w1) * (R(0, 1, 1) + w1));
+  const double diff = n - d, sum = n + d;
+  double v;
+  if (fabs(diff) < kSmallArg * sum) {
+    const double q = diff / sum;
+    v = 2.0 * small_series(q, q * q);  // log(n / d) = 2 atanh((n - d) / (n + d))
+  } else {
+    v = log(n / d);
+  }
+  return neg ? -v : v;
+}
+
+__device__ __forceinline__ void cuboid_tensor(const double *r, const double *c, const double *e, double out[6]) {
+  // offsets r - face in units of a power of two near the tile's size (exact):
+  // the products below stay far from under- and overflow in any unit of length
+  const double unit = scalbn(1.0, -ilogb(e[0] + e[1] + e[2]));
+  double d[3][2], R[8];  // [axis][face]; corner distance, index fx | fy << 1 | fz << 2
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    K.d[a][0] = r[a] - (c[a] - 0.5 * e[a]);
-    K.d[a][1] = r[a] - (c[a] + 0.5 * e[a]);
+    d[a][0] = unit * (r[a] - (c[a] - 0.5 * e[a]));
+    d[a][1] = unit * (r[a] - (c[a] + 0.5 * e[a]));
+  }
+  double xy[4], xz[4], yz[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    xy[q] = d[0][q & 1] * d[1][q >> 1];
+    xz[q] = d[0][q & 1] * d[2][q >> 1];
+    yz[q] = d[1][q & 1] * d[2][q >> 1];
   }
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const double x = K.d[0][q & 1], y = K.d[1][(q >> 1) & 1], z = K.d[2][(q >> 2) & 1];
-    K.R[q] = sqrt(x * x + y * y + z * z);
-  }
-  double txx = 0.0, tyy = 0.0, tzz = 0.0;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const double s = (__popc(q) & 1) ? 1.0 : -1.0;
-    const double x = K.d[0][q & 1], y = K.d[1][(q >> 1) & 1], z = K.d[2][(q >> 2) & 1];
-    txx += s * atan_ratio(y, z, x, K.R[q]);
-    tyy += s * atan_ratio(x, z, y, K.R[q]);
-    tzz += s * atan_ratio(x, y, z, K.R[q]);
-  }
-  // Off-diagonal entries: pair the two faces of the log's axis.  For a pair
-  // with the other two faces (f1, f2) fixed, the corner with the low face
-  // has sign s_lo = -(-1)^(f1+f2) and the high-face corner -s_lo, so the pair
-  // contributes s_lo (log(d_lo + R_lo) - log(d_hi + R_hi)) = -s_lo log_diff.
-  double txy = 0.0, txz = 0.0, tyz = 0.0;
-#pragma unroll
-  for (int f1 = 0; f1 < 2; ++f1) {
-#pragma unroll
-    for (int f2 = 0; f2 < 2; ++f2) {
-      const double s_lo = ((f1 + f2) & 1) ? 1.0 : -1.0;
-      // xy: log axis z, fixed (fx = f1, fy = f2)
-      txy -= s_lo * log_diff(K.d[2][0], K.R[f1 | (f2 << 1)], K.d[2][1], K.R[f1 | (f2 << 1) | 4]);
-      // xz: log axis y, fixed (fx = f1, fz = f2)
-      txz -= s_lo * log_diff(K.d[1][0], K.R[f1 | (f2 << 2)], K.d[1][1], K.R[f1 | 2 | (f2 << 2)]);
-      // yz: log axis x, fixed (fy = f1, fz = f2)
-      tyz -= s_lo * log_diff(K.d[0][0], K.R[(f1 << 1) | (f2 << 2)], K.d[0][1], K.R[1 | (f1 << 1) | (f2 << 2)]);
-    }
+    const double x = d[0][q & 1], y = d[1][(q >> 1) & 1], z = d[2][(q >> 2) & 1];
+    R[q] = sqrt(x * x + y * y + z * z);
   }
   const double k = 0.25 / MT_PI;
-  out[0] = -k * txx;
-  out[1] = k * txy;
-  out[2] = k * txz;
-  out[3] = -k * tyy;
-  out[4] = k * tyz;
-  out[5] = -k * tzz;
+  out[0] = -k * angle_sum(d[0], yz, [&](int x, int y, int z) { return R[x | (y << 1) | (z << 2)]; });
+  out[3] = -k * angle_sum(d[1], xz, [&](int y, int x, int z) { return R[x | (y << 1) | (z << 2)]; });
+  out[5] = -k * angle_sum(d[2], xy, [&](int z, int x, int y) { return R[x | (y << 1) | (z << 2)]; });
+  out[1] = k * log_sum(d[2], [&](int x, int y, int z) { return R[x | (y << 1) | (z << 2)]; });
+  out[2] = k * log_sum(d[1], [&](int x, int z, int y) { return R[x | (y << 1) | (z << 2)]; });
+  out[4] = k * log_sum(d[0], [&](int y, int z, int x) { return R[x | (y << 1) | (z << 2)]; });
 }
 
-// Tensor of a uniformly magnetised tetrahedron (vertices v[4][3]) at r.
-// The body's field is that of its face charges sigma_f = M.n_f, so with
-// H = -N M,  N = (1/4 pi) sum_f g_f n_f^T,  g_f = grad_r int_f dS / |r - r'|.
-// For a plane triangle the gradient splits into a part along n_f, -n_f times
-// the solid angle under which the face is seen (signed like the height of r
-// above the face), and an in-plane part from the 2-D divergence theorem:
-// minus the sum over the edges of the edge's outward in-plane normal times
-// int_edge dl / |r - r'|.  Solid angle: atan2 form of Van Oosterom and
-// Strackee (1983); edge integral: log((R_b + s_b) / (R_a + s_a)) with s the
-// projections on the edge direction, or the equal log((R_a - s_a) /
-// (R_b - s_b)) where the first would cancel.  FP64 throughout.
+// Tensor of a uniformly magnetised tetrahedron at r.  The body's field is that
+// of its face charges sigma_f = M.n_f, so with H = -N M,
+//   N = (1/4 pi) sum_f g_f n_f^T,  g_f = grad_r int_f dS / |r - r'|.
+// For a plane triangle the gradient splits into a part along n_f, minus the
+// signed solid angle of the face, and an in-plane part from the 2-D
+// divergence theorem: minus the sum over its edges of the edge's outward
+// in-plane normal u times l_e = int_e dl / |r - r'|.  Each edge belongs to
+// two faces and l_e is the same for both, so
+//   N = (1/4 pi) [ sum_f -omega_f n_f n_f^T - sum_e l_e (u n^T + u' n'^T) ]
+// with dyads that depend on the tetrahedron only (the polyhedron form of
+// Werner and Scheeres, 1997): they are formed once per tile (tetra_geom), and
+// a block takes 4 distances, 4 solid angles (atan2 form of Van Oosterom and
+// Strackee, 1983; the triple product as (a - r).(b - a) x (c - a)) and 6 edge
+// integrals, l_e = 2 atanh(|e| / (R_a + R_b)).  FP64 throughout; the FP64 pipe bounds it
+// (per-pair face geometry and every edge twice took three times the
+// operations): 5,760 tetrahedra, tensor and first field, 153.8 -> 35.8 ms; errors
+// against 128-bit arithmetic 0.3 to 0.65 of the per-face form's.
 __device__ __forceinline__ void sub3(const double *a, const double *b, double *c) {
   c[0] = a[0] - b[0];
   c[1] = a[1] - b[1];
@@ -114,73 +170,135 @@ __device__ __forceinline__ void crs3(const double *a, const double *b, double *c
   c[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-__device__ void tetra_tensor(const double *r, const double *v, double out[6]) {
-  double N[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+// per-tile geometry of a tetrahedron (doubles): vertices 4 x 3, outward face
+// normals (b - a) x (c - a) 4 x 3, face dyads n n^T 4 x 6, edge dyads 6 x 6
+// (symmetrised: the exact ones are symmetric), edge lengths 6, the largest
+// distance of a vertex from the centroid, the centroid.  Face f lies opposite
+// vertex f; edges 01, 02, 03, 12, 13, 23.  Dyad entries xx xy xz yy yz zz.
+constexpr int kTgVert = 0, kTgNorm = 12, kTgFace = 24, kTgEdge = 48, kTgLen = 84, kTgRad = 90, kTgCen = 91,
+              kTgSize = 94;
+__device__ __forceinline__ int tetra_edge(int a, int b) {  // a < b
+  return a == 0 ? b - 1 : a + b;
+}
+
+__device__ void tetra_geom(const double *c, const double *v, double *G) {
+  for (int q = 0; q < 12; ++q) G[kTgVert + q] = v[q];
+  for (int q = kTgEdge; q < kTgLen; ++q) G[q] = 0.0;
+  double rad = 0.0;
+  for (int a = 0; a < 4; ++a) {
+    double d[3];
+    sub3(v + 3 * a, c, d);
+    rad = fmax(rad, sqrt(dot3(d, d)));
+    for (int b = a + 1; b < 4; ++b) {
+      sub3(v + 3 * b, v + 3 * a, d);
+      G[kTgLen + tetra_edge(a, b)] = sqrt(dot3(d, d));
+    }
+  }
+  G[kTgRad] = rad;
+  for (int q = 0; q < 3; ++q) G[kTgCen + q] = c[q];
 #pragma unroll 1
   for (int f = 0; f < 4; ++f) {
     // face (a, b, c) opposite vertex f, made counter-clockwise about its
     // outward normal
-    const int ia = f == 0 ? 1 : 0;
-    const int ib = f <= 1 ? 2 : 1;
-    const int ic = f <= 2 ? 3 : 2;
-    const double *A = v + 3 * ia, *Bv = v + 3 * ib, *C = v + 3 * ic;
+    int id[3] = {f == 0 ? 1 : 0, f <= 1 ? 2 : 1, f <= 2 ? 3 : 2};
     double ab[3], ac[3], nf[3], to_f[3];
-    sub3(Bv, A, ab);
-    sub3(C, A, ac);
+    sub3(v + 3 * id[1], v + 3 * id[0], ab);
+    sub3(v + 3 * id[2], v + 3 * id[0], ac);
     crs3(ab, ac, nf);
-    sub3(v + 3 * f, A, to_f);
+    sub3(v + 3 * f, v + 3 * id[0], to_f);
     if (dot3(nf, to_f) > 0.0) {
-      const double *t = Bv;
-      Bv = C;
-      C = t;
-      nf[0] = -nf[0];
-      nf[1] = -nf[1];
-      nf[2] = -nf[2];
+      const int t = id[1];
+      id[1] = id[2];
+      id[2] = t;
+      for (int q = 0; q < 3; ++q) nf[q] = -nf[q];
     }
+    for (int q = 0; q < 3; ++q) G[kTgNorm + 3 * f + q] = nf[q];
     const double inv = 1.0 / sqrt(dot3(nf, nf));
-    nf[0] *= inv;
-    nf[1] *= inv;
-    nf[2] *= inv;
-    double ra[3], rb[3], rc[3], bxc[3];
-    sub3(A, r, ra);
-    sub3(Bv, r, rb);
-    sub3(C, r, rc);
-    crs3(rb, rc, bxc);
-    const double la = sqrt(dot3(ra, ra)), lb = sqrt(dot3(rb, rb)), lc = sqrt(dot3(rc, rc));
-    const double omega = -2.0 * atan2(dot3(ra, bxc), la * lb * lc + dot3(ra, rb) * lc + dot3(ra, rc) * lb +
-                                                         dot3(rb, rc) * la);
-    double g[3] = {-omega * nf[0], -omega * nf[1], -omega * nf[2]};
-    const double *P[3] = {A, Bv, C};
-    const double *Rv[3] = {ra, rb, rc};
-    const double L[3] = {la, lb, lc};
-#pragma unroll
+    for (int q = 0; q < 3; ++q) nf[q] *= inv;
+    int k = 0;
+    for (int a = 0; a < 3; ++a)
+      for (int b = a; b < 3; ++b) G[kTgFace + 6 * f + k++] = nf[a] * nf[b];
     for (int e = 0; e < 3; ++e) {
-      const int e2 = (e + 1) % 3;
+      const int p = id[e], q = id[(e + 1) % 3];
       double t[3], u[3];
-      sub3(P[e2], P[e], t);
+      sub3(v + 3 * q, v + 3 * p, t);
       const double len = sqrt(dot3(t, t));
-      t[0] /= len;
-      t[1] /= len;
-      t[2] /= len;
+      for (int a = 0; a < 3; ++a) t[a] /= len;
       crs3(t, nf, u);  // in-plane, out of the face
-      const double s1 = dot3(Rv[e], t), s2 = dot3(Rv[e2], t);
-      const double li = (s1 + s2 >= 0.0) ? log((L[e2] + s2) / (L[e] + s1)) : log((L[e] - s1) / (L[e2] - s2));
-      g[0] -= u[0] * li;
-      g[1] -= u[1] * li;
-      g[2] -= u[2] * li;
+      double *D = G + kTgEdge + 6 * tetra_edge(p < q ? p : q, p < q ? q : p);
+      k = 0;
+      for (int a = 0; a < 3; ++a)
+        for (int b = a; b < 3; ++b) D[k++] += 0.5 * (u[a] * nf[b] + u[b] * nf[a]);
+    }
+  }
+}
+
+__global__ void k_tetra_geom(int64_t n, const double *centre, const double *vert, double *geo) {
+  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (j < n) tetra_geom(centre + 3 * j, vert + 12 * j, geo + kTgSize * j);
+}
+
+__device__ __forceinline__ void tetra_tensor(const double *r, const double *G, double out[6]) {
+  double D[4][3], L[4], num[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    double *d = D[a];
+    sub3(G + kTgVert + 3 * a, r, d);
+    L[a] = sqrt(dot3(d, d));
+    // the faces that hold vertex a: any of a face's vertices gives its triple
+    // product; faces 1, 2, 3 take vertex 0, face 0 vertex 1
+    if (a == 0) {
+#pragma unroll
+      for (int f = 1; f < 4; ++f) num[f] = dot3(d, G + kTgNorm + 3 * f);
+    } else if (a == 1) {
+      num[0] = dot3(d, G + kTgNorm);
+    }
+  }
+  double N[6] = {0, 0, 0, 0, 0, 0}, dots[6];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = a + 1; b < 4; ++b) {
+      const int e = tetra_edge(a, b);
+      const double len = G[kTgLen + e];
+      dots[e] = dot3(D[a], D[b]);
+      const double s = L[a] + L[b];
+      double li;
+      if (8.0 * len < s) {  // 2 atanh(q), q = len / s: 10 terms leave q^20 / 21 < 5e-20
+        const double q = len / s, z = q * q;
+        li = 2.0 * q *
+             fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, 1.0 / 19, 1.0 / 17), 1.0 / 15), 1.0 / 13),
+                                                   1.0 / 11), 1.0 / 9), 1.0 / 7), 1.0 / 5), 1.0 / 3), 1.0);
+      } else if (dots[e] >= 0.0) {
+        li = log((s + len) / (s - len));
+      } else {
+        // near the edge s - len would cancel:
+        // s^2 - len^2 = 2 (R_a R_b + dot) = 2 |a x b|^2 / (R_a R_b - dot)
+        double x[3];
+        crs3(D[a], D[b], x);
+        li = log((s + len) * (s + len) * fma(L[a], L[b], -dots[e]) / (2.0 * dot3(x, x)));
+      }
+#pragma unroll
+      for (int q = 0; q < 6; ++q) N[q] = fma(-li, G[kTgEdge + 6 * e + q], N[q]);
     }
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+  for (int f = 0; f < 4; ++f) {
+    const int a = f == 0 ? 1 : 0, b = f <= 1 ? 2 : 1, c = f <= 2 ? 3 : 2;
+    const double den = fma(L[a] * L[b], L[c], fma(dots[tetra_edge(a, b)], L[c],
+                                                  fma(dots[tetra_edge(a, c)], L[b], dots[tetra_edge(b, c)] * L[a])));
+    double half;  // half the solid angle
+    if (fabs(num[f]) < kSmallArg * den) {
+      const double q = num[f] / den;
+      half = small_series(q, -q * q);
+    } else {
+      half = atan2(num[f], den);
+    }
 #pragma unroll
-      for (int b = 0; b < 3; ++b) N[a][b] += g[a] * nf[b];
+    for (int q = 0; q < 6; ++q) N[q] = fma(2.0 * half, G[kTgFace + 6 * f + q], N[q]);
   }
   const double k = 0.25 / MT_PI;
-  out[0] = k * N[0][0];
-  out[1] = 0.5 * k * (N[0][1] + N[1][0]);
-  out[2] = 0.5 * k * (N[0][2] + N[2][0]);
-  out[3] = k * N[1][1];
-  out[4] = 0.5 * k * (N[1][2] + N[2][1]);
-  out[5] = k * N[2][2];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) out[q] = k * N[q];
 }
 
 // One block per lattice offset (dx, dy, dz): the tensor of the tile at the
@@ -252,7 +370,7 @@ __device__ __forceinline__ int64_t scale_index(int64_t i, int64_t j, int TR, int
 struct AsmArgs {
   const double *centre, *edge;
   const double *vert;  // 12n, tetrahedral tiles
-  int kind;            // MT_TILE_CUBOID / MT_TILE_TETRA
+  const double *geo;   // kTgSize n, tetrahedral tiles (tetra_geom)
   // uniform lattice: block (i, j) = table[offset lat_i - lat_j] (nullptr: evaluate)
   const double *table;
   const int32_t *lat;
@@ -276,22 +394,108 @@ struct AsmArgs {
   int count_only;     // 1: only count near blocks per row into near_fill
 };
 
-// grid (Q, P); TC threads; thread = column j of the chunk, loop over the
-// panel's TR rows i.
+// Block (i, j) into the storage: apart, in FP64, if it is a touching pair of a
+// BF16 precision, else in the tensor's layout and precision.
+__device__ __forceinline__ void store_block(const AsmArgs &A, int64_t i, int64_t j, bool near, const double N6[6]) {
+  if (near) {
+    const int slot = atomicAdd(&A.near_fill[i], 1);
+    const int64_t at = A.near_ptr[i] + slot;
+    A.near_col[at] = (int32_t)j;
+#pragma unroll
+    for (int e = 0; e < 6; ++e) A.near_val[6 * at + e] = N6[e];
+    return;  // dense store keeps zeros there
+  }
+  if (A.dense) {
+    // all 9 entries: row 3i + a, column 3j + b (scales fixed to 1)
+    __nv_bfloat16 *D = (__nv_bfloat16 *)A.data;
+    const size_t plane = (size_t)A.Kp * A.Kp;
+    const int e_of[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const double v = N6[e_of[a][b]];
+        const size_t at = dense_a_index(3 * i + a, 3 * j + b, A.Kp / 64);
+        const __nv_bfloat16 hi = __double2bfloat16(v);
+        D[at] = hi;
+        if (A.prec == MT_BF16_SPLIT) D[plane + at] = __double2bfloat16(v - (double)__bfloat162float(hi));
+      }
+    return;
+  }
+  switch (A.prec) {
+    case MT_F64: {
+      double *D = (double *)A.data;
+#pragma unroll
+      for (int e = 0; e < 6; ++e) D[layout_index(i, j, e, A.TR, A.TC, 6, A.Q)] = N6[e];
+    } break;
+    case MT_F32: {
+      float *D = (float *)A.data;
+#pragma unroll
+      for (int e = 0; e < 6; ++e) {
+        const int pl = stream_plane(e, A.nplane);
+        if (pl >= 0) D[layout_index_h(i, j, pl, A.TR, A.TC, A.nplane, A.Q, A.half)] = (float)N6[e];
+        else if (traceless(A.nplane) && e == 5) {
+          // zz is not stored: the identity that gives it must hold here
+          const double tr = N6[0] + N6[3] + N6[5] - (i == j ? 1.0 : 0.0);
+          if (!(fabs(tr) <= kTraceTol * (fabs(N6[0]) + fabs(N6[3]) + fabs(N6[5])) + kPlanarTol))
+            *A.planar_bad = 1;
+        } else if (!(fabs(N6[e]) <= kPlanarTol)) *A.planar_bad = 1;
+      }
+    } break;
+    case MT_BF16_SCALED: {
+      // power-of-two scale of the block: 2^s with s = exponent of max |N|
+      double mx = 0.0;
+#pragma unroll
+      for (int e = 0; e < 6; ++e) mx = fmax(mx, fabs(N6[e]));
+      int s = 0;
+      if (mx > 0.0) {
+        frexp(mx, &s);
+        s = max(-126, min(126, s));
+      }
+      __nv_bfloat16 *D = (__nv_bfloat16 *)A.data;
+#pragma unroll
+      for (int e = 0; e < 6; ++e) {
+        const int pl = stream_plane(e, A.nplane);
+        if (pl >= 0) D[layout_index(i, j, pl, A.TR, A.TC, A.nplane, A.Q)] = __double2bfloat16(ldexp(N6[e], -s));
+        else if (!(fabs(N6[e]) <= kPlanarTol)) *A.planar_bad = 1;
+      }
+      A.scale[scale_index(i, j, A.TR, A.TC, A.Q)] = (int8_t)s;
+    } break;
+    case MT_BF16_SPLIT: {
+      __nv_bfloat16 *D = (__nv_bfloat16 *)A.data;
+      const int half = A.nplane / 2;  // hi planes, then as many lo planes
+#pragma unroll
+      for (int e = 0; e < 6; ++e) {
+        const int pl = stream_plane(e, half);
+        if (pl < 0) {
+          if (!(fabs(N6[e]) <= kPlanarTol)) *A.planar_bad = 1;
+          continue;
+        }
+        const __nv_bfloat16 hi = __double2bfloat16(N6[e]);
+        const __nv_bfloat16 lo = __double2bfloat16(N6[e] - (double)__bfloat162float(hi));
+        D[layout_index(i, j, pl, A.TR, A.TC, A.nplane, A.Q)] = hi;
+        D[layout_index(i, j, half + pl, A.TR, A.TC, A.nplane, A.Q)] = lo;
+      }
+    } break;
+  }
+}
+
+__device__ __forceinline__ bool kept_apart(const AsmArgs &A, int rel) {
+  return (rel & 2) && (A.prec == MT_BF16_SCALED || A.prec == MT_BF16_SPLIT);
+}
+
+// Cuboids: grid (Q, P); TC threads; thread = column j of the chunk, loop over
+// the panel's TR rows i.
 __global__ void k_assemble(AsmArgs A) {
   const int64_t q = blockIdx.x, p = blockIdx.y;
   const int64_t j = q * A.TC + threadIdx.x;
   if (j >= A.n) return;
-  const bool tet = A.kind == MT_TILE_TETRA;
-  double cj[3], ej[3], vj[12];
+  double cj[3], ej[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     cj[a] = A.centre[3 * j + a];
     ej[a] = A.edge[3 * j + a];
   }
-  if (tet)
-#pragma unroll
-    for (int a = 0; a < 12; ++a) vj[a] = A.vert[12 * j + a];
   for (int r = 0; r < A.TR; ++r) {
     const int64_t i = p * A.TR + r;
     if (i >= A.n) break;
@@ -313,13 +517,13 @@ __global__ void k_assemble(AsmArgs A) {
       rel = (i == j) ? 2 : ((same ? 1 : 0) | (touch ? 2 : 0));
       toff = ((int64_t)(dx + A.Lx - 1) * (2 * A.Ly - 1) + (dy + A.Ly - 1)) * (2 * A.Lz - 1) + (dz + A.Lz - 1);
     } else {
-      rel = (i == j) ? 2 : tet ? tetra_relation(ci, A.vert + 12 * i, vj) : pair_relation(ci, ei, cj, ej);
+      rel = (i == j) ? 2 : pair_relation(ci, ei, cj, ej);
     }
     if (rel & 1) atomicExch(A.bad, 1);
     // half storage: block (i, j) of an omitted chunk is block (j, i), which
     // its own chunk stores (the relation above is still checked for all pairs)
     if (A.half && half_q0(p, A.TC / A.TR) > q) continue;
-    const bool near = (rel & 2) && (A.prec == MT_BF16_SCALED || A.prec == MT_BF16_SPLIT);
+    const bool near = kept_apart(A, rel);
     if (A.count_only) {
       if (near) atomicAdd(&A.near_fill[i], 1);
       continue;
@@ -328,93 +532,60 @@ __global__ void k_assemble(AsmArgs A) {
     if (A.table) {
 #pragma unroll
       for (int e = 0; e < 6; ++e) N6[e] = A.table[6 * toff + e];
-    } else if (tet) {
-      tetra_tensor(ci, vj, N6);
     } else {
       cuboid_tensor(ci, cj, ej, N6);
     }
-    if (near) {
-      const int slot = atomicAdd(&A.near_fill[i], 1);
-      const int64_t at = A.near_ptr[i] + slot;
-      A.near_col[at] = (int32_t)j;
+    store_block(A, i, j, near, N6);
+  }
+}
+
+// Tetrahedra: a block needs the source tile's ~90 doubles of geometry, so the
+// roles are turned round: a CTA stages kTetCols source tiles in shared memory
+// (read by all its threads at once: broadcasts) and thread t takes field
+// point i = kTetRows blockIdx.y + t.
+constexpr int kTetCols = 16, kTetRows = 128;
+__global__ void __launch_bounds__(kTetRows) k_assemble_tetra(AsmArgs A) {
+  __shared__ double sg[kTetCols * kTgSize];
+  const int64_t j0 = blockIdx.x * (int64_t)kTetCols;
+  const int cols = (int)(A.n - j0 < kTetCols ? A.n - j0 : kTetCols);
+  for (int q = threadIdx.x; q < cols * kTgSize; q += kTetRows) sg[q] = A.geo[j0 * kTgSize + q];
+  __syncthreads();
+  const int64_t i = blockIdx.y * (int64_t)kTetRows + threadIdx.x;
+  if (i >= A.n) return;
+  double ci[3];
 #pragma unroll
-      for (int e = 0; e < 6; ++e) A.near_val[6 * at + e] = N6[e];
-      continue;  // dense store keeps zeros there
+  for (int a = 0; a < 3; ++a) ci[a] = A.centre[3 * i + a];
+  const double rad = A.geo[i * kTgSize + kTgRad];
+  for (int k = 0; k < cols; ++k) {
+    const int64_t j = j0 + k;
+    const double *G = sg + k * kTgSize;
+    int rel = 2;
+    if (i != j) {
+      // tiles further apart than their vertices reach from the centroids
+      // neither share a vertex nor hold each other's centroid
+      double d[3];
+      sub3(ci, G + kTgCen, d);
+      const double reach = (rad + G[kTgRad]) * (1.0 + 1e-9);
+      rel = dot3(d, d) > reach * reach ? 0 : tetra_relation(ci, A.vert + 12 * i, G + kTgVert);
     }
-    if (A.dense) {
-      // all 9 entries: row 3i + a, column 3j + b (scales fixed to 1)
-      __nv_bfloat16 *D = (__nv_bfloat16 *)A.data;
-      const size_t plane = (size_t)A.Kp * A.Kp;
-      const int e_of[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-          const double v = N6[e_of[a][b]];
-          const size_t at = dense_a_index(3 * i + a, 3 * j + b, A.Kp / 64);
-          const __nv_bfloat16 hi = __double2bfloat16(v);
-          D[at] = hi;
-          if (A.prec == MT_BF16_SPLIT) D[plane + at] = __double2bfloat16(v - (double)__bfloat162float(hi));
-        }
+    if (rel & 1) atomicExch(A.bad, 1);
+    const bool near = kept_apart(A, rel);
+    if (A.count_only) {
+      if (near) atomicAdd(&A.near_fill[i], 1);
       continue;
     }
-    switch (A.prec) {
-      case MT_F64: {
-        double *D = (double *)A.data;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) D[layout_index(i, j, e, A.TR, A.TC, 6, A.Q)] = N6[e];
-      } break;
-      case MT_F32: {
-        float *D = (float *)A.data;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-          const int pl = stream_plane(e, A.nplane);
-          if (pl >= 0) D[layout_index_h(i, j, pl, A.TR, A.TC, A.nplane, A.Q, A.half)] = (float)N6[e];
-          else if (traceless(A.nplane) && e == 5) {
-            // zz is not stored: the identity that gives it must hold here
-            const double tr = N6[0] + N6[3] + N6[5] - (i == j ? 1.0 : 0.0);
-            if (!(fabs(tr) <= kTraceTol * (fabs(N6[0]) + fabs(N6[3]) + fabs(N6[5])) + kPlanarTol))
-              *A.planar_bad = 1;
-          } else if (!(fabs(N6[e]) <= kPlanarTol)) *A.planar_bad = 1;
-        }
-      } break;
-      case MT_BF16_SCALED: {
-        // power-of-two scale of the block: 2^s with s = exponent of max |N|
-        double mx = 0.0;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) mx = fmax(mx, fabs(N6[e]));
-        int s = 0;
-        if (mx > 0.0) {
-          frexp(mx, &s);
-          s = max(-126, min(126, s));
-        }
-        __nv_bfloat16 *D = (__nv_bfloat16 *)A.data;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-          const int pl = stream_plane(e, A.nplane);
-          if (pl >= 0) D[layout_index(i, j, pl, A.TR, A.TC, A.nplane, A.Q)] = __double2bfloat16(ldexp(N6[e], -s));
-          else if (!(fabs(N6[e]) <= kPlanarTol)) *A.planar_bad = 1;
-        }
-        A.scale[scale_index(i, j, A.TR, A.TC, A.Q)] = (int8_t)s;
-      } break;
-      case MT_BF16_SPLIT: {
-        __nv_bfloat16 *D = (__nv_bfloat16 *)A.data;
-#pragma unroll
-        const int half = A.nplane / 2;  // hi planes, then as many lo planes
-        for (int e = 0; e < 6; ++e) {
-          const int pl = stream_plane(e, half);
-          if (pl < 0) {
-            if (!(fabs(N6[e]) <= kPlanarTol)) *A.planar_bad = 1;
-            continue;
-          }
-          const __nv_bfloat16 hi = __double2bfloat16(N6[e]);
-          const __nv_bfloat16 lo = __double2bfloat16(N6[e] - (double)__bfloat162float(hi));
-          D[layout_index(i, j, pl, A.TR, A.TC, A.nplane, A.Q)] = hi;
-          D[layout_index(i, j, half + pl, A.TR, A.TC, A.nplane, A.Q)] = lo;
-        }
-      } break;
-    }
+    double N6[6];
+    tetra_tensor(ci, G, N6);
+    store_block(A, i, j, near, N6);
   }
+}
+
+void launch_assemble(const AsmArgs &A, const mt_layout &L) {
+  if (A.geo)
+    k_assemble_tetra<<<dim3((unsigned)((A.n + kTetCols - 1) / kTetCols), (unsigned)((A.n + kTetRows - 1) / kTetRows)),
+                       kTetRows>>>(A);
+  else
+    k_assemble<<<dim3((unsigned)L.Q, (unsigned)L.P), L.TC>>>(A);
 }
 
 // sort each row's near blocks by column so that the FP64 near sum has a
@@ -455,9 +626,11 @@ __global__ void k_blocks(const double *centre, const double *edge, const double 
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= count) return;
   const int64_t i = pairs[2 * p], j = pairs[2 * p + 1];
-  if (kind == MT_TILE_TETRA)
-    tetra_tensor(&centre[3 * i], &vert[12 * j], &out[6 * p]);
-  else
+  if (kind == MT_TILE_TETRA) {
+    double G[kTgSize];
+    tetra_geom(&centre[3 * j], &vert[12 * j], G);
+    tetra_tensor(&centre[3 * i], G, &out[6 * p]);
+  } else
     cuboid_tensor(&centre[3 * i], &centre[3 * j], &edge[3 * j], &out[6 * p]);
 }
 
@@ -547,7 +720,6 @@ mt_status assemble(mt_tensor *T) {
   A.centre = t->d_centre;
   A.edge = t->d_edge;
   A.vert = t->d_vert;
-  A.kind = t->kind;
   A.n = n;
   A.TR = L.TR;
   A.TC = L.TC;
@@ -576,8 +748,14 @@ mt_status assemble(mt_tensor *T) {
     A.Ly = t->Ly;
     A.Lz = t->Lz;
   }
+  DevTemp<double> geo;
+  if (t->kind == MT_TILE_TETRA) {
+    MT_CUDA(geo.alloc((size_t)kTgSize * n));
+    k_tetra_geom<<<(unsigned)((n + 127) / 128), 128>>>(n, t->d_centre, t->d_vert, geo.p);
+    MT_CUDA(cudaGetLastError());
+    A.geo = geo.p;
+  }
   const bool has_near = (T->prec == MT_BF16_SCALED || T->prec == MT_BF16_SPLIT);
-  dim3 grid((unsigned)L.Q, (unsigned)L.P);
   if (has_near) {
     DevTemp<int> fill;
     MT_CUDA(fill.alloc(n));
@@ -585,7 +763,7 @@ mt_status assemble(mt_tensor *T) {
     MT_CUDA(cudaMemset(d_fill, 0, sizeof(int) * n));
     A.near_fill = d_fill;
     A.count_only = 1;
-    k_assemble<<<grid, L.TC>>>(A);
+    launch_assemble(A, L);
     MT_CUDA(cudaGetLastError());
     std::vector<int> cnt(n);
     MT_CUDA(cudaMemcpy(cnt.data(), d_fill, sizeof(int) * n, cudaMemcpyDeviceToHost));
@@ -601,7 +779,7 @@ mt_status assemble(mt_tensor *T) {
     A.near_col = T->d_near_col;
     A.near_val = T->d_near_val;
     A.count_only = 0;
-    k_assemble<<<grid, L.TC>>>(A);
+    launch_assemble(A, L);
     MT_CUDA(cudaGetLastError());
     k_sort_near<<<(unsigned)((n + 127) / 128), 128>>>(n, T->d_near_ptr, T->d_near_col, T->d_near_val);
     MT_CUDA(cudaGetLastError());
@@ -614,7 +792,7 @@ mt_status assemble(mt_tensor *T) {
     }
     MT_CUDA(cudaDeviceSynchronize());
   } else {
-    k_assemble<<<grid, L.TC>>>(A);
+    launch_assemble(A, L);
     MT_CUDA(cudaGetLastError());
     MT_CUDA(cudaDeviceSynchronize());
   }
@@ -650,7 +828,7 @@ mt_status assemble(mt_tensor *T) {
     A.TC = T->L.TC;
     A.nplane = T->L.nplane;
     A.Q = T->L.Q;
-    k_assemble<<<dim3((unsigned)T->L.Q, (unsigned)T->L.P), T->L.TC>>>(A);
+    launch_assemble(A, T->L);
     MT_CUDA(cudaGetLastError());
     MT_CUDA(cudaDeviceSynchronize());
   }
