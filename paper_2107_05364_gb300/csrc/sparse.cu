@@ -10,7 +10,7 @@
 // entry's two copies adjacent; the first k = floor(f * nonzeros) are dropped,
 // except that an entry whose two copies the cut splits stays (blocks stay
 // symmetric).  The magnitude t of the element of rank k is found exactly by
-// a two-pass radix select on the FP32 bit patterns (non-negative floats order
+// a three-pass radix select on the FP32 bit patterns (non-negative floats order
 // like their bits); every element below t goes, and of the elements equal
 // to t the first r = k - #(below t) in that order.
 //
@@ -39,6 +39,7 @@
 // the FP32 storage error.
 #include <algorithm>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "mt_internal.cuh"
@@ -48,60 +49,165 @@ namespace {
 __device__ __forceinline__ uint32_t abs_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 __device__ __forceinline__ float f4_at(const float4 &v, int q) { return q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w; }
 
-// entries of the streaming FP32 layout belonging to real tiles, with their
-// multiplicity in the full matrix (diagonal 1, off-diagonal 2)
-template <typename F>
-__device__ __forceinline__ void for_each_entry(const float *D, int64_t n, int TR, int TC, int np, int64_t Q,
-                                               int64_t blk, F &&f) {
-  // blk enumerates (p, q, r, c) chunk positions; the 6 entries of the block
-  // (np planes stored: 6, or 4 for a single-layer tensor without xz, yz)
-  const int64_t per_chunk = (int64_t)TR * TC;
-  const int64_t chunk = blk / per_chunk, rc = blk - chunk * per_chunk;
-  const int64_t p = chunk / Q, q = chunk - p * Q;
-  const int r = (int)(rc / TC), c = (int)(rc - (int64_t)(rc / TC) * TC);
-  const int64_t i = p * TR + r, j = q * TC + c;
-  if (i >= n || j >= n) return;
-  const float *base = D + chunk * np * per_chunk + (int64_t)r * TC + c;
-  const int mult[6] = {1, 2, 2, 1, 2, 1};
+// Multiplicity of a stored plane's entry in the full matrix: an off-diagonal
+// entry of a symmetric block stands for two elements (planes xx xy xz yy yz
+// zz, or xx xy yy zz of a single-layer tensor).
+template <int NP>
+__device__ __forceinline__ constexpr int plane_mult(int pl) {
+  return NP == 6 ? ((pl == 0 || pl == 3 || pl == 5) ? 1 : 2) : (pl == 1 ? 2 : 1);
+}
+
+// Radix select of the element of rank k, on the device: three passes over the
+// 31 magnitude bits (11, 10, 10), each a histogram of the elements whose
+// higher bits match the selection so far, then one block that finds the bin.
+struct Select {
+  unsigned long long nz;    // nonzero elements of the full matrix
+  unsigned long long rest;  // rank within the selected prefix; at the end the copies of t to drop
+  unsigned int prefix;      // selected high bits; at the end the bits of t
+  int active;               // 0: nothing to drop (t = 0)
+  unsigned long long kept;  // nonzero elements kept (k_rows)
+};
+__host__ __device__ constexpr int sel_shift(int pass) { return 20 - 10 * pass; }
+__host__ __device__ constexpr int sel_bins(int pass) { return pass == 0 ? 2048 : 1024; }
+constexpr int kHistCopies = 8, kHistThreads = 1024;
+constexpr size_t kHistSmem = (size_t)kHistCopies * 2 * 2048 * sizeof(unsigned int);
+
+// Adjacent tiles' entries have adjacent magnitudes, so a warp's atomics
+// collide: they go to shared memory, a copy of the histogram per 4 warps, as
+// plain increments (colliding lanes of an increment are counted together in
+// hardware), off-diagonal entries to a second histogram that counts double at
+// the end.  Global 64-bit atomics on 65,536 bins took 6.5 ms at n = 6,400
+// (single layer), a pass of this 0.14-0.16 (0.097: its 655 MB at copy rate).
+template <int NP>
+__global__ void __launch_bounds__(kHistThreads) k_hist(const float *D, int64_t n, int TR, int TC, int64_t Q,
+                                                       int64_t P, int pass, const Select *sel,
+                                                       unsigned long long *hist) {
+  extern __shared__ unsigned int sh[];  // [copy][2][bins]
+  if (pass > 0 && !sel->active) return;
+  const int bins = sel_bins(pass), shift = sel_shift(pass);
+  const uint32_t prefix = pass > 0 ? sel->prefix : 0;
+  for (int q = threadIdx.x; q < kHistCopies * 2 * bins; q += kHistThreads) sh[q] = 0;
+  __syncthreads();
+  unsigned int *mine = sh + (threadIdx.x >> 5) % kHistCopies * 2 * bins;
+  // positions: 4 adjacent columns of one row of one chunk
+  const int64_t c4 = TC / 4, per = TR * c4, plane = (int64_t)TR * TC, tot = P * Q * per;
+  for (int64_t t = blockIdx.x * (int64_t)kHistThreads + threadIdx.x; t < tot; t += (int64_t)gridDim.x * kHistThreads) {
+    const int64_t chunk = t / per, rc = t - chunk * per;
+    const int64_t p = chunk / Q, q = chunk - p * Q;
+    const int r = (int)(rc / c4), c = 4 * (int)(rc - (int64_t)r * c4);
+    if (p * TR + r >= n) continue;
+    const int64_t j = q * TC + c;
+    const float *base = D + chunk * NP * plane + (int64_t)r * TC + c;
+    float4 v[NP];
 #pragma unroll
-  for (int e = 0; e < 6; ++e) {
-    const int pl = stream_plane(e, np);
-    f(i, j, e, pl < 0 ? 0.0f : base[pl * per_chunk], mult[e]);
+    for (int pl = 0; pl < NP; ++pl) v[pl] = __ldcs(reinterpret_cast<const float4 *>(base + pl * plane));
+#pragma unroll
+    for (int pl = 0; pl < NP; ++pl)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t bits = abs_bits(f4_at(v[pl], u));
+        if (bits == 0 || j + u >= n) continue;
+        if (pass > 0 && (bits >> (shift + 10)) != prefix) continue;
+        atomicAdd(&mine[(plane_mult<NP>(pl) - 1) * bins + ((bits >> shift) & (bins - 1))], 1u);
+      }
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < bins; q += kHistThreads) {
+    unsigned long long h = 0;
+    for (int k = 0; k < kHistCopies; ++k)
+      h += (unsigned long long)sh[k * 2 * bins + q] + 2ull * sh[(k * 2 + 1) * bins + q];
+    if (h) atomicAdd(&hist[q], h);
   }
 }
 
-__global__ void k_hist(const float *D, int64_t n, int TR, int TC, int np, int64_t Q, int64_t nblk, int pass,
-                       uint32_t hi, unsigned long long *hist) {
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblk; b += (int64_t)gridDim.x * blockDim.x)
-    for_each_entry(D, n, TR, TC, np, Q, b, [&](int64_t, int64_t, int, float v, int mult) {
-      const uint32_t bits = abs_bits(v);
-      if (bits == 0) return;
-      if (pass == 0) atomicAdd(&hist[bits >> 16], (unsigned long long)mult);
-      else if ((bits >> 16) == hi) atomicAdd(&hist[bits & 0xffffu], (unsigned long long)mult);
-    });
+// inclusive sum over the block of 1,024 threads
+__device__ __forceinline__ unsigned long long block_scan(unsigned long long v, unsigned long long *sh) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  if (lane == 31) sh[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    unsigned long long x = sh[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    sh[lane] = x;
+  }
+  __syncthreads();
+  if (w > 0) v += sh[w - 1];
+  __syncthreads();
+  return v;
 }
 
-// copies of the cut value t in row tile i (counted for the tie order)
-__global__ void k_row_ties(const float *D, int64_t n, int TR, int TC, int np, int64_t Q, uint32_t tbits,
+// one block: the bin holding rank `rest` (pass 0: the number of elements and
+// the rank k = floor(fraction nz) first); clears the histogram for the next
+// pass
+__global__ void __launch_bounds__(1024) k_select(int pass, double fraction, unsigned long long *hist, Select *sel) {
+  __shared__ unsigned long long sh[32], s_rest;
+  __shared__ int s_active;
+  const int t = threadIdx.x;
+  // two adjacent bins per thread
+  const unsigned long long h0 = hist[2 * t], h1 = hist[2 * t + 1];
+  hist[2 * t] = hist[2 * t + 1] = 0;
+  const unsigned long long incl = block_scan(h0 + h1, sh);
+  if (pass == 0) {
+    if (t == 1023) {
+      sel->nz = incl;
+      s_rest = (unsigned long long)(fraction * (double)incl);
+      s_active = incl > 0 && s_rest > 0;
+      sel->active = s_active;
+      if (!s_active) {
+        sel->prefix = 0;
+        sel->rest = 0;
+      }
+    }
+  } else if (t == 0) {
+    s_rest = sel->rest;
+    s_active = sel->active;
+  }
+  __syncthreads();
+  if (!s_active) return;
+  const unsigned long long k = s_rest, ex = incl - (h0 + h1);
+  if (ex <= k && k < incl) {  // exactly one thread
+    const int second = ex + h0 <= k ? 1 : 0;
+    const unsigned int bin = 2 * t + second;
+    sel->rest = k - ex - (second ? h0 : 0);
+    sel->prefix = pass == 0 ? bin : (sel->prefix << 10) | bin;
+  }
+}
+
+// copies of the cut value t in row tile i (counted for the tie order; not
+// needed when none of them is dropped)
+template <int NP>
+__global__ void k_row_ties(const float *D, int64_t n, int TR, int TC, int64_t Q, const Select *sel,
                            unsigned long long *ties) {
   const int64_t i = blockIdx.x;
-  const int64_t p = i / TR;
-  const int r = (int)(i - p * TR);
-  unsigned long long local = 0;
-  const int mult[6] = {1, 2, 2, 1, 2, 1};
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-    const int64_t q = j / TC;
-    const int c = (int)(j - q * TC);
-    const float *base = D + (p * Q + q) * np * (int64_t)TR * TC + (int64_t)r * TC + c;
+  const uint32_t tbits = sel->prefix;
+  unsigned int local = 0;
+  if (sel->rest > 0) {
+    const int64_t p = i / TR, plane = (int64_t)TR * TC;
+    const int r = (int)(i - p * TR);
+    for (int64_t j = 4 * (int64_t)threadIdx.x; j < n; j += 4 * blockDim.x) {
+      const int64_t q = j / TC;
+      const float *base = D + (p * Q + q) * NP * plane + (int64_t)r * TC + (j - q * TC);
 #pragma unroll
-    for (int e = 0; e < 6; ++e) {
-      const int pl = stream_plane(e, np);
-      if (pl >= 0) local += abs_bits(base[pl * (int64_t)TR * TC]) == tbits ? mult[e] : 0;
+      for (int pl = 0; pl < NP; ++pl) {
+        const float4 v = __ldcs(reinterpret_cast<const float4 *>(base + pl * plane));
+#pragma unroll
+        for (int u = 0; u < 4; ++u)  // the padding past column n is zero, t is not
+          local += abs_bits(f4_at(v, u)) == tbits ? plane_mult<NP>(pl) : 0;
+      }
     }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) local += __shfl_xor_sync(0xffffffffu, local, off);
-  __shared__ unsigned long long sh[32];
+  __shared__ unsigned int sh[32];
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = local;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -111,104 +217,154 @@ __global__ void k_row_ties(const float *D, int64_t n, int TR, int TC, int np, in
   }
 }
 
+// one block: out[i] = sum of in[0 .. i - 1], i = 0 .. n (in place allowed for
+// 64-bit counts)
+template <typename In, typename Out>
+__global__ void __launch_bounds__(1024) k_scan(const In *in, int64_t n, Out *out) {
+  __shared__ unsigned long long sh[32];
+  unsigned long long carry = 0;
+  for (int64_t i0 = 0; i0 < n; i0 += 1024) {
+    const int64_t i = i0 + threadIdx.x;
+    const unsigned long long v = i < n ? (unsigned long long)in[i] : 0;
+    const unsigned long long incl = block_scan(v, sh);
+    if (i < n) out[i] = (Out)(carry + incl - v);
+    __shared__ unsigned long long s_tot;
+    if (threadIdx.x == 1023) s_tot = incl;
+    __syncthreads();
+    carry += s_tot;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) out[n] = (Out)carry;
+}
+
 // a later kept column joins the run when it lies at most this far past the
 // run's last kept column (the columns between are stored as zero blocks)
 constexpr int kRunJoin = 4;
 
-// Row tile i in increasing column order, one warp per row, 32 columns per
-// step.  An entry is kept if |v| > t, or if |v| == t and the copies of t up
-// to and including it (counted from tie_start[i], in column and entry order)
-// exceed r.  The kept columns are grouped into runs (see the storage note);
-// every lane walks the step's kept columns in order, so the run state is
-// the same in all lanes.  FILL = false: the row's stored blocks (runs padded
-// to 4) into cnt[i] and its runs into nrun[i]; FILL = true: each kept block
-// at its slot and each run's (first block, first column) pair (the value
-// planes were zeroed before).  With t = 0 every nonzero entry is kept.
-template <bool FILL>
-__global__ void k_rows(const float *D, int64_t n, int TR, int TC, int np, int64_t Q, uint32_t tbits,
-                       const unsigned long long *tie_start, unsigned long long r, int *cnt, int *nrun,
-                       const int64_t *ptr, const int64_t *rptr, int32_t *run, float *val) {
-  const int64_t i = blockIdx.x;
-  const int lane = threadIdx.x;
-  const int64_t p = i / TR;
+// Row tile i in increasing column order, one warp per row, a chunk of 128
+// columns per step as 4 words of 32 (lane = column), the next step's values
+// loaded ahead.  An entry is kept if |v| > t, or if |v| == t and the copies
+// of t up to and including it (counted from tie_start[i], in column and entry
+// order) exceed r.  The kept columns are grouped into runs (see the storage
+// note) from the word's ballot: the run state is the same in all lanes, and
+// only the starts of new runs are walked one by one.  FILL = false: the row's
+// stored blocks (runs padded to 4) into cnt[i], its runs into nrun[i], the
+// kept elements of the full matrix added to sel->kept; FILL = true: each kept
+// block at its slot and each run's (first block, first column) pair (the
+// value planes were zeroed before).  With t = 0 every nonzero entry is kept.
+// One 32-column word per step, walking every kept column, took 1.3 (count)
+// and 1.5 ms (fill) at n = 6,400 (single layer, 40 % dropped); this 0.17 and
+// 0.27 (0.10 and 0.16: the tensor read, the kept blocks written).
+constexpr int kRowsPerCta = 4;
+template <int NP, bool FILL>
+__global__ void __launch_bounds__(32 * kRowsPerCta) k_rows(const float *D, int64_t n, int TR, int TC, int64_t Q,
+                                                           const unsigned long long *tie_start, Select *sel, int *cnt,
+                                                           int *nrun, const int64_t *ptr, const int64_t *rptr,
+                                                           int32_t *run, float *val) {
+  const int64_t i = blockIdx.x * (int64_t)kRowsPerCta + (threadIdx.x >> 5);
+  if (i >= n) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t p = i / TR, plane = (int64_t)TR * TC;
   const int rr = (int)(i - p * TR);
-  const int mult[6] = {1, 2, 2, 1, 2, 1};
+  const uint32_t tbits = sel->prefix;
+  const unsigned long long r = sel->rest;
   const int64_t o = FILL ? ptr[i] : 0, K4 = FILL ? ptr[i + 1] - o : 0;
-  float *rv = FILL ? val + np * o : nullptr;  // np value planes, as the source
+  float *rv = FILL ? val + NP * o : nullptr;  // NP value planes, as the source
   int32_t *rd = FILL ? run + 2 * rptr[i] : nullptr;
-  unsigned long long carry = tie_start ? tie_start[i] : 0;
+  unsigned long long carry = r > 0 ? tie_start[i] : 0;
   // run state: stored blocks before the open run, its first and last column
   int64_t ofs = 0, col0 = -1, last = -1;
   int64_t runs = 0;
-  for (int64_t j0 = 0; j0 < n; j0 += 32) {
-    const int64_t j = j0 + lane;
-    float v[6] = {0, 0, 0, 0, 0, 0};
-    uint32_t bits[6] = {0, 0, 0, 0, 0, 0};
-    unsigned tm = 0;  // copies of t in this lane's block
-    if (j < n) {
-      const int64_t q = j / TC;
-      const int c = (int)(j - q * TC);
-      const float *base = D + (p * Q + q) * np * (int64_t)TR * TC + (int64_t)rr * TC + c;
+  unsigned int kept = 0;
+  const float *row = D + p * Q * NP * plane + (int64_t)rr * TC + lane;
+  float nx[4][NP];
+  auto load = [&](int64_t q) {
+    const float *base = row + q * NP * plane;
 #pragma unroll
-      for (int e = 0; e < 6; ++e) {
-        const int pl = stream_plane(e, np);
-        v[e] = pl < 0 ? 0.0f : base[pl * (int64_t)TR * TC];
-        bits[e] = abs_bits(v[e]);
-        tm += (bits[e] != 0 && bits[e] == tbits) ? mult[e] : 0;
+    for (int w = 0; w < 4; ++w)
+#pragma unroll
+      for (int e = 0; e < NP; ++e) nx[w][e] = q * 128 + 32 * w + lane < n ? __ldcs(base + e * plane + 32 * w) : 0.0f;
+  };
+  load(0);
+  for (int64_t q = 0; q < Q; ++q) {
+    float v[4][NP];
+#pragma unroll
+    for (int w = 0; w < 4; ++w)
+#pragma unroll
+      for (int e = 0; e < NP; ++e) v[w][e] = nx[w][e];
+    if (q + 1 < Q) load(q + 1);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int64_t j0 = q * 128 + 32 * w;
+      unsigned tm = 0;  // copies of t in this lane's block
+#pragma unroll
+      for (int e = 0; e < NP; ++e) {
+        const uint32_t bits = abs_bits(v[w][e]);
+        tm += (bits != 0 && bits == tbits) ? plane_mult<NP>(e) : 0;
       }
-    }
-    // inclusive scan of tm over the lanes (columns in order)
-    unsigned incl = tm;
+      unsigned long long cum = carry;
+      if (__any_sync(0xffffffffu, tm != 0)) {
+        // inclusive scan of tm over the lanes (columns in order)
+        unsigned incl = tm;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const unsigned y = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += y;
-    }
-    unsigned long long cum = carry + (incl - tm);
-    bool keep = false;
-#pragma unroll
-    for (int e = 0; e < 6; ++e) {
-      bool k = bits[e] != 0 && bits[e] > tbits;
-      if (bits[e] != 0 && bits[e] == tbits) {
-        cum += mult[e];
-        k = cum > r;
+        for (int off = 1; off < 32; off <<= 1) {
+          const unsigned y = __shfl_up_sync(0xffffffffu, incl, off);
+          if (lane >= off) incl += y;
+        }
+        cum += incl - tm;
+        carry += __shfl_sync(0xffffffffu, incl, 31);
       }
-      if (!k) v[e] = 0.0f;
-      keep = keep || k;
-    }
-    carry += __shfl_sync(0xffffffffu, incl, 31);
-    // runs: the kept columns of this step in order (the mask is the same in
-    // every lane, so is the walk)
-    unsigned mk = __ballot_sync(0xffffffffu, keep);
-    int64_t slot = -1;
-    while (mk) {
-      const int l = __ffs(mk) - 1;
-      mk &= mk - 1;
-      const int64_t jk = j0 + l;
-      if (col0 < 0 || jk - last > kRunJoin) {  // a new run
-        if (col0 >= 0) ofs += (last - col0 + 4) & ~(int64_t)3;  // close the open one, padded to 4
-        col0 = jk;
+      bool keep = false;
+#pragma unroll
+      for (int e = 0; e < NP; ++e) {
+        const uint32_t bits = abs_bits(v[w][e]);
+        bool k = bits != 0 && bits > tbits;
+        if (bits != 0 && bits == tbits) {
+          cum += plane_mult<NP>(e);
+          k = cum > r;
+        }
+        if (!k) v[w][e] = 0.0f;
+        keep = keep || k;
+        if (!FILL) kept += k ? plane_mult<NP>(e) : 0;
+      }
+      const unsigned mk = __ballot_sync(0xffffffffu, keep);
+      if (mk == 0) continue;
+      // a kept column starts a run when none of the kRunJoin columns before
+      // it is kept (in this word, or in earlier ones through `last`)
+      unsigned starts = mk & ~(mk << 1) & ~(mk << 2) & ~(mk << 3) & ~(mk << 4);
+      const int first = __ffs(mk) - 1;
+      if (col0 >= 0 && j0 + first - last <= kRunJoin) starts &= ~(1u << first);
+      int64_t shift = ofs - col0;  // slot of column j of the open run: shift + j
+      while (starts) {
+        const int sc = __ffs(starts) - 1;
+        starts &= starts - 1;
+        const unsigned below = mk & ((1u << sc) - 1u);
+        if (below) last = j0 + 31 - __clz(below);
+        if (col0 >= 0) ofs += (last - col0 + 4) & ~(int64_t)3;  // close the open run, padded to 4
+        col0 = j0 + sc;
         if (FILL && lane == 0) {
           rd[2 * runs] = (int32_t)ofs;
-          rd[2 * runs + 1] = (int32_t)jk;
+          rd[2 * runs + 1] = (int32_t)col0;
         }
         ++runs;
+        if (lane >= sc) shift = ofs - col0;
       }
-      if (l == lane) slot = ofs + (jk - col0);
-      last = jk;
-    }
-    if (FILL && keep) {
+      last = j0 + 31 - __clz(mk);
+      if (FILL && keep) {
 #pragma unroll
-      for (int e = 0; e < 6; ++e) {
-        const int pl = stream_plane(e, np);
-        if (pl >= 0) rv[pl * K4 + slot] = v[e];
+        for (int e = 0; e < NP; ++e) rv[e * K4 + shift + j0 + lane] = v[w][e];
       }
     }
   }
   if (col0 >= 0) ofs += (last - col0 + 4) & ~(int64_t)3;
-  if (!FILL && lane == 0) {
-    cnt[i] = (int)ofs;
-    nrun[i] = (int)runs;
+  if (!FILL) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, off);
+    if (lane == 0) {
+      cnt[i] = (int)ofs;
+      nrun[i] = (int)runs;
+      atomicAdd(&sel->kept, (unsigned long long)kept);
+    }
   }
 }
 
@@ -400,22 +556,6 @@ int sparse_split(int64_t n, int64_t nnzb, int sms) {
   return S;
 }
 
-// position of rank k in a 65536-bin histogram: bin and rank within it
-void select_bin(const std::vector<unsigned long long> &h, unsigned long long k, uint32_t *bin,
-                unsigned long long *rest) {
-  unsigned long long cum = 0;
-  for (uint32_t b = 0; b < h.size(); ++b) {
-    if (cum + h[b] > k) {
-      *bin = b;
-      *rest = k - cum;
-      return;
-    }
-    cum += h[b];
-  }
-  *bin = (uint32_t)h.size() - 1;
-  *rest = 0;
-}
-
 }  // namespace
 
 namespace mt {
@@ -466,72 +606,42 @@ extern "C" mt_status mt_tensor_threshold(mt_tensor *T, double fraction, mt_tenso
   const int64_t n = T->n;
   const mt_layout &L = T->L;
   const float *D = reinterpret_cast<const float *>(T->d_data);
-  const int64_t nblk = L.P * L.Q * (int64_t)L.TR * L.TC;
-  DevTemp<unsigned long long> hist;
-  MT_CUDA(hist.alloc(65536));
-  unsigned long long *d_hist = hist.p;
-  std::vector<unsigned long long> h(65536);
-  const int grid = 4 * T->tiles->ctx->num_sms;
-  // pass 1: top 16 bits
-  MT_CUDA(cudaMemset(d_hist, 0, sizeof(unsigned long long) * 65536));
-  k_hist<<<grid, 256>>>(D, n, L.TR, L.TC, L.nplane, L.Q, nblk, 0, 0, d_hist);
-  MT_CUDA(cudaGetLastError());
-  MT_CUDA(cudaMemcpy(h.data(), d_hist, sizeof(unsigned long long) * 65536, cudaMemcpyDeviceToHost));
-  unsigned long long nz = 0;
-  for (auto x : h) nz += x;
-  const unsigned long long k = (unsigned long long)(fraction * (double)nz);
-  uint32_t tbits = 0;
-  unsigned long long r = 0;  // copies of t to drop (the first r in tie order)
-  if (k > 0 && nz > 0) {
-    uint32_t b1 = 0;
-    unsigned long long rest = 0;
-    select_bin(h, k, &b1, &rest);
-    // pass 2: low 16 bits inside bin b1
-    MT_CUDA(cudaMemset(d_hist, 0, sizeof(unsigned long long) * 65536));
-    k_hist<<<grid, 256>>>(D, n, L.TR, L.TC, L.nplane, L.Q, nblk, 1, b1, d_hist);
-    MT_CUDA(cudaGetLastError());
-    MT_CUDA(cudaMemcpy(h.data(), d_hist, sizeof(unsigned long long) * 65536, cudaMemcpyDeviceToHost));
-    uint32_t b2 = 0;
-    unsigned long long rest2 = 0;
-    select_bin(h, rest, &b2, &rest2);
-    tbits = (b1 << 16) | b2;
-    r = rest2;
-  }
-  // tie order: copies of t before each row tile
-  DevTemp<unsigned long long> tie_start;
-  unsigned long long *d_tie = nullptr;
-  if (r > 0) {
-    MT_CUDA(tie_start.alloc(n));
-    d_tie = tie_start.p;
-    k_row_ties<<<(unsigned)n, 256>>>(D, n, L.TR, L.TC, L.nplane, L.Q, tbits, d_tie);
-    MT_CUDA(cudaGetLastError());
-    std::vector<unsigned long long> ties(n);
-    MT_CUDA(cudaMemcpy(ties.data(), d_tie, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost));
-    unsigned long long acc = 0;
-    for (int64_t i = 0; i < n; ++i) {
-      const unsigned long long c = ties[i];
-      ties[i] = acc;
-      acc += c;
-    }
-    MT_CUDA(cudaMemcpy(d_tie, ties.data(), sizeof(unsigned long long) * n, cudaMemcpyHostToDevice));
-  }
-  // stored blocks and runs per row
+  const int np = L.nplane;  // value planes: those the source stores (6, or 4 for a single layer)
+  MT_CHECK(L.TC == 128 && (np == 6 || np == 4), MT_EINVAL, "mt_tensor_threshold: unexpected storage");
+  // everything up to the sizes of the new arrays is decided on the device
+  DevTemp<Select> sel;
+  DevTemp<unsigned long long> hist, tie_start;
   DevTemp<int> cnt_rows, run_rows;
+  DevTemp<int64_t> row_ptr, row_rptr;
+  MT_CUDA(sel.alloc(1));
+  MT_CUDA(hist.alloc(sel_bins(0)));
+  MT_CUDA(tie_start.alloc(n + 1));
   MT_CUDA(cnt_rows.alloc(n));
   MT_CUDA(run_rows.alloc(n));
-  int *d_cnt = cnt_rows.p, *d_nrun = run_rows.p;
-  k_rows<false><<<(unsigned)n, 32>>>(D, n, L.TR, L.TC, L.nplane, L.Q, tbits, d_tie, r, d_cnt, d_nrun, nullptr,
-                                     nullptr, nullptr, nullptr);
-  MT_CUDA(cudaGetLastError());
-  std::vector<int> cnt(n), nrun(n);
-  MT_CUDA(cudaMemcpy(cnt.data(), d_cnt, sizeof(int) * n, cudaMemcpyDeviceToHost));
-  MT_CUDA(cudaMemcpy(nrun.data(), d_nrun, sizeof(int) * n, cudaMemcpyDeviceToHost));
-  std::vector<int64_t> ptr(n + 1, 0), rptr(n + 1, 0);
-  for (int64_t i = 0; i < n; ++i) {
-    ptr[i + 1] = ptr[i] + cnt[i];  // runs are padded to 4 blocks already
-    rptr[i + 1] = rptr[i] + nrun[i];
+  MT_CUDA(row_ptr.alloc(n + 1));
+  MT_CUDA(row_rptr.alloc(n + 1));
+  MT_CUDA(cudaMemset(sel.p, 0, sizeof(Select)));
+  MT_CUDA(cudaMemset(hist.p, 0, sizeof(unsigned long long) * sel_bins(0)));
+  const auto hist_k = np == 6 ? k_hist<6> : k_hist<4>;
+  MT_CUDA(cudaFuncSetAttribute(hist_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHistSmem));
+  const int sms = T->tiles->ctx->num_sms;
+  for (int pass = 0; pass < 3; ++pass) {
+    hist_k<<<sms, kHistThreads, kHistSmem>>>(D, n, L.TR, L.TC, L.Q, L.P, pass, sel.p, hist.p);
+    k_select<<<1, 1024>>>(pass, fraction, hist.p, sel.p);
   }
-  const int64_t nnzb = ptr[n], nruns = rptr[n];
+  (np == 6 ? k_row_ties<6> : k_row_ties<4>)<<<(unsigned)n, 256>>>(D, n, L.TR, L.TC, L.Q, sel.p, tie_start.p);
+  k_scan<<<1, 1024>>>(tie_start.p, n, tie_start.p);
+  const unsigned row_grid = (unsigned)((n + kRowsPerCta - 1) / kRowsPerCta);
+  (np == 6 ? k_rows<6, false> : k_rows<4, false>)<<<row_grid, 32 * kRowsPerCta>>>(
+      D, n, L.TR, L.TC, L.Q, tie_start.p, sel.p, cnt_rows.p, run_rows.p, nullptr, nullptr, nullptr, nullptr);
+  k_scan<<<1, 1024>>>(cnt_rows.p, n, row_ptr.p);  // runs are padded to 4 blocks already
+  k_scan<<<1, 1024>>>(run_rows.p, n, row_rptr.p);
+  MT_CUDA(cudaGetLastError());
+  Select hs;
+  int64_t nnzb = 0, nruns = 0;
+  MT_CUDA(cudaMemcpy(&hs, sel.p, sizeof(Select), cudaMemcpyDeviceToHost));
+  MT_CUDA(cudaMemcpy(&nnzb, row_ptr.p + n, sizeof(int64_t), cudaMemcpyDeviceToHost));
+  MT_CUDA(cudaMemcpy(&nruns, row_rptr.p + n, sizeof(int64_t), cudaMemcpyDeviceToHost));
   mt_ctx *ctx = T->tiles->ctx;
   mt_tensor *S = new mt_tensor();
   S->tiles = T->tiles;
@@ -543,7 +653,6 @@ extern "C" mt_status mt_tensor_threshold(mt_tensor *T, double fraction, mt_tenso
   S->sp_blocks = nnzb;
   S->sp_runs = nruns;
   S->sp_split = sparse_split(n, nnzb, ctx->num_sms);
-  const int np = T->L.nplane;  // value planes: those the source stores (6, or 4 for a single layer)
   S->bytes = 2 * sizeof(int64_t) * (n + 1) + 2 * sizeof(int32_t) * (size_t)std::max<int64_t>(1, nruns) +
              np * sizeof(float) * (size_t)std::max<int64_t>(1, nnzb) + sizeof(int32_t) * kSpSegMax * (size_t)n;
   {
@@ -557,21 +666,20 @@ extern "C" mt_status mt_tensor_threshold(mt_tensor *T, double fraction, mt_tenso
     }
     ctx->in_use += S->bytes;
   }
-  cudaError_t e = cudaMalloc(&S->d_sp_ptr, sizeof(int64_t) * (n + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&S->d_sp_rptr, sizeof(int64_t) * (n + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&S->d_sp_col, 2 * sizeof(int32_t) * std::max<int64_t>(1, nruns));
+  std::swap(S->d_sp_ptr, row_ptr.p);
+  std::swap(S->d_sp_rptr, row_rptr.p);
+  cudaError_t e = cudaMalloc(&S->d_sp_col, 2 * sizeof(int32_t) * std::max<int64_t>(1, nruns));
   if (e == cudaSuccess) e = cudaMalloc(&S->d_sp_val, np * sizeof(float) * std::max<int64_t>(1, nnzb));
   if (e == cudaSuccess) e = cudaMalloc(&S->d_sp_seg, sizeof(int32_t) * kSpSegMax * (size_t)n);
-  if (e == cudaSuccess) e = cudaMemcpy(S->d_sp_ptr, ptr.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(S->d_sp_rptr, rptr.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice);
   // gap and padding blocks are zero
   if (e == cudaSuccess) e = cudaMemset(S->d_sp_val, 0, np * sizeof(float) * std::max<int64_t>(1, nnzb));
   if (e != cudaSuccess) {
     mt::tensor_release(S);
     return mt::cuda_fail(e, "mt_tensor_threshold allocation", __FILE__, __LINE__);
   }
-  k_rows<true><<<(unsigned)n, 32>>>(D, n, L.TR, L.TC, L.nplane, L.Q, tbits, d_tie, r, nullptr, nullptr,
-                                    S->d_sp_ptr, S->d_sp_rptr, S->d_sp_col, S->d_sp_val);
+  (np == 6 ? k_rows<6, true> : k_rows<4, true>)<<<row_grid, 32 * kRowsPerCta>>>(
+      D, n, L.TR, L.TC, L.Q, tie_start.p, sel.p, nullptr, nullptr, S->d_sp_ptr, S->d_sp_rptr, S->d_sp_col,
+      S->d_sp_val);
   e = cudaGetLastError();
   if (e == cudaSuccess)
     k_seg_runs<<<(unsigned)((n * kSpSegMax + 255) / 256), 256>>>(
@@ -584,25 +692,10 @@ extern "C" mt_status mt_tensor_threshold(mt_tensor *T, double fraction, mt_tenso
   }
   if (threshold) {
     float tf;
-    std::memcpy(&tf, &tbits, sizeof(tf));
+    std::memcpy(&tf, &hs.prefix, sizeof(tf));
     *threshold = (double)tf;
   }
-  if (kept_elements) {
-    // kept elements of the full matrix (off-diagonal entries count twice)
-    std::vector<float> vals(np * (size_t)std::max<int64_t>(1, nnzb));
-    MT_CUDA(cudaMemcpy(vals.data(), S->d_sp_val, np * sizeof(float) * nnzb, cudaMemcpyDeviceToHost));
-    int64_t kept = 0;
-    const int mult[6] = {1, 2, 2, 1, 2, 1};
-    for (int64_t i = 0; i < n; ++i) {
-      const int64_t o = ptr[i], K4 = ptr[i + 1] - o;
-      for (int e = 0; e < 6; ++e)
-        for (int64_t a = 0; a < K4; ++a) {
-          const int pl = stream_plane(e, np);
-          kept += (pl >= 0 && vals[np * o + pl * K4 + a] != 0.0f) ? mult[e] : 0;
-        }
-    }
-    *kept_elements = kept;
-  }
+  if (kept_elements) *kept_elements = (int64_t)hs.kept;
   *out = S;
   return MT_OK;
 }
