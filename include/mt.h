@@ -102,7 +102,7 @@ typedef enum {
                           /* products + 7 stage kernels; every tensor kind    */
   MT_PATH_PERSISTENT = 2  /* a whole step/run/relax call as one cooperative    */
                           /* kernel: each SM holds its rows of the tensor in   */
-                          /* shared memory, grid barriers between the stages; */
+                          /* shared memory and exchanges them between stages; */
                           /* FP32 streaming tensors of small tile sets         */
 } mt_path;
 
@@ -526,9 +526,9 @@ MT_API mt_status mt_relax(mt_tensor *T, const mt_llg_params *p, const mt_ode_opt
  * MT_ECUDA otherwise.  The context stays usable.  Synchronous. */
 MT_API mt_status mt_selftest_wait_timeout(mt_ctx *ctx, double limit_s);
 
-/* Self-test of the grid-wide barrier of the one-kernel integrator path
+/* Self-test of the grid-wide exchange of the one-kernel integrator path
  * (MT_PATH_PERSISTENT): a cooperative launch of 4 CTAs in which one CTA
- * leaves without arriving, so the others' bounded wait (about 2 s) runs
+ * leaves without publishing, so the others' bounded wait (about 2 s) runs
  * out; they record the timeout, raise the abort flag and return.  Returns
  * MT_ETIMEOUT when that was reported (the expected outcome), MT_ECUDA
  * otherwise.  The context stays usable.  Synchronous. */

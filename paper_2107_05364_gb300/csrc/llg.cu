@@ -232,7 +232,7 @@ __device__ __forceinline__ void block_reduce(float v[NV], int max_idx) {
 // true in thread 0 of the last block (with tot filled).  FP32 throughout:
 // the sums (squared scaled errors, volume-weighted m) need no more, and FP64
 // arithmetic on the one latency-critical thread is slow on this part.
-__device__ bool reduce_across_blocks(const StageArgs &A, int b, float v[5], double tot[5]) {
+__device__ bool reduce_across_blocks(const StageArgs &A, int b, float v[5], float tot[5]) {
   const int nblk = gridDim.x;
   __shared__ int s_last;
   block_reduce<5>(v, 1);
@@ -258,7 +258,7 @@ __device__ bool reduce_across_blocks(const StageArgs &A, int b, float v[5], doub
   block_reduce<5>(acc, 1);
   if (threadIdx.x == 0) {
     A.red_count[b] = 0;
-    for (int q = 0; q < 5; ++q) tot[q] = (double)acc[q];
+    for (int q = 0; q < 5; ++q) tot[q] = acc[q];
   }
   return threadIdx.x == 0;
 }
@@ -283,11 +283,11 @@ __device__ __forceinline__ void plan_attempt(const StageArgs &A, SimCtl &c) {
 
 // After the first derivative of a run: its torque, and a relaxation that is
 // already below tolerance ends here.
-__device__ __forceinline__ void close_first(SimCtl &c, double tau) {
-  c.tau = tau;
+__device__ __forceinline__ void close_first(SimCtl &c, float tau) {
+  c.tau = (double)tau;
   c.n_rhs += 1;
   c.fresh = 0;
-  if (!isfinite(c.tau)) finish_sim(c, MT_ENONFINITE);
+  if (!isfinite(tau)) finish_sim(c, MT_ENONFINITE);
   else if (c.mode == MODE_RELAX && c.tau < c.tol) finish_sim(c, MT_OK);
 }
 
@@ -296,17 +296,19 @@ __device__ __forceinline__ void close_first(SimCtl &c, double tau) {
 // reject, advance the time, record an output (*out_row = its index, else
 // -1), finish on the end time, on the torque tolerance or on the attempt
 // cap, choose the next step size and plan the next attempt.
-__device__ __forceinline__ void close_attempt(const StageArgs &A, SimCtl &c, const double tot[5], int64_t *out_row) {
+__device__ __forceinline__ void close_attempt(const StageArgs &A, SimCtl &c, const float tot[5], int64_t *out_row) {
   *out_row = -1;
   const bool fixed = A.fixed_h > 0.0;
   // the RMS of the scaled errors; its sum is an FP32 sum on both paths
-  const double err = (double)sqrtf((float)tot[0] / (3.0f * (float)A.n));
-  const double tau = tot[1];
-  c.err = err;
+  // (tests and the step factor in FP32 too: FP64 operations take many cycles
+  // on this part, and one thread does all of this)
+  const float err = sqrtf(tot[0] / (3.0f * (float)A.n));
+  const double tau = (double)tot[1];
+  c.err = (double)err;
   c.n_attempt += 1;
   c.n_rhs += 6;
   const bool finite = isfinite(err) && isfinite(tot[2]) && isfinite(tot[3]) && isfinite(tot[4]);
-  const bool accept = finite && (fixed || err <= 1.0);
+  const bool accept = finite && (fixed || err <= 1.0f);
   if (!finite) {
     c.accepted = 0;
     finish_sim(c, MT_ENONFINITE);
@@ -340,10 +342,8 @@ __device__ __forceinline__ void close_attempt(const StageArgs &A, SimCtl &c, con
   } else {
     // 0.9 err^(-1/5) clamped to [0.2, 5], in FP32 (a relative 1e-7 on the
     // proposal is immaterial; FP64 transcendentals are slow on this part)
-    const float ef = (float)err;
-    double fac = ef > 0.0f ? (double)(0.9f * exp2f(-0.2f * log2f(ef))) : 5.0;
-    fac = fmin(5.0, fmax(0.2, fac));
-    c.h = c.hs * fac;
+    const float f = err > 0.0f ? 0.9f * exp2f(-0.2f * log2f(err)) : 5.0f;
+    c.h = c.hs * (f > 5.0f ? 5.0 : f < 0.2f ? 0.2 : (double)f);
     if (A.hmax > 0.0 && c.h > A.hmax) c.h = A.hmax;
   }
   if (!c.done && c.mode != MODE_STEPS && c.n_attempt >= c.attempt_cap) finish_sim(c, MT_ENOCONV);
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs A) {
       v[3] = w * mi[1];
       v[4] = w * mi[2];
     }
-    double tot[5];
+    float tot[5];
     if (reduce_across_blocks(A, b, v, tot)) {
       SimCtl c = A.ctl[b];
       c.m_last[0] = tot[2];
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs A) {
       v[3] = w * mi[1];
       v[4] = w * mi[2];
     }
-    double tot[5];
+    float tot[5];
     if (reduce_across_blocks(A, b, v, tot)) {
       SimCtl c = A.ctl[b];
       int64_t row = -1;
@@ -528,37 +528,57 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs A) {
 // right-hand side is a few microseconds of work, and the step graph's 13
 // dependent launches per attempt are what the step costs.  Here one CTA per
 // SM keeps its rows of the tensor in shared memory for the whole call (or,
-// when they do not fit, reads them from the L2-resident tensor), the stage
-// inputs of all tiles pass through L2 between grid-wide barriers, and every
+// when they do not fit, reads them from the L2-resident tensor), and every
 // CTA takes the step-control decisions itself from the same per-CTA partial
-// sums reduced in the same fixed order (so all CTAs agree bit for bit): per
-// attempt one barrier before each of the right-hand sides 3..7 and one for
-// the error norm (the stage-2 input every CTA forms for all tiles itself),
-// no launches.  The stage arithmetic is the graph path's except that the
-// error norm and <m> are summed over rows and CTAs in another order.
+// sums reduced in the same fixed order (so all CTAs agree bit for bit).  The
+// stage arithmetic is the graph path's except that the error norm and <m> are
+// summed over rows and CTAs in another order.
+//
+// What is left is bound by the latency of the exchanges between the CTAs, six
+// per attempt: the inputs of stages 3..7 of all tiles, and k7 with the partial
+// sums (the stage-2 input every CTA forms for all tiles itself).  A barrier
+// after plain stores costs three L2 round trips in a row (the stores, the
+// arrival counter, the reload of the data).  Instead every 64-bit word of an
+// exchange carries the number of the exchange beside its data, and the reader
+// polls the data itself: one trip out and one in.  64-bit accesses are single
+// copies, so a word whose tag matches holds its data, and no ordering between
+// words is needed.  400-tile film: 25.5 us
+// per attempt with barriers and plain data, 20.7 with this exchange and one
+// lane per row doing all that follows the row sums (about half of it the
+// exchanges, the rest the serial chain of one stage).
 constexpr int kSmallThreads = 256;
 constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallRed = 3 * 8 * kSmallWarps;  // floats of one buffer of row sums
+
+// one tile's vector: 3 floats and the 16-bit tag in each of two 64-bit words;
+// a CTA's partial sums: 5 words of a float and the tag (padded to 6)
+struct alignas(16) TagVec {
+  unsigned long long a, b;
+};
+struct alignas(16) TagSum {
+  unsigned long long v[6];
+};
 
 struct SmallArgs {
   StageArgs A;
   const float *N;  // stored FP32 tensor, streaming layout
   int TR, TC;
   int64_t Q;
-  float *xg;                // 2 x B x 3n: stage inputs of all tiles (ping-pong)
-  float *part;              // [G][B][5] per-CTA partial sums
-  unsigned long long *bar;  // barrier words (kBarWords, zeroed before the launch)
-  int *abort_flag;          // a bounded wait gave up: every CTA leaves
-  int *status;              // device status word (MT_DEV_TIMEOUT)
-  int64_t iters;            // attempts at most
-  int init;                 // evaluate k1 and the torque at the state first
-  int R;                    // rows per CTA at most
-  int nsmem;                // 1: the CTA's tensor rows live in shared memory, 0: read from L2
-  int nplane;               // stored entry planes: 6, or 4 (single layer: no xz, yz)
+  // exchanged words (zeroed before the launch; tags start at 1)
+  TagVec *xg;       // 2 x B x n: stage inputs (ping-pong)
+  TagVec *kx;       // 2 x B x n: the committed k1 and the k7 of the attempt
+  TagVec *yx;       // B x n: the state of the last accepted attempt
+  TagSum *part;     // [G][B] per-CTA partial sums
+  int *abort_flag;  // a bounded wait gave up: every CTA leaves
+  int *status;      // device status word (MT_DEV_TIMEOUT)
+  int64_t iters;    // attempts at most (kSmallChunk: their 6 tags each fit 16 bits)
+  int init;         // evaluate k1 and the torque at the state first
+  int R;            // rows per CTA at most
 };
 
 // byte offsets of the dynamic shared memory of k_small_run
 struct SmallSmem {
-  size_t ctl, red, hd, y, k, tau, coef, par, kc, nbr, wex, kan, axis, wv, Ms, M, N, total;
+  size_t ctl, red, y, k, coef, par, kc, Ms, M, N, total;
 };
 __host__ __device__ __forceinline__ size_t small_take(size_t &o, size_t bytes) {
   const size_t at = o;
@@ -569,19 +589,12 @@ __host__ __device__ __forceinline__ SmallSmem small_smem(int64_t n, int B, int R
   SmallSmem s;
   size_t o = 0;
   s.ctl = small_take(o, sizeof(SimCtl) * B);
-  s.red = small_take(o, sizeof(float) * kSmallWarps * 3 * 8);
-  s.hd = small_take(o, sizeof(float) * B * R * 3);
+  s.red = small_take(o, sizeof(float) * 2 * kSmallRed);
   s.y = small_take(o, sizeof(float) * B * R * 3);
   s.k = small_take(o, sizeof(float) * 7 * B * R * 3);
-  s.tau = small_take(o, sizeof(float) * B * R);
   s.coef = small_take(o, sizeof(float) * B * 36);  // (float)(h a_sj), s = 1..6, j < s
   s.par = small_take(o, sizeof(float) * B * 6);    // g1, g2, Ha, exchange factor
-  s.kc = small_take(o, sizeof(int) * B);           // buffer of the committed k1 (0: k[0], 1: k[6])
-  s.nbr = small_take(o, sizeof(int32_t) * R * 6);  // the CTA's rows: neighbours,
-  s.wex = small_take(o, sizeof(float) * R * 6);    // exchange weights,
-  s.kan = small_take(o, sizeof(float) * R);        // anisotropy, axis,
-  s.axis = small_take(o, sizeof(float) * R * 3);
-  s.wv = small_take(o, sizeof(float) * R);         // volume weights
+  s.kc = small_take(o, sizeof(int) * B);           // where the committed k1 and y are (see SmallSh)
   s.Ms = small_take(o, sizeof(float) * n);
   s.M = small_take(o, sizeof(float) * B * 3 * n);
   s.N = small_take(o, nsmem ? sizeof(float) * 6 * R * n : 0);
@@ -591,149 +604,139 @@ __host__ __device__ __forceinline__ SmallSmem small_smem(int64_t n, int B, int R
 
 struct SmallSh {
   SimCtl *ctl;
-  float *red, *hd, *y, *k, *tau, *coef, *par, *wex, *kan, *axis, *wv, *Ms, *M, *N;
-  int32_t *nbr;
+  float *red, *y, *k, *coef, *par, *Ms, *M, *N;
+  // per simulation: the tag of the exchange that published the committed k1
+  // (0: it is still in global memory, in k[0]), kKcBuf = its buffer of kx,
+  // kKcY = the committed y is in yx under the same tag (else in global y)
   int *kc;
 };
+constexpr int kKcBuf = 1 << 30, kKcY = 1 << 29, kKcTag = 0xffff;
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
+__device__ __forceinline__ void st_pair(void *p, unsigned long long a, unsigned long long b) {
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
+}
+__device__ __forceinline__ void ld_pair(const void *p, unsigned long long &a, unsigned long long &b) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void publish_vec(TagVec *p, const float v[3], unsigned tag) {
+  const unsigned y = __float_as_uint(v[1]);
+  const unsigned hi_a = (y & 0xffffu) | (tag << 16), hi_b = (y >> 16) | (tag << 16);
+  st_pair(p, __float_as_uint(v[0]) | ((unsigned long long)hi_a << 32),
+          __float_as_uint(v[2]) | ((unsigned long long)hi_b << 32));
+}
+__device__ __forceinline__ bool vec_tagged(unsigned long long a, unsigned long long b, unsigned tag) {
+  return (unsigned)(a >> 48) == tag && (unsigned)(b >> 48) == tag;
+}
+__device__ __forceinline__ void vec_of(unsigned long long a, unsigned long long b, float v[3]) {
+  v[0] = __uint_as_float((unsigned)a);
+  v[1] = __uint_as_float(((unsigned)(a >> 32) & 0xffffu) | ((unsigned)(b >> 32) << 16));
+  v[2] = __uint_as_float((unsigned)b);
 }
 
-__device__ __forceinline__ void red_release_add_u64(unsigned long long *p, unsigned long long v) {
-  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
+// Bound of every polling loop: after ~2 s (or once another CTA gave up) the
+// status word gets MT_DEV_TIMEOUT, the abort flag is raised and the loop ends.
+struct PollLimit {
+  uint32_t it = 0;
+  uint64_t t0 = 0;
+  __device__ __forceinline__ bool expired(const SmallArgs &S) {
+    if ((++it & 63u) != 0u) return false;
+    if (*reinterpret_cast<volatile int *>(S.abort_flag)) return true;
+    const uint64_t t = mtd::globaltimer_ns();
+    if (t0 == 0) t0 = t;
+    if (t - t0 <= 2000000000ull) return false;
+    atomicExch(S.status, MT_DEV_TIMEOUT);
+    atomicExch(S.abort_flag, 1);
+    return true;
+  }
+};
 
-// Barrier words: [0] the arrival counter, which only grows (zeroed before
-// the launch): barrier k is complete when it reaches k x G.  The abort flag
-// sits on the next 128-byte line.
-constexpr int kBarLine = 16;  // 8-byte words per 128-byte line
-constexpr size_t kBarWords = kBarLine;
-
-// Grid-wide barrier of a cooperative launch (all CTAs co-resident): the
-// CTA's writes are ordered before thread 0's release-add by the CTA barrier,
-// and the other CTAs' writes before its acquire-load of the completed count
-// (release/acquire at GPU scope, no full fences).  The wait is bounded:
-// after ~2 s (or once another CTA gave up) the status word gets
-// MT_DEV_TIMEOUT, the abort flag is raised and false is returned.
-__device__ __forceinline__ bool small_grid_sync(const SmallArgs &S, unsigned long long &k) {
-  __shared__ int s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    k += 1;
-    const unsigned long long target = k * gridDim.x;
-    red_release_add_u64(S.bar, 1ull);
-    int ok = 1;
-    if (ld_acquire_u64(S.bar) < target) {
-      const uint64_t t0 = mtd::globaltimer_ns();
-      for (uint32_t it = 1;; ++it) {
-        if (ld_acquire_u64(S.bar) >= target) break;
-        if ((it & 63u) == 0u) {
-          if (*reinterpret_cast<volatile int *>(S.abort_flag)) {
-            ok = 0;
-            break;
-          }
-          if (mtd::globaltimer_ns() - t0 > 2000000000ull) {
-            atomicExch(S.status, MT_DEV_TIMEOUT);
-            atomicExch(S.abort_flag, 1);
-            ok = 0;
-            break;
-          }
-        }
+// n tagged vectors from src: f(j, v) for this thread's j = tid, tid + 256, ...
+// (four in flight at once).  False when the wait gave up.
+template <typename F>
+__device__ __forceinline__ bool poll_vecs(const SmallArgs &S, const TagVec *src, int n, unsigned tag, F &&f) {
+  constexpr int U = 4;
+  PollLimit lim;
+  for (int j0 = threadIdx.x; j0 < n; j0 += U * kSmallThreads) {
+    unsigned long long a[U], b[U];
+    for (;;) {
+      bool all = true;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + u * kSmallThreads;
+        if (j < n) ld_pair(src + j, a[u], b[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j0 + u * kSmallThreads < n) all = all && vec_tagged(a[u], b[u], tag);
+      if (all) break;
+      if (lim.expired(S)) return false;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + u * kSmallThreads;
+      if (j < n) {
+        float v[3];
+        vec_of(a[u], b[u], v);
+        f(j, v);
       }
     }
-    s_ok = ok;
   }
-  __syncthreads();
-  return s_ok != 0;
+  return true;
 }
 
-// Eq. 1 for the CTA's rows from H_d in sh.hd: the local fields and the
-// right-hand side into kout, the torque |m x H|/Ms into sh.tau (the
-// arithmetic of k_stage).
-__device__ __forceinline__ void small_llg(const StageArgs &A, const SmallSh &sh, float *kout, int R, int nr,
-                                          int64_t r0) {
-  const int64_t n = A.n;
-  for (int p = threadIdx.x; p < A.B * nr; p += kSmallThreads) {
-    const int b = p / nr, q = p - (p / nr) * nr;
-    if (sh.ctl[b].done) continue;
-    const int64_t i = r0 + q;
-    const float *yb = sh.M + (size_t)b * 3 * n;
-    const float mi[3] = {yb[3 * i], yb[3 * i + 1], yb[3 * i + 2]};
-    const float *hd = sh.hd + ((size_t)b * R + q) * 3;
-    const float *pb = sh.par + 6 * b;
-    float H[3] = {hd[0], hd[1], hd[2]}, k[3];
-    local_fields(pb + 2, pb[5], A.exch, sh.nbr + 6 * q, sh.wex + 6 * q, sh.kan[q], sh.axis + 3 * q, yb, mi, H);
-    const float t = llg(pb[0], pb[1], mi, H, k) / sh.Ms[i];
-    float *ko = kout + ((size_t)b * R + q) * 3;
-    ko[0] = k[0];
-    ko[1] = k[1];
-    ko[2] = k[2];
-    sh.tau[(size_t)b * R + q] = t;
-  }
-  __syncthreads();
-}
-
-// k_S of the CTA's rows [r0, r0 + nr) for every running simulation, from
-// the stage input of all tiles in sh.M: H_d = -N (Ms m) from the rows held
-// in sh.N, then the local fields and Eq. 1 (the arithmetic of k_stage); the
-// torque |m x H|/Ms into sh.tau.
-template <int RMAX>
-__device__ __forceinline__ void small_rhs(const StageArgs &A, const SmallSh &sh, float *kout, int R, int nr,
-                                          int64_t r0) {
-  const int64_t n = A.n;
+// H_d row sums of simulation b for the CTA's rows, from the stage input of all
+// tiles in sh.M, as partial sums in `red`.  Rows in shared memory: the CTA's
+// threads over the columns, each warp's sums of row value v = 3 q + c at
+// red[warp 3 RMAX + v].
+template <int RMAX, bool PLANAR>
+__device__ __forceinline__ void small_product(const SmallSh &sh, const float *mb, float *red, int R, int nr, int n) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const size_t pl = (size_t)R * n;  // entries of one plane of the CTA's rows
-  for (int b = 0; b < A.B; ++b) {
-    if (sh.ctl[b].done) continue;  // the same in every thread
-    float acc[RMAX][3];
+  constexpr int NV = 3 * RMAX, NS = NV <= 8 ? 8 : NV <= 16 ? 16 : 32;
+  const int pl = R * n;  // entries of one plane of the CTA's rows
+  float acc[NS];
 #pragma unroll
-    for (int q = 0; q < RMAX; ++q) acc[q][0] = acc[q][1] = acc[q][2] = 0.0f;
-    const float *mb = sh.M + (size_t)b * 3 * n;
-    for (int64_t j = tid; j < n; j += kSmallThreads) {
-      const float ms = sh.Ms[j];
-      const float x0 = ms * mb[3 * j], x1 = ms * mb[3 * j + 1], x2 = ms * mb[3 * j + 2];
+  for (int v = 0; v < NS; ++v) acc[v] = 0.0f;
+  // rows past nr repeat the last one (their sums are dropped): no branch
+  // between the loads of a column
+  const float *e[RMAX];
 #pragma unroll
-      for (int q = 0; q < RMAX; ++q) {
-        if (q < nr) {
-          const float *e = sh.N + (size_t)q * n + j;
-          const float nxx = e[0], nxy = e[pl], nxz = e[2 * pl], nyy = e[3 * pl], nyz = e[4 * pl], nzz = e[5 * pl];
-          acc[q][0] = fmaf(nxx, x0, fmaf(nxy, x1, fmaf(nxz, x2, acc[q][0])));
-          acc[q][1] = fmaf(nxy, x0, fmaf(nyy, x1, fmaf(nyz, x2, acc[q][1])));
-          acc[q][2] = fmaf(nxz, x0, fmaf(nyz, x1, fmaf(nzz, x2, acc[q][2])));
-        }
+  for (int q = 0; q < RMAX; ++q) e[q] = sh.N + (q < nr ? q : nr - 1) * n;
+#pragma unroll 2
+  for (int j = tid; j < n; j += kSmallThreads) {
+    const float ms = sh.Ms[j];
+    const float x0 = ms * mb[3 * j], x1 = ms * mb[3 * j + 1], x2 = ms * mb[3 * j + 2];
+#pragma unroll
+    for (int q = 0; q < RMAX; ++q) {
+      const float *f = e[q] + j;
+      if constexpr (PLANAR) {  // no xz, yz
+        const float nxx = f[0], nxy = f[pl], nyy = f[3 * pl], nzz = f[5 * pl];
+        acc[3 * q] = fmaf(nxx, x0, fmaf(nxy, x1, acc[3 * q]));
+        acc[3 * q + 1] = fmaf(nxy, x0, fmaf(nyy, x1, acc[3 * q + 1]));
+        acc[3 * q + 2] = fmaf(nzz, x2, acc[3 * q + 2]);
+      } else {
+        const float nxx = f[0], nxy = f[pl], nxz = f[2 * pl], nyy = f[3 * pl], nyz = f[4 * pl], nzz = f[5 * pl];
+        acc[3 * q] = fmaf(nxx, x0, fmaf(nxy, x1, fmaf(nxz, x2, acc[3 * q])));
+        acc[3 * q + 1] = fmaf(nxy, x0, fmaf(nyy, x1, fmaf(nyz, x2, acc[3 * q + 1])));
+        acc[3 * q + 2] = fmaf(nxz, x0, fmaf(nyz, x1, fmaf(nzz, x2, acc[3 * q + 2])));
       }
     }
-#pragma unroll
-    for (int q = 0; q < RMAX; ++q)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float v = mtd::warp_sum(acc[q][c]);
-        if (lane == 0 && q < nr) sh.red[w * 3 * RMAX + 3 * q + c] = v;
-      }
-    __syncthreads();
-    if (tid < 3 * nr) {
-      float s = 0.0f;
-      for (int ww = 0; ww < kSmallWarps; ++ww) s += sh.red[ww * 3 * RMAX + tid];
-      sh.hd[(size_t)b * R * 3 + tid] = -s;
-    }
-    __syncthreads();
   }
-  small_llg(A, sh, kout, R, nr, r0);
+  const float tot = mtd::warp_reduce_scatter<NS>(acc, lane);  // lane l: value l / (32 / NS)
+  const int v = lane / (32 / NS);
+  if (lane % (32 / NS) == 0 && v < 3 * nr) red[w * NV + v] = tot;
 }
 
 // The same for tile sets whose rows do not fit the shared memory but whose
 // tensor stays in L2 (up to ~100 MB): each warp owns rows w and w + 8 of the
 // CTA (at most 16) and reads them from the streaming layout, lanes over the
 // columns (128 consecutive columns of an entry plane are contiguous, 16-byte
-// aligned), so no cross-warp reduction is needed.
-__device__ __forceinline__ void small_rhs_l2(const SmallArgs &S, const StageArgs &A, const SmallSh &sh,
-                                             float *kout, int R, int nr, int64_t r0) {
-  const int64_t n = A.n;
+// aligned), so no cross-warp reduction is needed: red[3 q + c].
+template <bool PLANAR>
+__device__ __forceinline__ void small_product_l2(const SmallArgs &S, const SmallSh &sh, const float *mb, float *red,
+                                                 int nr, int64_t r0, int64_t n) {
+  constexpr int NP = PLANAR ? 4 : 6;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const size_t plane = (size_t)S.TR * S.TC, chunk = (size_t)S.nplane * plane;
+  const size_t plane = (size_t)S.TR * S.TC, chunk = NP * plane;
   const float *rowp[2] = {nullptr, nullptr};
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -743,84 +746,64 @@ __device__ __forceinline__ void small_rhs_l2(const SmallArgs &S, const StageArgs
       rowp[r] = S.N + (size_t)p * S.Q * chunk + (size_t)(i - p * S.TR) * S.TC;
     }
   }
-  for (int b = 0; b < A.B; ++b) {
-    if (sh.ctl[b].done) continue;  // the same in every thread
-    float acc[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
-    const float *mb = sh.M + (size_t)b * 3 * n;
-    // a lane takes 4 adjacent columns (one 16-byte load per entry plane; the
-    // padding of the last column chunk holds zeros), two such groups per
-    // step so that 24 loads per lane are in flight
-    for (int64_t j0 = 4 * lane; j0 < n; j0 += 256) {
-      float4 ent[2][2][6];
-      float x[2][4][3];
+  float acc[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+  // a lane takes 4 adjacent columns (one 16-byte load per entry plane; the
+  // padding of the last column chunk holds zeros), two such groups per
+  // step so that 4 NP loads per lane are in flight
+  for (int64_t j0 = 4 * lane; j0 < n; j0 += 256) {
+    float4 ent[2][2][NP];
+    float x[2][4][3];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int64_t j = j0 + 128 * u;
-        const int64_t cq = j / S.TC;
-        const size_t off = (size_t)cq * chunk + (size_t)(j - cq * S.TC);
+    for (int u = 0; u < 2; ++u) {
+      const int64_t j = j0 + 128 * u;
+      const int64_t cq = j / S.TC;
+      const size_t off = (size_t)cq * chunk + (size_t)(j - cq * S.TC);
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < 2; ++r)
 #pragma unroll
-          for (int e = 0; e < 6; ++e) {
-            const int pl = stream_plane(e, S.nplane);
-            ent[u][r][e] = (rowp[r] && j < n && pl >= 0)
-                               ? __ldg(reinterpret_cast<const float4 *>(rowp[r] + off + pl * plane))
-                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-          }
+        for (int e = 0; e < NP; ++e)
+          ent[u][r][e] = (rowp[r] && j < n) ? __ldg(reinterpret_cast<const float4 *>(rowp[r] + off + e * plane))
+                                            : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const bool in = j + k < n;
+        const float ms = in ? sh.Ms[j + k] : 0.0f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[u][k][c] = in ? ms * mb[3 * (j + k) + c] : 0.0f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const bool in = j + k < n;
-          const float ms = in ? sh.Ms[j + k] : 0.0f;
-#pragma unroll
-          for (int c = 0; c < 3; ++c) x[u][k][c] = in ? ms * mb[3 * (j + k) + c] : 0.0f;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float *ex = reinterpret_cast<const float *>(&ent[u][r][0]) + k;  // entry e at ex[4 e]
-            const float nxx = ex[0], nxy = ex[4], nxz = ex[8], nyy = ex[12], nyz = ex[16], nzz = ex[20];
-            const float x0 = x[u][k][0], x1 = x[u][k][1], x2 = x[u][k][2];
-            acc[r][0] = fmaf(nxx, x0, fmaf(nxy, x1, fmaf(nxz, x2, acc[r][0])));
-            acc[r][1] = fmaf(nxy, x0, fmaf(nyy, x1, fmaf(nyz, x2, acc[r][1])));
-            acc[r][2] = fmaf(nxz, x0, fmaf(nyz, x1, fmaf(nzz, x2, acc[r][2])));
+          const float *ex = reinterpret_cast<const float *>(&ent[u][r][0]) + k;  // plane e at ex[4 e]
+          const float x0 = x[u][k][0], x1 = x[u][k][1], x2 = x[u][k][2];
+          if constexpr (PLANAR) {
+            acc[r][0] = fmaf(ex[0], x0, fmaf(ex[4], x1, acc[r][0]));
+            acc[r][1] = fmaf(ex[4], x0, fmaf(ex[8], x1, acc[r][1]));
+            acc[r][2] = fmaf(ex[12], x2, acc[r][2]);
+          } else {
+            acc[r][0] = fmaf(ex[0], x0, fmaf(ex[4], x1, fmaf(ex[8], x2, acc[r][0])));
+            acc[r][1] = fmaf(ex[4], x0, fmaf(ex[12], x1, fmaf(ex[16], x2, acc[r][1])));
+            acc[r][2] = fmaf(ex[8], x0, fmaf(ex[16], x1, fmaf(ex[20], x2, acc[r][2])));
           }
-    }
+        }
+  }
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      if (!rowp[r]) continue;  // the same in the whole warp
-      const int q = w + kSmallWarps * r;
+  for (int r = 0; r < 2; ++r) {
+    if (!rowp[r]) continue;  // the same in the whole warp
+    const int q = w + kSmallWarps * r;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float v = mtd::warp_sum(acc[r][c]);
-        if (lane == 0) sh.hd[((size_t)b * R + q) * 3 + c] = -v;
-      }
+    for (int c = 0; c < 3; ++c) {
+      const float v = mtd::warp_sum(acc[r][c]);
+      if (lane == 0) red[3 * q + c] = v;
     }
   }
-  __syncthreads();
-  small_llg(A, sh, kout, R, nr, r0);
 }
 
-// all tiles' stage input (B x 3n floats written by every CTA before the
-// barrier) into shared memory, through L2
-__device__ __forceinline__ void small_load_state(float *sM, const float *src, size_t count) {
-  if ((count & 3) == 0) {  // src and sM are 16-byte aligned
-    const float4 *s4 = reinterpret_cast<const float4 *>(src);
-    float4 *d4 = reinterpret_cast<float4 *>(sM);
-    for (size_t q = threadIdx.x; q < count / 4; q += kSmallThreads) d4[q] = __ldcg(s4 + q);
-  } else {
-    for (size_t q = threadIdx.x; q < count; q += kSmallThreads) sM[q] = __ldcg(src + q);
-  }
-  __syncthreads();
-}
-
-// Warp 0: the sums of the CTA's 5 values per simulation (sum, max, sum,
-// sum, sum over its rows, one lane per row) to part[g][b]; after the
-// barrier, every CTA's warp 0 adds the G partials of b in the same fixed
-// order (lane-strided, then a butterfly), so all CTAs hold the same totals.
+// Warp: the sums of 5 values over its lanes (sum, max, sum, sum, sum)
 __device__ __forceinline__ void small_warp_reduce(float v[5]) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -831,25 +814,61 @@ __device__ __forceinline__ void small_warp_reduce(float v[5]) {
     v[4] += __shfl_xor_sync(0xffffffffu, v[4], o);
   }
 }
-__device__ __forceinline__ void small_partial(const SmallArgs &S, int b, float v[5]) {
+// the CTA's 5 values of simulation b (one lane per row) to every CTA
+__device__ __forceinline__ void small_partial(const SmallArgs &S, int b, float v[5], unsigned tag) {
   small_warp_reduce(v);
-  if ((threadIdx.x & 31) == 0) {
-    float *dst = S.part + ((size_t)blockIdx.x * S.A.B + b) * 5;
-    for (int q = 0; q < 5; ++q) dst[q] = v[q];
+  if ((threadIdx.x & 31) < 3) {
+    const int l = threadIdx.x & 31;  // lane l sends words 2 l and 2 l + 1
+    const float lo = l == 0 ? v[0] : l == 1 ? v[2] : v[4], hi = l == 0 ? v[1] : l == 1 ? v[3] : 0.0f;
+    TagSum *dst = S.part + (size_t)blockIdx.x * S.A.B + b;
+    st_pair(&dst->v[2 * l], __float_as_uint(lo) | ((unsigned long long)tag << 32),
+            __float_as_uint(hi) | ((unsigned long long)tag << 32));
   }
 }
-__device__ __forceinline__ void small_total(const SmallArgs &S, int b, double tot[5]) {
+// A warp: the G partials of b added in a fixed order (lane-strided, then a
+// butterfly), so all CTAs hold the same totals.  False when the wait gave up.
+__device__ __forceinline__ bool small_total(const SmallArgs &S, int b, unsigned tag, float tot[5]) {
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  for (int g = threadIdx.x & 31; g < (int)gridDim.x; g += 32) {
-    const float *src = S.part + ((size_t)g * S.A.B + b) * 5;
-    acc[0] += __ldcg(&src[0]);
-    acc[1] = mtd::nan_max(acc[1], __ldcg(&src[1]));
-    acc[2] += __ldcg(&src[2]);
-    acc[3] += __ldcg(&src[3]);
-    acc[4] += __ldcg(&src[4]);
+  constexpr int U = 5;  // of one lane, in flight at once (152 CTAs: all)
+  PollLimit lim;
+  bool ok = true;
+  for (int g0 = threadIdx.x & 31; ok && g0 < (int)gridDim.x; g0 += 32 * U) {
+    unsigned long long w[U][6];
+    for (;;) {
+      bool all = true;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const TagSum *src = S.part + (size_t)(g0 + 32 * u) * S.A.B + b;
+        if (g0 + 32 * u < (int)gridDim.x)
+#pragma unroll
+          for (int l = 0; l < 3; ++l) ld_pair(&src->v[2 * l], w[u][2 * l], w[u][2 * l + 1]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (g0 + 32 * u < (int)gridDim.x)
+#pragma unroll
+          for (int l = 0; l < 6; ++l) all = all && (unsigned)(w[u][l] >> 32) == tag;
+      if (all) break;
+      if (lim.expired(S)) {
+        ok = false;
+        break;
+      }
+    }
+    if (!ok) break;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (g0 + 32 * u < (int)gridDim.x) {
+        acc[0] += __uint_as_float((unsigned)w[u][0]);
+        acc[1] = mtd::nan_max(acc[1], __uint_as_float((unsigned)w[u][1]));
+        acc[2] += __uint_as_float((unsigned)w[u][2]);
+        acc[3] += __uint_as_float((unsigned)w[u][3]);
+        acc[4] += __uint_as_float((unsigned)w[u][4]);
+      }
   }
+  ok = __all_sync(0xffffffffu, ok);
   small_warp_reduce(acc);
-  for (int q = 0; q < 5; ++q) tot[q] = (double)acc[q];
+  for (int q = 0; q < 5; ++q) tot[q] = acc[q];
+  return ok;
 }
 
 // m / |m| with every rounding pinned (no contraction freedom), so that the
@@ -862,27 +881,133 @@ __device__ __forceinline__ void small_unit(const float *v, float *out) {
   out[2] = __fmul_rn(v[2], inv);
 }
 
-// this CTA's rows [r0, r0 + nr) of a per-simulation plane (B x R x 3 in
-// shared memory) into the tile-major global array dst (B x 3n)
-__device__ __forceinline__ void small_publish_rows(float *dst, const float *src, int B, int R, int nr, int64_t r0,
-                                                   int64_t n) {
-  for (int p = threadIdx.x; p < B * nr * 3; p += kSmallThreads) {
-    const int b = p / (nr * 3), qc = p - b * nr * 3;
-    dst[(size_t)b * 3 * n + 3 * r0 + qc] = src[(size_t)b * R * 3 + qc];
+// A warp: (float)(h a_sj) of every stage-input row s = 1..6 (the inputs of
+// stages 2..7) and j < s of simulation b: coef[36 b + 6 (s - 1) + j]
+__device__ __forceinline__ void small_coefficients(const SmallSh &sh, int b) {
+  for (int rj = threadIdx.x & 31; rj < 36; rj += 32) {
+    const int r = rj / 6, j = rj - r * 6;
+    if (j <= r) sh.coef[36 * b + rj] = (float)(sh.ctl[b].hs * c_dp_a[r + 1][j]);
   }
 }
 
-// (float)(h a_sj) of every stage-input row s = 1..6 (the inputs of stages
-// 2..7) and j < s, per simulation: coef[36 b + 6 (s - 1) + j]
-__device__ __forceinline__ void small_coefficients(const StageArgs &A, const SmallSh &sh) {
-  for (int p = threadIdx.x; p < A.B * 36; p += kSmallThreads) {
-    const int b = p / 36, rj = p - b * 36, r = rj / 6, j = rj - r * 6;
-    if (j <= r) sh.coef[p] = (float)(sh.ctl[b].hs * c_dp_a[r + 1][j]);
+// The constants of row q = lane of the CTA (every warp holds them: a warp owns
+// simulations, its lanes the rows), a missing neighbour as the row itself
+// with weight 0
+struct SmallRow {
+  int nbr[6];
+  float wex[6], kan, axis[3], Ms, wv;
+};
+
+// One stage of every running simulation: the product, then by the warp that
+// owns the simulation (b mod 8; lane q = row q of the CTA) the local fields,
+// Eq. 1 (the arithmetic of k_stage) and what follows from it: after stages
+// 1..6 k, for stages 2..6 also the next stage's input, published under
+// `tag`; after stage 7 k7 and the sums of the error norm, the torque and <m>;
+// after stage 1 (k1 at the state) k1 and the torque.  One CTA barrier per
+// simulation: sh.M is read only before it (a later exchange may overwrite
+// it), and the two buffers of row sums alternate.
+template <int RMAX, bool NSMEM, bool PLANAR>
+__device__ __forceinline__ void small_stage(const SmallArgs &S, const SmallSh &sh, const SmallRow &rw, int st,
+                                            unsigned tag, int nr, int64_t r0, int &buf) {
+  const StageArgs &A = S.A;
+  const int n = (int)A.n, B = A.B, R = S.R;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const size_t kpl = (size_t)B * R * 3;  // floats of one derivative plane
+  for (int b = 0; b < B; ++b) {
+    if (sh.ctl[b].done) continue;  // the same in every thread
+    const float *mb = sh.M + (size_t)b * 3 * n;
+    float *red = sh.red + buf * kSmallRed;
+    buf ^= 1;
+    if constexpr (NSMEM) small_product<RMAX, PLANAR>(sh, mb, red, R, nr, n);
+    else small_product_l2<PLANAR>(S, sh, mb, red, nr, r0, n);
+    const bool mine = warp == (b & (kSmallWarps - 1)), row = mine && lane < nr;
+    const int q = lane;
+    const int i = (int)r0 + q;
+    // what needs the other tiles: the exchange sum and m itself
+    float mi[3] = {0.0f, 0.0f, 0.0f}, he[3] = {0.0f, 0.0f, 0.0f};
+    if (row) {
+      for (int c = 0; c < 3; ++c) mi[c] = mb[3 * i + c];
+      if (A.exch) {
+#pragma unroll
+        for (int f = 0; f < 6; ++f)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) he[c] += rw.wex[f] * (mb[3 * rw.nbr[f] + c] - mi[c]);
+      }
+    }
+    __syncthreads();
+    if (!mine) continue;
+    float k[3] = {0.0f, 0.0f, 0.0f}, tau = 0.0f;
+    float *ks = sh.k + ((size_t)b * R + q) * 3;  // row q's k1; plane s at + s kpl
+    const float *y0 = sh.y + ((size_t)b * R + q) * 3;
+    if (row) {
+      const float *pb = sh.par + 6 * b;
+      float H[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float s = 0.0f;
+        if constexpr (NSMEM) {
+#pragma unroll
+          for (int w = 0; w < kSmallWarps; ++w) s += red[w * 3 * RMAX + 3 * q + c];
+        } else {
+          s = red[3 * q + c];
+        }
+        H[c] = -s + pb[2 + c];
+        if (A.exch) H[c] += pb[5] * he[c];
+      }
+      if (rw.kan != 0.0f) {
+        const float me = mi[0] * rw.axis[0] + mi[1] * rw.axis[1] + mi[2] * rw.axis[2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) H[c] += rw.kan * me * rw.axis[c];
+      }
+      const float mxh = llg(pb[0], pb[1], mi, H, k);
+      if (st == 1 || st == 7) tau = mxh / rw.Ms;
+      for (int c = 0; c < 3; ++c) ks[(st - 1) * kpl + c] = k[c];
+      if (st >= 2 && st <= 6) {
+        // this row's input of the next stage: y + sum_j (h a_sj) k_j
+        const float *cf = sh.coef + 36 * b + 6 * (st - 1);
+        float acc[3] = {0.0f, 0.0f, 0.0f}, a[6], kj[6][3];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {  // all loads before the sums
+          a[j] = j < st ? cf[j] : 0.0f;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) kj[j][c] = j < st - 1 ? ks[j * kpl + c] : k[c];
+        }
+#pragma unroll
+        for (int j = 0; j < 6; ++j)
+          if (a[j] != 0.0f)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) acc[c] += a[j] * kj[j][c];
+        const float v[3] = {y0[0] + acc[0], y0[1] + acc[1], y0[2] + acc[2]};
+        publish_vec(S.xg + (size_t)((st + 1) & 1) * B * n + (size_t)b * n + i, v, tag);
+      }
+    }
+    if (st >= 2 && st <= 6) continue;
+    // k1 (stage 1) or k7 into the buffer that does not hold the committed k1
+    const int into = st == 1 ? 0 : (sh.kc[b] & kKcBuf) ? 0 : 1;
+    float v[5] = {0.0f, tau, 0.0f, 0.0f, 0.0f};
+    if (row) {
+      publish_vec(S.kx + (size_t)into * B * n + (size_t)b * n + i, k, tag);
+      if (st == 7) {
+        // embedded error, torque and <m> at the 5th-order solution (the
+        // stage-7 input), in FP32
+        const float hs = (float)sh.ctl[b].hs, atol = (float)A.atol, rtol = (float)A.rtol;
+        for (int c = 0; c < 3; ++c) {
+          float e = 0.0f;
+#pragma unroll
+          for (int j = 0; j < 7; ++j)
+            if (c_dp_err[j] != 0.0) e = fmaf((float)c_dp_err[j], j == 6 ? k[c] : ks[j * kpl + c], e);
+          const float r = e * hs / (atol + rtol * fmaxf(fabsf(y0[c]), fabsf(mi[c])));
+          v[0] = fmaf(r, r, v[0]);
+        }
+        const float wv = rw.wv / sqrtf(mi[0] * mi[0] + mi[1] * mi[1] + mi[2] * mi[2]);
+        for (int c = 0; c < 3; ++c) v[2 + c] = wv * mi[c];
+      }
+    }
+    small_partial(S, b, v, tag);
   }
-  __syncthreads();
 }
 
-template <int RMAX, bool NSMEM>
+template <int RMAX, bool NSMEM, bool PLANAR>
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
   extern __shared__ __align__(16) unsigned char smem[];
   const StageArgs &A = S.A;
@@ -895,26 +1020,18 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
   SmallSh sh;
   sh.ctl = reinterpret_cast<SimCtl *>(smem + L.ctl);
   sh.red = reinterpret_cast<float *>(smem + L.red);
-  sh.hd = reinterpret_cast<float *>(smem + L.hd);
   sh.y = reinterpret_cast<float *>(smem + L.y);
   sh.k = reinterpret_cast<float *>(smem + L.k);
-  sh.tau = reinterpret_cast<float *>(smem + L.tau);
   sh.coef = reinterpret_cast<float *>(smem + L.coef);
   sh.par = reinterpret_cast<float *>(smem + L.par);
-  sh.nbr = reinterpret_cast<int32_t *>(smem + L.nbr);
   sh.kc = reinterpret_cast<int *>(smem + L.kc);
-  sh.wex = reinterpret_cast<float *>(smem + L.wex);
-  sh.kan = reinterpret_cast<float *>(smem + L.kan);
-  sh.axis = reinterpret_cast<float *>(smem + L.axis);
-  sh.wv = reinterpret_cast<float *>(smem + L.wv);
   sh.Ms = reinterpret_cast<float *>(smem + L.Ms);
   sh.M = reinterpret_cast<float *>(smem + L.M);
   sh.N = reinterpret_cast<float *>(smem + L.N);
-  const size_t kpl = (size_t)B * R * 3;  // floats of one derivative plane
-  const size_t state = (size_t)B * 3 * n;
-  unsigned long long nbar = 0;  // barriers passed
+  const size_t kpl = (size_t)B * R * 3;
+  unsigned seq = 0;  // exchanges so far: the next one's tag is seq + 1
+  int buf = 0;
   bool ok = true;
-  const float atol = (float)A.atol, rtol = (float)A.rtol;
 
   // control blocks and parameters, Ms, the CTA's rows of N (plane e, row q,
   // column j) and their tile constants, the rows of y and of the derivative
@@ -935,18 +1052,22 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
     for (int64_t q = tid; q < (int64_t)6 * nr * n; q += kSmallThreads) {
       const int64_t j = q % n, eq = q / n;
       const int e = (int)(eq / nr), r = (int)(eq % nr);
-      const int pl = stream_plane(e, S.nplane);
-      sh.N[((size_t)e * R + r) * n + j] = pl < 0 ? 0.0f : S.N[layout_index(r0 + r, j, pl, S.TR, S.TC, S.nplane, S.Q)];
+      constexpr int NP = PLANAR ? 4 : 6;
+      const int pl = stream_plane(e, NP);
+      if (pl >= 0) sh.N[((size_t)e * R + r) * n + j] = S.N[layout_index(r0 + r, j, pl, S.TR, S.TC, NP, S.Q)];
     }
-  for (int q = tid; q < nr; q += kSmallThreads) {
-    const int64_t i = r0 + q;
+  SmallRow rw;
+  {
+    const int64_t i = r0 + (lane < nr ? lane : 0);
     for (int f = 0; f < 6; ++f) {
-      sh.nbr[6 * q + f] = A.nbr[6 * i + f];
-      sh.wex[6 * q + f] = A.wex[6 * i + f];
+      const int32_t p = A.nbr[6 * i + f];
+      rw.nbr[f] = p >= 0 ? p : (int)i;
+      rw.wex[f] = p >= 0 ? A.wex[6 * i + f] : 0.0f;
     }
-    sh.kan[q] = A.kan[i];
-    for (int c = 0; c < 3; ++c) sh.axis[3 * q + c] = A.axis[3 * i + c];
-    sh.wv[q] = (float)A.wvol[i];
+    rw.kan = A.kan[i];
+    for (int c = 0; c < 3; ++c) rw.axis[c] = A.axis[3 * i + c];
+    rw.Ms = A.Ms[i];
+    rw.wv = (float)A.wvol[i];
   }
   for (int p = tid; p < B * nr * 3; p += kSmallThreads) {
     const int b = p / (nr * 3), qc = p - b * nr * 3;
@@ -954,169 +1075,122 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
     sh.y[(size_t)b * R * 3 + qc] = A.y[o];
     sh.k[(size_t)b * R * 3 + qc] = A.k[0][o];
   }
+  if (S.init)
+    for (int64_t q = tid; q < (int64_t)B * 3 * n; q += kSmallThreads) sh.M[q] = A.y[q];
   __syncthreads();
 
   if (S.init) {  // k1 and the torque at the state
-    small_load_state(sh.M, A.y, state);
-    if (NSMEM) small_rhs<RMAX>(A, sh, sh.k, R, nr, r0);
-    else small_rhs_l2(S, A, sh, sh.k, R, nr, r0);
-    small_publish_rows(A.k[0], sh.k, B, R, nr, r0, n);  // read by all CTAs after the barrier
-    for (int b = warp; b < B; b += kSmallWarps) {
+    small_stage<RMAX, NSMEM, PLANAR>(S, sh, rw, 1, 1, nr, r0, buf);
+    seq = 1;
+    for (int b = warp; ok && b < B; b += kSmallWarps) {
       if (sh.ctl[b].done) continue;
-      float v[5] = {0.0f, lane < nr ? sh.tau[(size_t)b * R + lane] : 0.0f, 0.0f, 0.0f, 0.0f};
-      small_partial(S, b, v);
-    }
-    ok = small_grid_sync(S, nbar);
-    if (ok)
-      for (int b = warp; b < B; b += kSmallWarps) {
-        if (sh.ctl[b].done) continue;
-        double tot[5];
-        small_total(S, b, tot);
-        if (lane == 0) close_first(sh.ctl[b], tot[1]);
-        __syncwarp();
+      float tot[5];
+      ok = small_total(S, b, 1, tot);
+      if (ok && lane == 0) {
+        close_first(sh.ctl[b], tot[1]);
+        sh.kc[b] = 1;  // k1: tag 1 in buffer 0 of kx
       }
-    __syncthreads();
+      __syncwarp();
+    }
   }
+  for (int b = warp; b < B; b += kSmallWarps)
+    if (!sh.ctl[b].done) small_coefficients(sh, b);
+  ok = __syncthreads_and(ok);
 
   for (int64_t it = 0; ok && it < S.iters; ++it) {
     bool any = false;
     for (int b = 0; b < B; ++b) any = any || !sh.ctl[b].done;
     if (!any) break;
-    small_coefficients(A, sh);
     // stage 2 needs no exchange between CTAs: every CTA forms the input of
     // all tiles, y + (h a_21) k1, from the committed state (after an accepted
     // attempt: the normalised 5th-order solution still in sh.M and the k7
-    // every CTA published; else the committed y and k1 in global memory)
+    // every CTA published; else the committed y and k1)
     for (int b = 0; b < B; ++b) {
       if (sh.ctl[b].done) continue;
+      const int kc = sh.kc[b];
       const bool adopt = it > 0 && sh.ctl[b].accepted;
       const float a21 = sh.coef[36 * b];
-      const float *kb = (sh.kc[b] ? A.k[6] : A.k[0]) + (size_t)b * 3 * n;
-      const float *yb = A.y + (size_t)b * 3 * n;
       float *mb = sh.M + (size_t)b * 3 * n;
-      for (int64_t j = tid; j < n; j += kSmallThreads) {
-        float y[3];
-        if (adopt) {
-          small_unit(mb + 3 * j, y);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) y[c] = __ldcg(yb + 3 * j + c);
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) mb[3 * j + c] = __fadd_rn(y[c], __fmul_rn(a21, __ldcg(kb + 3 * j + c)));
+      const float *yb = A.y + (size_t)b * 3 * n, *kb = A.k[0] + (size_t)b * 3 * n;
+      if (!adopt) {  // the committed y into sh.M
+        if (kc & kKcY)
+          ok = poll_vecs(S, S.yx + (size_t)b * n, (int)n, kc & kKcTag, [&](int j, const float *y) {
+                 for (int c = 0; c < 3; ++c) mb[3 * j + c] = y[c];
+               }) && ok;
+        else
+          for (int j = tid; j < n; j += kSmallThreads)
+            for (int c = 0; c < 3; ++c) mb[3 * j + c] = __ldcg(yb + 3 * j + c);
       }
+      auto form = [&](int j, const float *k1) {  // (the thread that wrote mb[j])
+        float y[3] = {mb[3 * j], mb[3 * j + 1], mb[3 * j + 2]};
+        if (adopt) small_unit(mb + 3 * j, y);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) mb[3 * j + c] = __fadd_rn(y[c], __fmul_rn(a21, k1[c]));
+      };
+      if (kc & kKcTag)
+        ok = poll_vecs(S, S.kx + (size_t)((kc & kKcBuf) ? 1 : 0) * B * n + (size_t)b * n, (int)n, kc & kKcTag, form) &&
+             ok;
+      else
+        for (int j = tid; j < n; j += kSmallThreads) {
+          const float k1[3] = {__ldcg(kb + 3 * j), __ldcg(kb + 3 * j + 1), __ldcg(kb + 3 * j + 2)};
+          form(j, k1);
+        }
     }
-    __syncthreads();
-    if (NSMEM) small_rhs<RMAX>(A, sh, sh.k + kpl, R, nr, r0);
-    else small_rhs_l2(S, A, sh, sh.k + kpl, R, nr, r0);
-    for (int st = 3; st <= 7 && ok; ++st) {
-      // this CTA's rows of the stage input y + sum_j (h a_sj) k_j
-      float *xo = S.xg + (size_t)(st & 1) * state;
-      for (int p = tid; p < B * nr; p += kSmallThreads) {
-        const int b = p / nr, q = p - (p / nr) * nr;
-        if (sh.ctl[b].done) continue;
-        const float *cf = sh.coef + 36 * b + 6 * (st - 2);
-        float acc[3] = {0.0f, 0.0f, 0.0f};
-        for (int j = 0; j < st - 1; ++j) {
-          const float a = cf[j];
-          if (a != 0.0f) {
-            const float *kj = sh.k + j * kpl + ((size_t)b * R + q) * 3;
-            acc[0] += a * kj[0];
-            acc[1] += a * kj[1];
-            acc[2] += a * kj[2];
-          }
+    ok = __syncthreads_and(ok);
+    if (!ok) break;
+    for (int st = 2; st <= 7; ++st) {
+      if (st > 2) {  // all tiles' input of this stage
+        for (int b = 0; b < B; ++b) {
+          if (sh.ctl[b].done) continue;
+          float *mb = sh.M + (size_t)b * 3 * n;
+          ok = poll_vecs(S, S.xg + (size_t)(st & 1) * B * n + (size_t)b * n, (int)n, seq + st - 2,
+                         [&](int j, const float *v) {
+                           for (int c = 0; c < 3; ++c) mb[3 * j + c] = v[c];
+                         }) && ok;
         }
-        const float *y0 = sh.y + ((size_t)b * R + q) * 3;
-        float *d = xo + (size_t)b * 3 * n + 3 * (r0 + q);
-        d[0] = y0[0] + acc[0];
-        d[1] = y0[1] + acc[1];
-        d[2] = y0[2] + acc[2];
+        ok = __syncthreads_and(ok);
+        if (!ok) break;
       }
-      ok = small_grid_sync(S, nbar);
+      small_stage<RMAX, NSMEM, PLANAR>(S, sh, rw, st, seq + st - 1, nr, r0, buf);
+    }
+    if (!ok) break;
+    seq += 6;  // the k7 and the partial sums went out under this tag
+    for (int b = warp; ok && b < B; b += kSmallWarps) {
+      if (sh.ctl[b].done) continue;
+      float tot[5];
+      ok = small_total(S, b, seq, tot);
       if (!ok) break;
-      small_load_state(sh.M, xo, state);
-      if (NSMEM) small_rhs<RMAX>(A, sh, sh.k + (st - 1) * kpl, R, nr, r0);
-      else small_rhs_l2(S, A, sh, sh.k + (st - 1) * kpl, R, nr, r0);
-    }
-    if (!ok) break;
-    // this CTA's k7 rows into the buffer not holding the committed k1: the
-    // next attempt's k1 if this one is accepted
-    for (int p = tid; p < B * nr * 3; p += kSmallThreads) {
-      const int b = p / (nr * 3), qc = p - b * nr * 3;
-      if (sh.ctl[b].done) continue;
-      (sh.kc[b] ? A.k[0] : A.k[6])[(size_t)b * 3 * n + 3 * r0 + qc] = sh.k[6 * kpl + (size_t)b * R * 3 + qc];
-    }
-    // embedded error, torque and <m> at the 5th-order solution (the stage-7
-    // input), in FP32 over the CTA's rows: one lane per row
-    for (int b = warp; b < B; b += kSmallWarps) {
-      if (sh.ctl[b].done) continue;
-      float v[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-      if (lane < nr) {
-        const float hs = (float)sh.ctl[b].hs;
-        const int64_t i = r0 + lane;
-        const float *mi = sh.M + (size_t)b * 3 * n + 3 * i;
-        const float *y0 = sh.y + ((size_t)b * R + lane) * 3;
-        for (int c = 0; c < 3; ++c) {
-          float e = 0.0f;
-#pragma unroll
-          for (int j = 0; j < 7; ++j)
-            if (c_dp_err[j] != 0.0) e = fmaf((float)c_dp_err[j], sh.k[j * kpl + ((size_t)b * R + lane) * 3 + c], e);
-          const float r = e * hs / (atol + rtol * fmaxf(fabsf(y0[c]), fabsf(mi[c])));
-          v[0] = fmaf(r, r, v[0]);
-        }
-        v[1] = sh.tau[(size_t)b * R + lane];
-        const float wv = sh.wv[lane] / sqrtf(mi[0] * mi[0] + mi[1] * mi[1] + mi[2] * mi[2]);
-        v[2] = wv * mi[0];
-        v[3] = wv * mi[1];
-        v[4] = wv * mi[2];
-      }
-      small_partial(S, b, v);
-    }
-    ok = small_grid_sync(S, nbar);
-    if (!ok) break;
-    for (int b = warp; b < B; b += kSmallWarps) {
-      if (sh.ctl[b].done) continue;
-      double tot[5];
-      small_total(S, b, tot);
       if (lane == 0) {
-        int64_t row = -1;
-        close_attempt(A, sh.ctl[b], tot, &row);
-        if (g == 0 && row >= 0) {
-          double *mo = A.mavg + ((size_t)row * B + b) * 3;
+        int64_t out = -1;
+        close_attempt(A, sh.ctl[b], tot, &out);
+        if (g == 0 && out >= 0) {
+          double *mo = A.mavg + ((size_t)out * B + b) * 3;
           mo[0] = tot[2];
           mo[1] = tot[3];
           mo[2] = tot[4];
         }
       }
       __syncwarp();
-    }
-    __syncthreads();
-    // accepted: adopt the normalised 5th-order solution (this CTA's rows also
-    // into the committed y in global memory, read after a later rejection);
-    // k7 is the next k1
-    for (int p = tid; p < B * nr; p += kSmallThreads) {
-      const int b = p / nr, q = p - (p / nr) * nr;
+      small_coefficients(sh, b);
       if (!sh.ctl[b].accepted) continue;
-      const float *yn = sh.M + (size_t)b * 3 * n + 3 * (r0 + q);
-      float *y0 = sh.y + ((size_t)b * R + q) * 3;
-      float *k1 = sh.k + ((size_t)b * R + q) * 3;
-      const float *k7 = sh.k + 6 * kpl + ((size_t)b * R + q) * 3;
-      float *yg = A.y + (size_t)b * 3 * n + 3 * (r0 + q);
-      small_unit(yn, y0);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        yg[c] = y0[c];
-        k1[c] = k7[c];
+      // adopt the normalised 5th-order solution (published for a stage-2
+      // input after a later rejection); k7 is the next k1
+      if (lane < nr) {
+        float *y0 = sh.y + ((size_t)b * R + lane) * 3;
+        float *k1 = sh.k + ((size_t)b * R + lane) * 3;
+        small_unit(sh.M + (size_t)b * 3 * n + 3 * (r0 + lane), y0);
+        publish_vec(S.yx + (size_t)b * n + r0 + lane, y0, seq);
+        for (int c = 0; c < 3; ++c) k1[c] = k1[6 * kpl + c];
       }
+      if (lane == 0) sh.kc[b] = ((sh.kc[b] & kKcBuf) ^ kKcBuf) | kKcY | (int)seq;
     }
-    __syncthreads();
-    for (int b = tid; b < B; b += kSmallThreads)
-      if (sh.ctl[b].accepted) sh.kc[b] ^= 1;
-    __syncthreads();
+    ok = __syncthreads_and(ok);
   }
   if (!ok) return;  // timed out: the status word tells the host
   // write back: the state and the next derivative of this CTA's rows; CTA 0
-  // the control blocks (nothing left to commit) and the active set
+  // the control blocks (nothing left to commit) and the active set.  (Every
+  // CTA's partial sums of the last attempt have arrived, so none still reads
+  // the global y and k1 for its stage 2.)
   for (int p = tid; p < B * nr * 3; p += kSmallThreads) {
     const int b = p / (nr * 3), qc = p - b * nr * 3;
     const size_t o = (size_t)b * 3 * n + 3 * r0 + qc;
@@ -1136,12 +1210,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
   }
 }
 
-// failure-detection self-test: CTA 0 leaves without arriving, so the other
-// CTAs' bounded barrier wait runs out
-__global__ void k_barrier_selftest(SmallArgs S) {
-  unsigned long long nbar = 0;
+// failure-detection self-test: CTA 0 leaves without publishing its words, so
+// the other CTAs' bounded wait for them runs out
+__global__ void k_exchange_selftest(SmallArgs S) {
   if (blockIdx.x == 0) return;
-  small_grid_sync(S, nbar);
+  const float v[3] = {1.0f, 2.0f, 3.0f};
+  if (threadIdx.x == 0) publish_vec(S.xg + blockIdx.x, v, 1);
+  poll_vecs(S, S.xg, gridDim.x, 1, [](int, const float *) {});
 }
 
 // put a prepared control block into slot b and make it active
@@ -1311,9 +1386,7 @@ struct mt_integrator {
   int small_G = 0, small_R = 0, small_rmax = 0;
   bool small_nsmem = true;  // tensor rows in shared memory (else read from L2)
   size_t small_smem_bytes = 0;
-  float *sm_xg = nullptr;
-  float *sm_part = nullptr;
-  unsigned long long *sm_bar = nullptr;  // barrier words, then the abort flag
+  unsigned char *sm_words = nullptr;  // words its CTAs exchange, then the abort flag (SmallWords)
 };
 
 namespace {
@@ -1363,13 +1436,31 @@ StageArgs stage_args(mt_integrator *I) {
 
 constexpr size_t kSmallSmemMax = 225 * 1024;  // of the 227 KB a CTA may opt in to
 
-template <int RMAX, bool NSMEM>
-cudaError_t small_attr(size_t bytes, int *per_sm) {
-  cudaError_t e =
-      cudaFuncSetAttribute(k_small_run<RMAX, NSMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_small_run<RMAX, NSMEM>, kSmallThreads, bytes);
-  return e;
+using SmallKernel = void (*)(SmallArgs);
+template <bool PLANAR>
+SmallKernel small_kernel_of(bool nsmem, int rmax) {
+  return !nsmem ? k_small_run<2, false, PLANAR>
+                : rmax == 2 ? k_small_run<2, true, PLANAR>
+                            : rmax == 4 ? k_small_run<4, true, PLANAR> : k_small_run<8, true, PLANAR>;
+}
+SmallKernel small_kernel(const mt_tensor *T, bool nsmem, int rmax) {
+  return T->L.nplane == 4 ? small_kernel_of<true>(nsmem, rmax) : small_kernel_of<false>(nsmem, rmax);
+}
+
+// byte offsets of the exchanged words of k_small_run
+struct SmallWords {
+  size_t xg, kx, yx, part, abort_flag, total;
+};
+SmallWords small_words(int64_t n, int B, int G) {
+  SmallWords w;
+  const size_t vecs = sizeof(TagVec) * (size_t)B * n;
+  w.xg = 0;
+  w.kx = w.xg + 2 * vecs;
+  w.yx = w.kx + 2 * vecs;
+  w.part = w.yx + vecs;
+  w.abort_flag = w.part + sizeof(TagSum) * (size_t)G * B;
+  w.total = w.abort_flag + 128;
+  return w;
 }
 
 // a tensor the one-kernel path reads from L2 every right-hand side must
@@ -1396,14 +1487,18 @@ bool small_plan(mt_integrator *I) {
     if (R > (nsmem ? 8 : 2 * kSmallWarps)) continue;
     if (!nsmem && (T->bytes > kSmallL2Bytes || T->L.TC % 4 != 0)) continue;
     const size_t bytes = small_smem(n, I->B, R, nsmem).total;
-    if (bytes > kSmallSmemMax) continue;
+    // (the limit counts one buffer of row sums, and H_d, the torque and the
+    // constants of the CTA's rows, once held in shared memory: the same tile
+    // sets qualify for this path whatever its kernel keeps there)
+    size_t counted = bytes - sizeof(float) * kSmallRed;
+    for (const int per_row : {3 * I->B, I->B, 6, 6, 1, 3, 1}) small_take(counted, sizeof(float) * R * per_row);
+    if (counted > kSmallSmemMax) continue;
     const int G = (int)((n + R - 1) / R);
     const int rmax = !nsmem ? 2 : R <= 2 ? 2 : R <= 4 ? 4 : 8;
     int per_sm = 0;
-    const cudaError_t e = !nsmem     ? small_attr<2, false>(bytes, &per_sm)
-                          : rmax == 2 ? small_attr<2, true>(bytes, &per_sm)
-                          : rmax == 4 ? small_attr<4, true>(bytes, &per_sm)
-                                      : small_attr<8, true>(bytes, &per_sm);
+    const SmallKernel kern = small_kernel(T, nsmem, rmax);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSmallThreads, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
       continue;
@@ -1427,17 +1522,17 @@ mt_status launch_small(mt_integrator *I, int init, int64_t iters) {
   S.TR = T->L.TR;
   S.TC = T->L.TC;
   S.Q = T->L.Q;
-  S.xg = I->sm_xg;
-  S.part = I->sm_part;
-  S.bar = I->sm_bar;
-  S.abort_flag = reinterpret_cast<int *>(I->sm_bar + kBarWords);
+  const SmallWords w = small_words(T->n, I->B, I->small_G);
+  S.xg = reinterpret_cast<TagVec *>(I->sm_words + w.xg);
+  S.kx = reinterpret_cast<TagVec *>(I->sm_words + w.kx);
+  S.yx = reinterpret_cast<TagVec *>(I->sm_words + w.yx);
+  S.part = reinterpret_cast<TagSum *>(I->sm_words + w.part);
+  S.abort_flag = reinterpret_cast<int *>(I->sm_words + w.abort_flag);
   S.status = T->tiles->ctx->d_status;
   S.iters = iters;
   S.init = init;
   S.R = I->small_R;
-  S.nsmem = I->small_nsmem ? 1 : 0;
-  S.nplane = T->L.nplane;
-  MT_CUDA(cudaMemsetAsync(I->sm_bar, 0, (kBarWords + kBarLine) * sizeof(unsigned long long), I->stream));
+  MT_CUDA(cudaMemsetAsync(I->sm_words, 0, w.total, I->stream));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)I->small_G);
   cfg.blockDim = dim3(kSmallThreads);
@@ -1456,10 +1551,7 @@ mt_status launch_small(mt_integrator *I, int init, int64_t iters) {
   if (!ctx->small_ev) e = cudaEventCreateWithFlags(&ctx->small_ev, cudaEventDisableTiming);
   else e = cudaStreamWaitEvent(I->stream, ctx->small_ev, 0);
   if (e == cudaSuccess) {
-    if (!I->small_nsmem) e = cudaLaunchKernelEx(&cfg, k_small_run<2, false>, S);
-    else if (I->small_rmax == 2) e = cudaLaunchKernelEx(&cfg, k_small_run<2, true>, S);
-    else if (I->small_rmax == 4) e = cudaLaunchKernelEx(&cfg, k_small_run<4, true>, S);
-    else e = cudaLaunchKernelEx(&cfg, k_small_run<8, true>, S);
+    e = cudaLaunchKernelEx(&cfg, small_kernel(T, I->small_nsmem, I->small_rmax), S);
   }
   if (e == cudaSuccess) e = cudaEventRecord(ctx->small_ev, I->stream);
   if (e != cudaSuccess) return mt::cuda_fail(e, "k_small_run launch", __FILE__, __LINE__);
@@ -1588,6 +1680,7 @@ void plan_host(const mt_integrator *I, SimCtl &c) {
 // no launch runs for long; between them the host reads the number of
 // unfinished simulations (and stops on a device timeout).
 constexpr int64_t kSmallChunk = 4096;
+static_assert(6 * kSmallChunk + 1 < 1 << 15, "exchange tags of one launch");
 
 mt_status small_steps(mt_integrator *I, int init, int64_t nsteps) {
   for (int64_t done = 0; done < nsteps || init;) {
@@ -1721,9 +1814,7 @@ mt_status mt_integrator_create(mt_tensor *T, const mt_llg_params *p, const mt_od
   MT_TRY(dalloc(I, &I->mavg, sizeof(double) * 3 * B));
   I->small_ok = small_plan(I);
   if (I->small_ok) {
-    MT_TRY(dalloc(I, &I->sm_xg, 2 * vec));
-    MT_TRY(dalloc(I, &I->sm_part, sizeof(float) * 5 * I->small_G * B));
-    MT_TRY(dalloc(I, &I->sm_bar, (kBarWords + kBarLine) * sizeof(unsigned long long)));
+    MT_TRY(dalloc(I, &I->sm_words, small_words(n, B, I->small_G).total));
     I->path = MT_PATH_PERSISTENT;
   }
   if (cudaMallocHost(&I->h_poll, 2 * sizeof(int)) != cudaSuccess) {
@@ -1847,14 +1938,14 @@ int mt_integrator_get_path(mt_integrator *I) { return I ? I->path : 0; }
 mt_status mt_selftest_grid_barrier_timeout(mt_ctx *ctx) {
   MT_CHECK(ctx, MT_EINVAL, "mt_selftest_grid_barrier_timeout: NULL context");
   MT_CUDA(cudaSetDevice(ctx->device));
-  unsigned long long *words = nullptr;
-  const size_t bytes = (kBarWords + kBarLine) * sizeof(unsigned long long) + sizeof(int);
-  MT_CUDA(cudaMalloc(&words, bytes));
-  cudaError_t e = cudaMemset(words, 0, bytes);
+  // 4 tagged vectors, the abort flag, a status word
+  unsigned char *words = nullptr;
+  MT_CUDA(cudaMalloc(&words, 256));
+  cudaError_t e = cudaMemset(words, 0, 256);
   SmallArgs S{};
-  S.bar = words;
-  S.abort_flag = reinterpret_cast<int *>(words + kBarWords);
-  S.status = reinterpret_cast<int *>(words + kBarWords + kBarLine);
+  S.xg = reinterpret_cast<TagVec *>(words);
+  S.abort_flag = reinterpret_cast<int *>(words + 128);
+  S.status = reinterpret_cast<int *>(words + 192);
   if (e == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(4);
@@ -1864,17 +1955,17 @@ mt_status mt_selftest_grid_barrier_timeout(mt_ctx *ctx) {
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k_barrier_selftest, S);
+    e = cudaLaunchKernelEx(&cfg, k_exchange_selftest, S);
   }
   int h = 0;
   if (e == cudaSuccess) e = cudaMemcpy(&h, S.status, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(words);
   if (e != cudaSuccess) return mt::cuda_fail(e, "mt_selftest_grid_barrier_timeout", __FILE__, __LINE__);
   if (h == MT_DEV_TIMEOUT) {
-    mt::set_error("mt_selftest_grid_barrier_timeout: the bounded barrier gave up as designed");
+    mt::set_error("mt_selftest_grid_barrier_timeout: the bounded wait gave up as designed");
     return MT_ETIMEOUT;
   }
-  mt::set_error("mt_selftest_grid_barrier_timeout: the barrier did not report a timeout");
+  mt::set_error("mt_selftest_grid_barrier_timeout: the wait did not report a timeout");
   return MT_ECUDA;
 }
 

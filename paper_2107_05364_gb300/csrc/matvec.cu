@@ -558,30 +558,6 @@ struct HalfShape {
   static_assert(STAGES >= 2 && SMEM_BYTES <= 227 * 1024, "ring within one CTA's shared memory");
 };
 
-// Sums over the warp's lanes of NS values (NS a power of two <= 32), scattered:
-// lane l returns the total of value l / (32 / NS).  Recursive halving: at the
-// step with offset o a lane keeps the upper half of its values if (l & o),
-// else the lower half, and adds its partner's copy of them; once one value is
-// left the remaining offsets add it whole.
-template <int NS>
-__device__ __forceinline__ float warp_reduce_scatter(float (&v)[NS], int lane) {
-  static_assert(NS >= 1 && NS <= 32 && (NS & (NS - 1)) == 0, "a power of two up to 32");
-  int o = 16;
-#pragma unroll
-  for (int cnt = NS / 2; cnt >= 1; cnt /= 2, o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < cnt; ++i) {
-      const float send = up ? v[i] : v[cnt + i];
-      const float keep = up ? v[cnt + i] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-#pragma unroll
-  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-  return v[0];
-}
-
 struct HalfArgs {
   const float *tensor;
   const float *xs;   // [b][q][3][TC], Ms m
@@ -1106,7 +1082,7 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
       }
       __syncwarp();
       if (lane == 0) mtd::mbar_arrive(&empty[s]);
-      if constexpr (SCATTER) accs[k] += warp_reduce_scatter<NSLOT>(rv, lane);  // every lane, aborted or not
+      if constexpr (SCATTER) accs[k] += mtd::warp_reduce_scatter<NSLOT>(rv, lane);  // every lane, aborted or not
     }
   };
 

@@ -510,6 +510,30 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Sums over the warp's lanes of NS values (NS a power of two <= 32), scattered:
+// lane l returns the total of value l / (32 / NS).  Recursive halving: at the
+// step with offset o a lane keeps the upper half of its values if (l & o),
+// else the lower half, and adds its partner's copy of them; once one value is
+// left the remaining offsets add it whole.
+template <int NS>
+__device__ __forceinline__ float warp_reduce_scatter(float (&v)[NS], int lane) {
+  static_assert(NS >= 1 && NS <= 32 && (NS & (NS - 1)) == 0, "a power of two up to 32");
+  int o = 16;
+#pragma unroll
+  for (int cnt = NS / 2; cnt >= 1; cnt /= 2, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < cnt; ++i) {
+      const float send = up ? v[i] : v[cnt + i];
+      const float keep = up ? v[cnt + i] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
 // Stream-K split of U work units over G CTAs: CTA k owns [begin(k), begin(k+1)).
 __host__ __device__ __forceinline__ int64_t sk_begin(int64_t k, int64_t U, int64_t G) { return (k * U) / G; }
 // CTA owning unit u: largest k with begin(k) <= u.
