@@ -444,9 +444,10 @@ def run_batched(args, quiet=False):
     e1.record(cur)
     torch.cuda.synchronize()
     gemm_ms = e0.elapsed_time(e1) / reps
-    Kp = int(math.ceil(3 * n / 128) * 128)
+    Kp = int(math.ceil(n / 128) * 128)
     stored = info["bytes"]
-    flops = 2.0 * Kp * Kp * mt_pad(B) * (3 if args.prec == "split" else 1)
+    # plane products per block: off-diagonal planes are multiplied twice
+    flops = 2.0 * (5 if info["planes"] == 4 else 9) * Kp * Kp * mt_pad(B) * (3 if args.prec == "split" else 1)
     Td.close()
     I.close()
     # plain FP32 path, one simulation at a time

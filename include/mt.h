@@ -76,9 +76,10 @@ typedef enum {
 typedef enum {
   MT_LAYOUT_STREAM = 0, /* 6 unique entries per block, tile-blocked panels for  */
                         /* the streaming product (one simulation per pass)      */
-  MT_LAYOUT_DENSE = 1,  /* all 9 entries, row-major 3n x 3n BF16 (or hi + lo   */
-                        /* pair) for the batched tensor-core product; only      */
-                        /* MT_BF16_SCALED (scales fixed to 1) and MT_BF16_SPLIT */
+  MT_LAYOUT_DENSE = 1,  /* entry planes (6; 4 for a single layer) of n x n BF16 */
+                        /* (or hi + lo pairs) for the batched tensor-core       */
+                        /* product; only MT_BF16_SCALED (scales fixed to 1) and */
+                        /* MT_BF16_SPLIT                                        */
   MT_LAYOUT_SPARSE = 2, /* thresholded FP32 tensor in block-sparse rows       */
                         /* (made by mt_tensor_threshold, Sec. 4.3.1)            */
   MT_LAYOUT_STREAM6 = 3, /* MT_LAYOUT_STREAM with all 6 entry planes and every  */
@@ -152,7 +153,7 @@ typedef struct {
   int32_t rows_per_panel, cols_per_chunk; /* tile-blocked layout (stream)     */
   int32_t layout;      /* mt_layout_kind                                      */
   int32_t planes;      /* stored values per 3x3 block: 6 (4 single-layer),    */
-                       /* split 12 (8 single-layer), dense 9                  */
+                       /* streaming split 12 (8 single-layer)                 */
   int64_t bytes;       /* device bytes of the stored tensor                   */
   int64_t near_blocks; /* FP64 near-field blocks kept apart (0 if none)       */
   int32_t half;        /* 1: only the upper triangle of blocks is stored      */
@@ -271,8 +272,8 @@ MT_API mt_status mt_demag_assemble(mt_tiles *tiles, mt_prec prec, mt_tensor **ou
 /* As mt_demag_assemble, with an explicit storage layout (mt_layout_kind).
  * MT_LAYOUT_DENSE turns every product over a batch of B simulations into a
  * GEMM on the tensor cores (tcgen05, BF16 in, FP32 accumulate); the rows and
- * columns of the 3n x 3n matrix are padded to a multiple of 128 (zeros) and
- * the blocks of touching tiles are kept apart in FP64 as for the streaming
+ * columns of each entry plane are padded to a multiple of 128 (zeros), an
+ * off-diagonal plane serves both entries it stands for, and the blocks of touching tiles are kept apart in FP64 as for the streaming
  * layout.  Errors as mt_demag_assemble, plus MT_EINVAL for a precision the
  * layout does not support. */
 MT_API mt_status mt_demag_assemble_ex(mt_tiles *tiles, mt_prec prec, int layout, mt_tensor **out);

@@ -159,6 +159,14 @@ mt_status demag_apply(mt_tensor *T, const float *m, int B, float *H, cudaStream_
   return MT_OK;
 }
 
+// single-layer cuboid set: every tile has the same centre z and z edge
+bool single_layer(const mt_tiles *t) {
+  if (t->kind != MT_TILE_CUBOID) return false;
+  for (int64_t i = 1; i < t->n; ++i)
+    if (t->centre[3 * i + 2] != t->centre[2] || t->edge[3 * i + 2] != t->edge[2]) return false;
+  return true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -482,22 +490,16 @@ mt_status mt_demag_assemble_ex(mt_tiles *tiles, mt_prec prec, int layout, mt_ten
     // thread mapping of the assembly kernel: 16-row panels x 128-column chunks
     T->L.TR = 16;
     T->L.TC = 128;
-    T->L.nplane = 9;
+    T->L.nplane = single_layer(tiles) ? 4 : 6;
     T->L.elem_bytes = 2;
     T->L.P = (T->n + T->L.TR - 1) / T->L.TR;
     T->L.Q = (T->n + T->L.TC - 1) / T->L.TC;
-    T->Kp = ((3 * T->n + 127) / 128) * 128;
-    data_bytes = (size_t)T->Kp * T->Kp * 2 * (prec == MT_BF16_SPLIT ? 2 : 1);
+    T->Kp = ((T->n + 127) / 128) * 128;
+    data_bytes = mt::dense_tensor_bytes(T->n, prec, T->L.nplane);
   } else {
     mt::layout_for(prec, &T->L);
-    // single-layer cuboid set (every tile: the same centre z and z edge): the
-    // FP32 tensor's xz and yz entries vanish; 4 entry planes
-    if (allow_planar && prec != MT_F64 && tiles->kind == MT_TILE_CUBOID) {
-      bool planar = true;
-      for (int64_t i = 1; i < tiles->n && planar; ++i)
-        planar = tiles->centre[3 * i + 2] == tiles->centre[2] && tiles->edge[3 * i + 2] == tiles->edge[2];
-      if (planar) mt::layout_for_planar(prec, &T->L);
-    }
+    // single-layer set: the xz and yz entries vanish; 4 entry planes
+    if (allow_planar && prec != MT_F64 && single_layer(tiles)) mt::layout_for_planar(prec, &T->L);
     T->L.P = (T->n + T->L.TR - 1) / T->L.TR;
     T->L.Q = (T->n + T->L.TC - 1) / T->L.TC;
     // FP32 tiles of one shape: the tensor is symmetric (N_ij = N_ji), so
@@ -569,7 +571,7 @@ mt_status mt_tensor_get_info(const mt_tensor *T, mt_tensor_info *info) {
   info->rows_per_panel = T->L.TR;
   info->cols_per_chunk = T->L.TC;
   info->layout = T->layout;
-  info->planes = T->layout == MT_LAYOUT_DENSE ? 9 : T->L.nplane;  // sparse: as its source
+  info->planes = T->L.nplane;  // sparse: as its source
   info->bytes = (int64_t)T->bytes;
   info->near_blocks = T->near_count;
   info->half = T->L.half ? 1 : 0;
@@ -671,10 +673,7 @@ namespace mt {
 // device bytes of a tensor of n tiles in a precision and layout (as allocated
 // by mt_demag_assemble_ex)
 size_t tensor_bytes_for(int64_t n, int prec, int layout) {
-  if (layout == MT_LAYOUT_DENSE) {
-    const size_t Kp = (size_t)((3 * n + 127) / 128) * 128;
-    return Kp * Kp * 2 * (prec == MT_BF16_SPLIT ? 2 : 1);
-  }
+  if (layout == MT_LAYOUT_DENSE) return dense_tensor_bytes(n, prec, 6);
   mt_layout L;
   layout_for(prec, &L);
   L.P = (n + L.TR - 1) / L.TR;

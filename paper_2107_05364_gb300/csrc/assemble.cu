@@ -384,7 +384,7 @@ struct AsmArgs {
   int *bad;           // set to 1 on overlap
   int *planar_bad;    // set to 1 if a 4- or 3-plane (single-layer) tensor meets |N_xz| or |N_yz| >
                       // kPlanarTol, or (3 or 5 planes) a block's trace off delta_ij by more than kTraceTol
-  int dense;          // 1: 9-entry row-major matrix (Kp x Kp), else tile-blocked
+  int dense;          // 1: tensor-core planes (dense_a_index), else the streaming layout
   int half;           // 1: streaming FP32 tensor of one tile shape, upper triangle of chunks only
   int64_t Kp;
   int *near_fill;     // per-row fill counter (BF16 precisions)
@@ -406,20 +406,20 @@ __device__ __forceinline__ void store_block(const AsmArgs &A, int64_t i, int64_t
     return;  // dense store keeps zeros there
   }
   if (A.dense) {
-    // all 9 entries: row 3i + a, column 3j + b (scales fixed to 1)
     __nv_bfloat16 *D = (__nv_bfloat16 *)A.data;
-    const size_t plane = (size_t)A.Kp * A.Kp;
-    const int e_of[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+    const bool split = A.prec == MT_BF16_SPLIT;
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const double v = N6[e_of[a][b]];
-        const size_t at = dense_a_index(3 * i + a, 3 * j + b, A.Kp / 64);
-        const __nv_bfloat16 hi = __double2bfloat16(v);
-        D[at] = hi;
-        if (A.prec == MT_BF16_SPLIT) D[plane + at] = __double2bfloat16(v - (double)__bfloat162float(hi));
+    for (int e = 0; e < 6; ++e) {
+      const int pl = stream_plane(e, A.nplane);
+      if (pl < 0) {
+        if (!(fabs(N6[e]) <= kPlanarTol)) *A.planar_bad = 1;
+        continue;
       }
+      const size_t at = dense_a_index(i, j, pl, A.Kp / 64, A.nplane, split);
+      const __nv_bfloat16 hi = __double2bfloat16(N6[e]);
+      D[at] = hi;
+      if (split) D[at + kDenseLo] = __double2bfloat16(N6[e] - (double)__bfloat162float(hi));
+    }
     return;
   }
   switch (A.prec) {
@@ -677,18 +677,20 @@ __global__ void k_read_rows(const void *data, const int8_t *scale, int prec, int
 }
 
 // dense layout -> double, rows [i0, i1)
-__global__ void k_read_rows_dense(const __nv_bfloat16 *D, int split, int64_t n, int64_t Kp, int64_t i0, int64_t i1,
-                                  double *out) {
+__global__ void k_read_rows_dense(const __nv_bfloat16 *D, bool split, int64_t n, int64_t KB, int np, int64_t i0,
+                                  int64_t i1, double *out) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t rows = i1 - i0;
   if (t >= rows * n) return;
   const int64_t i = i0 + t / n, j = t % n;
-  const int ra[6] = {0, 0, 0, 1, 1, 2}, cb[6] = {0, 1, 2, 1, 2, 2};
-  const size_t plane = (size_t)Kp * Kp;
   for (int e = 0; e < 6; ++e) {
-    const size_t at = dense_a_index(3 * i + ra[e], 3 * j + cb[e], Kp / 64);
-    double v = (double)__bfloat162float(D[at]);
-    if (split) v += (double)__bfloat162float(D[plane + at]);
+    const int pl = stream_plane(e, np);
+    double v = 0.0;
+    if (pl >= 0) {
+      const size_t at = dense_a_index(i, j, pl, KB, np, split);
+      v = (double)__bfloat162float(D[at]);
+      if (split) v += (double)__bfloat162float(D[at + kDenseLo]);
+    }
     out[t * 6 + e] = v;
   }
 }
@@ -756,46 +758,46 @@ mt_status assemble(mt_tensor *T) {
     A.geo = geo.p;
   }
   const bool has_near = (T->prec == MT_BF16_SCALED || T->prec == MT_BF16_SPLIT);
+  DevTemp<int> fill;  // per-row counters of the blocks kept apart
   if (has_near) {
-    DevTemp<int> fill;
     MT_CUDA(fill.alloc(n));
-    int *d_fill = fill.p;
-    MT_CUDA(cudaMemset(d_fill, 0, sizeof(int) * n));
-    A.near_fill = d_fill;
+    MT_CUDA(cudaMemset(fill.p, 0, sizeof(int) * n));
+    A.near_fill = fill.p;
     A.count_only = 1;
     launch_assemble(A, L);
     MT_CUDA(cudaGetLastError());
     std::vector<int> cnt(n);
-    MT_CUDA(cudaMemcpy(cnt.data(), d_fill, sizeof(int) * n, cudaMemcpyDeviceToHost));
+    MT_CUDA(cudaMemcpy(cnt.data(), fill.p, sizeof(int) * n, cudaMemcpyDeviceToHost));
     std::vector<int32_t> ptr(n + 1, 0);
     for (int64_t i = 0; i < n; ++i) ptr[i + 1] = ptr[i] + cnt[i];
     T->near_count = ptr[n];
     MT_CUDA(cudaMalloc(&T->d_near_ptr, sizeof(int32_t) * (n + 1)));
     MT_CUDA(cudaMalloc(&T->d_near_col, sizeof(int32_t) * std::max<int64_t>(1, T->near_count)));
     MT_CUDA(cudaMalloc(&T->d_near_val, sizeof(double) * 6 * std::max<int64_t>(1, T->near_count)));
+    MT_CUDA(cudaMalloc(&T->d_near_hl, sizeof(float2) * 6 * std::max<int64_t>(1, T->near_count)));
     MT_CUDA(cudaMemcpy(T->d_near_ptr, ptr.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice));
-    MT_CUDA(cudaMemset(d_fill, 0, sizeof(int) * n));
     A.near_ptr = T->d_near_ptr;
     A.near_col = T->d_near_col;
     A.near_val = T->d_near_val;
     A.count_only = 0;
-    launch_assemble(A, L);
+  }
+  // every block into its place (again with another layout, should the first
+  // turn out not to hold the tensor)
+  auto fill_all = [&]() -> mt_status {
+    if (has_near) MT_CUDA(cudaMemset(fill.p, 0, sizeof(int) * n));
+    launch_assemble(A, T->L);
     MT_CUDA(cudaGetLastError());
-    k_sort_near<<<(unsigned)((n + 127) / 128), 128>>>(n, T->d_near_ptr, T->d_near_col, T->d_near_val);
-    MT_CUDA(cudaGetLastError());
-    const int64_t c6 = 6 * std::max<int64_t>(1, T->near_count);
-    MT_CUDA(cudaMalloc(&T->d_near_hl, sizeof(float2) * c6));
     if (T->near_count > 0) {
+      k_sort_near<<<(unsigned)((n + 127) / 128), 128>>>(n, T->d_near_ptr, T->d_near_col, T->d_near_val);
       k_near_split<<<(unsigned)((6 * T->near_count + 255) / 256), 256>>>(6 * T->near_count, T->d_near_val,
                                                                         T->d_near_col, t->d_Ms, T->d_near_hl);
       MT_CUDA(cudaGetLastError());
     }
     MT_CUDA(cudaDeviceSynchronize());
-  } else {
-    launch_assemble(A, L);
-    MT_CUDA(cudaGetLastError());
-    MT_CUDA(cudaDeviceSynchronize());
-  }
+    return MT_OK;
+  };
+  mt_status st = fill_all();
+  if (st != MT_OK) return st;
   int bad[2] = {0, 0};
   MT_CUDA(cudaMemcpy(bad, d_bad, 2 * sizeof(int), cudaMemcpyDeviceToHost));
   MT_CHECK(!bad[0], MT_EOVERLAP, "mt_demag_assemble: tiles overlap or a tile centre lies on another tile");
@@ -805,12 +807,19 @@ mt_status assemble(mt_tensor *T) {
     // all (within the budget reserved for them)
     mt_ctx *ctx = t->ctx;
     const bool half = T->L.half;
-    layout_for(T->prec, &T->L);
-    T->L.P = (n + T->L.TR - 1) / T->L.TR;
-    T->L.Q = (n + T->L.TC - 1) / T->L.TC;
-    T->L.half = half;
-    T->L.CH = half ? half_chunks(T->L.P, T->L.Q, T->L.TC / T->L.TR) : T->L.P * T->L.Q;
-    const size_t bytes = (size_t)T->L.CH * (T->L.chunk_bytes() + T->L.scale_bytes_per_chunk);
+    size_t data_bytes;
+    if (A.dense) {
+      T->L.nplane = 6;
+      data_bytes = dense_tensor_bytes(n, T->prec, 6);
+    } else {
+      layout_for(T->prec, &T->L);
+      T->L.P = (n + T->L.TR - 1) / T->L.TR;
+      T->L.Q = (n + T->L.TC - 1) / T->L.TC;
+      T->L.half = half;
+      T->L.CH = half ? half_chunks(T->L.P, T->L.Q, T->L.TC / T->L.TR) : T->L.P * T->L.Q;
+      data_bytes = (size_t)T->L.CH * T->L.chunk_bytes();
+    }
+    const size_t bytes = data_bytes + (A.dense ? 0 : (size_t)T->L.CH * T->L.scale_bytes_per_chunk);
     {
       std::lock_guard<std::mutex> lk(ctx->mu);
       MT_CHECK(ctx->in_use - T->bytes + bytes <= ctx->budget, MT_ENOMEM,
@@ -818,7 +827,6 @@ mt_status assemble(mt_tensor *T) {
       ctx->in_use += bytes - T->bytes;
       T->bytes = bytes;
     }
-    const size_t data_bytes = (size_t)T->L.CH * T->L.chunk_bytes();
     MT_CUDA(cudaFree(T->d_data));
     T->d_data = nullptr;
     MT_CUDA(cudaMalloc(&T->d_data, data_bytes));
@@ -828,9 +836,7 @@ mt_status assemble(mt_tensor *T) {
     A.TC = T->L.TC;
     A.nplane = T->L.nplane;
     A.Q = T->L.Q;
-    launch_assemble(A, T->L);
-    MT_CUDA(cudaGetLastError());
-    MT_CUDA(cudaDeviceSynchronize());
+    return fill_all();
   }
   return MT_OK;
 }
@@ -862,7 +868,8 @@ mt_status read_rows(const mt_tensor *T, int64_t i0, int64_t i1, double *out) {
   const int64_t tot = rows * n;
   if (T->layout == MT_LAYOUT_DENSE)
     k_read_rows_dense<<<(unsigned)((tot + 255) / 256), 256>>>((const __nv_bfloat16 *)T->d_data,
-                                                              T->prec == MT_BF16_SPLIT, n, T->Kp, i0, i1, d_out);
+                                                              T->prec == MT_BF16_SPLIT, n, T->Kp / 64, T->L.nplane,
+                                                              i0, i1, d_out);
   else
     k_read_rows<<<(unsigned)((tot + 255) / 256), 256>>>(T->d_data, T->d_scale, T->prec, n, T->L.TR, T->L.TC,
                                                          T->L.nplane, T->L.Q, T->L.half, i0, i1, d_out);

@@ -1,32 +1,44 @@
 // Batched demag product on the 5th-generation tensor cores (tcgen05).
 //
 // B simulations on one geometry turn the product H_d = -N (Ms m) (Eq. 9,
-// Eq. 17) into a GEMM: D[3n x B] = N[3n x 3n] X^T with X[b] = Ms m_b.  The
-// tensor is stored dense (all 9 entries of each block, row r = 3i + a,
-// column c = 3j + b) in BF16, or as a BF16 hi + lo pair ("split").  The
-// split product carries the operand as three BF16 terms x0 + x1 + x2 (24
-// significant bits: a relaxed, nearly uniform state would otherwise round
-// every x the same way and leave a coherent error) and forms
-// N_hi (x0 + x1 + x2) + N_lo (x0 + x1); the blocks of touching tiles are
-// zero there and are applied with FP64-class accuracy by the near-field
-// kernel.
+// Eq. 17) into GEMMs with X[b] = Ms m_b.  Every 3x3 block of N is symmetric,
+// so the tensor is stored as its 6 entry planes (xx xy xz yy yz zz; 4, without
+// xz and yz, for a single-layer tile set), each an n x n matrix in BF16 or as
+// a BF16 hi + lo pair ("split"), and an off-diagonal plane is read once and
+// multiplied twice: H_x += N_xy X_y and H_y += N_xy X_x.  The split product
+// carries the operand as three BF16 terms x0 + x1 + x2 (24 significant bits: a
+// relaxed, nearly uniform state would otherwise round every x the same way and
+// leave a coherent error) and forms N_hi (x0 + x1 + x2) + N_lo (x0 + x1); the
+// blocks of touching tiles are zero there and are applied with FP64-class
+// accuracy by the near-field kernel.
 //
-// The GEMM is HBM-bound for B <= ~300 (64 flop per tensor byte at B = 64),
-// so the design streams the tensor once per batched product:
-//   * persistent CTAs, one per SM; the (row tile, K block) units are split
-//     evenly over the CTAs in storage order (stream-K);
-//   * warp 0 issues 2-D TMA loads (128-byte swizzle) of a 128 x 64 tensor
-//     tile and the 64-wide slice of X^T into a shared-memory ring;
-//   * warp 1 issues tcgen05.mma (M = 128, N = B, K = 16, BF16 -> FP32) into
-//     a ring of four TMEM accumulators, each filled over a few K blocks (the
-//     tensor cores' FP32 accumulation rounds with a bias, so chains stay
-//     short), and releases ring slots with tcgen05.commit;
-//   * warps 2-5 drain each finished accumulator with tcgen05.ld (one TMEM
-//     lane = one row per thread) into FP32 register sums while the next ones
-//     fill; rows split between two CTAs are summed by whichever warp arrives
-//     last, in CTA order;
-//   * the number of K blocks per accumulator and the ring depth are chosen
-//     per tensor and batch width by timing candidates on first use.
+// The product is HBM-bound for B <= ~200 (96 flop per tensor byte at B = 64),
+// so the design streams the planes once per batched product:
+//   * persistent CTAs, one per SM; the (row tile, K block, plane) units are
+//     split evenly over the CTAs in storage order (stream-K);
+//   * warp 0 issues 2-D TMA loads (128-byte swizzle): a 128 x 64 plane tile
+//     (split: hi and lo together) per stage of a shared-memory ring, and the
+//     64-wide operand slices of the K block's components, each once per row
+//     tile and K block, in a ring of their own.  The first ring-full of plane
+//     tiles is issued before the wait on the kernel ahead (which writes the
+//     operand, never the tensor);
+//   * warp 1 issues tcgen05.mma (M = 128, N = B ... 3 B, K = 16, BF16 -> FP32)
+//     into one TMEM accumulator per component and K block (the tensor cores'
+//     FP32 accumulation rounds with a bias, so chains stay short: at most 192
+//     products), taken in rotation from a ring of accumulators, and releases
+//     ring slots with tcgen05.commit;
+//   * eight warps drain each finished accumulator with tcgen05.ld (one TMEM lane
+//     = one row per thread, half of the batch per warp) into FP32 register
+//     sums of the three components while the next ones fill; row tiles split
+//     between CTAs are summed by whichever warp arrives last, in CTA order;
+//   * the ring depth is chosen per tensor and batch width by timing
+//     candidates on first use.
+// Storing all 9 entries of a block moved 1.5 times the bytes (single layer:
+// 2.25 times).  Fields, before and after: n = 6,000, B = 8, BF16 110 -> 84 us
+// (product 98 -> 70, 0.92 of the copy bandwidth); n = 10,000, B = 64, BF16 328
+// -> 226 us (product 188, 0.97); split, B = 16 521 -> 370 us (product at the
+// copy bandwidth), B = 64 595 -> 537 us and at n = 20,000 2,187 -> 1,946 us:
+// there the five products of every entry bound it, 1.3 PFLOP/s.
 // Every wait is bounded; on a timeout the kernel records MT_DEV_TIMEOUT,
 // still frees its TMEM and returns.
 #include <cuda.h>
@@ -34,6 +46,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "mt_internal.cuh"
 
@@ -41,26 +54,72 @@ namespace {
 
 constexpr int GM = 128;  // rows per tile (MMA M)
 constexpr int GK = 64;   // K per ring stage: one 128-byte swizzle row of BF16
-constexpr int EPI_WARPS = 4;
-constexpr int NACC = 4;  // TMEM accumulators in flight between the MMA warp and the epilogue
+constexpr int EPI_WARPS = 8;
+constexpr int A_TILE = GM * GK * 2;  // bytes of one plane tile
 
-// The split product with a padded batch up to 64 "stacks" the three operand
-// planes x0 | x1 | x2 into one N = 3 Bp operand: one MMA gives N_hi x0,
-// N_hi x1, N_hi x2 side by side in TMEM and a second (N = 2 Bp) adds N_lo x0
-// and N_lo x1 onto the first two groups; the epilogue adds the groups in
-// FP32.  That reads each tensor tile from shared memory twice per K step
-// instead of five times (the split product was bound by the shared-memory
-// reads that feed the tensor cores).  N <= 256 limits it to Bp <= 64; wider
-// batches issue the five MMAs.
+// Shape of one batch width.  GROUPS: column groups of an accumulator (the
+// epilogue adds them).  The split product puts the operand terms side by side
+// so that a tensor tile is read from shared memory twice per K step instead of
+// five times (those reads, not the tensor pipe, would bound it):
+//   BP <= 32: N_hi [x0 | x1 | x2] (N = 3 BP) and N_lo [x0 | x1] (N = 2 BP);
+//   BP = 64:  three such groups of three components would not fit the 512 TMEM
+//             columns twice over, so N_hi [x0 | x1] and N_lo [x0 | x1]
+//             (N = 128), and N_hi x2 (N = 64) onto the second group;
+//   BP = 128: five products onto one group.
+// A ring stage holds one unit of 32 KB: a plane's hi and lo tiles, or two
+// consecutive planes' tiles (16 KB stages left the handshakes of the TMA, MMA
+// and commit path, a few hundred cycles each, above a tile's time in HBM).
+// XG: the three operand slices of a K block share a slot and its barriers
+// where two such slots fit, else each has its own.  AG: likewise the three
+// accumulators of a K block; else they are taken in rotation, at least 4 (the
+// next K block's first component starts while the last one's are drained).
 template <bool SPLIT, int BP>
 struct GemmShape {
-  static constexpr bool STACK = SPLIT && BP <= 64;
-  static constexpr int ACC_COLS = STACK ? 3 * BP : BP;  // TMEM columns of one accumulator
-  // accumulators (<= 512 TMEM columns); the BF16 product at BP <= 64 keeps 8
-  // in flight
-  static constexpr int NA = STACK ? (BP == 64 ? 2 : 4) : (BP <= 64 ? 2 * NACC : NACC);
+  static constexpr int GROUPS = !SPLIT ? 1 : BP <= 32 ? 3 : BP == 64 ? 2 : 1;
+  static constexpr int ACC_COLS = GROUPS * BP;
+  static constexpr bool AG = 512 / ACC_COLS >= 6;
+  static constexpr int NA = AG ? 2 : 512 / ACC_COLS;  // barriers: sets of three, or single accumulators
+  static constexpr int ACCS = AG ? 6 : NA;
+  static constexpr int TERMS = SPLIT ? 3 : 1;
+  static constexpr int X_SLICE = TERMS * BP * GK * 2;  // bytes: one component of one K block
+  static constexpr bool XG = !SPLIT || BP <= 32;
+  static constexpr int NX = XG ? 2 : BP == 64 ? 4 : 3;
+  static constexpr int X_SLOT = (XG ? 3 : 1) * X_SLICE;
+  static constexpr int X_ROWS = XG && !SPLIT && 3 * BP <= 256 ? 3 * BP : BP;  // rows of one operand copy
+  static constexpr int PPU = SPLIT ? 1 : 2;  // planes per unit
+  static constexpr int A_STAGE = 2 * A_TILE;
+  static constexpr int HB = BP / 2;  // simulations per epilogue warp
+  // the 3 HB register sums of an epilogue thread at BP = 128 exceed what 10
+  // warps may have (168): two warpgroups of epilogue warps then take over
+  // registers of a first one that holds the TMA and MMA warps (56 + 2 x 224 =
+  // 3 x 168)
+  static constexpr bool REGSPLIT = BP == 128;
+  static constexpr int EPI0 = REGSPLIT ? 4 : 2;  // first epilogue warp
+  static constexpr int THREADS = 32 * (EPI0 + EPI_WARPS);
+  static_assert(AG || NA >= 4, "accumulators of one K block and one spare");
 };
-constexpr int GEMM_THREADS = 32 * (2 + EPI_WARPS);
+
+// Planes in storage order (NP = 6, or 4 for a single layer): plane p couples
+// the components pc(p) <= pd(p).
+template <int NP>
+constexpr __host__ __device__ int pc(int p) {
+  return NP == 6 ? (p < 3 ? 0 : p < 5 ? 1 : 2) : (p < 2 ? 0 : p - 1);
+}
+template <int NP>
+constexpr __host__ __device__ int pd(int p) {
+  return NP == 6 ? (p < 3 ? p : p < 5 ? p - 2 : 2) : (p == 0 ? 0 : p < 3 ? 1 : 2);
+}
+// planes that a component takes part in, as a bit mask
+template <int NP>
+constexpr __host__ __device__ unsigned planes_of(int comp) {
+  return NP == 6 ? (comp == 0 ? 0b000111u : comp == 1 ? 0b011010u : 0b110100u)
+                 : (comp == 0 ? 0b0011u : comp == 1 ? 0b0110u : 0b1000u);
+}
+// does the component take part in none of the planes p + 1 .. e - 1?
+template <int NP>
+__device__ __forceinline__ bool last_plane(int comp, int p, int e) {
+  return (planes_of<NP>(comp) & ~((2u << p) - 1u) & ((1u << e) - 1u)) == 0;
+}
 
 // ---- tcgen05 / TMA wrappers -------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
@@ -76,6 +135,13 @@ __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
 
 // D (tmem) = A (smem) * B (smem) [+ D]; BF16 inputs, FP32 accumulate
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
@@ -102,6 +168,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t r[16]) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t r[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
                                        uint64_t policy) {
@@ -119,57 +190,96 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
 }
 
 struct GemmArgs {
-  int64_t n3;    // valid rows (3n)
+  int64_t n;     // tiles
   int64_t MT;    // row tiles
   int64_t KB;    // K blocks
-  int64_t KBU;   // units per row tile (a unit = KPS consecutive K blocks)
   int B, Bp;     // batch, padded batch (MMA N)
-  int chunk;     // K blocks per TMEM accumulation before the FP32 promotion
-  int stages;
-  int stage_bytes;
+  int stages;    // plane tiles in the ring
   uint32_t tmem_cols;
-  float *H;      // [B][n3]
-  float *part;   // [2G][Bp][GM]
+  float *H;      // [B][n][3]
+  float *part;   // [2G][3][Bp][GM]
   int *count;    // [MT][EPI_WARPS]
   const int *n_active;
   int *status;
 };
 
-template <bool SPLIT, int BP, int KPS>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-    k_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tAlo,
-           const __grid_constant__ CUtensorMap tX, const __grid_constant__ CUtensorMap tX1,
-           const __grid_constant__ CUtensorMap tX2, GemmArgs P) {
-  mtd::pdl_enter();
+// f(integral_constant<0>) ... f(integral_constant<N - 1>)
+template <int N, int I = 0, typename F>
+__device__ __forceinline__ void static_for(F &&f) {
+  if constexpr (I < N) {
+    f(std::integral_constant<int, I>{});
+    static_for<N, I + 1>(f);
+  }
+}
+
+// a ring position: slot and the parity of its current pass
+template <int DEPTH>
+struct RingPos {
+  uint32_t s = 0, ph = 0;
+  __device__ __forceinline__ void next(int depth = DEPTH) {
+    if (++s == (uint32_t)depth) {
+      s = 0;
+      ph ^= 1u;
+    }
+  }
+};
+
+// W consecutive columns of an accumulator, its column groups added (the small
+// ones first), onto run
+template <int W, int GROUPS, int BP>
+__device__ __forceinline__ void drain_cols(uint32_t acc, float *run) {
+  uint32_t v[GROUPS][W];
+#pragma unroll
+  for (int g = 0; g < GROUPS; ++g) {
+    if constexpr (W == 16) tmem_ld16(acc + (uint32_t)(g * BP), v[g]);
+    else tmem_ld8(acc + (uint32_t)(g * BP), v[g]);
+  }
+  tmem_wait_ld();
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    float x = __uint_as_float(v[GROUPS - 1][j]);
+#pragma unroll
+    for (int g = GROUPS - 2; g >= 0; --g) x = __uint_as_float(v[g][j]) + x;
+    run[j] += x;
+  }
+}
+
+template <bool SPLIT, int BP, int NP>
+__global__ void __launch_bounds__(GemmShape<SPLIT, BP>::THREADS, 1)
+    k_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tX, GemmArgs P) {
+  using SH = GemmShape<SPLIT, BP>;
+  constexpr int NA = SH::NA, NX = SH::NX, HB = SH::HB;
+  constexpr int NU = NP / SH::PPU;  // units of a (row tile, K block)
   extern __shared__ unsigned char smem_raw[];
-  // 1024-byte aligned base for the swizzled tiles
+  // 1024-byte aligned base for the swizzled tiles: the plane tiles, the
+  // operand slices, the barriers
   const uint32_t raw = mtd::smem_u32(smem_raw);
   unsigned char *smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  const int A_BYTES = GM * GK * 2;
-  const int X_BYTES = P.Bp * GK * 2;
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + (size_t)P.stages * P.stage_bytes);
+  unsigned char *smem_x = smem + (size_t)P.stages * SH::A_STAGE;
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem_x + NX * SH::X_SLOT);
   uint64_t *empty = full + P.stages;
-  uint64_t *accf = empty + P.stages;
-  using SH = GemmShape<SPLIT, BP>;
-  constexpr int NA = SH::NA;
+  uint64_t *xfull = empty + P.stages;
+  uint64_t *xempty = xfull + NX;
+  uint64_t *accf = xempty + NX;
   uint64_t *acce = accf + NA;
   uint64_t *mma_done = acce + NA;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (the same value in a form the compiler knows to be uniform)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int64_t G = gridDim.x, k = blockIdx.x;
-  // a unit is KPS consecutive K blocks of one row tile; a ring stage holds
-  // one unit: KPS sub-blocks of [A (| x0 | A_lo | x1 | x2) | X]
-  const int SB = SPLIT ? 2 * A_BYTES + 3 * X_BYTES : A_BYTES + X_BYTES;
-  const int64_t U = P.MT * P.KBU;
+  const int64_t U = P.MT * P.KB * NU;
   const int64_t u0 = mtd::sk_begin(k, U, G), u1 = mtd::sk_begin(k + 1, U, G);
-  const bool idle = P.n_active && *P.n_active == 0;  // every simulation finished
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < P.stages; ++s) {
       mtd::mbar_init(&full[s], 1);
       mtd::mbar_init(&empty[s], 1);
+    }
+    for (int s = 0; s < NX; ++s) {
+      mtd::mbar_init(&xfull[s], 1);
+      mtd::mbar_init(&xempty[s], 1);
     }
     for (int a = 0; a < NA; ++a) {
       mtd::mbar_init(&accf[a], 1);
@@ -184,216 +294,354 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // unit u into ring stage s
+  auto load_a = [&](int64_t u, int s, uint64_t pol) {
+    mtd::mbar_arrive_expect_tx(&full[s], SH::A_STAGE);
+    tma_2d(smem + (size_t)s * SH::A_STAGE, &tA, 0, (int)(u * 2 * GM), &full[s], pol);
+  };
+  const int pre = (int)(u1 - u0 < P.stages ? u1 - u0 : P.stages);
+  if (warp == 0 && elect_one()) {
+    const uint64_t pol = mtd::policy_evict_first();
+    for (int s = 0; s < pre; ++s) load_a(u0 + s, s, pol);
+  }
+  __syncwarp();
+  mtd::pdl_enter();
+  const bool idle = P.n_active && *P.n_active == 0;  // every simulation finished
 
-  if (!idle && warp == 0 && lane == 0) {
-    // ---------------- TMA producer ----------------
-    const uint64_t pol_stream = mtd::policy_evict_first();
-    const uint64_t pol_keep = mtd::policy_evict_last();
-    int it = 0;
-    for (int64_t u = u0; u < u1; ++u, ++it) {
-      const int64_t mt = u / P.KBU, kbu = u - mt * P.KBU;
-      const int s = it % P.stages;
-      const uint32_t ph = (uint32_t)(it / P.stages) & 1u;
-      if (it >= P.stages && (*abort_flag || !mtd::mbar_wait_bounded(&empty[s], ph ^ 1u, P.status))) {
-        *abort_flag = 1;
-        break;
-      }
-      unsigned char *st = smem + (size_t)s * P.stage_bytes;
-      mtd::mbar_arrive_expect_tx(&full[s], (uint32_t)(KPS * SB));
-#pragma unroll
-      for (int q = 0; q < KPS; ++q) {
-        // tile (mt, kb) is one contiguous 16 KB block; X block kb likewise
-        const int64_t kb = kbu * KPS + q;
-        const int ya = (int)((mt * P.KB + kb) * GM), yx = (int)(kb * P.Bp);
-        unsigned char *sb = st + q * SB;
-        tma_2d(sb, &tA, 0, ya, &full[s], pol_stream);
-        if (SPLIT) {
-          // sub-block: A_hi | A_lo | x0 | x1 | x2 (the planes of x adjacent:
-          // one 3 Bp-row operand)
-          tma_2d(sb + A_BYTES, &tAlo, 0, ya, &full[s], pol_stream);
-          tma_2d(sb + 2 * A_BYTES, &tX, 0, yx, &full[s], pol_keep);
-          tma_2d(sb + 2 * A_BYTES + X_BYTES, &tX1, 0, yx, &full[s], pol_keep);
-          tma_2d(sb + 2 * A_BYTES + 2 * X_BYTES, &tX2, 0, yx, &full[s], pol_keep);
-        } else {
-          tma_2d(sb + A_BYTES, &tX, 0, yx, &full[s], pol_keep);
-        }
-      }
-    }
-    // drain: every copy issued must have landed before the CTA may exit
-    for (int s = 0; s < P.stages && s < it; ++s) {
-      const int last = it - 1 - ((it - 1 - s) % P.stages);  // last issue on stage s
-      mtd::mbar_wait_bounded(&full[s], (uint32_t)(last / P.stages) & 1u, P.status);
-    }
-  } else if (!idle && warp == 1 && lane == 0) {
-    // ---------------- MMA issuer ----------------
-    const uint32_t idesc = (1u << 4)                       // D: FP32
-                           | (1u << 7) | (1u << 10)        // A, B: BF16
-                           | ((uint32_t)(P.Bp >> 3) << 17)  // N
-                           | ((uint32_t)(GM >> 4) << 24);   // M
-    // stacked split: N = 3 Bp (N_hi [x0 | x1 | x2]) and N = 2 Bp (N_lo [x0 | x1])
-    const uint32_t idesc3 = (idesc & ~(0x3Fu << 17)) | ((uint32_t)((3 * BP) >> 3) << 17);
-    const uint32_t idesc2 = (idesc & ~(0x3Fu << 17)) | ((uint32_t)((2 * BP) >> 3) << 17);
-    // The tensor cores' FP32 accumulation rounds with a bias, so a product
-    // is accumulated in TMEM over at most P.chunk K blocks and then handed to
-    // the epilogue, which adds the chunks in FP32 (round to nearest).
-    int it = 0, chunk = 0;
-    bool issued = false;
-    int64_t u = u0;
-    while (u < u1 && !*abort_flag) {
-      const int64_t mt = u / P.KBU;
-      const int64_t seg_end = u1 < (mt + 1) * P.KBU ? u1 : (mt + 1) * P.KBU;
-      while (u < seg_end && !*abort_flag) {
-        const int64_t c_end = seg_end < u + P.chunk ? seg_end : u + P.chunk;
-        const int a = chunk % NA;
-        if (chunk >= NA && !mtd::mbar_wait_bounded(&acce[a], (uint32_t)(chunk / NA - 1) & 1u, P.status)) {
+  if (warp < SH::EPI0) {
+    if constexpr (SH::REGSPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    // (One thread each issues the copies and the products, and a few hundred
+    // dependent instructions per plane tile would already exceed the tile's
+    // time in HBM: the planes are unrolled, ring positions counted, and the
+    // whole MMA warp walks the units, so that descriptors and addresses stay
+    // in uniform registers, as the instruction takes them.)
+    if (warp == 0) {
+      // ---------------- TMA producer ----------------
+      const bool leader = elect_one();
+      const uint64_t pol_stream = mtd::policy_evict_first();
+      const uint64_t pol_keep = mtd::policy_evict_last();
+      RingPos<0> a;
+      RingPos<NX> x;
+      int it = 0, xi = 0;
+      bool stop = idle;
+      int64_t kb = (u0 / NU) % P.KB;
+      int e0 = (int)(u0 % NU);
+      auto wait = [&](uint64_t *bar, uint32_t parity) {
+        if (*abort_flag || !mtd::mbar_wait_bounded(bar, parity, P.status)) {
           *abort_flag = 1;
-          break;
+          stop = true;
         }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(a * SH::ACC_COLS);
-        bool first = true;
-        for (; u < c_end; ++u, ++it) {
-          const int s = it % P.stages;
-          const uint32_t ph = (uint32_t)(it / P.stages) & 1u;
-          if (*abort_flag || !mtd::mbar_wait_bounded(&full[s], ph, P.status)) {
-            *abort_flag = 1;
-            break;
+      };
+      // operand rows of (term t, K block kb, component c): ((t KB + kb) 3 + c) Bp
+      auto copy_x = [&](uint32_t off, int t, int c) {
+        tma_2d(smem_x + x.s * SH::X_SLOT + off, &tX, 0, (int)(((t * P.KB + kb) * 3 + c) * BP), &xfull[x.s], pol_keep);
+      };
+      for (int64_t u = u0; u < u1 && !stop;) {
+        const int e1 = u1 - u < NU - e0 ? e0 + (int)(u1 - u) : NU;
+        unsigned have = 0;  // components whose slice is loaded
+        auto slice = [&](int comp) {
+          if (have >> comp & 1 || stop) return;
+          have |= SH::XG ? 7u : 1u << comp;
+          wait(&xempty[x.s], x.ph ^ 1u);  // (passes on the first round)
+          if (stop) return;
+          if (leader) {
+            mtd::mbar_arrive_expect_tx(&xfull[x.s], SH::X_SLOT);
+            constexpr int TB = BP * GK * 2;  // bytes of one operand term
+            if constexpr (SH::X_ROWS > BP) {
+              copy_x(0, 0, 0);
+            } else if constexpr (SH::XG) {
+#pragma unroll
+              for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int t = 0; t < SH::TERMS; ++t) copy_x(c * SH::X_SLICE + t * TB, t, c);
+            } else {
+#pragma unroll
+              for (int t = 0; t < SH::TERMS; ++t) copy_x(t * TB, t, comp);
+            }
+          }
+          x.next();
+          ++xi;
+        };
+        static_for<NU>([&](auto uu) {
+          constexpr int p0 = uu * SH::PPU;
+          if (uu < e0 || uu >= e1 || stop) return;
+          static_for<SH::PPU>([&](auto r) {
+            slice(pc<NP>(p0 + r));
+            slice(pd<NP>(p0 + r));
+          });
+          if (!stop && it >= pre) {
+            wait(&empty[a.s], a.ph ^ 1u);
+            if (!stop && leader) load_a(u + (uu - e0), (int)a.s, pol_stream);
+          }
+          if (!stop) {
+            ++it;
+            a.next(P.stages);
+          }
+        });
+        u += e1 - e0;
+        e0 = 0;
+        if (++kb == P.KB) kb = 0;
+      }
+      // drain: every copy issued must have landed before the CTA may exit
+      it = it > pre ? it : pre;
+      for (int s = 0; s < P.stages && s < it; ++s) {
+        const int last = it - 1 - ((it - 1 - s) % P.stages);  // last issue on stage s
+        mtd::mbar_wait_bounded(&full[s], (uint32_t)(last / P.stages) & 1u, P.status);
+      }
+      for (int s = 0; s < NX && s < xi; ++s) {
+        const int last = xi - 1 - ((xi - 1 - s) % NX);
+        mtd::mbar_wait_bounded(&xfull[s], (uint32_t)(last / NX) & 1u, P.status);
+      }
+    } else if (!idle && warp == 1) {
+      // ---------------- MMA issuer ----------------
+      // D: FP32; A, B: BF16; M = 128; N in units of 8 columns
+      constexpr uint32_t id0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GM >> 4) << 24);
+      constexpr uint32_t id1 = id0 | ((uint32_t)(BP >> 3) << 17), id2 = id0 | ((uint32_t)(2 * BP >> 3) << 17),
+                         id3 = id0 | ((uint32_t)(3 * BP >> 3) << 17);
+      const uint64_t da0 = sw128_desc(mtd::smem_u32(smem)), dx0 = sw128_desc(mtd::smem_u32(smem_x));
+      const bool leader = elect_one();
+      RingPos<0> a;
+      RingPos<NX> x;
+      RingPos<NA> c;
+      bool issued = false, ok = true;
+      int e0 = (int)(u0 % NU);
+      for (int64_t u = u0; u < u1 && ok;) {
+        const int e1 = u1 - u < NU - e0 ? e0 + (int)(u1 - u) : NU;
+        // per component: its operand (offset in the descriptor), its accumulator
+        // (column), its barriers
+        uint32_t opnd[3] = {0, 0, 0}, acc[3] = {0, 0, 0}, xbar[3] = {0, 0, 0}, abar[3] = {0, 0, 0};
+        unsigned have = 0, begun = 0;
+        // a component's first plane: its operand has arrived, an accumulator is free
+        auto begin = [&](auto comp) {
+          if (!SH::XG || have == 0) ok = ok && mtd::mbar_wait_bounded(&xfull[x.s], x.ph, P.status);
+          if (!SH::AG || have == 0)
+            ok = ok && mtd::mbar_wait_bounded(&acce[c.s], c.ph ^ 1u, P.status);  // (passes on the first round)
+          opnd[comp] = (x.s * SH::X_SLOT + (SH::XG ? comp * SH::X_SLICE : 0)) >> 4;
+          acc[comp] = (SH::AG ? 3 * c.s + comp : c.s) * SH::ACC_COLS;
+          xbar[comp] = x.s;
+          abar[comp] = c.s;
+          have |= 1u << comp;
+          if (!SH::XG) x.next();
+          if (!SH::AG) c.next();
+        };
+        static_for<NU>([&](auto uu) {
+          if (uu < e0 || uu >= e1 || !ok) return;
+          static_for<SH::PPU>([&](auto r) {
+            constexpr int p = uu * SH::PPU + r;
+            constexpr std::integral_constant<int, pc<NP>(p)> pa{};
+            constexpr std::integral_constant<int, pd<NP>(p)> pb{};
+            if (!(have >> pa & 1)) begin(pa);
+            if (!(have >> pb & 1)) begin(pb);
+          });
+          if (!ok || *abort_flag || !mtd::mbar_wait_bounded(&full[a.s], a.ph, P.status)) {
+            ok = false;
+            return;
           }
           tc_fence_after();
-          const uint32_t st = mtd::smem_u32(smem + (size_t)s * P.stage_bytes);
-#pragma unroll
-          for (int q = 0; q < KPS; ++q) {
-            const uint32_t sa = st + q * SB;
-#pragma unroll
-            for (int kk = 0; kk < GK / 16; ++kk) {
-              // K advance inside the 128-byte swizzle row: 16 BF16 = 32 bytes
-              const uint64_t da = sw128_desc(sa + 32 * kk);
-              if (!SPLIT) {
-                umma_bf16(d_tmem, da, sw128_desc(sa + A_BYTES + 32 * kk), idesc, first ? 0u : 1u);
-              } else if (SH::STACK) {
-                const uint32_t salo = sa + A_BYTES, sx = salo + A_BYTES;
-                const uint64_t dx = sw128_desc(sx + 32 * kk);
-                umma_bf16(d_tmem, da, dx, idesc3, first ? 0u : 1u);                  // N_hi [x0 | x1 | x2]
-                umma_bf16(d_tmem, sw128_desc(salo + 32 * kk), dx, idesc2, 1u);       // N_lo [x0 | x1]
-              } else {
-                const uint32_t salo = sa + A_BYTES, sx = salo + A_BYTES, sx1 = sx + X_BYTES, sx2 = sx1 + X_BYTES;
-                const uint64_t dx = sw128_desc(sx + 32 * kk), d1 = sw128_desc(sx1 + 32 * kk);
-                const uint64_t dlo = sw128_desc(salo + 32 * kk);
-                umma_bf16(d_tmem, da, dx, idesc, first ? 0u : 1u);            // N_hi x0
-                umma_bf16(d_tmem, da, d1, idesc, 1u);                         // N_hi x1
-                umma_bf16(d_tmem, da, sw128_desc(sx2 + 32 * kk), idesc, 1u);  // N_hi x2
-                umma_bf16(d_tmem, dlo, dx, idesc, 1u);                        // N_lo x0
-                umma_bf16(d_tmem, dlo, d1, idesc, 1u);                        // N_lo x1
+          static_for<SH::PPU>([&](auto r) {
+            constexpr int p = uu * SH::PPU + r;
+            constexpr std::integral_constant<int, pc<NP>(p)> pa{};
+            constexpr std::integral_constant<int, pd<NP>(p)> pb{};
+            const uint64_t da = da0 + ((a.s * SH::A_STAGE + (SPLIT ? 0 : r * A_TILE)) >> 4);
+            // the plane times one component's operand, onto the other's accumulator
+            auto product = [&](uint32_t to, uint32_t from, uint32_t keep) {
+              const uint32_t dt = tmem_base + to;
+              const uint64_t dx = dx0 + from;
+              if (!leader) return;
+  #pragma unroll
+              for (int kk = 0; kk < GK / 16; ++kk) {
+                // K advance inside the 128-byte swizzle row: 16 BF16 = 32 bytes
+                const uint64_t dak = da + 2 * kk, dxk = dx + 2 * kk;
+                const uint32_t k0 = kk == 0 ? keep : 1u;  // 0: the accumulator's first product
+                if constexpr (!SPLIT) {
+                  umma_bf16(dt, dak, dxk, id1, k0);
+                } else {
+                  const uint64_t dlo = dak + (A_TILE >> 4);
+                  constexpr int TB = (BP * GK * 2) >> 4;  // one operand term
+                  if constexpr (SH::GROUPS == 3) {
+                    umma_bf16(dt, dak, dxk, id3, k0);  // N_hi [x0 | x1 | x2]
+                    umma_bf16(dt, dlo, dxk, id2, 1u);  // N_lo [x0 | x1]
+                  } else if constexpr (SH::GROUPS == 2) {
+                    umma_bf16(dt, dak, dxk, id2, k0);                // N_hi [x0 | x1]
+                    umma_bf16(dt + BP, dak, dxk + 2 * TB, id1, 1u);  // N_hi x2
+                    umma_bf16(dt, dlo, dxk, id2, 1u);                // N_lo [x0 | x1]
+                  } else {
+                    umma_bf16(dt, dak, dxk, id1, k0);           // N_hi x0
+                    umma_bf16(dt, dak, dxk + TB, id1, 1u);      // N_hi x1
+                    umma_bf16(dt, dak, dxk + 2 * TB, id1, 1u);  // N_hi x2
+                    umma_bf16(dt, dlo, dxk, id1, 1u);           // N_lo x0
+                    umma_bf16(dt, dlo, dxk + TB, id1, 1u);      // N_lo x1
+                  }
+                }
               }
-              first = false;
-            }
-          }
+            };
+            product(acc[pa], opnd[pb], begun >> pa & 1);
+            if constexpr (pa != pb) product(acc[pb], opnd[pa], begun >> pb & 1);
+            begun |= 1u << pa | 1u << pb;
+          });
           issued = true;
-          umma_commit(&empty[s]);  // ring slot free once these MMAs are done
+          if (leader) umma_commit(&empty[a.s]);  // ring slot free once these MMAs are done
+          a.next(P.stages);
+          // a component's last plane: its slice is free, its accumulator complete
+          static_for<3>([&](auto comp) {
+            constexpr int pe = uu * SH::PPU + SH::PPU;  // planes so far
+            if (!leader || !(planes_of<NP>(comp) >> (pe - SH::PPU) & ((1u << SH::PPU) - 1u)) ||
+                !last_plane<NP>(comp, pe - 1, e1 * SH::PPU))
+              return;
+            if (!SH::XG) umma_commit(&xempty[xbar[comp]]);
+            if (!SH::AG) umma_commit(&accf[abar[comp]]);
+          });
+        });
+        if (!ok) break;
+        if (SH::XG) {
+          if (leader) umma_commit(&xempty[x.s]);
+          x.next();
         }
-        umma_commit(&accf[a]);  // accumulator a holds the chunk
-        ++chunk;
+        if (SH::AG) {
+          if (leader) umma_commit(&accf[c.s]);
+          c.next();
+        }
+        u += e1 - e0;
+        e0 = 0;
+      }
+      if (!ok) *abort_flag = 1;
+      if (leader) {
+        if (issued) umma_commit(mma_done);
+        else mtd::mbar_arrive(mma_done);
       }
     }
-    if (issued) umma_commit(mma_done);
-    else mtd::mbar_arrive(mma_done);
-  } else if (!idle && warp >= 2) {
-    // ---------------- epilogue ----------------
-    const int g = warp & 3;  // TMEM lane group accessible to this warp
-    const int row = g * 32 + lane;
-    const int64_t first_mt = u0 / P.KBU;
-    int chunk = 0;
-    int64_t u = u0;
-    float run[BP];  // FP32 sum of the chunks of the current row tile
-    while (u < u1) {
-      const int64_t mt = u / P.KBU;
-      const int64_t seg_end = u1 < (mt + 1) * P.KBU ? u1 : (mt + 1) * P.KBU;
+  } else {
+    if constexpr (SH::REGSPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+    if (!idle) {
+      // ---------------- epilogue ----------------
+      const int e = warp - SH::EPI0;
+      const int lg = warp & 3;           // TMEM lane group accessible to this warp
+      const int b0 = (e >> 2) * HB;      // this warp's half of the batch
+      const int row = lg * 32 + lane;
+      const int64_t KBU = P.KB * NU;
+      const int64_t first_mt = u0 / KBU;
+      RingPos<NA> c;
+      float run[3][HB];  // FP32 sums of the current row tile
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int j = 0; j < HB; ++j) run[q][j] = 0.0f;
       bool ok = true;
-      bool first_chunk = true;
-      while (u < seg_end) {
-        u = seg_end < u + P.chunk ? seg_end : u + P.chunk;
-        const int a = chunk % NA;
-        const bool got = !*abort_flag && mtd::mbar_wait_bounded(&accf[a], (uint32_t)(chunk / NA) & 1u, P.status);
-        if (!got) {
-          *abort_flag = 1;
-          ok = false;
-        }
-        tc_fence_after();
-        const uint32_t acc = tmem_base + ((uint32_t)(g * 32) << 16) + (uint32_t)(a * SH::ACC_COLS);
-        if (SH::STACK) {
-          // the three column groups x0, x1, x2 of each 16-column piece, the
-          // two small ones added first
-#pragma unroll
-          for (int c0 = 0; c0 < BP; c0 += 16) {
-            uint32_t v0[16], v1[16], v2[16];
-            tmem_ld16(acc + (uint32_t)c0, v0);
-            tmem_ld16(acc + (uint32_t)(BP + c0), v1);
-            tmem_ld16(acc + (uint32_t)(2 * BP + c0), v2);
-            tmem_wait_ld();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float x = __uint_as_float(v0[j]) + (__uint_as_float(v1[j]) + __uint_as_float(v2[j]));
-              run[c0 + j] = first_chunk ? x : run[c0 + j] + x;
+      int64_t mt = first_mt, kb = (u0 / NU) % P.KB;
+      int e0 = (int)(u0 % NU);
+      for (int64_t u = u0; u < u1 && ok;) {
+        const int e1 = u1 - u < NU - e0 ? e0 + (int)(u1 - u) : NU;
+        // components in the order the MMA warp takes their accumulators (4 bits
+        // each, + 1): x, y, z of a whole K block; of a partial one the planes tell
+        unsigned order = 0x321;
+        if (e0 != 0 || e1 != NU) {
+          unsigned have = 0;
+          int cnt = 0;
+          order = 0;
+#pragma unroll 1
+          for (int p = e0 * SH::PPU; p < e1 * SH::PPU; ++p)
+#pragma unroll 1
+            for (int side = 0; side < 2; ++side) {
+              const int comp = side ? pd<NP>(p) : pc<NP>(p);
+              if (have >> comp & 1) continue;
+              have |= 1u << comp;
+              order |= (unsigned)(comp + 1) << (4 * cnt++);
             }
+        }
+        bool first = true;
+#pragma unroll 1
+        for (; order && ok; order >>= 4) {
+          if (!SH::AG || first) {
+            if (!mtd::mbar_wait_warp_relaxed(&accf[c.s], c.ph, P.status) || *abort_flag) {
+              *abort_flag = 1;
+              ok = false;
+              break;
+            }
+            tc_fence_after();
           }
+          first = false;
+          const int comp = (int)(order & 15u) - 1;
+          const uint32_t acc = tmem_base + ((uint32_t)(lg * 32) << 16) +
+                               (uint32_t)((SH::AG ? 3 * c.s + comp : c.s) * SH::ACC_COLS + b0);
+          constexpr int W = HB < 16 ? HB : 16;
+          static_for<3>([&](auto q) {
+            if (comp != q) return;
+#pragma unroll
+            for (int c0 = 0; c0 < HB; c0 += W) drain_cols<W, SH::GROUPS, BP>(acc + (uint32_t)c0, &run[q][c0]);
+          });
+          if (!SH::AG || (order >> 4) == 0) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mtd::mbar_arrive(&acce[c.s]);
+            c.next();
+          }
+        }
+        if (!ok) break;
+        u += e1 - e0;
+        const bool tile_ends = u == u1 || (kb == P.KB - 1 && e1 == NU);
+        e0 = 0;
+        if (!tile_ends) {
+          ++kb;
+          continue;
+        }
+        const int64_t next_mt = mt + 1;
+        kb = 0;
+        // the row tile's sums (this CTA's share of them)
+        const int64_t kf = mtd::sk_owner(mt * KBU, U, G), kl = mtd::sk_owner(mt * KBU + KBU - 1, U, G);
+        const int64_t r = mt * GM + row;
+        const int nb = P.B - b0 < HB ? P.B - b0 : HB;  // simulations of this warp (may be <= 0)
+        if (kf == kl) {
+#pragma unroll
+          for (int j = 0; j < HB; ++j)
+            if (j < nb && r < P.n)
+#pragma unroll
+              for (int q = 0; q < 3; ++q) P.H[((size_t)(b0 + j) * P.n + r) * 3 + q] = -run[q][j];
         } else {
-          // all loads of the accumulator in flight at once, one wait
-          uint32_t v[BP];
+          const int64_t slot = (mt == first_mt) ? 2 * k : 2 * k + 1;
 #pragma unroll
-          for (int c0 = 0; c0 < BP; c0 += 16) tmem_ld16(acc + (uint32_t)c0, &v[c0]);
-          tmem_wait_ld();
+          for (int q = 0; q < 3; ++q)
 #pragma unroll
-          for (int j = 0; j < BP; ++j)
-            run[j] = first_chunk ? __uint_as_float(v[j]) : run[j] + __uint_as_float(v[j]);
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mtd::mbar_arrive(&acce[a]);
-        first_chunk = false;
-        ++chunk;
-      }
-      if (!ok) continue;
-      const int64_t kf = mtd::sk_owner(mt * P.KBU, U, G), kl = mtd::sk_owner(mt * P.KBU + P.KBU - 1, U, G);
-      const int64_t r = mt * GM + row;
-      if (kf == kl) {
+            for (int j = 0; j < HB; ++j) P.part[(((size_t)slot * 3 + q) * BP + b0 + j) * GM + row] = run[q][j];
+          __threadfence();
+          __syncwarp();
+          int last = 0;
+          if (lane == 0) last = (atomicAdd(&P.count[mt * EPI_WARPS + e], 1) == (int)(kl - kf));
+          last = __shfl_sync(0xffffffffu, last, 0);
+          if (last) {
+            __threadfence();
+            // 8 simulations at a time: all their parts loaded (in CTA order per
+            // value) before their stores to H, which the compiler cannot move
+            // loads across
+            for (int j0 = 0; j0 < nb; j0 += 8) {
+              float tot[3][8];
 #pragma unroll
-        for (int b = 0; b < BP; ++b)
-          if (b < P.B && r < P.n3) P.H[(size_t)b * P.n3 + r] = -run[b];
-        continue;
-      }
-      const int64_t slot = (mt == first_mt) ? 2 * k : 2 * k + 1;
+              for (int q = 0; q < 3; ++q)
 #pragma unroll
-      for (int b = 0; b < BP; ++b) P.part[((size_t)slot * BP + b) * GM + row] = run[b];
-      __threadfence();
-      __syncwarp();
-      int last = 0;
-      if (lane == 0) {
-        const int old = atomicAdd(&P.count[mt * EPI_WARPS + g], 1);
-        last = (old == (int)(kl - kf));
-      }
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (last) {
-        __threadfence();
-        // 16 simulations at a time: all their parts loaded (in CTA order per
-        // simulation) before their stores to H, which the compiler cannot
-        // move loads across
-        for (int b0 = 0; b0 < P.B; b0 += 16) {
-          float tot[16];
+                for (int j = 0; j < 8; ++j) tot[q][j] = 0.0f;
+              for (int64_t kk = kf; kk <= kl; ++kk) {
+                const int64_t fm = mtd::sk_begin(kk, U, G) / KBU;
+                const int64_t sl = (mt == fm) ? 2 * kk : 2 * kk + 1;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) tot[j] = 0.0f;
-          for (int64_t kk = kf; kk <= kl; ++kk) {
-            const int64_t fm = mtd::sk_begin(kk, U, G) / P.KBU;
-            const int64_t sl = (mt == fm) ? 2 * kk : 2 * kk + 1;
+                for (int q = 0; q < 3; ++q)
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (b0 + j < P.B) tot[j] += __ldcg(&P.part[((size_t)sl * BP + b0 + j) * GM + row]);
+                  for (int j = 0; j < 8; ++j)
+                    if (j0 + j < nb) tot[q][j] += __ldcg(&P.part[(((size_t)sl * 3 + q) * BP + b0 + j0 + j) * GM + row]);
+              }
+              if (r < P.n)
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                  if (j0 + j < nb)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) P.H[((size_t)(b0 + j0 + j) * P.n + r) * 3 + q] = -tot[q][j];
+            }
+            if (lane == 0) P.count[mt * EPI_WARPS + e] = 0;
           }
-          if (r < P.n3)
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (b0 + j < P.B) P.H[(size_t)(b0 + j) * P.n3 + r] = -tot[j];
         }
-        if (lane == 0) P.count[mt * EPI_WARPS + g] = 0;
+        mt = next_mt;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+          for (int j = 0; j < HB; ++j) run[q][j] = 0.0f;
       }
     }
   }
@@ -405,28 +653,55 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   }
 }
 
-// X[b][c] = BF16(Ms_j m_j[a]) for c = 3j + a (zero for padding), and the
-// low part X_lo = BF16(x - X_hi) for the split product
-__global__ void k_prep_dense_x(const float *m, const float *Ms, int64_t n, int64_t Kp, int B, int Bp,
-                               __nv_bfloat16 *X, __nv_bfloat16 *X1, __nv_bfloat16 *X2, float *mT) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int b = blockIdx.y;
-  if (t >= Kp) return;
-  float x = 0.0f;
-  if (t < 3 * n) {
-    const float mv = m[(size_t)b * 3 * n + t];
-    x = Ms[t / 3] * mv;
-    mT[(size_t)t * Bp + b] = mv;
+// Operand of the batch: X_c[b][j] = BF16(Ms_j m_j,c), for the split product
+// with the two further terms x1, x2 of x = x0 + x1 + x2 (zero for padding), and
+// the simulation-fastest copy of m for the near blocks, mT[(3 j + c) Bp + b].
+// A CTA takes the 64 tiles of one K block and up to 32 simulations through
+// shared memory, so that both sides of the transposition are whole rows: a warp
+// reads a simulation's 192 floats, writes rows of 64 BF16, and rows of 32
+// simulations of mT.  n = 20,000, B = 64, split: 28.5 us with one thread per
+// value (mT stored with a stride), 12.1 with this.
+constexpr int kPrepSims = 32, kPrepWarps = 8;
+__global__ void __launch_bounds__(32 * kPrepWarps) k_prep_dense_x(const float *m, const float *Ms, int64_t n,
+                                                                  int64_t KB, int B, int Bp, int terms,
+                                                                  __nv_bfloat16 *X, float *mT) {
+  __shared__ float sm[kPrepSims][3 * GK + 1];
+  const int64_t kb = blockIdx.x, j0 = kb * GK;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int b0 = blockIdx.y * kPrepSims, nb = B - b0 < kPrepSims ? B - b0 : kPrepSims;
+  const int cols = (int)(n - j0 < GK ? n - j0 : GK);  // tiles of this block (may be <= 0: padding)
+  const float ms[2] = {2 * lane < cols ? Ms[j0 + 2 * lane] : 0.0f, 2 * lane + 1 < cols ? Ms[j0 + 2 * lane + 1] : 0.0f};
+#pragma unroll
+  for (int q = 0; q < kPrepSims / kPrepWarps; ++q) {
+    const int b = w + kPrepWarps * q;
+    if (b >= nb) break;
+    const float *src = m + (size_t)(b0 + b) * 3 * n + 3 * j0;
+#pragma unroll
+    for (int t = lane; t < 3 * GK; t += 32) sm[b][t] = t < 3 * cols ? src[t] : 0.0f;
   }
-  const __nv_bfloat16 hi = __float2bfloat16(x);
-  const size_t at = dense_x_index(b, t, Bp);
-  X[at] = hi;
-  if (X1) {  // three-term split x = x0 + x1 + x2
-    const float r = x - __bfloat162float(hi);
-    const __nv_bfloat16 mid = __float2bfloat16(r);
-    X1[at] = mid;
-    X2[at] = __float2bfloat16(r - __bfloat162float(mid));
+  __syncthreads();
+  const size_t term = (size_t)3 * KB * Bp * GK;
+#pragma unroll
+  for (int q = 0; q < kPrepSims / kPrepWarps; ++q) {
+    const int b = w + kPrepWarps * q;
+    if (b >= nb) break;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      __nv_bfloat162 *dst = reinterpret_cast<__nv_bfloat162 *>(X + dense_x_index(c, b0 + b, j0 + 2 * lane, Bp));
+      float x[2] = {ms[0] * sm[b][6 * lane + c], ms[1] * sm[b][6 * lane + 3 + c]};
+      __nv_bfloat162 hi = __floats2bfloat162_rn(x[0], x[1]);
+      dst[0] = hi;
+      for (int t = 1; t < terms; ++t) {
+        x[0] -= __bfloat162float(hi.x);
+        x[1] -= __bfloat162float(hi.y);
+        hi = __floats2bfloat162_rn(x[0], x[1]);
+        dst[t * term / 2] = hi;
+      }
+    }
   }
+  if (lane < nb)
+#pragma unroll 4
+    for (int t = w; t < 3 * cols; t += kPrepWarps) mT[(size_t)(3 * j0 + t) * Bp + b0 + lane] = sm[lane][t];
 }
 
 using EncodeFn = PFN_cuTensorMapEncodeTiled_v12000;
@@ -459,20 +734,44 @@ mt_status make_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t r
   return MT_OK;
 }
 
-// Tile shape along K: the K blocks (64 columns each) one ring stage holds,
-// 1 or 2 (a stage of 16 or 32 KB of tensor per plane), chosen by the
-// autotuner together with the ring depth; the split product at a padded
-// batch of 128 holds one (two would need 160 KB a stage: no room for two).
-constexpr int kps_max(bool split, int Bp) { return split && Bp > 64 ? 1 : 2; }
-
-int stage_bytes_for(int Bp, bool split, int kps) {
-  return kps * (split ? 2 * GM * GK * 2 + 3 * Bp * GK * 2 : GM * GK * 2 + Bp * GK * 2);
+// ring depth in plane tiles: what fits beside the operand slices
+template <bool SPLIT, int BP>
+constexpr int stages_max() {
+  using SH = GemmShape<SPLIT, BP>;
+  constexpr int fit = (224 * 1024 - SH::NX * SH::X_SLOT) / SH::A_STAGE;
+  static_assert(fit >= 2, "at least a double-buffered ring");
+  return fit < 12 ? fit : 12;
 }
+template <bool SPLIT, int BP>
+constexpr size_t smem_for(int stages) {  // + alignment slack, barriers
+  using SH = GemmShape<SPLIT, BP>;
+  return (size_t)stages * SH::A_STAGE + SH::NX * SH::X_SLOT + 1024 + 512;
+}
+static_assert(8 * (2 * 12 + 2 * 6 + 2 * 8 + 1) + 8 <= 512, "barriers");
 
-int stages_for(int Bp, bool split, int kps) {
-  const int stage = stage_bytes_for(Bp, split, kps);
-  const int budget = 224 * 1024;
-  return std::max(2, std::min(8, budget / stage));  // >= 2 stages always fit (stage <= 112 KB)
+using GemmKernel = void (*)(const CUtensorMap, const CUtensorMap, GemmArgs);
+struct GemmVariant {
+  GemmKernel kernel;
+  int stages, x_rows, planes_per_unit;
+  size_t stage_bytes, fixed_bytes;
+  uint32_t tmem_cols;
+  int threads;
+};
+template <bool SPLIT, int BP>
+GemmVariant variant(int np) {
+  using SH = GemmShape<SPLIT, BP>;
+  uint32_t cols = 32;
+  while (cols < (uint32_t)(SH::ACCS * SH::ACC_COLS)) cols <<= 1;
+  return {np == 6 ? k_gemm<SPLIT, BP, 6> : k_gemm<SPLIT, BP, 4>, stages_max<SPLIT, BP>(), SH::X_ROWS, SH::PPU, (size_t)SH::A_STAGE, smem_for<SPLIT, BP>(0), cols,
+          SH::THREADS};
+}
+GemmVariant gemm_variant(bool split, int Bp, int np) {
+  switch (Bp) {
+    case 16: return split ? variant<true, 16>(np) : variant<false, 16>(np);
+    case 32: return split ? variant<true, 32>(np) : variant<false, 32>(np);
+    case 64: return split ? variant<true, 64>(np) : variant<false, 64>(np);
+    default: return split ? variant<true, 128>(np) : variant<false, 128>(np);
+  }
 }
 
 }  // namespace
@@ -486,192 +785,118 @@ int dense_pad_batch(int B) {
   return bp;
 }
 
-// operand planes: 1 (BF16) or 3 (split: x0, x1, x2)
-size_t dense_x_bytes(const mt_tensor *T, int B) {
-  const size_t x = (size_t)dense_pad_batch(B) * T->Kp * 2 * (T->prec == MT_BF16_SPLIT ? 3 : 1);
-  return x + (size_t)3 * T->n * dense_pad_batch(B) * sizeof(float);  // + simulation-fastest copy of m
+// operand: 3 components, 1 term (BF16) or 3 (split: x0, x1, x2)
+static size_t dense_operand_bytes(const mt_tensor *T, int B) {
+  return (size_t)dense_pad_batch(B) * 3 * T->Kp * 2 * (T->prec == MT_BF16_SPLIT ? 3 : 1);
 }
-
+size_t dense_x_bytes(const mt_tensor *T, int B) {  // + the simulation-fastest copy of m
+  return dense_operand_bytes(T, B) + (size_t)3 * T->n * dense_pad_batch(B) * sizeof(float);
+}
 float *dense_mT(const mt_tensor *T, int B, void *X) {
-  const size_t x = (size_t)dense_pad_batch(B) * T->Kp * 2 * (T->prec == MT_BF16_SPLIT ? 3 : 1);
-  return reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(X) + x);
+  return reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(X) + dense_operand_bytes(T, B));
 }
 size_t dense_part_bytes(const mt_tensor *T, int B) {
-  return (size_t)2 * matvec_grid(T) * dense_pad_batch(B) * GM * sizeof(float);
+  return (size_t)2 * matvec_grid(T) * 3 * dense_pad_batch(B) * GM * sizeof(float);
 }
 size_t dense_count_bytes(const mt_tensor *T) { return (size_t)(T->Kp / GM) * EPI_WARPS * sizeof(int); }
 
-// (Measured when a stage first held two K blocks: the per-stage handshakes
-// of the TMA, MMA and commit path cost a fixed few hundred cycles, so 16 KB
-// tiles alone left the BF16 product at 0.70 of HBM and two per stage reached
-// 0.87; the split product went from 0.73 to 0.83 with a 2-deep ring of
-// 112 KB.  Both shapes stay candidates of the autotuner.)
-template <bool SPLIT, int BP>
-cudaError_t prep_one() {
-  cudaError_t e = cudaFuncSetAttribute(k_gemm<SPLIT, BP, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       227 * 1024);
-  if (e == cudaSuccess && kps_max(SPLIT, BP) == 2)
-    e = cudaFuncSetAttribute(k_gemm<SPLIT, BP, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  return e;
-}
-
 cudaError_t gemm_prepare() {
-  cudaError_t e;
-  if ((e = prep_one<false, 16>()) != cudaSuccess || (e = prep_one<false, 32>()) != cudaSuccess ||
-      (e = prep_one<false, 64>()) != cudaSuccess || (e = prep_one<false, 128>()) != cudaSuccess ||
-      (e = prep_one<true, 16>()) != cudaSuccess || (e = prep_one<true, 32>()) != cudaSuccess ||
-      (e = prep_one<true, 64>()) != cudaSuccess || (e = prep_one<true, 128>()) != cudaSuccess)
-    return e;
+  for (const bool split : {false, true})
+    for (const int Bp : {16, 32, 64, 128})
+      for (const int np : {4, 6}) {
+        const cudaError_t e = cudaFuncSetAttribute(gemm_variant(split, Bp, np).kernel,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+      }
   return cudaSuccess;
 }
 
 void launch_prep_dense_x(const mt_tensor *T, const float *m, int B, void *X, cudaStream_t s) {
-  const int Bp = dense_pad_batch(B);
-  __nv_bfloat16 *x = reinterpret_cast<__nv_bfloat16 *>(X);
-  const bool split = T->prec == MT_BF16_SPLIT;
-  __nv_bfloat16 *x1 = split ? x + (size_t)Bp * T->Kp : nullptr;
-  __nv_bfloat16 *x2 = split ? x + (size_t)2 * Bp * T->Kp : nullptr;
-  dim3 grid((unsigned)((T->Kp + 255) / 256), (unsigned)B);
-  k_prep_dense_x<<<grid, 256, 0, s>>>(m, T->tiles->d_Ms, T->n, T->Kp, B, Bp, x, x1, x2, dense_mT(T, B, X));
+  const int64_t KB = T->Kp / GK;
+  const dim3 grid((unsigned)KB, (unsigned)((B + kPrepSims - 1) / kPrepSims));
+  k_prep_dense_x<<<grid, 32 * kPrepWarps, 0, s>>>(m, T->tiles->d_Ms, T->n, KB, B, dense_pad_batch(B),
+                                      T->prec == MT_BF16_SPLIT ? 3 : 1, reinterpret_cast<__nv_bfloat16 *>(X),
+                                      dense_mT(T, B, X));
 }
 
 mt_status gemm_plan(const mt_tensor *T, int B, const void *X, GemmPlan *plan) {
   const int Bp = dense_pad_batch(B);
   MT_CHECK(B >= 1 && B <= 128, MT_EINVAL, "batched product: B = %d outside 1..128 simulations per pass", B);
-  // TMA row coordinates are 32-bit: (row tile * K blocks + K block) * 128
-  MT_CHECK((T->Kp / GM) * (T->Kp / GK) * (int64_t)GM < ((int64_t)1 << 31), MT_EINVAL,
-           "batched product: the dense tensor (3n = %lld) exceeds the 32-bit TMA coordinate range",
-           (long long)(3 * T->n));
   const bool split = T->prec == MT_BF16_SPLIT;
-  const __nv_bfloat16 *A = reinterpret_cast<const __nv_bfloat16 *>(T->d_data);
-  const __nv_bfloat16 *x = reinterpret_cast<const __nv_bfloat16 *>(X);
+  const GemmVariant v = gemm_variant(split, Bp, T->L.nplane);
+  const int64_t MT = T->Kp / GM, KB = T->Kp / GK, rows = MT * KB * (T->L.nplane / v.planes_per_unit) * 2 * GM;
+  MT_CHECK(rows < ((int64_t)1 << 31), MT_EINVAL,
+           "batched product: the dense tensor (n = %lld) exceeds the 32-bit TMA coordinate range", (long long)T->n);
   mt_status st;
-  // blocked storage seen as a [tiles * 128][64] array (A) and [KB * Bp][64] (X)
-  const uint64_t a_rows = (uint64_t)T->Kp * T->Kp / GK, x_rows = (uint64_t)(T->Kp / GK) * Bp;
-  if ((st = make_map(&plan->tA, A, GK, a_rows, GM)) != MT_OK) return st;
-  if ((st = make_map(&plan->tX, x, GK, x_rows, Bp)) != MT_OK) return st;
-  if (split) {
-    if ((st = make_map(&plan->tAlo, A + (size_t)T->Kp * T->Kp, GK, a_rows, GM)) != MT_OK) return st;
-    if ((st = make_map(&plan->tX1, x + (size_t)Bp * T->Kp, GK, x_rows, Bp)) != MT_OK) return st;
-    if ((st = make_map(&plan->tX2, x + (size_t)2 * Bp * T->Kp, GK, x_rows, Bp)) != MT_OK) return st;
-  } else {
-    plan->tAlo = plan->tA;
-    plan->tX1 = plan->tX;
-    plan->tX2 = plan->tX;
-  }
+  // blocked storage seen as a [units * 256][64] array and the operand as [terms * KB * 3 * Bp][64]
+  if ((st = make_map(&plan->tA, T->d_data, GK, (uint64_t)rows, 2 * GM)) != MT_OK) return st;
+  if ((st = make_map(&plan->tX, X, GK, (uint64_t)((split ? 9 : 3) * KB * Bp), (uint32_t)v.x_rows)) != MT_OK) return st;
   plan->B = B;
   plan->Bp = Bp;
   plan->split = split;
-  plan->kps = kps_max(split, Bp);
-  plan->stages = stages_for(Bp, split, plan->kps);
-  plan->chunk = 4 / plan->kps;  // units per accumulator chunk: 4 K blocks either way
+  plan->stages = v.stages;
   return MT_OK;
 }
 
 // The autotuner: per tensor and padded batch width, time the product for
-// each tile shape along K (1 or 2 K blocks per ring stage) and three ring
-// depths (the deepest that fits in shared memory and one and two stages
-// shallower) and keep the fastest; numerics do not depend on the choice.
+// three ring depths (the deepest that fits in shared memory and one and two
+// stages shallower) and keep the fastest; numerics do not depend on the choice.
 mt_status gemm_tune(mt_tensor *T, GemmPlan *plan, float *H, float *part, int *count, int *status, cudaStream_t s) {
   int key = 0;
   while ((16 << key) < plan->Bp) ++key;
   if (T->gemm_stages[key] > 0) {
     plan->stages = T->gemm_stages[key];
-    plan->kps = T->gemm_kps[key];
-    plan->chunk = 4 / plan->kps;
     return MT_OK;
   }
   cudaEvent_t e0, e1;
   MT_CUDA(cudaEventCreate(&e0));
   MT_CUDA(cudaEventCreate(&e1));
   float best_ms = 1e30f;
-  int best = 0, best_kps = plan->kps;
-  for (int kps = kps_max(plan->split, plan->Bp); kps >= 1; --kps) {
-    const int smax = stages_for(plan->Bp, plan->split, kps);
-    const int cand[3] = {smax, std::max(2, smax - 1), std::max(2, smax - 2)};
-    for (int c = 0; c < 3; ++c) {
-      if (c > 0 && cand[c] == cand[c - 1]) continue;
-      plan->kps = kps;
-      plan->chunk = 4 / kps;
-      plan->stages = cand[c];
-      launch_gemm(T, *plan, H, part, count, nullptr, status, s);  // warm
-      MT_CUDA(cudaEventRecord(e0, s));
-      for (int r = 0; r < 3; ++r) launch_gemm(T, *plan, H, part, count, nullptr, status, s);
-      MT_CUDA(cudaEventRecord(e1, s));
-      MT_CUDA(cudaEventSynchronize(e1));
-      float ms = 0.0f;
-      MT_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < best_ms) {
-        best_ms = ms;
-        best = cand[c];
-        best_kps = kps;
-      }
+  int best = plan->stages;
+  const int smax = plan->stages;
+  for (int st = smax; st >= std::max(2, smax - 2); --st) {
+    plan->stages = st;
+    launch_gemm(T, *plan, H, part, count, nullptr, status, s);  // warm
+    MT_CUDA(cudaEventRecord(e0, s));
+    for (int r = 0; r < 3; ++r) launch_gemm(T, *plan, H, part, count, nullptr, status, s);
+    MT_CUDA(cudaEventRecord(e1, s));
+    MT_CUDA(cudaEventSynchronize(e1));
+    float ms = 0.0f;
+    MT_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+    if (ms < best_ms) {
+      best_ms = ms;
+      best = st;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   MT_CUDA(cudaGetLastError());
   T->gemm_stages[key] = best;
-  T->gemm_kps[key] = best_kps;
   plan->stages = best;
-  plan->kps = best_kps;
-  plan->chunk = 4 / best_kps;
   return MT_OK;
 }
 
 void launch_gemm(const mt_tensor *T, const GemmPlan &plan, float *H, float *part, int *count, const int *n_active,
                  int *status, cudaStream_t s) {
+  const GemmVariant v = gemm_variant(plan.split, plan.Bp, T->L.nplane);
   GemmArgs P;
-  P.n3 = 3 * T->n;
+  P.n = T->n;
   P.MT = T->Kp / GM;
   P.KB = T->Kp / GK;
-  P.KBU = P.KB / plan.kps;
   P.B = plan.B;
   P.Bp = plan.Bp;
-  P.chunk = plan.chunk;
   P.stages = plan.stages;
-  P.stage_bytes = stage_bytes_for(plan.Bp, plan.split, plan.kps);
-  const bool stack = plan.split && plan.Bp <= 64;
-  const int acc_cols = stack ? 3 * plan.Bp : plan.Bp;
-  const int na = stack ? (plan.Bp == 64 ? 2 : 4) : (plan.Bp <= 64 ? 2 * NACC : NACC);  // as GemmShape
-  uint32_t cols = 32;
-  while (cols < (uint32_t)(na * acc_cols)) cols <<= 1;
-  P.tmem_cols = cols;
+  P.tmem_cols = v.tmem_cols;
   P.H = H;
   P.part = part;
   P.count = count;
   P.n_active = n_active;
   P.status = status;
-  const int64_t U = P.MT * P.KBU;
-  const int grid = (int)std::min<int64_t>(matvec_grid(T), U);
-  const size_t smem = (size_t)P.stages * P.stage_bytes + 1024 + 512;  // + alignment slack, barriers
-#define MT_GEMM_LAUNCH_K(SP, BPV, K)                                                                            \
-  mt::launch_pdl(k_gemm<SP, BPV, K>, dim3(grid), dim3(GEMM_THREADS), smem, s, plan.tA, plan.tAlo, plan.tX, plan.tX1, \
-                 plan.tX2, P)
-#define MT_GEMM_LAUNCH(SP, BPV)                          \
-  do {                                                   \
-    if (plan.kps == 2 && kps_max(SP, BPV) == 2)          \
-      MT_GEMM_LAUNCH_K(SP, BPV, kps_max(SP, BPV));       \
-    else                                                 \
-      MT_GEMM_LAUNCH_K(SP, BPV, 1);                      \
-  } while (0)
-  if (plan.split) {
-    switch (plan.Bp) {
-      case 16: MT_GEMM_LAUNCH(true, 16); break;
-      case 32: MT_GEMM_LAUNCH(true, 32); break;
-      case 64: MT_GEMM_LAUNCH(true, 64); break;
-      default: MT_GEMM_LAUNCH(true, 128); break;
-    }
-  } else {
-    switch (plan.Bp) {
-      case 16: MT_GEMM_LAUNCH(false, 16); break;
-      case 32: MT_GEMM_LAUNCH(false, 32); break;
-      case 64: MT_GEMM_LAUNCH(false, 64); break;
-      default: MT_GEMM_LAUNCH(false, 128); break;
-    }
-  }
-#undef MT_GEMM_LAUNCH
-#undef MT_GEMM_LAUNCH_K
+  // never more CTAs than units: every CTA then owns at least one, which the
+  // bookkeeping of split row tiles relies on
+  const int grid = (int)std::min<int64_t>(matvec_grid(T), P.MT * P.KB * (T->L.nplane / v.planes_per_unit));
+  launch_pdl(v.kernel, dim3(grid), dim3(v.threads), plan.stages * v.stage_bytes + v.fixed_bytes, s, plan.tA,
+             plan.tX, P);
 }
 
 }  // namespace mt

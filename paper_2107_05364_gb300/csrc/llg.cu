@@ -78,7 +78,7 @@ struct StageArgs {
   float *k[7];
   int64_t Q;
   int TC;
-  // operand of the batched tensor-core product (dense layout): X[b][Kp] BF16
+  // operand of the batched tensor-core product (dense layout; dense_x_index): BF16
   // (+ low part for the split precision); xs_mode 0 = streaming layout
   int xs_mode;  // 0 streaming FP32 chunks, 1 dense BF16, 2 dense split BF16, 3 sparse float4
   int64_t Kp;
@@ -185,19 +185,18 @@ __device__ __forceinline__ void write_stage_input(const StageArgs &A, float *ysn
     reinterpret_cast<float4 *>(A.xs)[(size_t)b * sparse_x_stride(A.n) + i] =
         make_float4(ms * v[0], ms * v[1], ms * v[2], 0.0f);
   } else {
-    __nv_bfloat16 *x1 = A.X + (size_t)A.Bp * A.Kp;  // split: second and third operand terms
-    __nv_bfloat16 *x2 = x1 + (size_t)A.Bp * A.Kp;
+    const size_t term = (size_t)3 * A.Kp * A.Bp;  // split: to the second and third operand terms
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const float f = ms * v[c];
       const __nv_bfloat16 hi = __float2bfloat16(f);
-      const size_t at = dense_x_index(b, 3 * i + c, A.Bp);
-      A.X[at] = hi;
+      __nv_bfloat16 *x = A.X + dense_x_index(c, b, i, A.Bp);
+      x[0] = hi;
       if (A.xs_mode == 2) {
         const float r = f - __bfloat162float(hi);
         const __nv_bfloat16 mid = __float2bfloat16(r);
-        x1[at] = mid;
-        x2[at] = __float2bfloat16(r - __bfloat162float(mid));
+        x[term] = mid;
+        x[2 * term] = __float2bfloat16(r - __bfloat162float(mid));
       }
       A.mT[(size_t)(3 * i + c) * A.Bp + b] = v[c];
     }

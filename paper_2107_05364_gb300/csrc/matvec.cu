@@ -1342,10 +1342,15 @@ __global__ void k_near(int64_t n, int B, const int32_t *ptr, const int32_t *col,
 }
 
 // The same for the simulation-fastest copy of a batch (element (b, j, c) at
-// mT[(3 j + c) Bp + b]): a thread takes V adjacent simulations of one tile
-// (one vector load per component), so a warp covers 32 V simulations and
-// shares the tile's blocks; the column of the next block is fetched one step
-// ahead.
+// mT[(3 j + c) Bp + b]).  LS lanes take one tile, V adjacent simulations each
+// (one vector load per component, the tile's blocks shared); three blocks'
+// loads are in flight at a time (one where the double-FP32 arithmetic, not the
+// latency, bounds it), their sums in column order.  The sums of a
+// CTA's tiles (16 or more) pass through shared memory, so that H, one row of
+// three floats per tile in every simulation's own vector, is read and written
+// in runs of whole tiles; a thread that wrote its own tile and
+// simulation touched a 32-byte sector for each value.  n = 10,000, B = 64, BF16:
+// 53 -> 36 us (split, n = 20,000: 118 -> 114, its double-FP32 sums bound it).
 template <int V>
 struct VecF;
 template <>
@@ -1361,74 +1366,92 @@ struct VecF<2> {
     o[1] = v.y;
   }
 };
-template <>
-struct VecF<4> {
-  using T = float4;
-  static __device__ __forceinline__ void get(T v, float *o) {
-    o[0] = v.x;
-    o[1] = v.y;
-    o[2] = v.z;
-    o[3] = v.w;
-  }
-};
 
-template <bool FF, int V>
-__global__ void k_near_v(int64_t n, int B, int Bp, const int32_t *ptr, const int32_t *col, const float2 *val,
-                         const float *mT, float *H, const int *active) {
+constexpr int kNearThreads = 256;
+// tiles of a CTA: a pass of its threads, at least 16
+template <int LS>
+constexpr int kNearTilesOf = kNearThreads / LS > 16 ? kNearThreads / LS : 16;
+template <bool FF, int LS, int V>
+__global__ void __launch_bounds__(kNearThreads) k_near_v(int64_t n, int B, int Bp, const int32_t *ptr,
+                                                         const int32_t *col, const float2 *val, const float *mT,
+                                                         float *H, const int *active) {
   mtd::pdl_enter();
   using VT = typename VecF<V>::T;
-  const int Bv = (B + V - 1) / V;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= n * Bv) return;
-  const int64_t i = t / Bv;
-  const int b0 = (int)(t - i * Bv) * V;
-  ff hx[V], hy[V], hz[V];
+  constexpr int SIMS = LS * V;             // simulations of a CTA
+  constexpr int PASS = kNearThreads / LS;  // tiles in one pass of the CTA
+  constexpr int TILES = kNearTilesOf<LS>;
+  constexpr int UN = FF ? 1 : 3;  // blocks in flight
+  constexpr int ROW = 3 * TILES + 1;
+  __shared__ float s_hi[SIMS][ROW], s_lo[FF ? SIMS : 1][FF ? ROW : 1];
+  const int64_t i0 = blockIdx.x * (int64_t)TILES;
+  const int bs = blockIdx.y * SIMS;  // first simulation
+  const int l = threadIdx.x % LS, b0 = bs + l * V;
+#pragma unroll 1
+  for (int ti = threadIdx.x / LS; ti < TILES; ti += PASS) {
+    const int64_t i = i0 + ti;
+    if (i >= n || b0 >= Bp) break;
+    ff h[3][V];
 #pragma unroll
-  for (int v = 0; v < V; ++v) hx[v] = hy[v] = hz[v] = ff{0.0f, 0.0f};
-  const int32_t a0 = ptr[i], a1 = ptr[i + 1];
-  int64_t jn = a0 < a1 ? col[a0] : 0;
-  for (int32_t a = a0; a < a1; ++a) {
-    const int64_t j = jn;
-    if (a + 1 < a1) jn = col[a + 1];
-    const float4 *vp = reinterpret_cast<const float4 *>(val + 6 * (size_t)a);
-    const float4 w0 = vp[0], w1 = vp[1], w2 = vp[2];
-    float x0[V], x1[V], x2[V];
-    VecF<V>::get(*reinterpret_cast<const VT *>(mT + (size_t)(3 * j) * Bp + b0), x0);
-    VecF<V>::get(*reinterpret_cast<const VT *>(mT + (size_t)(3 * j + 1) * Bp + b0), x1);
-    VecF<V>::get(*reinterpret_cast<const VT *>(mT + (size_t)(3 * j + 2) * Bp + b0), x2);
-    const float2 v0 = make_float2(w0.x, w0.y), v1 = make_float2(w0.z, w0.w), v2 = make_float2(w1.x, w1.y);
-    const float2 v3 = make_float2(w1.z, w1.w), v4 = make_float2(w2.x, w2.y), v5 = make_float2(w2.z, w2.w);
+    for (int c = 0; c < 3; ++c)
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      if (!FF) {
-        hx[v].hi = fmaf(v0.x, x0[v], fmaf(v1.x, x1[v], fmaf(v2.x, x2[v], hx[v].hi)));
-        hy[v].hi = fmaf(v1.x, x0[v], fmaf(v3.x, x1[v], fmaf(v4.x, x2[v], hy[v].hi)));
-        hz[v].hi = fmaf(v2.x, x0[v], fmaf(v4.x, x1[v], fmaf(v5.x, x2[v], hz[v].hi)));
-      } else {
-        ff_fma_lazy(hx[v], v0, x0[v]);
-        ff_fma_lazy(hx[v], v1, x1[v]);
-        ff_fma_lazy(hx[v], v2, x2[v]);
-        ff_fma_lazy(hy[v], v1, x0[v]);
-        ff_fma_lazy(hy[v], v3, x1[v]);
-        ff_fma_lazy(hy[v], v4, x2[v]);
-        ff_fma_lazy(hz[v], v2, x0[v]);
-        ff_fma_lazy(hz[v], v4, x1[v]);
-        ff_fma_lazy(hz[v], v5, x2[v]);
+      for (int v = 0; v < V; ++v) h[c][v] = ff{0.0f, 0.0f};
+    const int32_t a1 = ptr[i + 1];
+    int32_t a = ptr[i], jn[UN];  // the next columns, fetched a round ahead
+#pragma unroll
+    for (int q = 0; q < UN; ++q) jn[q] = a + q < a1 ? col[a + q] : 0;
+    for (; a < a1; a += UN) {
+      float4 w[UN][3];
+      float x[UN][3][V];
+#pragma unroll
+      for (int q = 0; q < UN; ++q) {
+        const int64_t j = jn[q];
+        jn[q] = a + UN + q < a1 ? col[a + UN + q] : 0;
+        if (a + q >= a1) continue;
+        const float4 *vp = reinterpret_cast<const float4 *>(val + 6 * (size_t)(a + q));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          w[q][c] = vp[c];
+          VecF<V>::get(*reinterpret_cast<const VT *>(mT + (size_t)(3 * j + c) * Bp + b0), x[q][c]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < UN; ++q) {
+        if (a + q >= a1) continue;
+        const float4 w0 = w[q][0], w1 = w[q][1], w2 = w[q][2];
+        const float2 e[6] = {{w0.x, w0.y}, {w0.z, w0.w}, {w1.x, w1.y}, {w1.z, w1.w}, {w2.x, w2.y}, {w2.z, w2.w}};
+        constexpr int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float x0 = x[q][0][v], x1 = x[q][1][v], x2 = x[q][2][v];
+            if (!FF) {
+              h[c][v].hi = fmaf(e[at[c][0]].x, x0, fmaf(e[at[c][1]].x, x1, fmaf(e[at[c][2]].x, x2, h[c][v].hi)));
+            } else {
+              ff_fma_lazy(h[c][v], e[at[c][0]], x0);
+              ff_fma_lazy(h[c][v], e[at[c][1]], x1);
+              ff_fma_lazy(h[c][v], e[at[c][2]], x2);
+            }
+          }
       }
     }
-  }
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    const int b = b0 + v;
-    if (b >= B || (active && !active[b])) continue;
-    float *Hb = H + (size_t)b * 3 * n + 3 * i;
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        s_hi[l * V + v][3 * ti + c] = h[c][v].hi;
+        if (FF) s_lo[l * V + v][3 * ti + c] = h[c][v].lo;
+      }
+  }
+  __syncthreads();
+  const int cnt = 3 * (int)(n - i0 < TILES ? n - i0 : TILES);
+  for (int q = threadIdx.x; q < SIMS * 3 * TILES; q += kNearThreads) {
+    const int s = q / (3 * TILES), t = q - s * 3 * TILES, b = bs + s;
+    if (t >= cnt || b >= B || (active && !active[b])) continue;
+    float *Hb = H + (size_t)b * 3 * n + 3 * i0 + t;
     // H = far - near, rounded once
-    const ff rx = ff_add({Hb[0], 0.0f}, -hx[v].hi, -hx[v].lo);
-    const ff ry = ff_add({Hb[1], 0.0f}, -hy[v].hi, -hy[v].lo);
-    const ff rz = ff_add({Hb[2], 0.0f}, -hz[v].hi, -hz[v].lo);
-    Hb[0] = rx.hi + rx.lo;
-    Hb[1] = ry.hi + ry.lo;
-    Hb[2] = rz.hi + rz.lo;
+    const ff r = ff_add({*Hb, 0.0f}, -s_hi[s][t], FF ? -s_lo[s][t] : 0.0f);
+    *Hb = r.hi + r.lo;
   }
 }
 
@@ -1720,22 +1743,19 @@ void launch_near(const mt_tensor *T, const float *m, int64_t sb, int64_t se, int
   const float2 *hl = T->d_near_hl;
   const int64_t n = T->n;
   if (sb == 1 && se >= B && se % 4 == 0) {  // simulation-fastest copy, rows of se >= B floats
-    const int V = B >= 128 ? 4 : B >= 64 ? 2 : 1;
-    const int64_t threads = n * ((B + V - 1) / V);
-    const unsigned g = (unsigned)((threads + 255) / 256);
     const int Bp = (int)se;
     const bool split = T->prec == MT_BF16_SPLIT;
-#define MT_NEAR_V(FF, VV) \
-  mt::launch_pdl(k_near_v<FF, VV>, dim3(g), dim3(256), 0, s, n, B, Bp, ptr, col, hl, m, H, active)
-    if (split) {
-      if (V == 4) MT_NEAR_V(true, 4);
-      else if (V == 2) MT_NEAR_V(true, 2);
-      else MT_NEAR_V(true, 1);
-    } else {
-      if (V == 4) MT_NEAR_V(false, 4);
-      else if (V == 2) MT_NEAR_V(false, 2);
-      else MT_NEAR_V(false, 1);
-    }
+    // lanes per tile: as many as there are simulations, at least 8, at most
+    // 32, two simulations each from 64 on
+#define MT_NEAR_V(LS, VV)                                                                                   \
+  mt::launch_pdl(split ? k_near_v<true, LS, VV> : k_near_v<false, LS, VV>,                                 \
+                 dim3((unsigned)((n + kNearTilesOf<LS> - 1) / kNearTilesOf<LS>),                           \
+                      (unsigned)((B + LS * VV - 1) / (LS * VV))),                                          \
+                 dim3(kNearThreads), 0, s, n, B, Bp, ptr, col, hl, m, H, active)
+    if (B <= 8) MT_NEAR_V(8, 1);
+    else if (B <= 16) MT_NEAR_V(16, 1);
+    else if (B <= 32) MT_NEAR_V(32, 1);
+    else MT_NEAR_V(32, 2);
 #undef MT_NEAR_V
     return;
   }

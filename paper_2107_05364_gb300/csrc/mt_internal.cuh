@@ -182,9 +182,9 @@ struct mt_tensor {
   std::atomic<int> refs{1};
   mt_tiles *tiles = nullptr;
   int prec = MT_F32;
-  int layout = MT_LAYOUT_STREAM;  // MT_LAYOUT_DENSE: 9-entry BF16 matrix for tensor cores
+  int layout = MT_LAYOUT_STREAM;  // MT_LAYOUT_DENSE: BF16 entry planes for tensor cores
   int64_t n = 0;
-  int64_t Kp = 0;                 // dense layout: rows = columns = 3n padded to 128
+  int64_t Kp = 0;                 // dense layout: rows = columns of a plane, n padded to 128
   mt_layout L;
   void *d_data = nullptr;
   size_t bytes = 0;
@@ -206,7 +206,6 @@ struct mt_tensor {
   float *d_colpart = nullptr;  // half storage: column work area of the standalone calls
   int colpart_B = 0;
   int gemm_stages[4] = {0, 0, 0, 0};  // tuned ring depth per padded batch 16/32/64/128
-  int gemm_kps[4] = {0, 0, 0, 0};     // tuned K blocks per ring stage (tile shape along K)
   // thresholded layout: block-sparse rows (kept blocks, 6 FP32 entries each)
   int64_t sp_blocks = 0;         // stored blocks (runs padded to 4)
   int64_t sp_runs = 0;           // runs of consecutive columns
@@ -275,25 +274,26 @@ __host__ __device__ __forceinline__ int64_t layout_index_h(int64_t i, int64_t j,
 // may reach 3 columns past the last tile).
 __host__ __device__ __forceinline__ int64_t sparse_x_stride(int64_t n) { return n + 4; }
 
-// Dense layout, tile-blocked: the 3n x 3n matrix (padded to Kp = 128 k) is
-// cut into 128-row x 64-column BF16 tiles, each stored contiguously (16 KB,
-// rows of 128 bytes), tiles ordered by (row tile, K block); the low part of
-// the split precision is a second such plane.  The operand X of a batch is
-// cut the same way along K: block kb holds Bp rows of 64 values.
-__host__ __device__ __forceinline__ size_t dense_a_index(int64_t r, int64_t c, int64_t KB) {
-  return ((size_t)((r >> 7) * KB + (c >> 6)) * 128 + (size_t)(r & 127)) * 64 + (size_t)(c & 63);
+// Dense layout, tile-blocked: each stored entry plane (6, or 4 for a single
+// layer) is an n x n matrix padded to Kp = 128 k, cut into 128-row x 64-column
+// BF16 tiles, each stored contiguously (16 KB, rows of 128 bytes; for the
+// split precision followed by the tile of low parts), tiles ordered by (row
+// tile, K block, plane).  The operand X of a batch is cut the same way along
+// K: for each term (split: 3), K block and component, Bp rows of 64 values.
+__host__ __device__ __forceinline__ size_t dense_a_index(int64_t i, int64_t j, int pl, int64_t KB, int np,
+                                                         bool split) {
+  const size_t tile = (size_t)((i >> 7) * KB + (j >> 6)) * np + pl;
+  return (tile * (split ? 256 : 128) + (size_t)(i & 127)) * 64 + (size_t)(j & 63);
 }
-__host__ __device__ __forceinline__ size_t dense_x_index(int64_t b, int64_t c, int64_t Bp) {
-  return ((size_t)(c >> 6) * Bp + (size_t)b) * 64 + (size_t)(c & 63);
+constexpr size_t kDenseLo = 128 * 64;  // from a high part to its low part
+__host__ __device__ __forceinline__ size_t dense_x_index(int c, int64_t b, int64_t j, int64_t Bp) {
+  return ((size_t)((j >> 6) * 3 + c) * Bp + (size_t)b) * 64 + (size_t)(j & 63);
 }
 
 // Tensor maps and shape of one batched tensor-core product (dense layout).
 struct GemmPlan {
-  CUtensorMap tA, tAlo, tX, tX1, tX2;  // tensor hi/lo; operand terms (split: x0, x1, x2)
-  const float *mT = nullptr;           // simulation-fastest copy of m (near blocks)
+  CUtensorMap tA, tX;  // tensor planes; operand terms
   int B = 0, Bp = 0, stages = 0;
-  int kps = 1;    // K blocks per ring stage (one unit of work)
-  int chunk = 4;  // units accumulated in TMEM before the FP32 promotion (4 K blocks)
   bool split = false;
 };
 
@@ -334,6 +334,11 @@ void launch_near(const mt_tensor *T, const float *m, int64_t sb, int64_t se, int
                  cudaStream_t s);
 
 // batched product on tcgen05 (dense layout)
+// bytes of a dense-layout tensor of np planes
+inline size_t dense_tensor_bytes(int64_t n, int prec, int np) {
+  const size_t Kp = (size_t)((n + 127) / 128) * 128;
+  return Kp * Kp * np * 2 * (prec == MT_BF16_SPLIT ? 2 : 1);
+}
 cudaError_t gemm_prepare();
 int dense_pad_batch(int B);
 size_t dense_x_bytes(const mt_tensor *T, int B);
@@ -452,6 +457,29 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
       }
     }
   }
+}
+
+// The same for a whole warp that has time: lane 0 polls, with pauses, so that
+// the warp does not take issue slots from the threads that feed it.
+__device__ __forceinline__ bool mbar_wait_warp_relaxed(uint64_t *bar, uint32_t parity, int *status,
+                                                       uint64_t limit_ns = 2000000000ull) {
+  int ok = 1;
+  if ((threadIdx.x & 31) == 0) {
+    uint64_t t0 = 0;
+    for (uint32_t it = 1; !mbar_try_wait(bar, parity); ++it) {
+      __nanosleep(128);
+      if ((it & 1023u) == 0u) {
+        const uint64_t t = globaltimer_ns();
+        if (t0 == 0) t0 = t;
+        if (t - t0 > limit_ns) {
+          if (status) atomicExch(status, MT_DEV_TIMEOUT);
+          ok = 0;
+          break;
+        }
+      }
+    }
+  }
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
 // 1-D bulk prefetch of global memory into L2 (no completion to wait for).
