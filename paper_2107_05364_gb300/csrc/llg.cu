@@ -547,7 +547,8 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs A) {
 // exchanges, the rest the serial chain of one stage).
 constexpr int kSmallThreads = 256;
 constexpr int kSmallWarps = kSmallThreads / 32;
-constexpr int kSmallRed = 3 * 8 * kSmallWarps;  // floats of one buffer of row sums
+constexpr int kSmallRed = 3 * 8 * kSmallWarps;       // floats of one buffer of row sums: one simulation's
+constexpr int kSmallRedL2 = 3 * 16 * kSmallWarps;    // rows read from L2: those of 8 simulations
 
 // one tile's vector: 3 floats and the 16-bit tag in each of two 64-bit words;
 // a CTA's partial sums: 5 words of a float and the tag (padded to 6)
@@ -584,18 +585,22 @@ __host__ __device__ __forceinline__ size_t small_take(size_t &o, size_t bytes) {
   o += (bytes + 15) & ~(size_t)15;
   return at;
 }
+// floats of a simulation's state in shared memory: rows of 4 tiles are read as
+// three float4 from 16-byte boundaries (12 floats past the last one's end are
+// allocated for a last row of fewer tiles)
+__host__ __device__ __forceinline__ int small_stride(int64_t n) { return (int)((3 * n + 3) & ~(int64_t)3); }
 __host__ __device__ __forceinline__ SmallSmem small_smem(int64_t n, int B, int R, bool nsmem) {
   SmallSmem s;
   size_t o = 0;
   s.ctl = small_take(o, sizeof(SimCtl) * B);
-  s.red = small_take(o, sizeof(float) * 2 * kSmallRed);
+  s.red = small_take(o, sizeof(float) * 2 * (nsmem ? kSmallRed : kSmallRedL2));
   s.y = small_take(o, sizeof(float) * B * R * 3);
   s.k = small_take(o, sizeof(float) * 7 * B * R * 3);
   s.coef = small_take(o, sizeof(float) * B * 36);  // (float)(h a_sj), s = 1..6, j < s
   s.par = small_take(o, sizeof(float) * B * 6);    // g1, g2, Ha, exchange factor
   s.kc = small_take(o, sizeof(int) * B);           // where the committed k1 and y are (see SmallSh)
   s.Ms = small_take(o, sizeof(float) * n);
-  s.M = small_take(o, sizeof(float) * B * 3 * n);
+  s.M = small_take(o, sizeof(float) * ((size_t)B * small_stride(n) + 12));
   s.N = small_take(o, nsmem ? sizeof(float) * 6 * R * n : 0);
   s.total = o;
   return s;
@@ -729,11 +734,17 @@ __device__ __forceinline__ void small_product(const SmallSh &sh, const float *mb
 // tensor stays in L2 (up to ~100 MB): each warp owns rows w and w + 8 of the
 // CTA (at most 16) and reads them from the streaming layout, lanes over the
 // columns (128 consecutive columns of an entry plane are contiguous, 16-byte
-// aligned), so no cross-warp reduction is needed: red[3 q + c].
-template <bool PLANAR>
-__device__ __forceinline__ void small_product_l2(const SmallArgs &S, const SmallSh &sh, const float *mb, float *red,
-                                                 int nr, int64_t r0, int64_t n) {
+// aligned), so no cross-warp reduction is needed: simulation s of the SB that
+// start at b at red[s 3 kSmallRowsL2 + 3 q + c].  The L2 reads bound it, so up
+// to 4 simulations share them (2,016-tile prism, 4 simulations, 8 attempts:
+// 2,302 us with a pass per simulation, 1,377 so; one simulation of an
+// 1,190-tile film 568 -> 388).
+constexpr int kSmallRowsL2 = 2 * kSmallWarps;
+template <int SB, bool PLANAR>
+__device__ __forceinline__ void small_product_l2(const SmallArgs &S, const SmallSh &sh, int b, float *red, int nr,
+                                                 int64_t r0, int n) {
   constexpr int NP = PLANAR ? 4 : 6;
+  constexpr int U = SB == 1 ? 2 : 1;  // groups of 128 columns in flight
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const size_t plane = (size_t)S.TR * S.TC, chunk = NP * plane;
   const float *rowp[2] = {nullptr, nullptr};
@@ -745,17 +756,22 @@ __device__ __forceinline__ void small_product_l2(const SmallArgs &S, const Small
       rowp[r] = S.N + (size_t)p * S.Q * chunk + (size_t)(i - p * S.TR) * S.TC;
     }
   }
-  float acc[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
-  // a lane takes 4 adjacent columns (one 16-byte load per entry plane; the
-  // padding of the last column chunk holds zeros), two such groups per
-  // step so that 4 NP loads per lane are in flight
-  for (int64_t j0 = 4 * lane; j0 < n; j0 += 256) {
-    float4 ent[2][2][NP];
-    float x[2][4][3];
+  const float *mb[SB];  // (a group past the last simulation repeats it)
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int64_t j = j0 + 128 * u;
-      const int64_t cq = j / S.TC;
+  for (int s = 0; s < SB; ++s) mb[s] = sh.M + (b + s < S.A.B ? b + s : S.A.B - 1) * small_stride(n);
+  float acc[SB][2][3];
+#pragma unroll
+  for (int s = 0; s < SB; ++s)
+#pragma unroll
+    for (int r = 0; r < 2; ++r) acc[s][r][0] = acc[s][r][1] = acc[s][r][2] = 0.0f;
+  // a lane takes 4 adjacent columns (one 16-byte load per entry plane; the
+  // padding of the last column chunk holds zeros)
+  for (int j0 = 4 * lane; j0 < n; j0 += 128 * U) {
+    float4 ent[U][2][NP];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 128 * u;
+      const int cq = j / S.TC;
       const size_t off = (size_t)cq * chunk + (size_t)(j - cq * S.TC);
 #pragma unroll
       for (int r = 0; r < 2; ++r)
@@ -763,42 +779,53 @@ __device__ __forceinline__ void small_product_l2(const SmallArgs &S, const Small
         for (int e = 0; e < NP; ++e)
           ent[u][r][e] = (rowp[r] && j < n) ? __ldg(reinterpret_cast<const float4 *>(rowp[r] + off + e * plane))
                                             : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const bool in = j + k < n;
-        const float ms = in ? sh.Ms[j + k] : 0.0f;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) x[u][k][c] = in ? ms * mb[3 * (j + k) + c] : 0.0f;
-      }
     }
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 128 * u;
+      if (j >= n) break;
+      float ms[4];
+      *reinterpret_cast<float4 *>(ms) = *reinterpret_cast<const float4 *>(sh.Ms + j);
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
+      for (int s = 0; s < SB; ++s) {
+        float x[12];  // 4 tiles' vectors, times Ms (0 past the last tile)
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          reinterpret_cast<float4 *>(x)[q] = *reinterpret_cast<const float4 *>(mb[s] + 3 * j + 4 * q);
+#pragma unroll
+        for (int q = 0; q < 12; ++q) x[q] = j + q / 3 < n ? ms[q / 3] * x[q] : 0.0f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const float *ex = reinterpret_cast<const float *>(&ent[u][r][0]) + k;  // plane e at ex[4 e]
-          const float x0 = x[u][k][0], x1 = x[u][k][1], x2 = x[u][k][2];
-          if constexpr (PLANAR) {
-            acc[r][0] = fmaf(ex[0], x0, fmaf(ex[4], x1, acc[r][0]));
-            acc[r][1] = fmaf(ex[4], x0, fmaf(ex[8], x1, acc[r][1]));
-            acc[r][2] = fmaf(ex[12], x2, acc[r][2]);
-          } else {
-            acc[r][0] = fmaf(ex[0], x0, fmaf(ex[4], x1, fmaf(ex[8], x2, acc[r][0])));
-            acc[r][1] = fmaf(ex[4], x0, fmaf(ex[12], x1, fmaf(ex[16], x2, acc[r][1])));
-            acc[r][2] = fmaf(ex[8], x0, fmaf(ex[16], x1, fmaf(ex[20], x2, acc[r][2])));
+          const float x0 = x[3 * k], x1 = x[3 * k + 1], x2 = x[3 * k + 2];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const float *ex = reinterpret_cast<const float *>(&ent[u][r][0]) + k;  // plane e at ex[4 e]
+            float *h = acc[s][r];
+            if constexpr (PLANAR) {
+              h[0] = fmaf(ex[0], x0, fmaf(ex[4], x1, h[0]));
+              h[1] = fmaf(ex[4], x0, fmaf(ex[8], x1, h[1]));
+              h[2] = fmaf(ex[12], x2, h[2]);
+            } else {
+              h[0] = fmaf(ex[0], x0, fmaf(ex[4], x1, fmaf(ex[8], x2, h[0])));
+              h[1] = fmaf(ex[4], x0, fmaf(ex[12], x1, fmaf(ex[16], x2, h[1])));
+              h[2] = fmaf(ex[8], x0, fmaf(ex[16], x1, fmaf(ex[20], x2, h[2])));
+            }
           }
         }
+      }
+    }
   }
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     if (!rowp[r]) continue;  // the same in the whole warp
     const int q = w + kSmallWarps * r;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float v = mtd::warp_sum(acc[r][c]);
-      if (lane == 0) red[3 * q + c] = v;
-    }
+    for (int s = 0; s < SB; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float v = mtd::warp_sum(acc[s][r][c]);
+        if (lane == 0) red[s * 3 * kSmallRowsL2 + 3 * q + c] = v;
+      }
   }
 }
 
@@ -902,107 +929,148 @@ struct SmallRow {
 // Eq. 1 (the arithmetic of k_stage) and what follows from it: after stages
 // 1..6 k, for stages 2..6 also the next stage's input, published under
 // `tag`; after stage 7 k7 and the sums of the error norm, the torque and <m>;
-// after stage 1 (k1 at the state) k1 and the torque.  One CTA barrier per
-// simulation: sh.M is read only before it (a later exchange may overwrite
-// it), and the two buffers of row sums alternate.
+// after stage 1 (k1 at the state) k1 and the torque.  One CTA barrier between
+// the product of a simulation (rows read from L2: of eight) and the rest:
+// sh.M is read only before it (a later exchange may overwrite it), and the
+// two buffers of row sums alternate.
+//
+// What a row needs of the other tiles: m itself and the exchange sum.
+struct SmallPre {
+  float mi[3], he[3];
+};
+__device__ __forceinline__ void small_pre(const StageArgs &A, const SmallRow &rw, const float *mb, int i,
+                                          SmallPre &pr) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    pr.mi[c] = mb[3 * i + c];
+    pr.he[c] = 0.0f;
+  }
+  if (A.exch) {
+#pragma unroll
+    for (int f = 0; f < 6; ++f)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) pr.he[c] += rw.wex[f] * (mb[3 * rw.nbr[f] + c] - pr.mi[c]);
+  }
+}
+
+// the owning warp's part after the barrier; WSUM partial sums per row value
+// (value v of part w at red[w WSTRIDE + v])
+template <int WSUM, int WSTRIDE>
+__device__ __forceinline__ void small_rows(const SmallArgs &S, const SmallSh &sh, const SmallRow &rw,
+                                           const SmallPre &pr, const float *red, int b, int st, unsigned tag, int nr,
+                                           int64_t r0) {
+  const StageArgs &A = S.A;
+  const int n = (int)A.n, B = A.B, R = S.R;
+  const size_t kpl = (size_t)B * R * 3;  // floats of one derivative plane
+  const int q = threadIdx.x & 31, i = (int)r0 + q;
+  const bool row = q < nr;
+  const float *mi = pr.mi, *he = pr.he;
+  float k[3] = {0.0f, 0.0f, 0.0f}, tau = 0.0f;
+  float *ks = sh.k + ((size_t)b * R + q) * 3;  // row q's k1; plane s at + s kpl
+  const float *y0 = sh.y + ((size_t)b * R + q) * 3;
+  if (row) {
+    const float *pb = sh.par + 6 * b;
+    float H[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float s = 0.0f;
+#pragma unroll
+      for (int w = 0; w < WSUM; ++w) s += red[w * WSTRIDE + 3 * q + c];
+      H[c] = -s + pb[2 + c];
+      if (A.exch) H[c] += pb[5] * he[c];
+    }
+    if (rw.kan != 0.0f) {
+      const float me = mi[0] * rw.axis[0] + mi[1] * rw.axis[1] + mi[2] * rw.axis[2];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) H[c] += rw.kan * me * rw.axis[c];
+    }
+    const float mxh = llg(pb[0], pb[1], mi, H, k);
+    if (st == 1 || st == 7) tau = mxh / rw.Ms;
+    for (int c = 0; c < 3; ++c) ks[(st - 1) * kpl + c] = k[c];
+    if (st >= 2 && st <= 6) {
+      // this row's input of the next stage: y + sum_j (h a_sj) k_j
+      const float *cf = sh.coef + 36 * b + 6 * (st - 1);
+      float acc[3] = {0.0f, 0.0f, 0.0f}, a[6], kj[6][3];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) {  // all loads before the sums
+        a[j] = j < st ? cf[j] : 0.0f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) kj[j][c] = j < st - 1 ? ks[j * kpl + c] : k[c];
+      }
+#pragma unroll
+      for (int j = 0; j < 6; ++j)
+        if (a[j] != 0.0f)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) acc[c] += a[j] * kj[j][c];
+      const float v[3] = {y0[0] + acc[0], y0[1] + acc[1], y0[2] + acc[2]};
+      publish_vec(S.xg + (size_t)((st + 1) & 1) * B * n + (size_t)b * n + i, v, tag);
+    }
+  }
+  if (st >= 2 && st <= 6) return;
+  // k1 (stage 1) or k7 into the buffer that does not hold the committed k1
+  const int into = st == 1 ? 0 : (sh.kc[b] & kKcBuf) ? 0 : 1;
+  float v[5] = {0.0f, tau, 0.0f, 0.0f, 0.0f};
+  if (row) {
+    publish_vec(S.kx + (size_t)into * B * n + (size_t)b * n + i, k, tag);
+    if (st == 7) {
+      // embedded error, torque and <m> at the 5th-order solution (the
+      // stage-7 input), in FP32
+      const float hs = (float)sh.ctl[b].hs, atol = (float)A.atol, rtol = (float)A.rtol;
+      for (int c = 0; c < 3; ++c) {
+        float e = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 7; ++j)
+          if (c_dp_err[j] != 0.0) e = fmaf((float)c_dp_err[j], j == 6 ? k[c] : ks[j * kpl + c], e);
+        const float r = e * hs / (atol + rtol * fmaxf(fabsf(y0[c]), fabsf(mi[c])));
+        v[0] = fmaf(r, r, v[0]);
+      }
+      const float wv = rw.wv / sqrtf(mi[0] * mi[0] + mi[1] * mi[1] + mi[2] * mi[2]);
+      for (int c = 0; c < 3; ++c) v[2 + c] = wv * mi[c];
+    }
+  }
+  small_partial(S, b, v, tag);
+}
+
 template <int RMAX, bool NSMEM, bool PLANAR>
 __device__ __forceinline__ void small_stage(const SmallArgs &S, const SmallSh &sh, const SmallRow &rw, int st,
                                             unsigned tag, int nr, int64_t r0, int &buf) {
   const StageArgs &A = S.A;
-  const int n = (int)A.n, B = A.B, R = S.R;
+  const int n = (int)A.n, B = A.B;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const size_t kpl = (size_t)B * R * 3;  // floats of one derivative plane
-  for (int b = 0; b < B; ++b) {
-    if (sh.ctl[b].done) continue;  // the same in every thread
-    const float *mb = sh.M + (size_t)b * 3 * n;
-    float *red = sh.red + buf * kSmallRed;
-    buf ^= 1;
-    if constexpr (NSMEM) small_product<RMAX, PLANAR>(sh, mb, red, R, nr, n);
-    else small_product_l2<PLANAR>(S, sh, mb, red, nr, r0, n);
-    const bool mine = warp == (b & (kSmallWarps - 1)), row = mine && lane < nr;
-    const int q = lane;
-    const int i = (int)r0 + q;
-    // what needs the other tiles: the exchange sum and m itself
-    float mi[3] = {0.0f, 0.0f, 0.0f}, he[3] = {0.0f, 0.0f, 0.0f};
-    if (row) {
-      for (int c = 0; c < 3; ++c) mi[c] = mb[3 * i + c];
-      if (A.exch) {
-#pragma unroll
-        for (int f = 0; f < 6; ++f)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) he[c] += rw.wex[f] * (mb[3 * rw.nbr[f] + c] - mi[c]);
-      }
+  SmallPre pr = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+  if constexpr (NSMEM) {
+    for (int b = 0; b < B; ++b) {
+      if (sh.ctl[b].done) continue;  // the same in every thread
+      const float *mb = sh.M + b * small_stride(n);
+      float *red = sh.red + buf * kSmallRed;
+      buf ^= 1;
+      small_product<RMAX, PLANAR>(sh, mb, red, S.R, nr, n);
+      const bool mine = warp == (b & (kSmallWarps - 1));
+      if (mine && lane < nr) small_pre(A, rw, mb, (int)r0 + lane, pr);
+      __syncthreads();
+      if (mine) small_rows<kSmallWarps, 3 * RMAX>(S, sh, rw, pr, red, b, st, tag, nr, r0);
     }
-    __syncthreads();
-    if (!mine) continue;
-    float k[3] = {0.0f, 0.0f, 0.0f}, tau = 0.0f;
-    float *ks = sh.k + ((size_t)b * R + q) * 3;  // row q's k1; plane s at + s kpl
-    const float *y0 = sh.y + ((size_t)b * R + q) * 3;
-    if (row) {
-      const float *pb = sh.par + 6 * b;
-      float H[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float s = 0.0f;
-        if constexpr (NSMEM) {
-#pragma unroll
-          for (int w = 0; w < kSmallWarps; ++w) s += red[w * 3 * RMAX + 3 * q + c];
-        } else {
-          s = red[3 * q + c];
-        }
-        H[c] = -s + pb[2 + c];
-        if (A.exch) H[c] += pb[5] * he[c];
+  } else {
+    for (int base = 0; base < B; base += kSmallWarps) {
+      const int end = base + kSmallWarps < B ? base + kSmallWarps : B;
+      float *red = sh.red + buf * kSmallRedL2;
+      buf ^= 1;
+      for (int b = base; b < end; b += 4) {
+        float *rb = red + (b - base) * 3 * kSmallRowsL2;
+        bool live = false;  // the same in every thread
+        for (int s = b; s < b + 4 && s < end; ++s) live = live || !sh.ctl[s].done;
+        if (!live) continue;
+        if (end - b >= 4) small_product_l2<4, PLANAR>(S, sh, b, rb, nr, r0, n);
+        else if (end - b == 3) small_product_l2<3, PLANAR>(S, sh, b, rb, nr, r0, n);
+        else if (end - b == 2) small_product_l2<2, PLANAR>(S, sh, b, rb, nr, r0, n);
+        else small_product_l2<1, PLANAR>(S, sh, b, rb, nr, r0, n);
       }
-      if (rw.kan != 0.0f) {
-        const float me = mi[0] * rw.axis[0] + mi[1] * rw.axis[1] + mi[2] * rw.axis[2];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) H[c] += rw.kan * me * rw.axis[c];
-      }
-      const float mxh = llg(pb[0], pb[1], mi, H, k);
-      if (st == 1 || st == 7) tau = mxh / rw.Ms;
-      for (int c = 0; c < 3; ++c) ks[(st - 1) * kpl + c] = k[c];
-      if (st >= 2 && st <= 6) {
-        // this row's input of the next stage: y + sum_j (h a_sj) k_j
-        const float *cf = sh.coef + 36 * b + 6 * (st - 1);
-        float acc[3] = {0.0f, 0.0f, 0.0f}, a[6], kj[6][3];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {  // all loads before the sums
-          a[j] = j < st ? cf[j] : 0.0f;
-#pragma unroll
-          for (int c = 0; c < 3; ++c) kj[j][c] = j < st - 1 ? ks[j * kpl + c] : k[c];
-        }
-#pragma unroll
-        for (int j = 0; j < 6; ++j)
-          if (a[j] != 0.0f)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc[c] += a[j] * kj[j][c];
-        const float v[3] = {y0[0] + acc[0], y0[1] + acc[1], y0[2] + acc[2]};
-        publish_vec(S.xg + (size_t)((st + 1) & 1) * B * n + (size_t)b * n + i, v, tag);
-      }
+      const int b = base + warp;
+      const bool mine = b < end && !sh.ctl[b].done;
+      if (mine && lane < nr) small_pre(A, rw, sh.M + b * small_stride(n), (int)r0 + lane, pr);
+      __syncthreads();
+      if (mine) small_rows<1, 0>(S, sh, rw, pr, red + warp * 3 * kSmallRowsL2, b, st, tag, nr, r0);
     }
-    if (st >= 2 && st <= 6) continue;
-    // k1 (stage 1) or k7 into the buffer that does not hold the committed k1
-    const int into = st == 1 ? 0 : (sh.kc[b] & kKcBuf) ? 0 : 1;
-    float v[5] = {0.0f, tau, 0.0f, 0.0f, 0.0f};
-    if (row) {
-      publish_vec(S.kx + (size_t)into * B * n + (size_t)b * n + i, k, tag);
-      if (st == 7) {
-        // embedded error, torque and <m> at the 5th-order solution (the
-        // stage-7 input), in FP32
-        const float hs = (float)sh.ctl[b].hs, atol = (float)A.atol, rtol = (float)A.rtol;
-        for (int c = 0; c < 3; ++c) {
-          float e = 0.0f;
-#pragma unroll
-          for (int j = 0; j < 7; ++j)
-            if (c_dp_err[j] != 0.0) e = fmaf((float)c_dp_err[j], j == 6 ? k[c] : ks[j * kpl + c], e);
-          const float r = e * hs / (atol + rtol * fmaxf(fabsf(y0[c]), fabsf(mi[c])));
-          v[0] = fmaf(r, r, v[0]);
-        }
-        const float wv = rw.wv / sqrtf(mi[0] * mi[0] + mi[1] * mi[1] + mi[2] * mi[2]);
-        for (int c = 0; c < 3; ++c) v[2 + c] = wv * mi[c];
-      }
-    }
-    small_partial(S, b, v, tag);
   }
 }
 
@@ -1075,7 +1143,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
     sh.k[(size_t)b * R * 3 + qc] = A.k[0][o];
   }
   if (S.init)
-    for (int64_t q = tid; q < (int64_t)B * 3 * n; q += kSmallThreads) sh.M[q] = A.y[q];
+    for (int b = 0; b < B; ++b)
+      for (int q = tid; q < 3 * (int)n; q += kSmallThreads) sh.M[b * small_stride(n) + q] = A.y[(size_t)b * 3 * n + q];
   __syncthreads();
 
   if (S.init) {  // k1 and the torque at the state
@@ -1109,7 +1178,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
       const int kc = sh.kc[b];
       const bool adopt = it > 0 && sh.ctl[b].accepted;
       const float a21 = sh.coef[36 * b];
-      float *mb = sh.M + (size_t)b * 3 * n;
+      float *mb = sh.M + b * small_stride(n);
       const float *yb = A.y + (size_t)b * 3 * n, *kb = A.k[0] + (size_t)b * 3 * n;
       if (!adopt) {  // the committed y into sh.M
         if (kc & kKcY)
@@ -1141,7 +1210,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
       if (st > 2) {  // all tiles' input of this stage
         for (int b = 0; b < B; ++b) {
           if (sh.ctl[b].done) continue;
-          float *mb = sh.M + (size_t)b * 3 * n;
+          float *mb = sh.M + b * small_stride(n);
           ok = poll_vecs(S, S.xg + (size_t)(st & 1) * B * n + (size_t)b * n, (int)n, seq + st - 2,
                          [&](int j, const float *v) {
                            for (int c = 0; c < 3; ++c) mb[3 * j + c] = v[c];
@@ -1177,7 +1246,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
       if (lane < nr) {
         float *y0 = sh.y + ((size_t)b * R + lane) * 3;
         float *k1 = sh.k + ((size_t)b * R + lane) * 3;
-        small_unit(sh.M + (size_t)b * 3 * n + 3 * (r0 + lane), y0);
+        small_unit(sh.M + b * small_stride(n) + 3 * (r0 + lane), y0);
         publish_vec(S.yx + (size_t)b * n + r0 + lane, y0, seq);
         for (int c = 0; c < 3; ++c) k1[c] = k1[6 * kpl + c];
       }
@@ -1486,10 +1555,14 @@ bool small_plan(mt_integrator *I) {
     if (R > (nsmem ? 8 : 2 * kSmallWarps)) continue;
     if (!nsmem && (T->bytes > kSmallL2Bytes || T->L.TC % 4 != 0)) continue;
     const size_t bytes = small_smem(n, I->B, R, nsmem).total;
-    // (the limit counts one buffer of row sums, and H_d, the torque and the
+    // (the limit counts one buffer of row sums, unpadded states, and H_d, the torque and the
     // constants of the CTA's rows, once held in shared memory: the same tile
     // sets qualify for this path whatever its kernel keeps there)
-    size_t counted = bytes - sizeof(float) * kSmallRed;
+    size_t counted = bytes - sizeof(float) * (2 * (nsmem ? kSmallRed : kSmallRedL2) - kSmallRed);
+    size_t state = 0, unpadded = 0;
+    small_take(state, sizeof(float) * ((size_t)I->B * small_stride(n) + 12));
+    small_take(unpadded, sizeof(float) * I->B * 3 * n);
+    counted += unpadded - state;
     for (const int per_row : {3 * I->B, I->B, 6, 6, 1, 3, 1}) small_take(counted, sizeof(float) * R * per_row);
     if (counted > kSmallSmemMax) continue;
     const int G = (int)((n + R - 1) / R);

@@ -30,7 +30,8 @@ def ctx(mt):
 
 
 @pytest.mark.parametrize("shape,B", [((1, 1, 1), 1), ((2, 1, 1), 1), ((5, 3, 1), 9), ((17, 9, 1), 2), ((19, 8, 2), 1),
-                                     ((32, 16, 2), 1), ((40, 26, 1), 1), ((60, 30, 1), 2)])
+                                     ((32, 16, 2), 1), ((40, 26, 1), 1), ((60, 30, 1), 2),
+                                     ((60, 30, 1), 1), ((14, 12, 12), 3), ((40, 20, 2), 9)])
 def test_rejections_and_splits_match_graph(mt, ctx, shape, B):
     nx, ny, nz = shape
     t = wl.film(nx, ny, nz, size=(nx * 6e-9, ny * 6e-9, nz * 4e-9))
