@@ -247,9 +247,9 @@ MT_API mt_status mt_demag_assemble(mt_tiles *tiles, mt_prec prec, mt_tensor **ou
  * tensor of tile j at the centre of tile i depends only on c_i - c_j and is
  * even in it, so N_ij = N_ji and the whole tensor is symmetric (Sec. 3.2).
  * An FP32 streaming tensor of more than 4,096 such tiles (any number with
- * MT_LAYOUT_STREAM_HALF; below ~3,600 tiles the full storage's product is
- * the faster one, one simulation) then stores only the upper triangle: 16-row panel p keeps its 128-column chunks from the
- * one holding its own rows on (about n^2 / 2 blocks); the product applies
+ * MT_LAYOUT_STREAM_HALF) then stores only the upper triangle: 16-row panel
+ * p keeps its 128-column chunks from the one holding its own rows on (about
+ * n^2 / 2 blocks); the product applies
  * each off-diagonal chunk to its rows and, transposed, to its columns (a
  * column work area of 1.5 KB per stored chunk and simulation, held by the
  * tensor or the integrator).  Stored half, the tensor leaves out zz: a
@@ -259,14 +259,13 @@ MT_API mt_status mt_demag_assemble(mt_tiles *tiles, mt_prec prec, mt_tensor **ou
  * others 5 (xx, xy, xz, yy, yz); assembly checks the identity on every block
  * and otherwise stores all 6 planes (mt_tensor_info.planes tells).
  * mt_tensor_info.half tells;
- * MT_LAYOUT_STREAM_FULL stores every block.  The half storage's product is
- * the faster one for products over 1 or 2 simulations (n = 10,000 film:
- * 0.11 against 0.25 ms for one, 0.15 against 0.26 ms for two); over 3 or
- * more simulations the full storage is (two passes, 0.31 against 0.24 ms
- * for four), so a caller that batches 3 or more should assemble
- * MT_LAYOUT_STREAM_FULL.  A pass over two simulations forms the row sums in
- * another order than a pass over one (each chunk's warp total first), so a
- * simulation's field from a half-stored tensor in a pair and alone agree to
+ * MT_LAYOUT_STREAM_FULL stores every block.  Up to four simulations share a
+ * read of either storage; the half storage's product is the faster one for
+ * every batch (n = 10,000 film, half against full: 0.11 and 0.25 ms for one
+ * simulation, 0.14 and 0.25 for two, 0.20 and 0.24 for four, 0.37 and 0.46 for
+ * eight).  A pass over two or more simulations forms the row sums in another
+ * order than a pass over one (each chunk's warp total first), so a
+ * simulation's field from a half-stored tensor in a batch and alone agree to
  * rounding, not bit for bit.
  * Thresholding and the allocation-free product need every block stored. */
 /* As mt_demag_assemble, with an explicit storage layout (mt_layout_kind).
@@ -567,11 +566,7 @@ typedef struct {
   int32_t layout;           /* mt_layout_kind of cached tensors (not        */
                             /* MT_LAYOUT_SPARSE; MT_LAYOUT_STREAM_HALF      */
                             /* fails the jobs of geometries whose tiles     */
-                            /* differ in shape); with MT_LAYOUT_STREAM and  */
-                            /* max_batch >= 3 every block is stored         */
-                            /* (MT_LAYOUT_STREAM_FULL): the half storage's  */
-                            /* product is faster for one or two simulations */
-                            /* per pass only                                */
+                            /* differ in shape)                             */
   int32_t form;             /* mt_form of every job                         */
   double gamma;             /* m/(A s)                                      */
   mt_ode_opts ode;          /* integrator options; max_steps caps each job  */

@@ -22,7 +22,7 @@
 //   * before waiting on the kernel ahead of it (which writes the operand,
 //     never the tensor), each CTA prefetches its first chunks into L2.
 // A tensor of tiles of one shape is symmetric and stored as its upper
-// triangle (Sec. 3.2); k_matvec_half and k_half_cols below apply it, each
+// triangle (Sec. 3.2); k_matvec_half and k_half_sum below apply it, each
 // stored chunk above the diagonal also to its columns.
 #include <algorithm>
 #include <cstdio>
@@ -523,13 +523,18 @@ __global__ void __launch_bounds__(MvShape<PREC, SB>::THREADS, 1) k_matvec(MvArgs
 // applied to its rows; a group above the diagonal (q > R) is applied,
 // transposed, to its columns too.  Its K chunks arrive one after the other,
 // so a thread keeps its columns' sums over the whole group in registers, and
-// the consumer warps meet once per group (not per chunk) to add them.  A
-// group's column sums go to the work area (a group split between two CTAs
-// is finished by the last of them to arrive, adding the parts in CTA
-// order); k_half_cols then adds, for each column chunk q, the sums of the
-// groups (R, q), R < q, in order of R and subtracts them from H.  Up to 2
-// simulations share a chunk read (more take several passes: their row
-// sums would not fit the registers).
+// the consumer warps meet once per group (not per chunk) to add them.  Up to 4
+// simulations share a chunk read.
+// Where a CTA's range ends inside a group or a super-row, another CTA holds
+// the rest.  Nobody waits for the other: the CTA with a group's last chunk
+// leaves its column sums in the group's place of the work area, the CTA with a
+// super-row's last chunk its row sums in H, and a CTA whose range ends inside
+// one leaves what it has in a place of its own, with a tag that says which
+// (at most one group and one super-row per CTA).  k_half_sum then adds, for each
+// column chunk q, the sums of the groups (R, q), R < q, and the tagged parts, in
+// a fixed order.  (Split sums finished by the last CTA to arrive, with fences,
+// counters and dependent loads at the end of every CTA, took 5 to 9 us of each
+// product.)
 // chunks a half-product CTA prefetches into L2 before the PDL wait
 constexpr int kHalfPrefetch = 18;
 
@@ -543,30 +548,71 @@ struct HalfShape {
   static constexpr int XS_BYTES = 3 * C::TC * 4;
   static constexpr int STAGE_BYTES = DATA_BYTES + SB * XS_BYTES;
   static constexpr int CB_BYTES = NCW * SB * 3 * C::TC * 4;  // the warps' column sums of a group
-  static constexpr int XI_BYTES = NCW * SB * K * RPW * 16;   // each warp's row operand (x, y, z, 0)
-  static constexpr int STAGES = (C::STAGES * STAGE_BYTES + CB_BYTES + XI_BYTES <= 226 * 1024)
+  static constexpr int XI_BYTES = NCW * SB * K * RPW * 32;   // each warp's row operand (x x y y z z - -)
+  static constexpr int RS_BYTES = SB > 1 ? NCW * K * 32 * 4 : 0;  // running row sums per warp, panel and lane
+  static constexpr int FIXED_BYTES = CB_BYTES + XI_BYTES + RS_BYTES;
+  static constexpr int STAGES = (C::STAGES * STAGE_BYTES + FIXED_BYTES <= 226 * 1024)
                                     ? C::STAGES
-                                    : (226 * 1024 - CB_BYTES - XI_BYTES) / STAGE_BYTES;
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + CB_BYTES + XI_BYTES + 2 * STAGES * 8 + 16;
+                                    : (226 * 1024 - FIXED_BYTES) / STAGE_BYTES;
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + FIXED_BYTES + 2 * STAGES * 8 + 16;
   static constexpr int THREADS = (NCW + 1) * 32;
   static constexpr int NV = K * RPW * 3;  // row values a warp holds per simulation
   static constexpr int NVAL = SB * RPW * 3;        // a warp's row values per chunk
-  static constexpr int NSLOT = NVAL <= 8 ? 8 : 16;  // padded for the reduce-scatter
-  static_assert(SB == 1 || SB == 2, "one or two simulations per chunk read");
+  static constexpr int NSLOT = NVAL <= 8 ? 8 : NVAL <= 16 ? 16 : 32;  // padded for the reduce-scatter
+  static_assert(SB == 1 || SB == 2 || SB == 4, "simulations per chunk read");
   static_assert(C::VEC == 4 && C::TC == 32 * C::VEC && C::TR % NCW == 0, "float4 columns, whole rows per warp");
-  static_assert((NCW * 32) % C::TC == 0 && NV <= 64 && 16 * SB <= 32, "flush and operand lanes");
+  static_assert((NCW * 32) % C::TC == 0 && NV <= 64, "flush lanes");
   static_assert(STAGES >= 2 && SMEM_BYTES <= 227 * 1024, "ring within one CTA's shared memory");
+};
+
+// Packed pairs of FP32 (two adjacent columns): one instruction multiplies and
+// adds both, each rounded as a scalar would be.  With two consumer warps per
+// scheduler the half product is bound by its instructions' issue and latency,
+// not by the FP32 lanes (8,000-tile cube, two simulations: 122 us with scalar
+// multiply-adds, 109 with pairs, 99 with nothing waited for at the ranges'
+// ends).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 pair2(float v) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
+  return d;
+}
+__device__ __forceinline__ float lo2(f32x2 a) { return __uint_as_float((unsigned)a); }
+__device__ __forceinline__ float hi2(f32x2 a) { return __uint_as_float((unsigned)(a >> 32)); }
+// 4 floats (16-byte aligned) as two pairs
+__device__ __forceinline__ void load_pairs(const void *p, f32x2 *v) {
+  const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(p);
+  v[0] = u.x;
+  v[1] = u.y;
+}
+// a row's operand, each component twice (as the pairs multiply it)
+struct alignas(16) RowOperand {
+  float x[2], y[2], z[2], pad[2];
 };
 
 struct HalfArgs {
   const float *tensor;
   const float *xs;   // [b][q][3][TC], Ms m
   float *H;
-  float *part;       // row partials of super-rows shared by CTAs [2 G][SB][K TR][3]
-  int *count;        // arrival counters per (simulation group, super-row, warp)
-  int *gcount;       // arrival counters per (simulation group, group)
+  float *rowsplit;   // row sums of the super-row a CTA's range ends in [G][SB][K TR][3]
+  int2 *tag;         // per CTA: that super-row (g Q + R) and that group's column chunk (g Q + q), -1: none [G]
   float *colpart;    // column sums of every group above the diagonal [NG][NGR][SB][3][TC]
-  float *colsplit;   // parts of the groups shared by CTAs [2 G][SB][3][TC]
+  float *colsplit;   // column sums of the group a CTA's range ends in [G][SB][3][TC]
   const int *active;
   int *status;
   int64_t n, P, Q, CH, NGR;  // NGR = Q (Q + 1) / 2 groups
@@ -626,21 +672,11 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
   using C = MvCfg<PREC>;
   using S = HalfShape<PREC, SB>;
   constexpr int K = S::K, TR = C::TR, TC = C::TC;
-  {
-    // before waiting on the previous kernel (which writes the operand, not
-    // the tensor): the CTA's first ring-full of tensor chunks into L2
-    const int64_t G = gridDim.x, NG = (A.B + SB - 1) / SB, U = NG * A.CH;
-    const int64_t u0 = mtd::sk_begin(blockIdx.x, U, G), u1 = mtd::sk_begin(blockIdx.x + 1, U, G);
-    const int64_t c0 = u0 % A.CH;
-    if (threadIdx.x < kHalfPrefetch && u0 + threadIdx.x < u1 && c0 + threadIdx.x < A.CH)
-      mtd::bulk_prefetch_l2(reinterpret_cast<const unsigned char *>(A.tensor) + (size_t)(c0 + threadIdx.x) * S::DATA_BYTES,
-                            S::DATA_BYTES);
-  }
-  mtd::pdl_enter();
   extern __shared__ __align__(128) unsigned char smem[];
   float *cb = reinterpret_cast<float *>(smem + S::STAGES * S::STAGE_BYTES);
-  float4 *xi_all = reinterpret_cast<float4 *>(smem + S::STAGES * S::STAGE_BYTES + S::CB_BYTES);
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + S::STAGES * S::STAGE_BYTES + S::CB_BYTES + S::XI_BYTES);
+  RowOperand *xi_all = reinterpret_cast<RowOperand *>(smem + S::STAGES * S::STAGE_BYTES + S::CB_BYTES);
+  float *rs_all = reinterpret_cast<float *>(smem + S::STAGES * S::STAGE_BYTES + S::CB_BYTES + S::XI_BYTES);
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + S::STAGES * S::STAGE_BYTES + S::FIXED_BYTES);
   uint64_t *empty = full + S::STAGES;
   volatile int *abort_flag = reinterpret_cast<volatile int *>(empty + S::STAGES);
 
@@ -659,13 +695,38 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
     mtd::fence_mbar_init();
   }
   __syncthreads();
+  // Before the wait on the previous kernel (which writes the operand, not the
+  // tensor nor the active set): the CTA's first chunks, the ring's into shared
+  // memory (as far as they are the first ones the loop below takes: units of
+  // one live simulation group), the next ones into L2
+  const int64_t g0 = u0 / A.CH, pre_end = u1 < (g0 + 1) * A.CH ? u1 : (g0 + 1) * A.CH;
+  const int pre = !half_live(A, g0, SB) ? 0 : (int)(pre_end - u0 < S::STAGES ? pre_end - u0 : S::STAGES);
+  auto chunk_at = [&](int64_t u) {
+    return reinterpret_cast<const unsigned char *>(A.tensor) + (size_t)(u % A.CH) * S::DATA_BYTES;
+  };
+  if (threadIdx.x == S::NCW * 32) {
+    const uint64_t pol_stream = mtd::policy_evict_first();
+    for (int j = 0; j < pre; ++j) {
+      mtd::mbar_arrive_expect_tx(&full[j], S::STAGE_BYTES);
+      mtd::bulk_g2s(smem + (size_t)j * S::STAGE_BYTES, chunk_at(u0 + j), S::DATA_BYTES, &full[j], pol_stream);
+    }
+  }
+  if (threadIdx.x >= pre && threadIdx.x < kHalfPrefetch && u0 + threadIdx.x < u1)
+    mtd::bulk_prefetch_l2(chunk_at(u0 + threadIdx.x), S::DATA_BYTES);
+  mtd::pdl_enter();
 
   if (warp == S::NCW) {
     // ---------------- producer: the CTA's units in storage order ----------------
+    if (lane == 1) {  // what the range ends in: a super-row, a group above the diagonal
+      GroupCursor gc;
+      const int64_t gs = group_decode<K>(A, u1 - 1, gc);
+      const int64_t su1 = gc.R == A.Q - 1 ? (gc.g + 1) * A.CH : gc.g * A.CH + (int64_t)K * half_gbase(gc.R + 1, A.Q);
+      const bool in_group = u1 < gs + group_len<K>(A, gc) && gc.q > gc.R;
+      A.tag[kcta] = make_int2(u1 < su1 ? (int)(gc.g * A.Q + gc.R) : -1, in_group ? (int)(gc.g * A.Q + gc.q) : -1);
+    }
     if (lane == 0) {
       const uint64_t pol_stream = mtd::policy_evict_first();
       const uint64_t pol_keep = mtd::policy_evict_last();
-      const unsigned char *tens = reinterpret_cast<const unsigned char *>(A.tensor);
       const unsigned char *xs = reinterpret_cast<const unsigned char *>(A.xs);
       int it = 0;
       GroupCursor gc;
@@ -685,9 +746,10 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
             }
           }
           unsigned char *st = smem + (size_t)s * S::STAGE_BYTES;
-          const int64_t c = gs - gc.g * A.CH + k;  // stored chunk
-          mtd::mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
-          mtd::bulk_g2s(st, tens + (size_t)c * S::DATA_BYTES, S::DATA_BYTES, &full[s], pol_stream);
+          if (it >= pre) {
+            mtd::mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
+            mtd::bulk_g2s(st, chunk_at(gs + k), S::DATA_BYTES, &full[s], pol_stream);
+          }
 #pragma unroll
           for (int m = 0; m < SB; ++m) {
             const int64_t b = gc.g * SB + m < A.B ? gc.g * SB + m : 0;
@@ -712,210 +774,91 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
   // - One simulation: lane l keeps the running sums of its part of every row
   //   value of every panel (acc, K RPW 3 registers) and the warp adds them
   //   over its lanes at the super-row's flush.
-  // - Two (twice those sums spilled registers): after each chunk the warp's
-  //   NVAL row values (value (m RPW + r) 3 + c: simulation m, row r,
+  // - Two or four (twice those sums spilled registers): after each chunk the
+  //   warp's NVAL row values (value (m RPW + r) 3 + c: simulation m, row r,
   //   component c) are added over the lanes by a reduce-scatter that leaves
   //   value l / LPS in lane l, which keeps its running sum for the chunk's
-  //   panel k in accs[k].  A simulation's sums then run in another order
-  //   than alone (each chunk's warp total first): equal to rounding.
-  constexpr bool SCATTER = SB == 2;
+  //   panel k in shared memory, rs[32 k] (so that the chunks' loop need not be
+  //   unrolled: K unrolled bodies of four simulations waited for instructions
+  //   more than for anything else).  A simulation's sums then run in another
+  //   order than alone (each chunk's warp total first): equal to rounding.
+  constexpr bool SCATTER = SB >= 2;
   constexpr int NVAL = S::NVAL, NSLOT = S::NSLOT, LPS = 32 / NSLOT;
   float acc[SCATTER ? 1 : SB][SCATTER ? 1 : K][S::RPW][3];
-  float accs[SCATTER ? K : 1];
-  const int my_val = lane / LPS;
-  float4 *xi = xi_all + warp * SB * K * S::RPW;  // [m][k RPW + r]
+  float *rs = rs_all + warp * K * 32 + lane;
+  RowOperand *xi = xi_all + warp * SB * K * S::RPW;  // [m][k RPW + r]
   int64_t sr_cur = -1;  // current (simulation group, super-row) = g Q + R
   int it = 0;
   bool aborted = false;
   const int ct = threadIdx.x;  // consumer thread 0 .. 32 NCW - 1
-  __shared__ int split_last;
 
   auto out = [&](int64_t b) -> float * {
     return (b < A.B && (!A.active || A.active[b])) ? A.H + (size_t)b * 3 * A.n : nullptr;
   };
 
-  // rows of super-row sr: warp totals, then written (or, for a super-row
-  // shared by CTAs, parked and added in CTA order by the last to arrive)
-  auto flush_lane = [&](int64_t sr) {
-    if constexpr (!SCATTER) {
-#pragma unroll
-      for (int m = 0; m < SB; ++m)
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-#pragma unroll
-          for (int r = 0; r < S::RPW; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc[m][k][r][c] = mtd::warp_sum(acc[m][k][r][c]);
-      const int64_t g = sr / A.Q, R = sr - g * A.Q;
-      const int64_t su0 = g * A.CH + (int64_t)K * half_gbase(R, A.Q);
-      const int64_t su1 = (R == A.Q - 1) ? (g + 1) * A.CH : g * A.CH + (int64_t)K * half_gbase(R + 1, A.Q);
-      const int64_t kf = mtd::sk_owner(su0, U, G), kl = mtd::sk_owner(su1 - 1, U, G);
-      // lane l holds values v = l and l + 32 (v = (k RPW + r) 3 + c)
-      float mine[SB][2];
-#pragma unroll
-      for (int m = 0; m < SB; ++m) {
-        mine[m][0] = mine[m][1] = 0.0f;
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-#pragma unroll
-          for (int r = 0; r < S::RPW; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const int v = (k * S::RPW + r) * 3 + c;
-              if (v == lane) mine[m][0] = acc[m][k][r][c];
-              if (v == lane + 32) mine[m][1] = acc[m][k][r][c];
-            }
+  // rows of super-row sr: warp totals, written to H by the CTA with the
+  // super-row's last chunk, else parked
+  auto flush_rows = [&](int64_t sr) {
+    const int64_t g = sr / A.Q, R = sr - g * A.Q;
+    const int64_t su1 = (R == A.Q - 1) ? (g + 1) * A.CH : g * A.CH + (int64_t)K * half_gbase(R + 1, A.Q);
+    const bool last = su1 <= u1;
+    const int64_t row0 = R * K * TR;
+    // value c of the row in super-row row `row_in`, simulation m, row slot kr
+    auto store = [&](int m, int kr, int c, int row_in, float v) {
+      if (!last) {
+        A.rowsplit[((kcta * SB + m) * K * TR + row_in) * 3 + c] = v;
+        return;
       }
-      auto row_of = [&](int v) {  // row within the super-row
-        const int k = v / (S::RPW * 3), r = (v / 3) % S::RPW;
-        return k * TR + warp * S::RPW + r;
-      };
       // traceless storage: the self block's N_zz is 1 - xx - yy, the stream
       // gave -(xx + yy), so the row's z sum lacks Ms_i m_i,z (its operand)
-      auto self_z = [&](int m, int v) -> float {
-        if constexpr (C::NPLANE == 3 || C::NPLANE == 5) {
-          if (v % 3 != 2) return 0.0f;
-          const int k = v / (S::RPW * 3), r = (v / 3) % S::RPW;
-          return xi[m * K * S::RPW + k * S::RPW + r].z;
-        } else {
-          return 0.0f;
-        }
-      };
-      const int64_t row0 = R * K * TR;
-      if (kf == kl) {
+      if (traceless(C::NPLANE) && c == 2) v += xi[m * K * S::RPW + kr].z[0];
+      float *H = out(g * SB + m);
+      if (H && row0 + row_in < A.n) H[3 * (row0 + row_in) + c] = -v;
+    };
+    if constexpr (!SCATTER) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int v = lane + 32 * h;
-          if (v >= S::NV) continue;
-          const int64_t row = row0 + row_of(v);
-          if (row >= A.n) continue;
+      for (int k = 0; k < K; ++k)
 #pragma unroll
-          for (int m = 0; m < SB; ++m)
-            if (float *H = out(g * SB + m)) H[3 * row + v % 3] = -(mine[m][h] + self_z(m, v));
-        }
-        return;
-      }
-      const int64_t slot = (u0 >= su0) ? 2 * kcta : 2 * kcta + 1;  // the super-row is this CTA's first or last
+        for (int r = 0; r < S::RPW; ++r)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int v = lane + 32 * h;
-        if (v >= S::NV) continue;
+          for (int c = 0; c < 3; ++c) acc[0][k][r][c] = mtd::warp_sum(acc[0][k][r][c]);
+      // lane l holds values v = l and l + 32 (v = (k RPW + r) 3 + c)
+      float mine[2] = {0.0f, 0.0f};
 #pragma unroll
-        for (int m = 0; m < SB; ++m) A.part[((slot * SB + m) * K * TR + row_of(v)) * 3 + v % 3] = mine[m][h];
-      }
-      __threadfence();
-      __syncwarp();
-      int last = 0;
-      if (lane == 0) last = (atomicAdd(&A.count[sr * S::NCW + warp], 1) == (int)(kl - kf));
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (!last) return;
-      __threadfence();
-      // the parts in CTA order, each CTA's values loaded together
-      float tot[2][SB];
+      for (int k = 0; k < K; ++k)
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+        for (int r = 0; r < S::RPW; ++r)
 #pragma unroll
-        for (int m = 0; m < SB; ++m) tot[h][m] = 0.0f;
-      for (int64_t kk = kf; kk <= kl; ++kk) {
-        const int64_t sl = (mtd::sk_begin(kk, U, G) >= su0) ? 2 * kk : 2 * kk + 1;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int v = lane + 32 * h;
-          if (v >= S::NV) continue;
-#pragma unroll
-          for (int m = 0; m < SB; ++m)
-            tot[h][m] += __ldcg(&A.part[((sl * SB + m) * K * TR + row_of(v)) * 3 + v % 3]);
-        }
-      }
+          for (int c = 0; c < 3; ++c) {
+            const int v = (k * S::RPW + r) * 3 + c;
+            if (v == lane) mine[0] = acc[0][k][r][c];
+            if (v == lane + 32) mine[1] = acc[0][k][r][c];
+          }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int v = lane + 32 * h;
-        if (v >= S::NV) continue;
-        const int64_t row = row0 + row_of(v);
-#pragma unroll
-        for (int m = 0; m < SB; ++m) {
-          float *H = out(g * SB + m);
-          if (H && row < A.n) H[3 * row + v % 3] = -(tot[h][m] + self_z(m, v));
-        }
+        const int v = lane + 32 * h, kr = v / 3;
+        if (v < S::NV) store(0, kr, v % 3, (kr / S::RPW) * TR + warp * S::RPW + kr % S::RPW, mine[h]);
       }
-      if (lane == 0) A.count[sr * S::NCW + warp] = 0;  // ready for the next launch
-        }
-  };
-
-  // the same for SCATTER: lane l holds value j = l / LPS of every panel; the
-  // LPS lanes of a value share the panels (lane l takes k = l % LPS,
-  // l % LPS + LPS, ...)
-  auto flush_scatter = [&](int64_t sr) {
-    if constexpr (SCATTER) {
-      const int64_t g = sr / A.Q, R = sr - g * A.Q;
-      const int64_t su0 = g * A.CH + (int64_t)K * half_gbase(R, A.Q);
-      const int64_t su1 = (R == A.Q - 1) ? (g + 1) * A.CH : g * A.CH + (int64_t)K * half_gbase(R + 1, A.Q);
-      const int64_t kf = mtd::sk_owner(su0, U, G), kl = mtd::sk_owner(su1 - 1, U, G);
-      const bool valid = my_val < NVAL;
-      const int m = my_val / (S::RPW * 3), r = (my_val / 3) % S::RPW, c = my_val % 3;
-      const int row_in = warp * S::RPW + r;  // row within each panel
-      auto self_z = [&](int k) -> float {  // as in flush_lane
-        if constexpr (C::NPLANE == 3 || C::NPLANE == 5) {
-          return c == 2 ? xi[m * K * S::RPW + k * S::RPW + r].z : 0.0f;
-        } else {
-          return 0.0f;
-        }
-      };
-      const int64_t row0 = R * K * TR;
-      float *H = valid ? out(g * SB + m) : nullptr;
-      if (kf == kl) {
+    } else {
+      // lane l holds value l / LPS of every panel; the LPS lanes of a value
+      // share the panels
+      const int v = lane / LPS, m = v / (S::RPW * 3), r = (v / 3) % S::RPW;
+      if (v < NVAL)
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-          if (!valid || k % LPS != lane % LPS) continue;
-          const int64_t row = row0 + k * TR + row_in;
-          if (H && row < A.n) H[3 * row + c] = -(accs[k] + self_z(k));
-        }
-        return;
-      }
-      const int64_t slot = (u0 >= su0) ? 2 * kcta : 2 * kcta + 1;  // the super-row is this CTA's first or last
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        if (!valid || k % LPS != lane % LPS) continue;
-        A.part[((slot * SB + m) * K * TR + k * TR + row_in) * 3 + c] = accs[k];
-      }
-      __threadfence();
-      __syncwarp();
-      int last = 0;
-      if (lane == 0) last = (atomicAdd(&A.count[sr * S::NCW + warp], 1) == (int)(kl - kf));
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (!last) return;
-      __threadfence();
-      // the parts in CTA order, each CTA's values loaded together
-      float tot[K];
-#pragma unroll
-      for (int k = 0; k < K; ++k) tot[k] = 0.0f;
-      for (int64_t kk = kf; kk <= kl; ++kk) {
-        const int64_t sl = (mtd::sk_begin(kk, U, G) >= su0) ? 2 * kk : 2 * kk + 1;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          if (!valid || k % LPS != lane % LPS) continue;
-          tot[k] += __ldcg(&A.part[((sl * SB + m) * K * TR + k * TR + row_in) * 3 + c]);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        if (!valid || k % LPS != lane % LPS) continue;
-        const int64_t row = row0 + k * TR + row_in;
-        if (H && row < A.n) H[3 * row + c] = -(tot[k] + self_z(k));
-      }
-      if (lane == 0) A.count[sr * S::NCW + warp] = 0;  // ready for the next launch
-        }
-  };
-  auto flush_rows = [&](int64_t sr) {
-    if constexpr (SCATTER) flush_scatter(sr);
-    else flush_lane(sr);
+        for (int k = lane % LPS; k < K; k += LPS)
+          store(m, k * S::RPW + r, v % 3, k * TR + warp * S::RPW + r, rs[32 * k]);
+    }
   };
 
   // the chunks kb .. ke - 1 of one group; STRICT: also its column sums
-  auto run_group = [&](auto strict_c, const GroupCursor &gc, int kb, int ke, float colp[SB][4][3]) {
+  auto run_group = [&](auto strict_c, const GroupCursor &gc, int kb, int ke, f32x2 (&colp)[SB][3][2]) {
     constexpr bool STRICT = decltype(strict_c)::value;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
+    // planes: xx xy (xz) yy (yz) (zz); FLAT: no xz, yz (a single layer);
+    // TRACE: zz = -(xx + yy) (the self blocks' +1 is added in flush_rows)
+    constexpr bool FLAT = C::PLANAR, TRACE = traceless(C::NPLANE);
+    constexpr int YY = FLAT ? 2 : 3;
+#pragma unroll(SCATTER ? 1 : K)
+    for (int k = SCATTER ? kb : 0; k < (SCATTER ? ke : K); ++k) {
       if (k < kb || k >= ke) continue;
       const int s = it % S::STAGES;
       const uint32_t ph = (uint32_t)(it / S::STAGES) & 1u;
@@ -933,156 +876,71 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
       }
       if (!aborted) {
         const unsigned char *st = smem + (size_t)s * S::STAGE_BYTES;
-        float X[SB][4], Y[SB][4], Z[SB][4];
+        // one or two simulations' operands stay in registers over the rows
+        constexpr bool HOLD = SB <= 2;
+        f32x2 X[HOLD ? SB : 1][3][2];
+        auto load_x = [&](int m, f32x2 (&x)[3][2]) {
 #pragma unroll
-        for (int m = 0; m < SB; ++m) {
-          const unsigned char *xsm = st + S::DATA_BYTES + m * S::XS_BYTES;
-          load_xs<PREC>(xsm, 0, lane, X[m]);
-          load_xs<PREC>(xsm, 1, lane, Y[m]);
-          load_xs<PREC>(xsm, 2, lane, Z[m]);
+          for (int c = 0; c < 3; ++c)
+            load_pairs(st + S::DATA_BYTES + m * S::XS_BYTES + c * TC * 4 + lane * 16, x[c]);
+        };
+        if constexpr (HOLD) {
+#pragma unroll
+          for (int m = 0; m < SB; ++m) load_x(m, X[m]);
         }
 #pragma unroll
         for (int r = 0; r < S::RPW; ++r) {
           const int row = warp * S::RPW + r;
-          float4 xr[SB];
-          if constexpr (STRICT) {
+          f32x2 n[C::NPLANE][2], zz[2];
 #pragma unroll
-            for (int m = 0; m < SB; ++m) xr[m] = xi[m * K * S::RPW + k * S::RPW + r];
-          }
-          if constexpr (C::NPLANE == 3) {
-            // zz = -(xx + yy) (trace 0; the self blocks' +1 is added in
-            // flush_rows)
-            float nxx[4], nxy[4], nyy[4];
-            load_vals<PREC>(st, 0, row, lane, nxx);
-            load_vals<PREC>(st, 1, row, lane, nxy);
-            load_vals<PREC>(st, 2, row, lane, nyy);
+          for (int e = 0; e < C::NPLANE; ++e) load_pairs(st + ((e * TR + row) * TC + lane * 4) * 4, n[e]);
 #pragma unroll
-            for (int m = 0; m < SB; ++m) {
-              float sx = 0.0f, sy = 0.0f, sz = 0.0f;
+          for (int p = 0; p < 2; ++p)
+            zz[p] = TRACE ? mul2(add2(n[0][p], n[YY][p]), pair2(-1.0f)) : n[C::NPLANE - 1][p];
 #pragma unroll
-              for (int v = 0; v < 4; ++v) {
-                const float nzz = -(nxx[v] + nyy[v]);
-                sx = fmaf(nxx[v], X[m][v], fmaf(nxy[v], Y[m][v], sx));
-                sy = fmaf(nxy[v], X[m][v], fmaf(nyy[v], Y[m][v], sy));
-                sz = fmaf(nzz, Z[m][v], sz);
-                if constexpr (STRICT) {
-                  colp[m][v][0] = fmaf(nxx[v], xr[m].x, fmaf(nxy[v], xr[m].y, colp[m][v][0]));
-                  colp[m][v][1] = fmaf(nxy[v], xr[m].x, fmaf(nyy[v], xr[m].y, colp[m][v][1]));
-                  colp[m][v][2] = fmaf(nzz, xr[m].z, colp[m][v][2]);
-                }
+          for (int m = 0; m < SB; ++m) {
+            if constexpr (!HOLD) load_x(m, X[0]);
+            const f32x2(&x)[3][2] = X[HOLD ? m : 0];
+            f32x2 sum[3] = {0, 0, 0};  // over columns 0, 2 and 1, 3
+            f32x2 xr[3];
+            if constexpr (STRICT) {
+              const RowOperand *o = &xi[m * K * S::RPW + k * S::RPW + r];
+              load_pairs(o, xr);  // (x, x), (y, y)
+              xr[2] = reinterpret_cast<const f32x2 *>(o)[2];
+            }
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+              sum[0] = fma2(n[0][p], x[0][p], fma2(n[1][p], x[1][p], sum[0]));
+              sum[1] = fma2(n[1][p], x[0][p], fma2(n[YY][p], x[1][p], sum[1]));
+              sum[2] = fma2(zz[p], x[2][p], sum[2]);
+              if constexpr (!FLAT) {
+                sum[0] = fma2(n[2][p], x[2][p], sum[0]);
+                sum[1] = fma2(n[4][p], x[2][p], sum[1]);
+                sum[2] = fma2(n[2][p], x[0][p], fma2(n[4][p], x[1][p], sum[2]));
               }
-              if constexpr (SCATTER) {
-                rv[(m * S::RPW + r) * 3 + 0] = sx;
-                rv[(m * S::RPW + r) * 3 + 1] = sy;
-                rv[(m * S::RPW + r) * 3 + 2] = sz;
-              } else {
-                acc[m][k][r][0] += sx;
-                acc[m][k][r][1] += sy;
-                acc[m][k][r][2] += sz;
+              if constexpr (STRICT) {
+                colp[m][0][p] = fma2(n[0][p], xr[0], fma2(n[1][p], xr[1], colp[m][0][p]));
+                colp[m][1][p] = fma2(n[1][p], xr[0], fma2(n[YY][p], xr[1], colp[m][1][p]));
+                colp[m][2][p] = fma2(zz[p], xr[2], colp[m][2][p]);
+                if constexpr (!FLAT) {
+                  colp[m][0][p] = fma2(n[2][p], xr[2], colp[m][0][p]);
+                  colp[m][1][p] = fma2(n[4][p], xr[2], colp[m][1][p]);
+                  colp[m][2][p] = fma2(n[2][p], xr[0], fma2(n[4][p], xr[1], colp[m][2][p]));
+                }
               }
             }
-          } else if constexpr (C::NPLANE == 5) {
-            // zz = -(xx + yy) (trace 0; the self blocks' +1 is added in
-            // flush_rows)
-            float nxx[4], nxy[4], nxz[4], nyy[4], nyz[4];
-            load_vals<PREC>(st, 0, row, lane, nxx);
-            load_vals<PREC>(st, 1, row, lane, nxy);
-            load_vals<PREC>(st, 2, row, lane, nxz);
-            load_vals<PREC>(st, 3, row, lane, nyy);
-            load_vals<PREC>(st, 4, row, lane, nyz);
 #pragma unroll
-            for (int m = 0; m < SB; ++m) {
-              float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-#pragma unroll
-              for (int v = 0; v < 4; ++v) {
-                const float nzz = -(nxx[v] + nyy[v]);
-                sx = fmaf(nxx[v], X[m][v], fmaf(nxy[v], Y[m][v], fmaf(nxz[v], Z[m][v], sx)));
-                sy = fmaf(nxy[v], X[m][v], fmaf(nyy[v], Y[m][v], fmaf(nyz[v], Z[m][v], sy)));
-                sz = fmaf(nxz[v], X[m][v], fmaf(nyz[v], Y[m][v], fmaf(nzz, Z[m][v], sz)));
-                if constexpr (STRICT) {
-                  colp[m][v][0] = fmaf(nxx[v], xr[m].x, fmaf(nxy[v], xr[m].y, fmaf(nxz[v], xr[m].z, colp[m][v][0])));
-                  colp[m][v][1] = fmaf(nxy[v], xr[m].x, fmaf(nyy[v], xr[m].y, fmaf(nyz[v], xr[m].z, colp[m][v][1])));
-                  colp[m][v][2] = fmaf(nxz[v], xr[m].x, fmaf(nyz[v], xr[m].y, fmaf(nzz, xr[m].z, colp[m][v][2])));
-                }
-              }
-              if constexpr (SCATTER) {
-                rv[(m * S::RPW + r) * 3 + 0] = sx;
-                rv[(m * S::RPW + r) * 3 + 1] = sy;
-                rv[(m * S::RPW + r) * 3 + 2] = sz;
-              } else {
-                acc[m][k][r][0] += sx;
-                acc[m][k][r][1] += sy;
-                acc[m][k][r][2] += sz;
-              }
-            }
-          } else if constexpr (C::PLANAR) {
-            float nxx[4], nxy[4], nyy[4], nzz[4];
-            load_vals<PREC>(st, 0, row, lane, nxx);
-            load_vals<PREC>(st, 1, row, lane, nxy);
-            load_vals<PREC>(st, 2, row, lane, nyy);
-            load_vals<PREC>(st, 3, row, lane, nzz);
-#pragma unroll
-            for (int m = 0; m < SB; ++m) {
-              float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-#pragma unroll
-              for (int v = 0; v < 4; ++v) {
-                sx = fmaf(nxx[v], X[m][v], fmaf(nxy[v], Y[m][v], sx));
-                sy = fmaf(nxy[v], X[m][v], fmaf(nyy[v], Y[m][v], sy));
-                sz = fmaf(nzz[v], Z[m][v], sz);
-                if constexpr (STRICT) {
-                  colp[m][v][0] = fmaf(nxx[v], xr[m].x, fmaf(nxy[v], xr[m].y, colp[m][v][0]));
-                  colp[m][v][1] = fmaf(nxy[v], xr[m].x, fmaf(nyy[v], xr[m].y, colp[m][v][1]));
-                  colp[m][v][2] = fmaf(nzz[v], xr[m].z, colp[m][v][2]);
-                }
-              }
-              if constexpr (SCATTER) {
-                rv[(m * S::RPW + r) * 3 + 0] = sx;
-                rv[(m * S::RPW + r) * 3 + 1] = sy;
-                rv[(m * S::RPW + r) * 3 + 2] = sz;
-              } else {
-                acc[m][k][r][0] += sx;
-                acc[m][k][r][1] += sy;
-                acc[m][k][r][2] += sz;
-              }
-            }
-          } else {
-            float nxx[4], nxy[4], nxz[4], nyy[4], nyz[4], nzz[4];
-            load_vals<PREC>(st, 0, row, lane, nxx);
-            load_vals<PREC>(st, 1, row, lane, nxy);
-            load_vals<PREC>(st, 2, row, lane, nxz);
-            load_vals<PREC>(st, 3, row, lane, nyy);
-            load_vals<PREC>(st, 4, row, lane, nyz);
-            load_vals<PREC>(st, 5, row, lane, nzz);
-#pragma unroll
-            for (int m = 0; m < SB; ++m) {
-              float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-#pragma unroll
-              for (int v = 0; v < 4; ++v) {
-                sx = fmaf(nxx[v], X[m][v], fmaf(nxy[v], Y[m][v], fmaf(nxz[v], Z[m][v], sx)));
-                sy = fmaf(nxy[v], X[m][v], fmaf(nyy[v], Y[m][v], fmaf(nyz[v], Z[m][v], sy)));
-                sz = fmaf(nxz[v], X[m][v], fmaf(nyz[v], Y[m][v], fmaf(nzz[v], Z[m][v], sz)));
-                if constexpr (STRICT) {
-                  colp[m][v][0] = fmaf(nxx[v], xr[m].x, fmaf(nxy[v], xr[m].y, fmaf(nxz[v], xr[m].z, colp[m][v][0])));
-                  colp[m][v][1] = fmaf(nxy[v], xr[m].x, fmaf(nyy[v], xr[m].y, fmaf(nyz[v], xr[m].z, colp[m][v][1])));
-                  colp[m][v][2] = fmaf(nxz[v], xr[m].x, fmaf(nyz[v], xr[m].y, fmaf(nzz[v], xr[m].z, colp[m][v][2])));
-                }
-              }
-              if constexpr (SCATTER) {
-                rv[(m * S::RPW + r) * 3 + 0] = sx;
-                rv[(m * S::RPW + r) * 3 + 1] = sy;
-                rv[(m * S::RPW + r) * 3 + 2] = sz;
-              } else {
-                acc[m][k][r][0] += sx;
-                acc[m][k][r][1] += sy;
-                acc[m][k][r][2] += sz;
-              }
+            for (int c = 0; c < 3; ++c) {
+              const float v = lo2(sum[c]) + hi2(sum[c]);
+              if constexpr (SCATTER) rv[(m * S::RPW + r) * 3 + c] = v;
+              else acc[0][k][r][c] += v;
             }
           }
         }
       }
       __syncwarp();
       if (lane == 0) mtd::mbar_arrive(&empty[s]);
-      if constexpr (SCATTER) accs[k] += mtd::warp_reduce_scatter<NSLOT>(rv, lane);  // every lane, aborted or not
+      if constexpr (SCATTER) rs[32 * k] += mtd::warp_reduce_scatter<NSLOT>(rv, lane);  // every lane, aborted or not
     }
   };
 
@@ -1097,7 +955,7 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
       sr_cur = sr;
       if constexpr (SCATTER) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) accs[k] = 0.0f;
+        for (int k = 0; k < K; ++k) rs[32 * k] = 0.0f;
       } else {
 #pragma unroll
         for (int m = 0; m < SB; ++m)
@@ -1107,26 +965,28 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
             for (int r = 0; r < S::RPW; ++r) acc[m][k][r][0] = acc[m][k][r][1] = acc[m][k][r][2] = 0.0f;
       }
       // the operand of this warp's rows of the super-row (column chunk R of
-      // the operand): lane l < 16 SB takes simulation l / 16, row slot l % 16
+      // the operand), one (simulation, row slot) per lane and round
       __syncwarp();
-      if (lane < SB * K * S::RPW) {
-        const int m = lane / (K * S::RPW), kr = lane % (K * S::RPW);
+#pragma unroll
+      for (int l = lane; l < SB * K * S::RPW; l += 32) {
+        const int m = l / (K * S::RPW), kr = l % (K * S::RPW);
         const int k = kr / S::RPW, r = kr % S::RPW;
         const int64_t b = gc.g * SB + m < A.B ? gc.g * SB + m : 0;
         const float *x = A.xs + (size_t)(b * A.Q + gc.R) * 3 * TC + k * TR + warp * S::RPW + r;
-        xi[m * K * S::RPW + kr] = make_float4(__ldg(x), __ldg(x + TC), __ldg(x + 2 * TC), 0.0f);
+        const float v0 = __ldg(x), v1 = __ldg(x + TC), v2 = __ldg(x + 2 * TC);
+        xi[l] = RowOperand{{v0, v0}, {v1, v1}, {v2, v2}, {0.0f, 0.0f}};
       }
       __syncwarp();
     }
-    if (gc.q == gc.R) {  // the diagonal group: rows only
-      run_group(std::false_type{}, gc, kb, ke, nullptr);
-      continue;
-    }
-    float colp[SB][4][3];
+    f32x2 colp[SB][3][2];  // column sums of columns 0, 1 and 2, 3
 #pragma unroll
     for (int m = 0; m < SB; ++m)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) colp[m][v][0] = colp[m][v][1] = colp[m][v][2] = 0.0f;
+      for (int c = 0; c < 3; ++c) colp[m][c][0] = colp[m][c][1] = 0;
+    if (gc.q == gc.R) {  // the diagonal group: rows only
+      run_group(std::false_type{}, gc, kb, ke, colp);
+      continue;
+    }
     run_group(std::true_type{}, gc, kb, ke, colp);
     // column sums of the group: each warp's (its rows) to shared memory,
     // then thread t adds column t % TC, components t / TC, t / TC + 2, ...,
@@ -1135,13 +995,13 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
     for (int m = 0; m < SB; ++m)
 #pragma unroll
       for (int c = 0; c < 3; ++c)
-        *reinterpret_cast<float4 *>(cb + ((warp * SB + m) * 3 + c) * TC + lane * 4) =
-            make_float4(colp[m][0][c], colp[m][1][c], colp[m][2][c], colp[m][3][c]);
+        *reinterpret_cast<ulonglong2 *>(cb + ((warp * SB + m) * 3 + c) * TC + lane * 4) =
+            make_ulonglong2(colp[m][c][0], colp[m][c][1]);
     asm volatile("bar.sync 1, %0;" ::"r"(S::NCW * 32) : "memory");
     constexpr int NT = S::NCW * 32 / TC;  // thread sets over the columns
     const int col = ct % TC;
-    const bool whole = (kb == 0 && ke == len);
-    const int64_t slot = (u0 >= gs) ? 2 * kcta : 2 * kcta + 1;  // a split group: this CTA's first or last
+    // the group's place, or, without its last chunk, this CTA's own
+    float *dst = ke == len ? A.colpart + (gc.g * A.NGR + gc.gi) * SB * 3 * TC : A.colsplit + kcta * SB * 3 * TC;
 #pragma unroll
     for (int c0 = 0; c0 < 3; c0 += NT) {
       const int c = c0 + ct / TC;
@@ -1151,68 +1011,61 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
         float tot = 0.0f;
 #pragma unroll
         for (int w = 0; w < S::NCW; ++w) tot += cb[((w * SB + m) * 3 + c) * TC + col];
-        if (whole) A.colpart[(((gc.g * A.NGR + gc.gi) * SB + m) * 3 + c) * TC + col] = tot;
-        else A.colsplit[((slot * SB + m) * 3 + c) * TC + col] = tot;
+        dst[(m * 3 + c) * TC + col] = tot;
       }
     }
-    if (!whole) __threadfence();
-    asm volatile("bar.sync 1, %0;" ::"r"(S::NCW * 32) : "memory");  // CB free; a split part is out
-    if (whole) continue;
-    // a group split between CTAs: the last to arrive adds the parts in CTA order
-    const int64_t kf = mtd::sk_owner(gs, U, G), kl = mtd::sk_owner(gs + len - 1, U, G);
-    int *gcount = &A.gcount[gc.g * A.NGR + gc.gi];
-    if (ct == 0) split_last = (atomicAdd(gcount, 1) == (int)(kl - kf));
-    asm volatile("bar.sync 1, %0;" ::"r"(S::NCW * 32) : "memory");
-    if (!split_last) continue;
-    __threadfence();
-    constexpr int NC = (3 + NT - 1) / NT;  // components per thread
-    float tot[NC][SB];
-#pragma unroll
-    for (int i = 0; i < NC; ++i)
-#pragma unroll
-      for (int m = 0; m < SB; ++m) tot[i][m] = 0.0f;
-    for (int64_t kk = kf; kk <= kl; ++kk) {  // the parts in CTA order, each CTA's loaded together
-      const int64_t sl = (mtd::sk_begin(kk, U, G) >= gs) ? 2 * kk : 2 * kk + 1;
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        const int c = i * NT + ct / TC;
-        if (c >= 3) break;
-#pragma unroll
-        for (int m = 0; m < SB; ++m) tot[i][m] += __ldcg(&A.colsplit[((sl * SB + m) * 3 + c) * TC + col]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < NC; ++i) {
-      const int c = i * NT + ct / TC;
-      if (c >= 3) break;
-#pragma unroll
-      for (int m = 0; m < SB; ++m) A.colpart[(((gc.g * A.NGR + gc.gi) * SB + m) * 3 + c) * TC + col] = tot[i][m];
-    }
-    if (ct == 0) *gcount = 0;  // ready for the next launch
+    asm volatile("bar.sync 1, %0;" ::"r"(S::NCW * 32) : "memory");  // CB free
   }
   if (sr_cur >= 0) flush_rows(sr_cur);
 }
 
-// The transposed part of a half-stored product.  Column j of column chunk q
-// gets the sum over the groups (R, q), R < q, of their column sums.  One CTA
-// per (q, simulation), kHalfColLanes threads per column: thread (r, t) adds
-// column t of the groups R = r, r + kHalfColLanes, ... in increasing R, and
-// the lanes' sums are added in order of r (a fixed order: the result does
-// not depend on timing) before H_j -= total.  Every load of a CTA is issued
-// in one round (the group sums were just written and sit in L2), and no
-// CTA waits on another.
+// The end of a half-stored product, H_j -= what is not in H yet: the column
+// sums of the groups (R, q), R < q, of j's column chunk q, and the parts of
+// split groups and super-rows (see above).  One CTA per (q, simulation),
+// kHalfColLanes threads per tile: thread (r, t) adds for tile t the groups R =
+// r, r + kHalfColLanes, ... in increasing R and every kHalfColLanes-th part in
+// order of the CTAs, and the lanes' sums are added in order of r (a fixed
+// order: the result does not depend on timing).  Every load of a CTA is issued
+// in one or two rounds (the sums were just written and sit in L2), and no CTA
+// waits on another.
 constexpr int kHalfColLanes = 8;
+constexpr int kHalfMaxCtas = 1024;  // CTAs of a product (one per SM)
 template <int TC>
-__global__ void __launch_bounds__(kHalfColLanes *TC) k_half_cols(HalfArgs A, int SB) {
+__global__ void __launch_bounds__(kHalfColLanes *TC) k_half_sum(HalfArgs A, int SB, int G) {
+  constexpr int L = kHalfColLanes, ROWS = TC;  // a super-row holds as many tiles as a column chunk
+  __shared__ float lane_sum[L][3][TC];
+  __shared__ short list[2][kHalfMaxCtas];  // CTAs with a part of this super-row, of this column chunk
+  __shared__ int cnt[2];
   mtd::pdl_enter();
   const int64_t q = blockIdx.x;
   const int b = blockIdx.y;
   const int t = threadIdx.x % TC, r = threadIdx.x / TC;
   const int64_t g = b / SB, m = b - g * SB;
+  const int64_t j = q * TC + t;
+  const bool writer = r == 0 && j < A.n && (!A.active || A.active[b]);
+  float *H = A.H + (size_t)b * 3 * A.n + 3 * j;
+  float h[3] = {0.0f, 0.0f, 0.0f};
+  if (writer) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) h[c] = __ldcg(H + c);
+  }
+  if (r >= L - 2 && t < 32) {  // a warp each: the tags in order of the CTAs
+    const int which = r - (L - 2);
+    const int want = (int)(g * A.Q + q);
+    int c = 0;
+    for (int k0 = 0; k0 < G; k0 += 32) {
+      const int k = k0 + t;
+      const int2 tg = k < G ? __ldcg(A.tag + k) : make_int2(-1, -1);
+      const bool hit = (which ? tg.y : tg.x) == want;
+      const unsigned mask = __ballot_sync(0xffffffffu, hit);
+      if (hit) list[which][c + __popc(mask & ((1u << t) - 1u))] = (short)k;
+      c += __popc(mask);
+    }
+    if (t == 0) cnt[which] = c;
+  }
   // group (R, q) is number half_gbase(R) + q - R
   const float *base = A.colpart + ((g * A.NGR * SB + m) * 3) * TC + t;
   const int64_t gstride = (int64_t)SB * 3 * TC;
-  constexpr int L = kHalfColLanes;
   float tot[3] = {0.0f, 0.0f, 0.0f};
   int64_t R = r;
   for (; R + 3 * L < q; R += 4 * L) {  // four groups' loads in flight
@@ -1238,26 +1091,30 @@ __global__ void __launch_bounds__(kHalfColLanes *TC) k_half_cols(HalfArgs A, int
     tot[1] += __ldcg(cp + TC);
     tot[2] += __ldcg(cp + 2 * TC);
   }
-  __shared__ float lane_sum[L][3][TC];
-  lane_sum[r][0][t] = tot[0];
-  lane_sum[r][1][t] = tot[1];
-  lane_sum[r][2][t] = tot[2];
   __syncthreads();
-  if (r != 0) return;
-  const int64_t j = q * TC + t;
-  if (j >= A.n || (A.active && !A.active[b])) return;
-  float v[3];
+  for (int s = r; s < cnt[1]; s += L) {
+    const float *cp = A.colsplit + ((int64_t)list[1][s] * SB + m) * 3 * TC + t;
+    tot[0] += __ldcg(cp);
+    tot[1] += __ldcg(cp + TC);
+    tot[2] += __ldcg(cp + 2 * TC);
+  }
+  for (int s = L - 1 - r; s < cnt[0]; s += L) {
+    const float *rp = A.rowsplit + (((int64_t)list[0][s] * SB + m) * ROWS + t) * 3;
+    tot[0] += __ldcg(rp);
+    tot[1] += __ldcg(rp + 1);
+    tot[2] += __ldcg(rp + 2);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) lane_sum[r][c][t] = tot[c];
+  __syncthreads();
+  if (!writer) return;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     float s = 0.0f;
 #pragma unroll
     for (int k2 = 0; k2 < L; ++k2) s += lane_sum[k2][c][t];
-    v[c] = s;
+    H[c] = h[c] - s;
   }
-  float *H = A.H + (size_t)b * 3 * A.n + 3 * j;
-  H[0] -= v[0];
-  H[1] -= v[1];
-  H[2] -= v[2];
 }
 
 // xs[b][q][c][t] = Ms_j m_j[c] with j = q*TC + t (0 beyond n)
@@ -1462,13 +1319,22 @@ constexpr bool has_half() {
 }
 
 template <int PREC, int SB>
+cudaError_t prepare_half_one() {
+  return cudaFuncSetAttribute(k_matvec_half<PREC, SB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              HalfShape<PREC, SB>::SMEM_BYTES);
+}
+template <int PREC>
+cudaError_t prepare_half() {
+  cudaError_t e;
+  if ((e = prepare_half_one<PREC, 1>()) != cudaSuccess || (e = prepare_half_one<PREC, 2>()) != cudaSuccess) return e;
+  return prepare_half_one<PREC, 4>();
+}
+template <int PREC, int SB>
 cudaError_t prepare_mv_one() {
   cudaError_t e = cudaFuncSetAttribute(k_matvec<PREC, SB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        MvShape<PREC, SB>::SMEM_BYTES);
-  if constexpr (has_half<PREC>() && SB <= 2) {
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_matvec_half<PREC, SB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               HalfShape<PREC, SB>::SMEM_BYTES);
+  if constexpr (has_half<PREC>()) {
+    if (e == cudaSuccess) e = prepare_half_one<PREC, SB>();
   }
   return e;
 }
@@ -1483,10 +1349,10 @@ cudaError_t prepare_mv() {
 
 // simulations per chunk read: 1, 2 or 4 (2 at most for the scaled BF16
 // tensor, whose 8-wide rows with 4 operands spill registers: measured 0.56 ms
-// for 4 simulations at n = 10,000 against 0.21 ms for one; 2 at most for a
-// half-stored tensor, whose threads hold the sums of 16 rows per simulation)
-inline int mv_group(int B, int prec, bool half) {
-  const int cap = (half || prec == MT_BF16_SCALED || prec == kBF16Planar) ? 2 : 4;
+// for 4 simulations at n = 10,000 against 0.21 ms for one; a half-stored
+// tensor's 4 at a time take 86 us on the 5,120-tile prism, 2 at a time twice 60)
+inline int mv_group(int B, int prec) {
+  const int cap = (prec == MT_BF16_SCALED || prec == kBF16Planar) ? 2 : 4;
   return B <= 1 ? 1 : (B == 2 || cap == 2) ? 2 : 4;
 }
 
@@ -1503,7 +1369,7 @@ void launch_mv_sb(const MvArgs &A, int grid_cap, cudaStream_t s) {
 
 // work area of a half-stored product over B simulations, SB per chunk read
 // (floats): the column sums of every group [NG][NGR][SB][3][TC]; the parts of
-// groups split between CTAs [2 grid_cap][SB][3][TC]
+// groups split between CTAs [grid_cap][SB][3][TC]
 struct HalfArea {
   size_t colpart, colsplit, bytes;
 };
@@ -1512,7 +1378,7 @@ inline HalfArea half_area(int64_t Q, int64_t B, int SB, int grid_cap, int TC) {
   HalfArea h;
   h.colpart = 0;
   h.colsplit = h.colpart + (size_t)NG * NGR * SB * 3 * TC;
-  h.bytes = (h.colsplit + (size_t)2 * grid_cap * SB * 3 * TC) * sizeof(float);
+  h.bytes = (h.colsplit + (size_t)grid_cap * SB * 3 * TC) * sizeof(float);
   return h;
 }
 
@@ -1527,9 +1393,8 @@ void launch_half(const mt_tensor *T, const float *xs, int B, float *H, float *pa
   A.tensor = reinterpret_cast<const float *>(T->d_data);
   A.xs = xs;
   A.H = H;
-  A.part = part;
-  A.count = count;
-  A.gcount = count + (size_t)B * T->L.P * 8;  // after the row counters (all counters rest at zero)
+  A.rowsplit = part;
+  A.tag = reinterpret_cast<int2 *>(count);
   A.colpart = work + h.colpart;
   A.colsplit = work + h.colsplit;
   A.active = active;
@@ -1541,19 +1406,17 @@ void launch_half(const mt_tensor *T, const float *xs, int B, float *H, float *pa
   A.NGR = half_groups(T->L.Q);
   A.B = B;
   const int64_t U = (int64_t)((B + SB - 1) / SB) * A.CH;
-  const int grid = (int)std::min<int64_t>(cap, U);
+  const int grid = (int)std::min<int64_t>(std::min(cap, kHalfMaxCtas), U);
   mt::launch_pdl(k_matvec_half<PREC, SB>, dim3(grid), dim3(S::THREADS), S::SMEM_BYTES, s, A);
-  mt::launch_pdl(k_half_cols<TC>, dim3((unsigned)A.Q, (unsigned)B), dim3(kHalfColLanes * TC), 0, s, A, SB);
+  mt::launch_pdl(k_half_sum<TC>, dim3((unsigned)A.Q, (unsigned)B), dim3(kHalfColLanes * TC), 0, s, A, SB, grid);
 }
 
-// a layout that exists only stored half (3 planes)
 template <int PREC>
-void launch_half_only(const mt_tensor *T, const void *xs, int B, void *H, void *part, int *count,
-                      const int *active, int *status, float *colpart, cudaStream_t s) {
-  if (mv_group(B, PREC, true) == 1)
-    launch_half<PREC, 1>(T, (const float *)xs, B, (float *)H, (float *)part, count, active, status, colpart, s);
-  else
-    launch_half<PREC, 2>(T, (const float *)xs, B, (float *)H, (float *)part, count, active, status, colpart, s);
+void launch_half_any(const mt_tensor *T, const void *xs, int B, void *H, void *part, int *count, const int *active,
+                     int *status, float *colpart, cudaStream_t s) {
+  const int sb = mv_group(B, PREC);
+  const auto launch = sb == 1 ? launch_half<PREC, 1> : sb == 2 ? launch_half<PREC, 2> : launch_half<PREC, 4>;
+  launch(T, (const float *)xs, B, (float *)H, (float *)part, count, active, status, colpart, s);
 }
 
 template <int PREC>
@@ -1561,10 +1424,7 @@ void launch_mv(const mt_tensor *T, const void *xs, int B, void *H, void *part, i
                int *status, float *colpart, cudaStream_t s) {
   if constexpr (has_half<PREC>()) {
     if (T->L.half) {
-      if (mv_group(B, PREC, true) == 1)
-        launch_half<PREC, 1>(T, (const float *)xs, B, (float *)H, (float *)part, count, active, status, colpart, s);
-      else
-        launch_half<PREC, 2>(T, (const float *)xs, B, (float *)H, (float *)part, count, active, status, colpart, s);
+      launch_half_any<PREC>(T, xs, B, H, part, count, active, status, colpart, s);
       return;
     }
   }
@@ -1583,7 +1443,7 @@ void launch_mv(const mt_tensor *T, const void *xs, int B, void *H, void *part, i
   A.CH = T->L.CH;
   A.B = B;
   const int cap = mt::matvec_grid(T);
-  switch (mv_group(B, PREC, false)) {
+  switch (mv_group(B, PREC)) {
     case 1: launch_mv_sb<PREC, 1>(A, cap, s); break;
     case 2: launch_mv_sb<PREC, 2>(A, cap, s); break;
     default:
@@ -1602,19 +1462,9 @@ cudaError_t matvec_prepare() {
   cudaError_t e;
   if ((e = prepare_mv<MT_F32>()) != cudaSuccess) return e;
   if ((e = prepare_mv<kF32Planar>()) != cudaSuccess) return e;
-  // the traceless layout is always stored half: its half kernels only
-  if ((e = cudaFuncSetAttribute(k_matvec_half<kF32Traceless, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                HalfShape<kF32Traceless, 1>::SMEM_BYTES)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(k_matvec_half<kF32Traceless, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                HalfShape<kF32Traceless, 2>::SMEM_BYTES)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(k_matvec_half<kF32Traceless5, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                HalfShape<kF32Traceless5, 1>::SMEM_BYTES)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(k_matvec_half<kF32Traceless5, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                HalfShape<kF32Traceless5, 2>::SMEM_BYTES)) != cudaSuccess)
-    return e;
+  // the traceless layouts are always stored half: their half kernels only
+  if ((e = prepare_half<kF32Traceless>()) != cudaSuccess) return e;
+  if ((e = prepare_half<kF32Traceless5>()) != cudaSuccess) return e;
   if ((e = prepare_mv<kBF16Planar>()) != cudaSuccess) return e;
   if ((e = prepare_mv<kSplitPlanar>()) != cudaSuccess) return e;
   if ((e = prepare_mv<MT_F64>()) != cudaSuccess) return e;
@@ -1672,23 +1522,23 @@ int64_t xs_floats(const mt_tensor *T) {
 
 size_t matvec_part_bytes(const mt_tensor *T) {
   const size_t el = T->prec == MT_F64 ? 8 : 4;
-  if (T->L.half)  // super-rows of K panels, up to 2 simulations per chunk read
-    return (size_t)2 * matvec_grid(T) * 2 * (T->L.TC / T->L.TR) * T->L.TR * 3 * el;
+  if (T->L.half)  // one super-row of K panels per CTA, up to 4 simulations per chunk read
+    return (size_t)matvec_grid(T) * 4 * T->L.TC * 3 * el;
   return (size_t)2 * matvec_grid(T) * 4 /*simulations per chunk read, at most*/ * T->L.TR * 3 * el;
 }
 
-// per (simulation, panel) up to 8 warp counters; a half-stored tensor adds
-// one counter per (simulation, group)
+// per (simulation, panel) up to 8 warp counters; a half-stored tensor: a tag
+// per CTA
 size_t matvec_count_bytes(const mt_tensor *T, int B) {
-  const size_t rows = (size_t)B * T->L.P * 8;
-  return (rows + (T->L.half ? (size_t)B * half_groups(T->L.Q) : 0)) * sizeof(int);
+  if (T->L.half) return matvec_grid(T) * sizeof(int2);
+  return (size_t)B * T->L.P * 8 * sizeof(int);
 }
 
 // half storage: the work area of the product over B simulations (a call
 // with fewer simulations uses less of each part)
 size_t matvec_colpart_bytes(const mt_tensor *T, int B) {
   if (!T->L.half) return 0;
-  const int sb = mv_group(B, MT_F32, true);
+  const int sb = mv_group(B, MT_F32);
   return half_area(T->L.Q, B, sb, matvec_grid(T), T->L.TC).bytes;
 }
 
@@ -1716,9 +1566,9 @@ void launch_matvec(const mt_tensor *T, const float *xs, int B, float *H, float *
                    const int *active, int *status, cudaStream_t s, float *colpart) {
   switch (T->prec) {
     case MT_F32:
-      if (T->L.nplane == 3) launch_half_only<kF32Traceless>(T, xs, B, H, part, count, active, status, colpart, s);
+      if (T->L.nplane == 3) launch_half_any<kF32Traceless>(T, xs, B, H, part, count, active, status, colpart, s);
       else if (T->L.nplane == 5)
-        launch_half_only<kF32Traceless5>(T, xs, B, H, part, count, active, status, colpart, s);
+        launch_half_any<kF32Traceless5>(T, xs, B, H, part, count, active, status, colpart, s);
       else if (T->L.nplane == 4) launch_mv<kF32Planar>(T, xs, B, H, part, count, active, status, colpart, s);
       else launch_mv<MT_F32>(T, xs, B, H, part, count, active, status, colpart, s);
       break;

@@ -230,7 +230,7 @@ __host__ __device__ __forceinline__ int stream_plane(int e, int nplane) {
   return e;
 }
 // zz is given by the trace (not stored) in a 3- or 5-plane layout
-__host__ __device__ __forceinline__ bool traceless(int nplane) { return nplane == 3 || nplane == 5; }
+__host__ __device__ __forceinline__ constexpr bool traceless(int nplane) { return nplane == 3 || nplane == 5; }
 // bound on |N_xz|, |N_yz| of a single-layer tile set (FP64 round-off of
 // entries that vanish by mirror symmetry)
 constexpr double kPlanarTol = 1e-12;
