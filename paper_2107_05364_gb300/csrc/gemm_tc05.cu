@@ -609,27 +609,31 @@ __global__ void __launch_bounds__(GemmShape<SPLIT, BP>::THREADS, 1)
           last = __shfl_sync(0xffffffffu, last, 0);
           if (last) {
             __threadfence();
-            // 8 simulations at a time: all their parts loaded (in CTA order per
-            // value) before their stores to H, which the compiler cannot move
-            // loads across
-            for (int j0 = 0; j0 < nb; j0 += 8) {
-              float tot[3][8];
+            // up to 16 simulations at a time, two parts' loads in flight (a
+            // small tensor's row tile has a dozen parts, and the sums in CTA
+            // order are a chain: 1,476-tile film, BF16, 29 simulations, four
+            // attempts, 1,233 us with 8 simulations and one part at a time,
+            // 833 with this).  Of the CTAs that share the tile only the first
+            // may have begun before it.
+            const int64_t slot_f = mtd::sk_begin(kf, U, G) / KBU == mt ? 2 * kf : 2 * kf + 1;
+            constexpr int JW = HB < 16 ? HB : 16;
+            for (int j0 = 0; j0 < nb; j0 += JW) {
+              float tot[3][JW];
 #pragma unroll
               for (int q = 0; q < 3; ++q)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) tot[q][j] = 0.0f;
+                for (int j = 0; j < JW; ++j) tot[q][j] = 0.0f;
+#pragma unroll 2
               for (int64_t kk = kf; kk <= kl; ++kk) {
-                const int64_t fm = mtd::sk_begin(kk, U, G) / KBU;
-                const int64_t sl = (mt == fm) ? 2 * kk : 2 * kk + 1;
+                const float *src = P.part + ((size_t)(kk == kf ? slot_f : 2 * kk) * 3 * BP + b0 + j0) * GM + row;
 #pragma unroll
                 for (int q = 0; q < 3; ++q)
 #pragma unroll
-                  for (int j = 0; j < 8; ++j)
-                    if (j0 + j < nb) tot[q][j] += __ldcg(&P.part[(((size_t)sl * 3 + q) * BP + b0 + j0 + j) * GM + row]);
+                  for (int j = 0; j < JW; ++j) tot[q][j] += __ldcg(src + (size_t)(q * BP + j) * GM);
               }
               if (r < P.n)
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
+                for (int j = 0; j < JW; ++j)
                   if (j0 + j < nb)
 #pragma unroll
                     for (int q = 0; q < 3; ++q) P.H[((size_t)(b0 + j0 + j) * P.n + r) * 3 + q] = -tot[q][j];
@@ -656,23 +660,28 @@ __global__ void __launch_bounds__(GemmShape<SPLIT, BP>::THREADS, 1)
 // Operand of the batch: X_c[b][j] = BF16(Ms_j m_j,c), for the split product
 // with the two further terms x1, x2 of x = x0 + x1 + x2 (zero for padding), and
 // the simulation-fastest copy of m for the near blocks, mT[(3 j + c) Bp + b].
-// A CTA takes the 64 tiles of one K block and up to 32 simulations through
+// A CTA takes the 64 tiles of one K block and up to SIMS simulations through
 // shared memory, so that both sides of the transposition are whole rows: a warp
-// reads a simulation's 192 floats, writes rows of 64 BF16, and rows of 32
+// reads a simulation's 192 floats, writes rows of 64 BF16, and rows of SIMS
 // simulations of mT.  n = 20,000, B = 64, split: 28.5 us with one thread per
-// value (mT stored with a stride), 12.1 with this.
-constexpr int kPrepSims = 32, kPrepWarps = 8;
+// value (mT stored with a stride), 12.1 with this.  SIMS = 32 fills a row of
+// mT's 128 bytes; where that gives fewer CTAs than SMs the chain of a warp's
+// simulations is the time, and SIMS = 8 gives each warp one
+// (n = 729, B = 64: 6.9 us alone with 32).
+constexpr int kPrepWarps = 8;
+template <int SIMS>
 __global__ void __launch_bounds__(32 * kPrepWarps) k_prep_dense_x(const float *m, const float *Ms, int64_t n,
                                                                   int64_t KB, int B, int Bp, int terms,
                                                                   __nv_bfloat16 *X, float *mT) {
-  __shared__ float sm[kPrepSims][3 * GK + 1];
+  __shared__ float sm[SIMS][3 * GK + 1];
   const int64_t kb = blockIdx.x, j0 = kb * GK;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int b0 = blockIdx.y * kPrepSims, nb = B - b0 < kPrepSims ? B - b0 : kPrepSims;
+  const int b0 = blockIdx.y * SIMS, nb = B - b0 < SIMS ? B - b0 : SIMS;
   const int cols = (int)(n - j0 < GK ? n - j0 : GK);  // tiles of this block (may be <= 0: padding)
   const float ms[2] = {2 * lane < cols ? Ms[j0 + 2 * lane] : 0.0f, 2 * lane + 1 < cols ? Ms[j0 + 2 * lane + 1] : 0.0f};
+  mtd::pdl_enter();
 #pragma unroll
-  for (int q = 0; q < kPrepSims / kPrepWarps; ++q) {
+  for (int q = 0; q < SIMS / kPrepWarps; ++q) {
     const int b = w + kPrepWarps * q;
     if (b >= nb) break;
     const float *src = m + (size_t)(b0 + b) * 3 * n + 3 * j0;
@@ -682,7 +691,7 @@ __global__ void __launch_bounds__(32 * kPrepWarps) k_prep_dense_x(const float *m
   __syncthreads();
   const size_t term = (size_t)3 * KB * Bp * GK;
 #pragma unroll
-  for (int q = 0; q < kPrepSims / kPrepWarps; ++q) {
+  for (int q = 0; q < SIMS / kPrepWarps; ++q) {
     const int b = w + kPrepWarps * q;
     if (b >= nb) break;
 #pragma unroll
@@ -699,9 +708,11 @@ __global__ void __launch_bounds__(32 * kPrepWarps) k_prep_dense_x(const float *m
       }
     }
   }
-  if (lane < nb)
+  const int b = lane % SIMS;
+  if (b < nb)
 #pragma unroll 4
-    for (int t = w; t < 3 * cols; t += kPrepWarps) mT[(size_t)(3 * j0 + t) * Bp + b0 + lane] = sm[lane][t];
+    for (int t = threadIdx.x / SIMS; t < 3 * cols; t += 32 * kPrepWarps / SIMS)
+      mT[(size_t)(3 * j0 + t) * Bp + b0 + b] = sm[b][t];
 }
 
 using EncodeFn = PFN_cuTensorMapEncodeTiled_v12000;
@@ -813,10 +824,12 @@ cudaError_t gemm_prepare() {
 
 void launch_prep_dense_x(const mt_tensor *T, const float *m, int B, void *X, cudaStream_t s) {
   const int64_t KB = T->Kp / GK;
-  const dim3 grid((unsigned)KB, (unsigned)((B + kPrepSims - 1) / kPrepSims));
-  k_prep_dense_x<<<grid, 32 * kPrepWarps, 0, s>>>(m, T->tiles->d_Ms, T->n, KB, B, dense_pad_batch(B),
-                                      T->prec == MT_BF16_SPLIT ? 3 : 1, reinterpret_cast<__nv_bfloat16 *>(X),
-                                      dense_mT(T, B, X));
+  const bool wide = KB * ((B + 31) / 32) >= T->tiles->ctx->num_sms;
+  const int sims = wide ? 32 : 8;
+  const dim3 grid((unsigned)KB, (unsigned)((B + sims - 1) / sims));
+  launch_pdl(wide ? k_prep_dense_x<32> : k_prep_dense_x<8>, grid, dim3(32 * kPrepWarps), 0, s, m,
+             (const float *)T->tiles->d_Ms, T->n, KB, B, dense_pad_batch(B), T->prec == MT_BF16_SPLIT ? 3 : 1,
+             reinterpret_cast<__nv_bfloat16 *>(X), dense_mT(T, B, X));
 }
 
 mt_status gemm_plan(const mt_tensor *T, int B, const void *X, GemmPlan *plan) {

@@ -1200,10 +1200,9 @@ __global__ void k_near(int64_t n, int B, const int32_t *ptr, const int32_t *col,
 
 // The same for the simulation-fastest copy of a batch (element (b, j, c) at
 // mT[(3 j + c) Bp + b]).  LS lanes take one tile, V adjacent simulations each
-// (one vector load per component, the tile's blocks shared); three blocks'
-// loads are in flight at a time (one where the double-FP32 arithmetic, not the
-// latency, bounds it), their sums in column order.  The sums of a
-// CTA's tiles (16 or more) pass through shared memory, so that H, one row of
+// (one vector load per component, the tile's blocks shared), UN blocks' loads in
+// flight at a time, their sums in column order.  The sums of a
+// CTA's tiles (8 to 32) pass through shared memory, so that H, one row of
 // three floats per tile in every simulation's own vector, is read and written
 // in runs of whole tiles; a thread that wrote its own tile and
 // simulation touched a 32-byte sector for each value.  n = 10,000, B = 64, BF16:
@@ -1224,47 +1223,48 @@ struct VecF<2> {
   }
 };
 
+// SP groups of LS lanes share a tile's blocks, every SP-th each, and their sums
+// are added in group order: SP = 4 where few CTAs make the chain of one list the
+// time (n = 729, split, B = 5, four attempts: 963 -> 662 us), 1 otherwise.  The lists are read before the
+// wait on the product.
 constexpr int kNearThreads = 256;
-// tiles of a CTA: a pass of its threads, at least 16
-template <int LS>
-constexpr int kNearTilesOf = kNearThreads / LS > 16 ? kNearThreads / LS : 16;
-template <bool FF, int LS, int V>
+template <int LS, int SP>
+constexpr int kNearTilesOf = kNearThreads / (LS * SP);  // tiles of a CTA
+template <bool FF, int LS, int V, int UN, int SP>
 __global__ void __launch_bounds__(kNearThreads) k_near_v(int64_t n, int B, int Bp, const int32_t *ptr,
                                                          const int32_t *col, const float2 *val, const float *mT,
                                                          float *H, const int *active) {
-  mtd::pdl_enter();
   using VT = typename VecF<V>::T;
-  constexpr int SIMS = LS * V;             // simulations of a CTA
-  constexpr int PASS = kNearThreads / LS;  // tiles in one pass of the CTA
-  constexpr int TILES = kNearTilesOf<LS>;
-  constexpr int UN = FF ? 1 : 3;  // blocks in flight
+  constexpr int SIMS = LS * V;  // simulations of a CTA
+  constexpr int TILES = kNearTilesOf<LS, SP>;
   constexpr int ROW = 3 * TILES + 1;
-  __shared__ float s_hi[SIMS][ROW], s_lo[FF ? SIMS : 1][FF ? ROW : 1];
+  __shared__ float s_hi[SP][SIMS][ROW], s_lo[FF ? SP : 1][FF ? SIMS : 1][FF ? ROW : 1];
   const int64_t i0 = blockIdx.x * (int64_t)TILES;
   const int bs = blockIdx.y * SIMS;  // first simulation
   const int l = threadIdx.x % LS, b0 = bs + l * V;
-#pragma unroll 1
-  for (int ti = threadIdx.x / LS; ti < TILES; ti += PASS) {
-    const int64_t i = i0 + ti;
-    if (i >= n || b0 >= Bp) break;
+  const int g = threadIdx.x / LS % SP, ti = threadIdx.x / (LS * SP);
+  const int64_t i = i0 + ti;
+  const bool live = i < n && b0 < Bp;
+  int32_t a = live ? ptr[i] + g : 0, jn[UN];  // the next columns, fetched a round ahead
+  const int32_t a1 = live ? ptr[i + 1] : 0;
+#pragma unroll
+  for (int q = 0; q < UN; ++q) jn[q] = a + SP * q < a1 ? col[a + SP * q] : 0;
+  mtd::pdl_enter();
+  if (live) {
     ff h[3][V];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
       for (int v = 0; v < V; ++v) h[c][v] = ff{0.0f, 0.0f};
-    const int32_t a1 = ptr[i + 1];
-    int32_t a = ptr[i], jn[UN];  // the next columns, fetched a round ahead
-#pragma unroll
-    for (int q = 0; q < UN; ++q) jn[q] = a + q < a1 ? col[a + q] : 0;
-    for (; a < a1; a += UN) {
+    for (; a < a1; a += SP * UN) {
       float4 w[UN][3];
       float x[UN][3][V];
 #pragma unroll
       for (int q = 0; q < UN; ++q) {
         const int64_t j = jn[q];
-        jn[q] = a + UN + q < a1 ? col[a + UN + q] : 0;
-        if (a + q >= a1) continue;
-        const float4 *vp = reinterpret_cast<const float4 *>(val + 6 * (size_t)(a + q));
+        jn[q] = a + SP * (UN + q) < a1 ? col[a + SP * (UN + q)] : 0;
+        if (a + SP * q >= a1) continue;
+        const float4 *vp = reinterpret_cast<const float4 *>(val + 6 * (size_t)(a + SP * q));
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           w[q][c] = vp[c];
@@ -1273,7 +1273,7 @@ __global__ void __launch_bounds__(kNearThreads) k_near_v(int64_t n, int B, int B
       }
 #pragma unroll
       for (int q = 0; q < UN; ++q) {
-        if (a + q >= a1) continue;
+        if (a + SP * q >= a1) continue;
         const float4 w0 = w[q][0], w1 = w[q][1], w2 = w[q][2];
         const float2 e[6] = {{w0.x, w0.y}, {w0.z, w0.w}, {w1.x, w1.y}, {w1.z, w1.w}, {w2.x, w2.y}, {w2.z, w2.w}};
         constexpr int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
@@ -1296,8 +1296,8 @@ __global__ void __launch_bounds__(kNearThreads) k_near_v(int64_t n, int B, int B
     for (int v = 0; v < V; ++v)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        s_hi[l * V + v][3 * ti + c] = h[c][v].hi;
-        if (FF) s_lo[l * V + v][3 * ti + c] = h[c][v].lo;
+        s_hi[g][l * V + v][3 * ti + c] = h[c][v].hi;
+        if (FF) s_lo[g][l * V + v][3 * ti + c] = h[c][v].lo;
       }
   }
   __syncthreads();
@@ -1306,8 +1306,11 @@ __global__ void __launch_bounds__(kNearThreads) k_near_v(int64_t n, int B, int B
     const int s = q / (3 * TILES), t = q - s * 3 * TILES, b = bs + s;
     if (t >= cnt || b >= B || (active && !active[b])) continue;
     float *Hb = H + (size_t)b * 3 * n + 3 * i0 + t;
+    ff near = {s_hi[0][s][t], FF ? s_lo[0][s][t] : 0.0f};
+#pragma unroll
+    for (int p = 1; p < SP; ++p) near = ff_add(near, s_hi[p][s][t], FF ? s_lo[p][s][t] : 0.0f);
     // H = far - near, rounded once
-    const ff r = ff_add({*Hb, 0.0f}, -s_hi[s][t], FF ? -s_lo[s][t] : 0.0f);
+    const ff r = ff_add({*Hb, 0.0f}, -near.hi, -near.lo);
     *Hb = r.hi + r.lo;
   }
 }
@@ -1596,17 +1599,33 @@ void launch_near(const mt_tensor *T, const float *m, int64_t sb, int64_t se, int
     const int Bp = (int)se;
     const bool split = T->prec == MT_BF16_SPLIT;
     // lanes per tile: as many as there are simulations, at least 8, at most
-    // 32, two simulations each from 64 on
-#define MT_NEAR_V(LS, VV)                                                                                   \
-  mt::launch_pdl(split ? k_near_v<true, LS, VV> : k_near_v<false, LS, VV>,                                 \
-                 dim3((unsigned)((n + kNearTilesOf<LS> - 1) / kNearTilesOf<LS>),                           \
-                      (unsigned)((B + LS * VV - 1) / (LS * VV))),                                          \
+    // 32, two simulations each from 33 on.  Three blocks in flight; one where
+    // the double-FP32 sums of many CTAs, not the latency, bound it (split: a
+    // field of 10,000 tiles, B = 128, 480 us with one, 486 with three; 2,520
+    // tiles, B = 128, 140 with one, 122 with three).  Four groups share a list
+    // while the CTAs of one group to a list do not fill the device twice; with
+    // long lists (17 to 27 blocks: more than one layer) and double-FP32 sums up to eight
+    // times (2,520 tiles in three layers, B = 64: 88 -> 76 us; lists of 9
+    // blocks, 4,800 tiles, B = 128: 147 -> 162, so not there).
+    const bool many = split && n * B > 600 * 1024;
+    const int sims = B <= 8 ? 8 : B <= 16 ? 16 : B <= 32 ? 32 : 64, lanes = sims < 32 ? sims : 32;
+    const int waves = split && T->near_count >= 16 * n ? 8 : 2;
+    const bool few = n * lanes / kNearThreads * ((B + sims - 1) / sims) < waves * T->tiles->ctx->num_sms;
+#define MT_NEAR_SP(LS, VV, UN, SP)                                                                        \
+  mt::launch_pdl(split ? k_near_v<true, LS, VV, UN, SP> : k_near_v<false, LS, VV, 3, SP>,                 \
+                 dim3((unsigned)((n + kNearTilesOf<LS, SP> - 1) / kNearTilesOf<LS, SP>),                  \
+                      (unsigned)((B + LS * VV - 1) / (LS * VV))),                                         \
                  dim3(kNearThreads), 0, s, n, B, Bp, ptr, col, hl, m, H, active)
-    if (B <= 8) MT_NEAR_V(8, 1);
-    else if (B <= 16) MT_NEAR_V(16, 1);
-    else if (B <= 32) MT_NEAR_V(32, 1);
-    else MT_NEAR_V(32, 2);
+#define MT_NEAR_V(LS, VV)                   \
+  if (few) MT_NEAR_SP(LS, VV, 3, 4);        \
+  else if (many) MT_NEAR_SP(LS, VV, 1, 1);  \
+  else MT_NEAR_SP(LS, VV, 3, 1)
+    if (sims == 8) { MT_NEAR_V(8, 1); }
+    else if (sims == 16) { MT_NEAR_V(16, 1); }
+    else if (sims == 32) { MT_NEAR_V(32, 1); }
+    else { MT_NEAR_V(32, 2); }
 #undef MT_NEAR_V
+#undef MT_NEAR_SP
     return;
   }
   if (T->prec == MT_BF16_SPLIT)
