@@ -1120,6 +1120,7 @@ __global__ void __launch_bounds__(kHalfColLanes *TC) k_half_sum(HalfArgs A, int 
 // xs[b][q][c][t] = Ms_j m_j[c] with j = q*TC + t (0 beyond n)
 template <typename In, typename Out>
 __global__ void k_prep_xs(const In *m, const float *Ms, int64_t n, int64_t Q, int TC, int B, Out *xs) {
+  mtd::pdl_enter();
   const int64_t tot = (int64_t)B * Q * TC;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = t / (Q * TC), rem = t - b * Q * TC;
@@ -1142,29 +1143,37 @@ __global__ void k_prep_xs(const In *m, const float *Ms, int64_t n, int64_t Q, in
 
 // Near-field blocks (BF16 precisions of the streaming layout): double-FP32
 // sums (mtd::ff) of N_ij Ms_j m_j over the touching tiles, added to the far
-// field and rounded once.  Threads enumerate (tile, simulation) pairs with
-// the simulation fastest, so a warp of a wide batch shares its tile's blocks
-// (broadcast loads); m element (b, j, c) sits at m[b * sb + (3 j + c) * se]:
-// se = 1 for the tile-major state, sb = 1 for a simulation-fastest copy.
+// field and rounded once.  LN lanes take one (tile, simulation) pair, every
+// LN-th block of the tile's list each; pairs are enumerated with the simulation
+// fastest, so neighbouring groups read the same blocks.  LN = 8 makes a list
+// three or four rounds of dependent loads instead of 27 (field of 10,800 graded
+// tiles, BF16, B = 1: 281 -> 242 us).  The lists are read before the wait on
+// the product.  m element (b, j, c) sits at m[b * sb + (3 j + c) * se]: se = 1
+// for the tile-major state, sb = 1 for a simulation-fastest copy.
 using mtd::ff;
 using mtd::ff_add;
 using mtd::ff_fma_lazy;
 
 // FF = false (the BF16 precision, whose far part carries ~1e-4 errors):
 // plain FP32 sums of the high words, H = far - near in FP32
-template <bool FF>
+template <bool FF, int LN>
 __global__ void k_near(int64_t n, int B, const int32_t *ptr, const int32_t *col, const float2 *val,
                        const float *m, int64_t sb, int64_t se, float *H, const int *active) {
-  mtd::pdl_enter();
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= n * B) return;
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LN;
+  const int l = threadIdx.x % LN;
   const int64_t i = t / B;
   const int b = (int)(t - i * B);
-  if (active && !active[b]) return;
+  const bool inside = t < n * B;
+  int32_t a = inside ? ptr[i] + l : 0;
+  const int32_t a1 = inside ? ptr[i + 1] : 0;
+  int32_t jn = a < a1 ? col[a] : 0;  // the next column, fetched a round ahead
+  mtd::pdl_enter();
+  if (!inside || (active && !active[b])) return;  // the same for the lanes of a group
   const float *mb = m + (size_t)b * sb;
   ff hx = {0, 0}, hy = {0, 0}, hz = {0, 0};
-  for (int32_t a = ptr[i]; a < ptr[i + 1]; ++a) {
-    const int64_t j = col[a];
+  for (; a < a1; a += LN) {
+    const int64_t j = jn;
+    jn = a + LN < a1 ? col[a + LN] : 0;
     // val holds N_ij Ms_j: the operand is m itself, exact in FP32
     const float x0 = mb[(3 * j) * se], x1 = mb[(3 * j + 1) * se], x2 = mb[(3 * j + 2) * se];
     // 48 bytes per block, 16-byte aligned: three float4 requests
@@ -1187,6 +1196,19 @@ __global__ void k_near(int64_t n, int B, const int32_t *ptr, const int32_t *col,
     ff_fma_lazy(hz, v2, x0);
     ff_fma_lazy(hz, v4, x1);
     ff_fma_lazy(hz, v5, x2);
+  }
+  if (LN > 1) {
+    const unsigned group = (LN < 32 ? (1u << (LN & 31)) - 1u : ~0u) << ((threadIdx.x & 31) - l);
+    ff *const h[3] = {&hx, &hy, &hz};
+#pragma unroll
+    for (int d = LN / 2; d >= 1; d >>= 1)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float hi = __shfl_xor_sync(group, h[c]->hi, d), lo = FF ? __shfl_xor_sync(group, h[c]->lo, d) : 0.0f;
+        if (FF) *h[c] = ff_add(*h[c], hi, lo);
+        else h[c]->hi += hi;
+      }
+    if (l != 0) return;
   }
   float *Hb = H + (size_t)b * 3 * n + 3 * i;
   // H = far - near, rounded once
@@ -1553,16 +1575,18 @@ void launch_prep_xs(const mt_tensor *T, const float *m, int B, float *xs, cudaSt
   const int64_t tot = (int64_t)B * T->L.Q * T->L.TC;
   const int blocks = (int)std::min<int64_t>((tot + 255) / 256, 4096);
   if (T->prec == MT_F64)
-    k_prep_xs<float, double><<<blocks, 256, 0, s>>>(m, T->tiles->d_Ms, T->n, T->L.Q, T->L.TC, B,
-                                                     reinterpret_cast<double *>(xs));
+    mt::launch_pdl(k_prep_xs<float, double>, dim3(blocks), dim3(256), 0, s, m, (const float *)T->tiles->d_Ms, T->n,
+                   T->L.Q, T->L.TC, B, reinterpret_cast<double *>(xs));
   else
-    k_prep_xs<float, float><<<blocks, 256, 0, s>>>(m, T->tiles->d_Ms, T->n, T->L.Q, T->L.TC, B, xs);
+    mt::launch_pdl(k_prep_xs<float, float>, dim3(blocks), dim3(256), 0, s, m, (const float *)T->tiles->d_Ms, T->n,
+                   T->L.Q, T->L.TC, B, xs);
 }
 
 void launch_prep_xs_f64(const mt_tensor *T, const double *m, int B, double *xs, cudaStream_t s) {
   const int64_t tot = (int64_t)B * T->L.Q * T->L.TC;
   const int blocks = (int)std::min<int64_t>((tot + 255) / 256, 4096);
-  k_prep_xs<double, double><<<blocks, 256, 0, s>>>(m, T->tiles->d_Ms, T->n, T->L.Q, T->L.TC, B, xs);
+  mt::launch_pdl(k_prep_xs<double, double>, dim3(blocks), dim3(256), 0, s, m, (const float *)T->tiles->d_Ms, T->n,
+                 T->L.Q, T->L.TC, B, xs);
 }
 
 void launch_matvec(const mt_tensor *T, const float *xs, int B, float *H, float *part, int *count,
@@ -1591,7 +1615,6 @@ void launch_near(const mt_tensor *T, const float *m, int64_t sb, int64_t se, int
                  cudaStream_t s) {
   if (T->near_count == 0) return;
   const int64_t tot = T->n * (int64_t)B;
-  const unsigned grid = (unsigned)((tot + 255) / 256);
   const int32_t *ptr = T->d_near_ptr, *col = T->d_near_col;
   const float2 *hl = T->d_near_hl;
   const int64_t n = T->n;
@@ -1628,10 +1651,15 @@ void launch_near(const mt_tensor *T, const float *m, int64_t sb, int64_t se, int
 #undef MT_NEAR_SP
     return;
   }
-  if (T->prec == MT_BF16_SPLIT)
-    mt::launch_pdl(k_near<true>, dim3(grid), dim3(256), 0, s, n, B, ptr, col, hl, m, sb, se, H, active);
-  else
-    mt::launch_pdl(k_near<false>, dim3(grid), dim3(256), 0, s, n, B, ptr, col, hl, m, sb, se, H, active);
+  // Eight lanes to a list while the pairs do not fill the device by themselves
+  // (4,096 tiles in a cube, split, B = 1: field 83 -> 66 us; B = 4: 111 -> 90).
+  // Short lists of four simulations and more stay with a thread each: eight
+  // lanes idle over 9 blocks (film of 10,000 tiles, BF16, B = 4: 305 -> 310).
+  const bool split = T->prec == MT_BF16_SPLIT;
+  const bool few = tot <= 128 * 1024 && (B < 4 || T->near_count >= 16 * n);
+  const unsigned grid = (unsigned)((tot * (few ? 8 : 1) + 255) / 256);
+  mt::launch_pdl(few ? (split ? k_near<true, 8> : k_near<false, 8>) : (split ? k_near<true, 1> : k_near<false, 1>),
+                 dim3(grid), dim3(256), 0, s, n, B, ptr, col, hl, m, sb, se, H, active);
 }
 
 }  // namespace mt

@@ -533,6 +533,7 @@ __global__ void __launch_bounds__(S == 1 ? 64 : 32 * S) k_spmv(int64_t n, int B,
 
 // xs[b][j] = (Ms_j m_j, 0) (the 4 padding entries per simulation stay zero)
 __global__ void k_prep_sparse_x(const float *m, const float *Ms, int64_t n, int B, float4 *xs) {
+  mtd::pdl_enter();
   const int64_t tot = (int64_t)B * n;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = t / n, j = t - b * n;
@@ -589,7 +590,8 @@ void launch_spmv(const mt_tensor *T, const float *xs, int B, float *H, const int
 void launch_prep_sparse_x(const mt_tensor *T, const float *m, int B, float *xs, cudaStream_t s) {
   const int64_t tot = (int64_t)B * T->n;
   const int blocks = (int)std::min<int64_t>((tot + 255) / 256, 4096);
-  k_prep_sparse_x<<<blocks, 256, 0, s>>>(m, T->tiles->d_Ms, T->n, B, reinterpret_cast<float4 *>(xs));
+  mt::launch_pdl(k_prep_sparse_x, dim3(blocks), dim3(256), 0, s, m, (const float *)T->tiles->d_Ms, T->n, B,
+                 reinterpret_cast<float4 *>(xs));
 }
 
 }  // namespace mt
