@@ -628,20 +628,12 @@ mt_status mt_llg_rhs(mt_tensor *T, const mt_llg_params *p, const float *m, int B
   std::vector<float> g1, g2, ha;
   std::vector<float> xsc;
   mt::llg_prefactors(p, B, g1, g2, ha, xsc);
-  float *d_par = nullptr;
-  MT_CUDA(cudaMalloc(&d_par, sizeof(float) * 6 * B));
   cudaStream_t s = (cudaStream_t)stream;
-  MT_CUDA(cudaMemcpyAsync(d_par, g1.data(), sizeof(float) * B, cudaMemcpyHostToDevice, s));
-  MT_CUDA(cudaMemcpyAsync(d_par + B, g2.data(), sizeof(float) * B, cudaMemcpyHostToDevice, s));
-  MT_CUDA(cudaMemcpyAsync(d_par + 2 * B, ha.data(), sizeof(float) * 3 * B, cudaMemcpyHostToDevice, s));
-  MT_CUDA(cudaMemcpyAsync(d_par + 5 * B, xsc.data(), sizeof(float) * B, cudaMemcpyHostToDevice, s));
-  if ((st = demag_apply(T, m, B, T->d_Hd, s)) != MT_OK) return st;
   if (tau) MT_CUDA(cudaMemsetAsync(tau, 0, sizeof(float) * B, s));
-  mt::launch_rhs_plain(T, m, T->d_Hd, B, d_par, d_par + B, d_par + 2 * B, d_par + 5 * B, dmdt, tau, s);
+  if ((st = demag_apply(T, m, B, T->d_Hd, s)) != MT_OK) return st;
+  mt::launch_rhs_plain(T, m, T->d_Hd, B, g1.data(), g2.data(), ha.data(), xsc.data(), dmdt, tau, s);
   MT_CUDA(cudaGetLastError());
-  // the parameter block must outlive the kernels
-  MT_CUDA(cudaStreamSynchronize(s));
-  cudaFree(d_par);
+  MT_CUDA(cudaStreamSynchronize(s));  // the results are complete when the call returns
   return MT_OK;
 }
 
