@@ -30,13 +30,27 @@ namespace {
 // ulps of the angle or of the ratio, as much as that of the sums it replaces
 // (whose logarithms of lengths in metres are of order 20); against 128-bit
 // arithmetic distant blocks come out 7 to 13 times closer, touching ones as
-// before.  n = 6,000 graded film, tensor and first field: 150.1 -> 39.3 ms.
+// before.  n = 6,000 graded film, tensor and first field: 150.1 -> 39.3 ms, and
+// 33.6 with signs and sizes tested on the high words and pairs that do not
+// touch told apart by that test alone.
 __device__ __forceinline__ double small_series(double t, double z) {
   // t (1 + z/3 + z^2/5 + z^3/7 + z^4/9 + z^5/11): atan t with z = -t^2,
   // atanh t with z = t^2; |t| < 2^-5 leaves z^6 / 13 < 7e-20
   return t * fma(z, fma(z, fma(z, fma(z, fma(z, 1.0 / 11, 1.0 / 9), 1.0 / 7), 1.0 / 5), 1.0 / 3), 1.0);
 }
 constexpr double kSmallArg = 0.03125;
+
+// Tests of signs and sizes on the high words: a comparison of doubles costs
+// the FP64 pipe as much as a product, and a block has about forty of them.
+__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) << 1) == 0; }
+__device__ __forceinline__ bool is_neg(double a) { return __double2hiint(a) < 0; }
+__device__ __forceinline__ double flip_sign(double a, double of) {  // -a where of is negative
+  return __hiloint2double(__double2hiint(a) ^ (__double2hiint(of) & (int)0x80000000), __double2loint(a));
+}
+// |a| 32 < b by the high words (b >= 0): |a| < kSmallArg b follows
+__device__ __forceinline__ bool is_small(double a, double b) {
+  return (unsigned)(__double2hiint(a) & 0x7fffffff) + (5u << 20) < (unsigned)__double2hiint(b);
+}
 
 // Arguments p of one face pair: theta_1 - theta_0 with theta = atan(b / a),
 // a > 0, as a complex number (its argument is in (-pi, pi)).
@@ -57,27 +71,25 @@ __device__ __forceinline__ Cplx cmul(Cplx p, Cplx q) {
 template <typename RF>
 __device__ __forceinline__ double angle_sum(const double u[2], const double vw[4], RF R) {
   Cplx pa[2], pb[2], f[2];
-  bool plain = true;  // every partial argument within (-pi/2, pi/2): the products keep the branch
+  int least = 1;  // > 0: every partial argument within (-pi/2, pi/2), the products keep the branch
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const double a = fabs(u[k]);
-    if (a == 0.0) {
+    if (is_zero(a)) {
       pa[k] = pb[k] = f[k] = {1.0, 0.0};
       continue;
     }
     pa[k] = arg_diff(a * R(k, 1, 0), vw[1], a * R(k, 0, 0), vw[0]);
     pb[k] = arg_diff(a * R(k, 0, 1), vw[2], a * R(k, 1, 1), vw[3]);
     f[k] = cmul(pa[k], pb[k]);
-    if (u[k] < 0.0) {
-      pa[k].im = -pa[k].im;
-      pb[k].im = -pb[k].im;
-      f[k].im = -f[k].im;
-    }
-    plain = plain && pa[k].re > 0.0 && pb[k].re > 0.0 && f[k].re > 0.0;
+    pa[k].im = flip_sign(pa[k].im, u[k]);
+    pb[k].im = flip_sign(pb[k].im, u[k]);
+    f[k].im = flip_sign(f[k].im, u[k]);
+    least = min(min(least, __double2hiint(f[k].re)), min(__double2hiint(pa[k].re), __double2hiint(pb[k].re)));
   }
-  if (plain) {
+  if (least > 0) {
     const Cplx t = cmul(f[0], {f[1].re, -f[1].im});
-    if (fabs(t.im) < kSmallArg * t.re) {
+    if (!is_neg(t.re) && is_small(t.im, t.re)) {
       const double q = t.im / t.re;
       return small_series(q, -q * q);
     }
@@ -93,13 +105,13 @@ __device__ __forceinline__ double angle_sum(const double u[2], const double vw[4
 // w + R for a point far on the negative side.
 template <typename RF>
 __device__ __forceinline__ double log_sum(const double w[2], RF R) {
-  const bool neg = w[0] < 0.0 && w[1] < 0.0;
+  const bool neg = is_neg(w[0]) && is_neg(w[1]);
   const double w0 = neg ? -w[0] : w[0], w1 = neg ? -w[1] : w[1];
   const double n = ((R(0, 0, 1) + w1) * (R(1, 1, 1) + w1)) * ((R(1, 0, 0) + w0) * (R(0, 1, 0) + w0));
   const double d = ((R(0, 0, 0) + w0) * (R(1, 1, 0) + w0)) * ((R(1, 0, 1) + w1) * (R(0, 1, 1) + w1));
   const double diff = n - d, sum = n + d;
   double v;
-  if (fabs(diff) < kSmallArg * sum) {
+  if (is_small(diff, sum)) {
     const double q = diff / sum;
     v = 2.0 * small_series(q, q * q);  // log(n / d) = 2 atanh((n - d) / (n + d))
   } else {
@@ -115,8 +127,9 @@ __device__ __forceinline__ void cuboid_tensor(const double *r, const double *c, 
   double d[3][2], R[8];  // [axis][face]; corner distance, index fx | fy << 1 | fz << 2
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    d[a][0] = unit * (r[a] - (c[a] - 0.5 * e[a]));
-    d[a][1] = unit * (r[a] - (c[a] + 0.5 * e[a]));
+    const double ur = unit * r[a];
+    d[a][0] = ur - unit * (c[a] - 0.5 * e[a]);
+    d[a][1] = ur - unit * (c[a] + 0.5 * e[a]);
   }
   double xy[4], xz[4], yz[4];
 #pragma unroll
@@ -154,7 +167,7 @@ __device__ __forceinline__ void cuboid_tensor(const double *r, const double *c, 
 // Strackee, 1983; the triple product as (a - r).(b - a) x (c - a)) and 6 edge
 // integrals, l_e = 2 atanh(|e| / (R_a + R_b)).  FP64 throughout; the FP64 pipe bounds it
 // (per-pair face geometry and every edge twice took three times the
-// operations): 5,760 tetrahedra, tensor and first field, 153.8 -> 35.8 ms; errors
+// operations): 5,760 tetrahedra, tensor and first field, 153.8 -> 34.2 ms; errors
 // against 128-bit arithmetic 0.3 to 0.65 of the per-face form's.
 __device__ __forceinline__ void sub3(const double *a, const double *b, double *c) {
   c[0] = a[0] - b[0];
@@ -264,7 +277,8 @@ __device__ __forceinline__ void tetra_tensor(const double *r, const double *G, d
       dots[e] = dot3(D[a], D[b]);
       const double s = L[a] + L[b];
       double li;
-      if (8.0 * len < s) {  // 2 atanh(q), q = len / s: 10 terms leave q^20 / 21 < 5e-20
+      // 8 len < s by the high words; 2 atanh(q), q = len / s: 10 terms leave q^20 / 21 < 5e-20
+      if (__double2hiint(len) + (3 << 20) < __double2hiint(s)) {
         const double q = len / s, z = q * q;
         li = 2.0 * q *
              fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, fma(z, 1.0 / 19, 1.0 / 17), 1.0 / 15), 1.0 / 13),
@@ -287,7 +301,7 @@ __device__ __forceinline__ void tetra_tensor(const double *r, const double *G, d
     const double den = fma(L[a] * L[b], L[c], fma(dots[tetra_edge(a, b)], L[c],
                                                   fma(dots[tetra_edge(a, c)], L[b], dots[tetra_edge(b, c)] * L[a])));
     double half;  // half the solid angle
-    if (fabs(num[f]) < kSmallArg * den) {
+    if (!is_neg(den) && is_small(num[f], den)) {
       const double q = num[f] / den;
       half = small_series(q, -q * q);
     } else {
@@ -348,7 +362,13 @@ __device__ int tetra_relation(const double *ci, const double *vi, const double *
 // (a "near" pair, kept in FP64 for the BF16 precisions).
 __device__ __forceinline__ int pair_relation(const double *ci, const double *ei, const double *cj,
                                              const double *ej) {
+  // boxes that do not touch share no volume and hold no centre either (their
+  // bounds lie 1e-9 inside the touching one's): most pairs end here
   bool vol = true, pt = true, touch = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    touch = touch && (fabs(ci[a] - cj[a]) <= 0.5 * (ei[a] + ej[a]) * (1.0 + 1e-9));
+  if (!touch) return 0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const double d = fabs(ci[a] - cj[a]);
@@ -356,7 +376,6 @@ __device__ __forceinline__ int pair_relation(const double *ci, const double *ei,
     const double tol = 1e-12 * (ei[a] + ej[a]);
     vol = vol && (d < half - tol);
     pt = pt && (d <= 0.5 * ej[a] + tol);
-    touch = touch && (d <= half * (1.0 + 1e-9));
   }
   return ((vol || pt) ? 1 : 0) | (touch ? 2 : 0);
 }
