@@ -48,11 +48,12 @@ MU0 = 4e-7 * math.pi
 MATVEC_F32_N10000_TRAFFIC = {4: 1618117632 + 2918912}  # tensors storing every block
 # The same film with the tensor stored half (upper triangle of chunks, in
 # super-row order) and traceless (3 planes: xx, xy, yy), one ncu capture of
-# each kernel of a product: k_matvec_half<f32, 3 planes> read 621,368,064 and
-# wrote 4,680,192 bytes, k_half_cols read 4,864,000 (the column sums of the
-# groups above the diagonal) and wrote 15,360 -- 1.051 x the 0.60 GB
-# algorithmic bytes.  Valid while both kernels are unchanged.
-MATVEC_F32_HALF_N10000_TRAFFIC = {3: 621368064 + 4680192 + 4864000 + 15360}
+# each kernel of a product: k_matvec_half<f32, 3 planes> read 621,367,296 and
+# wrote 3,282,688 bytes, k_half_sum read 5,303,808 (the column sums of the
+# groups above the diagonal and the parts of split ones) and wrote none to
+# DRAM -- 1.050 x the 0.60 GB algorithmic bytes.  Valid while both kernels are
+# unchanged.
+MATVEC_F32_HALF_N10000_TRAFFIC = {3: 621367296 + 3282688 + 5303808}
 
 
 def f32_alg_bytes(info, n):
@@ -62,10 +63,10 @@ def f32_alg_bytes(info, n):
     one shape is stored half (N_ij = N_ji)."""
     blocks = n * (n + 1) / 2.0 if info.get("half") else float(n) * n
     return 4.0 * info["planes"] * blocks
-# The tensor-core products at n = 8,000 read 1.0040 (split) and 1.0028 (BF16)
+# The tensor-core products at n = 8,000 read 1.0060 (split) and 1.0041 (BF16)
 # x their stored tensors and wrote their fields (one ncu capture each of the
 # current kernels); the batched line scales that per stored byte.
-GEMM_READ_PER_STORED_BYTE = {"split": 1.0040, "bf16": 1.0028}
+GEMM_READ_PER_STORED_BYTE = {"split": 1.0060, "bf16": 1.0041}
 FIELD1 = np.array([-24.6e-3, 4.3e-3, 0.0]) / MU0
 WORKLOAD = "sp4_film_200x50x1_n10000_f32"
 METRIC = "LLG RHS evals/s"
@@ -365,7 +366,7 @@ def run_ours(args):
                                                          else MATVEC_F32_N10000_TRAFFIC).get(planes),
                      "kernel": (("k_matvec_half<f32" if info["half"] else "k_matvec<f32") +
                                 (", %d planes" % planes if planes != 6 else "") +
-                                ("> + k_half_cols" if info["half"] else ">")),
+                                ("> + k_half_sum" if info["half"] else ">")),
                      "stored": "upper triangle of blocks (N_ij = N_ji: tiles of one shape)" if info["half"]
                      else "every block",
                      "peak_kind": kind, "algorithmic_bytes_per_launch": alg_bytes,
@@ -381,7 +382,7 @@ def run_ours(args):
         "cpu_baseline": cpu,
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": 12 * n, "d2h_bytes_per_step": 12 * n,
                 "note": "set_state(pinned host) + 1 step + get_state(host); 6 RHS counted per step"},
-        "gpu_launches": 13 * args.steps,
+        "gpu_launches": (19 if info["half"] else 13) * args.steps,  # k_half_sum after each half product
         "clocks": clk.summary(),
     }
     line.update(extra)
@@ -1181,7 +1182,7 @@ def run_cube(args):
             "assemble_s": t_asm,
             "roofline": {"bound": "hbm", "achieved": alg / (launch * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": alg / (launch * 1e-3) / 1e9 / peak, "traffic": None,
-                         "kernel": "k_matvec_half<f32> + k_half_cols" if info["half"] else "k_matvec<f32>",
+                         "kernel": "k_matvec_half<f32> + k_half_sum" if info["half"] else "k_matvec<f32>",
                          "stored": "upper triangle of blocks (N_ij = N_ji: tiles of one shape)" if info["half"]
                          else "every block",
                          "algorithmic_bytes_per_launch": alg, "launch_ms": launch,
@@ -1189,7 +1190,7 @@ def run_cube(args):
                          "standalone_launch_ms": alone, "peak_kind": kind},
             "relax": {"tol": args.tol, "t_max_s": args.cube_tmax, "rtol_atol": args.cube_rtol, "alpha": 0.5,
                       "wall_s": relax_wall, "status": int(s), "states": states},
-            "cpu_baseline": cpu, "gpu_launches": 13 * args.steps, "clocks": clk.summary()}
+            "cpu_baseline": cpu, "gpu_launches": (19 if info["half"] else 13) * args.steps, "clocks": clk.summary()}
     T.close()
     tiles.close()
     print(json.dumps(line), flush=True)

@@ -1228,7 +1228,7 @@ __global__ void k_near(int64_t n, int B, const int32_t *ptr, const int32_t *col,
 // three floats per tile in every simulation's own vector, is read and written
 // in runs of whole tiles; a thread that wrote its own tile and
 // simulation touched a 32-byte sector for each value.  n = 10,000, B = 64, BF16:
-// 53 -> 36 us (split, n = 20,000: 118 -> 114, its double-FP32 sums bound it).
+// 53 -> 36 us (split, n = 20,000: 118 -> 104, its double-FP32 sums bound it).
 template <int V>
 struct VecF;
 template <>
