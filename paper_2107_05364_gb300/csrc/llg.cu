@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs A) {
 // exchanges, the rest the serial chain of one stage).
 constexpr int kSmallThreads = 256;
 constexpr int kSmallWarps = kSmallThreads / 32;
-constexpr int kSmallRed = 3 * 8 * kSmallWarps;       // floats of one buffer of row sums: one simulation's
+constexpr int kSmallRed = 3 * 8 * kSmallWarps;       // floats of one simulation's row sums
 constexpr int kSmallRedL2 = 3 * 16 * kSmallWarps;    // rows read from L2: those of 8 simulations
 
 // one tile's vector: 3 floats and the 16-bit tag in each of two 64-bit words;
@@ -600,6 +600,8 @@ struct SmallArgs {
   int64_t iters;    // attempts at most (kSmallChunk: their 6 tags each fit 16 bits)
   int init;         // evaluate k1 and the torque at the state first
   int R;            // rows per CTA at most
+  int group;        // rows in shared memory: simulations between two CTA barriers (1, 2, 4 or 8)
+  int lanes;        // threads that poll one simulation's vectors (a power of two)
 };
 
 // byte offsets of the dynamic shared memory of k_small_run
@@ -615,11 +617,11 @@ __host__ __device__ __forceinline__ size_t small_take(size_t &o, size_t bytes) {
 // three float4 from 16-byte boundaries (12 floats past the last one's end are
 // allocated for a last row of fewer tiles)
 __host__ __device__ __forceinline__ int small_stride(int64_t n) { return (int)((3 * n + 3) & ~(int64_t)3); }
-__host__ __device__ __forceinline__ SmallSmem small_smem(int64_t n, int B, int R, bool nsmem) {
+__host__ __device__ __forceinline__ SmallSmem small_smem(int64_t n, int B, int R, bool nsmem, int group) {
   SmallSmem s;
   size_t o = 0;
   s.ctl = small_take(o, sizeof(SimCtl) * B);
-  s.red = small_take(o, sizeof(float) * 2 * (nsmem ? kSmallRed : kSmallRedL2));
+  s.red = small_take(o, sizeof(float) * 2 * (nsmem ? group * kSmallRed : kSmallRedL2));
   s.y = small_take(o, sizeof(float) * B * R * 3);
   s.k = small_take(o, sizeof(float) * 7 * B * R * 3);
   s.coef = small_take(o, sizeof(float) * B * 36);  // (float)(h a_sj), s = 1..6, j < s
@@ -680,30 +682,31 @@ struct PollLimit {
   }
 };
 
-// n tagged vectors from src: f(j, v) for this thread's j = tid, tid + 256, ...
-// (four in flight at once).  False when the wait gave up.
+// n tagged vectors from src: f(j, v) for this thread's j = first, first +
+// lanes, ... (four in flight at once).  False when the wait gave up.
 template <typename F>
-__device__ __forceinline__ bool poll_vecs(const SmallArgs &S, const TagVec *src, int n, unsigned tag, F &&f) {
+__device__ __forceinline__ bool poll_vecs(const SmallArgs &S, const TagVec *src, int n, unsigned tag, int first,
+                                          int lanes, F &&f) {
   constexpr int U = 4;
   PollLimit lim;
-  for (int j0 = threadIdx.x; j0 < n; j0 += U * kSmallThreads) {
+  for (int j0 = first; j0 < n; j0 += U * lanes) {
     unsigned long long a[U], b[U];
     for (;;) {
       bool all = true;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int j = j0 + u * kSmallThreads;
+        const int j = j0 + u * lanes;
         if (j < n) ld_pair(src + j, a[u], b[u]);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (j0 + u * kSmallThreads < n) all = all && vec_tagged(a[u], b[u], tag);
+        if (j0 + u * lanes < n) all = all && vec_tagged(a[u], b[u], tag);
       if (all) break;
       if (lim.expired(S)) return false;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int j = j0 + u * kSmallThreads;
+      const int j = j0 + u * lanes;
       if (j < n) {
         float v[3];
         vec_of(a[u], b[u], v);
@@ -956,9 +959,9 @@ struct SmallRow {
 // 1..6 k, for stages 2..6 also the next stage's input, published under
 // `tag`; after stage 7 k7 and the sums of the error norm, the torque and <m>;
 // after stage 1 (k1 at the state) k1 and the torque.  One CTA barrier between
-// the product of a simulation (rows read from L2: of eight) and the rest:
-// sh.M is read only before it (a later exchange may overwrite it), and the
-// two buffers of row sums alternate.
+// the product of a simulation (MANY: of S.group of them; rows read from L2: of
+// eight) and the rest: sh.M is read only before it (a later exchange may
+// overwrite it), and the two buffers of row sums alternate.
 //
 // What a row needs of the other tiles: m itself and the exchange sum.
 struct SmallPre {
@@ -1057,14 +1060,33 @@ __device__ __forceinline__ void small_rows(const SmallArgs &S, const SmallSh &sh
   small_partial(S, b, v, tag);
 }
 
-template <int RMAX, bool NSMEM, bool PLANAR>
+template <int RMAX, bool NSMEM, bool PLANAR, bool MANY>
 __device__ __forceinline__ void small_stage(const SmallArgs &S, const SmallSh &sh, const SmallRow &rw, int st,
                                             unsigned tag, int nr, int64_t r0, int &buf) {
   const StageArgs &A = S.A;
   const int n = (int)A.n, B = A.B;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   SmallPre pr = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
-  if constexpr (NSMEM) {
+  if constexpr (MANY) {
+    for (int base = 0; base < B; base += S.group) {
+      const int end = base + S.group < B ? base + S.group : B;
+      float *red = sh.red + buf * S.group * kSmallRed;
+      buf ^= 1;
+      bool live = false;  // the same in every thread
+      for (int b = base; b < end; ++b) {
+        if (sh.ctl[b].done) continue;
+        live = true;
+        small_product<RMAX, PLANAR>(sh, sh.M + b * small_stride(n), red + (b - base) * kSmallRed, S.R, nr, n);
+      }
+      if (!live) continue;
+      const int b = base + ((warp - base) & (kSmallWarps - 1));  // this warp's simulation of the group
+      const bool mine = b < end && !sh.ctl[b].done;
+      if (mine && lane < nr) small_pre(A, rw, sh.M + b * small_stride(n), (int)r0 + lane, pr);
+      __syncthreads();
+      if (mine)
+        small_rows<kSmallWarps, 3 * RMAX>(S, sh, rw, pr, red + (b - base) * kSmallRed, b, st, tag, nr, r0);
+    }
+  } else if constexpr (NSMEM) {
     for (int b = 0; b < B; ++b) {
       if (sh.ctl[b].done) continue;  // the same in every thread
       const float *mb = sh.M + b * small_stride(n);
@@ -1100,7 +1122,7 @@ __device__ __forceinline__ void small_stage(const SmallArgs &S, const SmallSh &s
   }
 }
 
-template <int RMAX, bool NSMEM, bool PLANAR>
+template <int RMAX, bool NSMEM, bool PLANAR, bool MANY>
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
   extern __shared__ __align__(16) unsigned char smem[];
   const StageArgs &A = S.A;
@@ -1109,7 +1131,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
   const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r0 = (int64_t)g * n / G, r1 = (int64_t)(g + 1) * n / G;
   const int nr = (int)(r1 - r0);
-  const SmallSmem L = small_smem(n, B, R, NSMEM);
+  const SmallSmem L = small_smem(n, B, R, NSMEM, MANY ? S.group : 1);
   SmallSh sh;
   sh.ctl = reinterpret_cast<SimCtl *>(smem + L.ctl);
   sh.red = reinterpret_cast<float *>(smem + L.red);
@@ -1122,6 +1144,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
   sh.M = reinterpret_cast<float *>(smem + L.M);
   sh.N = reinterpret_cast<float *>(smem + L.N);
   const size_t kpl = (size_t)B * R * 3;
+  // `lanes` threads poll the vectors of one simulation: this one b0, b0 + sims, ...
+  const int lanes = MANY ? S.lanes : kSmallThreads, sims = MANY ? kSmallThreads / lanes : 1;
+  const int b0 = MANY ? tid / lanes : 0, j0 = MANY ? tid & (lanes - 1) : tid;
   unsigned seq = 0;  // exchanges so far: the next one's tag is seq + 1
   int buf = 0;
   bool ok = true;
@@ -1174,7 +1199,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
   __syncthreads();
 
   if (S.init) {  // k1 and the torque at the state
-    small_stage<RMAX, NSMEM, PLANAR>(S, sh, rw, 1, 1, nr, r0, buf);
+    small_stage<RMAX, NSMEM, PLANAR, MANY>(S, sh, rw, 1, 1, nr, r0, buf);
     seq = 1;
     for (int b = warp; ok && b < B; b += kSmallWarps) {
       if (sh.ctl[b].done) continue;
@@ -1199,7 +1224,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
     // all tiles, y + (h a_21) k1, from the committed state (after an accepted
     // attempt: the normalised 5th-order solution still in sh.M and the k7
     // every CTA published; else the committed y and k1)
-    for (int b = 0; b < B; ++b) {
+    for (int b = b0; b < B; b += sims) {
       if (sh.ctl[b].done) continue;
       const int kc = sh.kc[b];
       const bool adopt = it > 0 && sh.ctl[b].accepted;
@@ -1208,11 +1233,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
       const float *yb = A.y + (size_t)b * 3 * n, *kb = A.k[0] + (size_t)b * 3 * n;
       if (!adopt) {  // the committed y into sh.M
         if (kc & kKcY)
-          ok = poll_vecs(S, S.yx + (size_t)b * n, (int)n, kc & kKcTag, [&](int j, const float *y) {
+          ok = poll_vecs(S, S.yx + (size_t)b * n, (int)n, kc & kKcTag, j0, lanes, [&](int j, const float *y) {
                  for (int c = 0; c < 3; ++c) mb[3 * j + c] = y[c];
                }) && ok;
         else
-          for (int j = tid; j < n; j += kSmallThreads)
+          for (int j = j0; j < n; j += lanes)
             for (int c = 0; c < 3; ++c) mb[3 * j + c] = __ldcg(yb + 3 * j + c);
       }
       auto form = [&](int j, const float *k1) {  // (the thread that wrote mb[j])
@@ -1222,10 +1247,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
         for (int c = 0; c < 3; ++c) mb[3 * j + c] = __fadd_rn(y[c], __fmul_rn(a21, k1[c]));
       };
       if (kc & kKcTag)
-        ok = poll_vecs(S, S.kx + (size_t)((kc & kKcBuf) ? 1 : 0) * B * n + (size_t)b * n, (int)n, kc & kKcTag, form) &&
+        ok = poll_vecs(S, S.kx + (size_t)((kc & kKcBuf) ? 1 : 0) * B * n + (size_t)b * n, (int)n, kc & kKcTag, j0,
+                       lanes, form) &&
              ok;
       else
-        for (int j = tid; j < n; j += kSmallThreads) {
+        for (int j = j0; j < n; j += lanes) {
           const float k1[3] = {__ldcg(kb + 3 * j), __ldcg(kb + 3 * j + 1), __ldcg(kb + 3 * j + 2)};
           form(j, k1);
         }
@@ -1234,10 +1260,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
     if (!ok) break;
     for (int st = 2; st <= 7; ++st) {
       if (st > 2) {  // all tiles' input of this stage
-        for (int b = 0; b < B; ++b) {
+        for (int b = b0; b < B; b += sims) {
           if (sh.ctl[b].done) continue;
           float *mb = sh.M + b * small_stride(n);
-          ok = poll_vecs(S, S.xg + (size_t)(st & 1) * B * n + (size_t)b * n, (int)n, seq + st - 2,
+          ok = poll_vecs(S, S.xg + (size_t)(st & 1) * B * n + (size_t)b * n, (int)n, seq + st - 2, j0, lanes,
                          [&](int j, const float *v) {
                            for (int c = 0; c < 3; ++c) mb[3 * j + c] = v[c];
                          }) && ok;
@@ -1245,7 +1271,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(SmallArgs S) {
         ok = __syncthreads_and(ok);
         if (!ok) break;
       }
-      small_stage<RMAX, NSMEM, PLANAR>(S, sh, rw, st, seq + st - 1, nr, r0, buf);
+      small_stage<RMAX, NSMEM, PLANAR, MANY>(S, sh, rw, st, seq + st - 1, nr, r0, buf);
     }
     if (!ok) break;
     seq += 6;  // the k7 and the partial sums went out under this tag
@@ -1310,7 +1336,7 @@ __global__ void k_exchange_selftest(SmallArgs S) {
   if (blockIdx.x == 0) return;
   const float v[3] = {1.0f, 2.0f, 3.0f};
   if (threadIdx.x == 0) publish_vec(S.xg + blockIdx.x, v, 1);
-  poll_vecs(S, S.xg, gridDim.x, 1, [](int, const float *) {});
+  poll_vecs(S, S.xg, gridDim.x, 1, threadIdx.x, blockDim.x, [](int, const float *) {});
 }
 
 // put a prepared control block into slot b and make it active
@@ -1500,7 +1526,8 @@ struct mt_integrator {
   // small tile sets: the whole call in one cooperative kernel (k_small_run)
   int path = MT_PATH_GRAPH;  // the one in use
   bool small_ok = false;     // the tile set and batch fit it
-  int small_G = 0, small_R = 0, small_rmax = 0;
+  int small_G = 0, small_R = 0, small_rmax = 0, small_group = 1, small_lanes = kSmallThreads;
+  bool small_many = false;  // its form for several simulations
   bool small_nsmem = true;  // tensor rows in shared memory (else read from L2)
   size_t small_smem_bytes = 0;
   unsigned char *sm_words = nullptr;  // words its CTAs exchange, then the abort flag (SmallWords)
@@ -1554,14 +1581,17 @@ StageArgs stage_args(mt_integrator *I) {
 constexpr size_t kSmallSmemMax = 225 * 1024;  // of the 227 KB a CTA may opt in to
 
 using SmallKernel = void (*)(SmallArgs);
-template <bool PLANAR>
-SmallKernel small_kernel_of(bool nsmem, int rmax) {
-  return !nsmem ? k_small_run<2, false, PLANAR>
-                : rmax == 2 ? k_small_run<2, true, PLANAR>
-                            : rmax == 4 ? k_small_run<4, true, PLANAR> : k_small_run<8, true, PLANAR>;
+template <bool PLANAR, bool MANY>
+SmallKernel small_kernel_of(int rmax) {
+  return rmax == 2   ? k_small_run<2, true, PLANAR, MANY>
+         : rmax == 4 ? k_small_run<4, true, PLANAR, MANY>
+                     : k_small_run<8, true, PLANAR, MANY>;
 }
-SmallKernel small_kernel(const mt_tensor *T, bool nsmem, int rmax) {
-  return T->L.nplane == 4 ? small_kernel_of<true>(nsmem, rmax) : small_kernel_of<false>(nsmem, rmax);
+SmallKernel small_kernel(const mt_tensor *T, bool nsmem, int rmax, bool many) {
+  const bool planar = T->L.nplane == 4;
+  if (!nsmem) return planar ? k_small_run<2, false, true, false> : k_small_run<2, false, false, false>;
+  if (many) return planar ? small_kernel_of<true, true>(rmax) : small_kernel_of<false, true>(rmax);
+  return planar ? small_kernel_of<true, false>(rmax) : small_kernel_of<false, false>(rmax);
 }
 
 // byte offsets of the exchanged words of k_small_run
@@ -1603,7 +1633,7 @@ bool small_plan(mt_integrator *I) {
     const int R = (int)r_sm;
     if (R > (nsmem ? 8 : 2 * kSmallWarps)) continue;
     if (!nsmem && (T->bytes > kSmallL2Bytes || T->L.TC % 4 != 0)) continue;
-    const size_t bytes = small_smem(n, I->B, R, nsmem).total;
+    size_t bytes = small_smem(n, I->B, R, nsmem, 1).total;
     // (the limit counts one buffer of row sums, unpadded states, and H_d, the torque and the
     // constants of the CTA's rows, once held in shared memory: the same tile
     // sets qualify for this path whatever its kernel keeps there)
@@ -1614,10 +1644,26 @@ bool small_plan(mt_integrator *I) {
     counted += unpadded - state;
     for (const int per_row : {3 * I->B, I->B, 6, 6, 1, 3, 1}) small_take(counted, sizeof(float) * R * per_row);
     if (counted > kSmallSmemMax) continue;
+    // Several simulations: `group` of them (as many as fit) between two CTA
+    // barriers, one to a warp, and the threads divided among as many as keep
+    // the poll of one a single round of four vectors per thread.  One after
+    // the other, a barrier, a round trip and a chain each, 16 simulations of
+    // 10 tiles took 114 us per attempt, so 46; 16 of 400 tiles 149, so 100
+    // (one simulation: 12 and 20).  Three and four go two at a time: all at
+    // once, the polls of 100 to 150 CTAs with a row each get in the way of
+    // the stores (150 tiles, 4: 38 us against 29).  Two, and three whose poll
+    // takes more than a round, are as fast one after the other (400 tiles, 2:
+    // 23 us against 27; 1,000 tiles, 3: 46 and 47).
+    const bool many = nsmem && (I->B >= 4 || (I->B == 3 && n <= 4 * kSmallThreads / 2));
+    const int at_once = I->B <= 4 ? 2 : kSmallWarps;
+    int group = 1, lanes = kSmallThreads;
+    while (many && group < at_once && small_smem(n, I->B, R, nsmem, 2 * group).total <= kSmallSmemMax) group *= 2;
+    while (many && kSmallThreads / lanes < (at_once == 2 ? 2 : I->B) && lanes > 1 && n <= 4 * (lanes / 2)) lanes /= 2;
+    bytes = small_smem(n, I->B, R, nsmem, group).total;
     const int G = (int)((n + R - 1) / R);
     const int rmax = !nsmem ? 2 : R <= 2 ? 2 : R <= 4 ? 4 : 8;
     int per_sm = 0;
-    const SmallKernel kern = small_kernel(T, nsmem, rmax);
+    const SmallKernel kern = small_kernel(T, nsmem, rmax, many);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSmallThreads, bytes);
     if (e != cudaSuccess) {
@@ -1629,6 +1675,9 @@ bool small_plan(mt_integrator *I) {
     I->small_R = R;
     I->small_rmax = rmax;
     I->small_nsmem = nsmem;
+    I->small_many = many;
+    I->small_group = group;
+    I->small_lanes = lanes;
     I->small_smem_bytes = bytes;
     return true;
   }
@@ -1653,6 +1702,8 @@ mt_status launch_small(mt_integrator *I, int init, int64_t iters) {
   S.iters = iters;
   S.init = init;
   S.R = I->small_R;
+  S.group = I->small_group;
+  S.lanes = I->small_lanes;
   MT_CUDA(cudaMemsetAsync(I->sm_words, 0, w.total, I->stream));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)I->small_G);
@@ -1672,7 +1723,7 @@ mt_status launch_small(mt_integrator *I, int init, int64_t iters) {
   if (!ctx->small_ev) e = cudaEventCreateWithFlags(&ctx->small_ev, cudaEventDisableTiming);
   else e = cudaStreamWaitEvent(I->stream, ctx->small_ev, 0);
   if (e == cudaSuccess) {
-    e = cudaLaunchKernelEx(&cfg, small_kernel(T, I->small_nsmem, I->small_rmax), S);
+    e = cudaLaunchKernelEx(&cfg, small_kernel(T, I->small_nsmem, I->small_rmax, I->small_many), S);
   }
   if (e == cudaSuccess) e = cudaEventRecord(ctx->small_ev, I->stream);
   if (e != cudaSuccess) return mt::cuda_fail(e, "k_small_run launch", __FILE__, __LINE__);
