@@ -1579,6 +1579,7 @@ StageArgs stage_args(mt_integrator *I) {
 }
 
 constexpr size_t kSmallSmemMax = 225 * 1024;  // of the 227 KB a CTA may opt in to
+constexpr int kSmallSmemLimit = 227 * 1024;
 
 using SmallKernel = void (*)(SmallArgs);
 template <bool PLANAR, bool MANY>
@@ -1664,7 +1665,9 @@ bool small_plan(mt_integrator *I) {
     const int rmax = !nsmem ? 2 : R <= 2 ? 2 : R <= 4 ? 4 : 8;
     int per_sm = 0;
     const SmallKernel kern = small_kernel(T, nsmem, rmax, many);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the limit is the kernel's, for every integrator that uses it: a later and
+    // smaller one must not lower it
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemLimit);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSmallThreads, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
