@@ -785,6 +785,23 @@ GemmVariant gemm_variant(bool split, int Bp, int np) {
   }
 }
 
+// CTAs of a product: one per SM, but at least four units to each (every CTA
+// must own one, which the bookkeeping of split row tiles relies on): the last
+// CTA of a row tile adds the parts of all others, a chain that grows with
+// them.  Fields with a unit per CTA, with four (and with the nine-entry form
+// that came before), split precision, 33 simulations: 130 tiles 29.1, 18.3
+// (24.5) us, 392 tiles 56.5, 30.6 (46.1), 729 tiles 50.0, 40.8 (46.2); from
+// 1,700 tiles on every SM has that many.  Eight gain more at some sizes (1,000
+// tiles of a film 35.3 -> 29.9) and lose at others (350 tiles, BF16, 4
+// simulations: 10.4 -> 13.9), as the ranges fall on the row tiles.  One row
+// tile, up to 128 tiles, is left to one CTA (8 tiles, BF16, 128 simulations
+// 21.3 -> 13.2 us; 64 tiles in a cube, split, 33: 26.0 -> 20.2).
+constexpr int kMinUnits = 4;
+int gemm_grid(const mt_tensor *T, int planes_per_unit) {
+  const int64_t MT = T->Kp / GM, KB = T->Kp / GK, units = MT * KB * (T->L.nplane / planes_per_unit);
+  return MT == 1 ? 1 : (int)std::min<int64_t>(mt::matvec_grid(T), std::max<int64_t>(1, units / kMinUnits));
+}
+
 }  // namespace
 
 namespace mt {
@@ -905,9 +922,7 @@ void launch_gemm(const mt_tensor *T, const GemmPlan &plan, float *H, float *part
   P.count = count;
   P.n_active = n_active;
   P.status = status;
-  // never more CTAs than units: every CTA then owns at least one, which the
-  // bookkeeping of split row tiles relies on
-  const int grid = (int)std::min<int64_t>(matvec_grid(T), P.MT * P.KB * (T->L.nplane / v.planes_per_unit));
+  const int grid = gemm_grid(T, v.planes_per_unit);
   launch_pdl(v.kernel, dim3(grid), dim3(v.threads), plan.stages * v.stage_bytes + v.fixed_bytes, s, plan.tA,
              plan.tX, P);
 }
