@@ -468,66 +468,21 @@ mt_status mt_demag_assemble_ex(mt_tiles *tiles, mt_prec prec, int layout, mt_ten
   MT_CHECK(layout == MT_LAYOUT_STREAM || layout == MT_LAYOUT_DENSE || layout == MT_LAYOUT_STREAM6 ||
                layout == MT_LAYOUT_STREAM_FULL || layout == MT_LAYOUT_STREAM_HALF,
            MT_EINVAL, "mt_demag_assemble: bad layout %d", layout);
-  const bool allow_planar =
-      layout == MT_LAYOUT_STREAM || layout == MT_LAYOUT_STREAM_FULL || layout == MT_LAYOUT_STREAM_HALF;
-  const bool force_half = layout == MT_LAYOUT_STREAM_HALF;
-  const bool allow_half = layout == MT_LAYOUT_STREAM || force_half;
-  MT_CHECK(!force_half || (prec == MT_F32 && tiles->kind == MT_TILE_CUBOID), MT_EINVAL,
-           "mt_demag_assemble: MT_LAYOUT_STREAM_HALF stores FP32 tensors of cuboid tiles only");
-  if (layout != MT_LAYOUT_DENSE) layout = MT_LAYOUT_STREAM;
-  MT_CHECK(layout == MT_LAYOUT_STREAM || prec == MT_BF16_SCALED || prec == MT_BF16_SPLIT, MT_EINVAL,
-           "mt_demag_assemble: the dense layout stores BF16 or split BF16 only");
   mt_ctx *ctx = tiles->ctx;
   MT_CUDA(cudaSetDevice(ctx->device));
   mt_tensor *T = new mt_tensor();
   T->tiles = tiles;
   tiles->refs++;
   T->prec = prec;
-  T->layout = layout;
   T->n = tiles->n;
-  size_t data_bytes = 0, scale_bytes = 0;
-  if (layout == MT_LAYOUT_DENSE) {
-    // thread mapping of the assembly kernel: 16-row panels x 128-column chunks
-    T->L.TR = 16;
-    T->L.TC = 128;
-    T->L.nplane = single_layer(tiles) ? 4 : 6;
-    T->L.elem_bytes = 2;
-    T->L.P = (T->n + T->L.TR - 1) / T->L.TR;
-    T->L.Q = (T->n + T->L.TC - 1) / T->L.TC;
-    T->Kp = ((T->n + 127) / 128) * 128;
-    data_bytes = mt::dense_tensor_bytes(T->n, prec, T->L.nplane);
-  } else {
-    mt::layout_for(prec, &T->L);
-    // single-layer set: the xz and yz entries vanish; 4 entry planes
-    if (allow_planar && prec != MT_F64 && single_layer(tiles)) mt::layout_for_planar(prec, &T->L);
-    T->L.P = (T->n + T->L.TR - 1) / T->L.TR;
-    T->L.Q = (T->n + T->L.TC - 1) / T->L.TC;
-    // FP32 tiles of one shape: the tensor is symmetric (N_ij = N_ji), so
-    // only the upper triangle of chunks is stored (Sec. 3.2); by default
-    // from kHalfMinTiles tiles on, where the half product is the faster one
-    if (allow_half && prec == MT_F32 && tiles->kind == MT_TILE_CUBOID && (force_half || T->n > kHalfMinTiles)) {
-      // one shape: equal edges to 1e-12 (as for the lattice test; the
-      // tensor then differs from a symmetric one far below FP32 rounding)
-      bool same = true;
-      for (int64_t i = 1; i < tiles->n && same; ++i)
-        for (int a = 0; a < 3; ++a)
-          same = same && std::fabs(tiles->edge[3 * i + a] - tiles->edge[a]) <= 1e-12 * tiles->edge[a];
-      T->L.half = same;
-    }
-    // an FP32 tensor stored half leaves out zz, which the trace gives
-    // (traceless; checked on every block at assembly): 3 planes for a single
-    // layer, 5 otherwise
-    if (T->L.half && prec == MT_F32) mt::layout_for_traceless(&T->L, T->L.nplane == 4);
-    if (force_half && !T->L.half) {
-      delete T;
-      mt::tiles_release(tiles);
-      MT_CHECK(false, MT_EINVAL, "mt_demag_assemble: MT_LAYOUT_STREAM_HALF needs tiles of one shape");
-    }
-    T->L.CH = T->L.half ? half_chunks(T->L.P, T->L.Q, T->L.TC / T->L.TR) : T->L.P * T->L.Q;
-    data_bytes = (size_t)T->L.CH * T->L.chunk_bytes();
-    scale_bytes = (size_t)T->L.CH * T->L.scale_bytes_per_chunk;
+  size_t scale_bytes = 0;
+  const mt_status planned = mt::plan_storage(T, layout, &scale_bytes);
+  if (planned != MT_OK) {
+    delete T;
+    mt::tiles_release(tiles);
+    return planned;
   }
-  T->bytes = data_bytes + scale_bytes;
+  const size_t data_bytes = T->bytes - scale_bytes;
   {
     std::lock_guard<std::mutex> lk(ctx->mu);
     if (ctx->in_use + T->bytes > ctx->budget) {
@@ -662,15 +617,99 @@ void tensor_release(mt_tensor *T) {
 
 namespace mt {
 
-// device bytes of a tensor of n tiles in a precision and layout (as allocated
-// by mt_demag_assemble_ex)
-size_t tensor_bytes_for(int64_t n, int prec, int layout) {
-  if (layout == MT_LAYOUT_DENSE) return dense_tensor_bytes(n, prec, 6);
-  mt_layout L;
-  layout_for(prec, &L);
-  L.P = (n + L.TR - 1) / L.TR;
-  L.Q = (n + L.TC - 1) / L.TC;
-  return (size_t)L.P * L.Q * (L.chunk_bytes() + L.scale_bytes_per_chunk);
+// Storage of a tensor of T->tiles in T->prec, decided before anything is
+// allocated: layout, planes, chunks and bytes (scale_bytes of them block
+// scales).  Assembly may still find that a set needs all 6 planes.
+mt_status plan_storage(mt_tensor *T, int layout, size_t *scale_bytes) {
+  const mt_tiles *tiles = T->tiles;
+  const int prec = T->prec;
+  const bool allow_planar =
+      layout == MT_LAYOUT_STREAM || layout == MT_LAYOUT_STREAM_FULL || layout == MT_LAYOUT_STREAM_HALF;
+  const bool force_half = layout == MT_LAYOUT_STREAM_HALF;
+  const bool allow_half = layout == MT_LAYOUT_STREAM || force_half;
+  MT_CHECK(!force_half || (prec == MT_F32 && tiles->kind == MT_TILE_CUBOID), MT_EINVAL,
+           "mt_demag_assemble: MT_LAYOUT_STREAM_HALF stores FP32 tensors of cuboid tiles only");
+  if (layout != MT_LAYOUT_DENSE) layout = MT_LAYOUT_STREAM;
+  MT_CHECK(layout == MT_LAYOUT_STREAM || prec == MT_BF16_SCALED || prec == MT_BF16_SPLIT, MT_EINVAL,
+           "mt_demag_assemble: the dense layout stores BF16 or split BF16 only");
+  T->layout = layout;
+  *scale_bytes = 0;
+  if (layout == MT_LAYOUT_DENSE) {
+    // thread mapping of the assembly kernel: 16-row panels x 128-column chunks
+    T->L.TR = 16;
+    T->L.TC = 128;
+    T->L.nplane = single_layer(tiles) ? 4 : 6;
+    T->L.elem_bytes = 2;
+    T->L.P = (T->n + T->L.TR - 1) / T->L.TR;
+    T->L.Q = (T->n + T->L.TC - 1) / T->L.TC;
+    T->Kp = ((T->n + 127) / 128) * 128;
+    T->bytes = dense_tensor_bytes(T->n, prec, T->L.nplane);
+    return MT_OK;
+  }
+  layout_for(prec, &T->L);
+  // single-layer set: the xz and yz entries vanish; 4 entry planes
+  if (allow_planar && prec != MT_F64 && single_layer(tiles)) layout_for_planar(prec, &T->L);
+  T->L.P = (T->n + T->L.TR - 1) / T->L.TR;
+  T->L.Q = (T->n + T->L.TC - 1) / T->L.TC;
+  // FP32 tiles of one shape: the tensor is symmetric (N_ij = N_ji), so
+  // only the upper triangle of chunks is stored (Sec. 3.2), by default above
+  // kHalfMinTiles tiles
+  if (allow_half && prec == MT_F32 && tiles->kind == MT_TILE_CUBOID && (force_half || T->n > kHalfMinTiles)) {
+    // one shape: equal edges to 1e-12 (as for the lattice test; the
+    // tensor then differs from a symmetric one far below FP32 rounding)
+    bool same = true;
+    for (int64_t i = 1; i < tiles->n && same; ++i)
+      for (int a = 0; a < 3; ++a)
+        same = same && std::fabs(tiles->edge[3 * i + a] - tiles->edge[a]) <= 1e-12 * tiles->edge[a];
+    T->L.half = same;
+  }
+  // an FP32 tensor stored half leaves out zz, which the trace gives
+  // (traceless; checked on every block at assembly): 3 planes for a single
+  // layer, 5 otherwise
+  if (T->L.half && prec == MT_F32) layout_for_traceless(&T->L, T->L.nplane == 4);
+  MT_CHECK(!force_half || T->L.half, MT_EINVAL,
+           "mt_demag_assemble: MT_LAYOUT_STREAM_HALF needs tiles of one shape");
+  T->L.CH = T->L.half ? half_chunks(T->L.P, T->L.Q, T->L.TC / T->L.TR) : T->L.P * T->L.Q;
+  *scale_bytes = (size_t)T->L.CH * T->L.scale_bytes_per_chunk;
+  T->bytes = (size_t)T->L.CH * T->L.chunk_bytes() + *scale_bytes;
+  return MT_OK;
+}
+
+// Device bytes to reserve for the tensor of cuboid tiles (centre, edge) and an
+// integrator of B simulations on it, before either exists: the tensor with all
+// the planes that its assembly may turn out to need.
+size_t engine_bytes_bound(mt_ctx *ctx, int64_t n, const std::vector<double> &centre, const std::vector<double> &edge,
+                          int prec, int layout, int B) {
+  mt_tiles tiles;
+  tiles.ctx = ctx;
+  tiles.n = n;
+  tiles.centre = centre;
+  tiles.edge = edge;
+  mt_tensor T;
+  T.tiles = &tiles;
+  T.prec = prec;
+  T.n = n;
+  size_t scale_bytes = 0;
+  if (plan_storage(&T, layout, &scale_bytes) != MT_OK &&  // (its assembly will say so)
+      plan_storage(&T, MT_LAYOUT_STREAM_FULL, &scale_bytes) != MT_OK)
+    return 0;
+  if (T.layout == MT_LAYOUT_DENSE) {
+    T.L.nplane = 6;
+    T.bytes = dense_tensor_bytes(n, prec, 6);
+  } else {
+    mt_layout all;
+    layout_for(prec, &all);
+    T.bytes = (size_t)T.L.CH * (all.chunk_bytes() + all.scale_bytes_per_chunk);
+  }
+  return T.bytes + integ_bytes(&T, B);
+}
+
+// device bytes of an assembled tensor, the blocks kept apart among them
+size_t tensor_device_bytes(const mt_tensor *T) {
+  const size_t near = T->d_near_ptr ? sizeof(int32_t) * (T->n + 1 + T->near_count) +
+                                          6 * (sizeof(double) + sizeof(float2)) * (size_t)T->near_count
+                                    : 0;
+  return T->bytes + near;
 }
 
 }  // namespace mt

@@ -824,7 +824,7 @@ float *dense_mT(const mt_tensor *T, int B, void *X) {
   return reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(X) + dense_operand_bytes(T, B));
 }
 size_t dense_part_bytes(const mt_tensor *T, int B) {
-  return (size_t)2 * matvec_grid(T) * 3 * dense_pad_batch(B) * GM * sizeof(float);
+  return (size_t)2 * gemm_grid(T, T->prec == MT_BF16_SPLIT ? 1 : 2) * 3 * dense_pad_batch(B) * GM * sizeof(float);
 }
 size_t dense_count_bytes(const mt_tensor *T) { return (size_t)(T->Kp / GM) * EPI_WARPS * sizeof(int); }
 

@@ -2640,6 +2640,19 @@ void integ_slot_mavg(const void *ctl_host, int b, double m[3]) {
   for (int q = 0; q < 3; ++q) m[q] = c.m_last[q];
 }
 
+// Device bytes of an integrator of B simulations (mt_integrator_create): states,
+// fields and derivatives, operand and work areas of the product, and 4 MB for
+// the rest (control blocks, reductions, the words of the one-kernel path, at
+// most 2.5 MB as its states fit a CTA's shared memory, the step graph).
+size_t integ_bytes(const mt_tensor *T, int B) {
+  const bool dense = T->layout == MT_LAYOUT_DENSE;
+  const size_t vec = sizeof(float) * 3 * T->n * B;
+  const size_t product = dense ? dense_x_bytes(T, B) + dense_part_bytes(T, B) + dense_count_bytes(T)
+                               : sizeof(float) * xs_floats(T) * B + matvec_part_bytes(T) + matvec_count_bytes(T, B) +
+                                     matvec_colpart_bytes(T, B);
+  return 11 * vec + product + ((size_t)4 << 20);
+}
+
 // k1 for the freshly admitted slots (one demag product for the batch)
 mt_status integ_init_fresh(mt_integrator *I) { return enqueue_init(I, 1); }
 

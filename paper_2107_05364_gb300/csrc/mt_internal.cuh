@@ -366,6 +366,13 @@ void ctx_release(mt_ctx *c);
 void tiles_release(mt_tiles *t);
 void tensor_release(mt_tensor *T);
 
+// storage of a tensor, and device bytes of a tensor and an integrator on it
+mt_status plan_storage(mt_tensor *T, int layout, size_t *scale_bytes);
+size_t engine_bytes_bound(mt_ctx *ctx, int64_t n, const std::vector<double> &centre, const std::vector<double> &edge,
+                          int prec, int layout, int B);
+size_t tensor_device_bytes(const mt_tensor *T);
+size_t integ_bytes(const mt_tensor *T, int B);
+
 // assembly (FP64) and packing
 mt_status assemble(mt_tensor *T);
 mt_status blocks_fp64(mt_tiles *t, int64_t count, const int64_t *pairs, double *out);

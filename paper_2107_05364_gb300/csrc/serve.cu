@@ -49,7 +49,6 @@ mt_status integ_poll(mt_integrator *I, void *ctl_host, cudaEvent_t ev);
 bool integ_slot_done(const void *ctl_host, int b, mt_stats *st);
 mt_status integ_fetch_slot(mt_integrator *I, int b, float *m_host);
 mt_status integ_create_idle(mt_tensor *T, const mt_llg_params *p, const mt_ode_opts *o, int B, mt_integrator **out);
-size_t tensor_bytes_for(int64_t n, int prec, int layout);
 }  // namespace mt
 
 namespace {
@@ -97,6 +96,7 @@ struct Geometry {
   std::unique_ptr<Engine> eng;
   std::deque<std::shared_ptr<Job>> waiting;
   double last_used = 0;
+  size_t need = 0;  // device bytes to reserve for its engine (0: not yet known)
 };
 
 }  // namespace
@@ -122,12 +122,6 @@ struct mt_server {
 };
 
 namespace {
-
-size_t engine_state_bytes(int64_t n, int B) {
-  // state, two stage inputs, H_d, seven stage derivatives (FP32, B x 3n each),
-  // operand copies and reductions: a conservative estimate
-  return (size_t)B * 3 * n * sizeof(float) * 14 + ((size_t)4 << 20);
-}
 
 void destroy_engine(mt_server *S, Geometry &g) {
   Engine *e = g.eng.get();
@@ -157,7 +151,9 @@ void fail_job(mt_server *S, const std::shared_ptr<Job> &j, mt_status st) {
 // make g resident: evict idle engines (least recently used) until the tensor
 // and batch state fit the budget.  Returns false if it cannot be done now.
 bool make_resident(mt_server *S, Geometry &g, const std::vector<Geometry *> &all) {
-  const size_t need = mt::tensor_bytes_for(g.n, S->o.prec, S->o.layout) + engine_state_bytes(g.n, S->o.max_batch);
+  if (g.need == 0)
+    g.need = mt::engine_bytes_bound(S->ctx, g.n, g.centre, g.edge, S->o.prec, S->o.layout, S->o.max_batch);
+  const size_t need = g.need;
   if (need > S->budget) {
     // can never fit: fail the geometry's waiting jobs
     while (!g.waiting.empty()) {
@@ -206,10 +202,11 @@ bool make_resident(mt_server *S, Geometry &g, const std::vector<Geometry *> &all
                       cudaMallocHost(&e->ctl, mt::integ_ctl_bytes(e->I)) != cudaSuccess ||
                       cudaEventCreateWithFlags(&e->ev, cudaEventDisableTiming) != cudaSuccess))
     st = MT_ENOMEM;
-  e->bytes = need;
+  // what it took, now that the tensor's planes are known
+  e->bytes = st == MT_OK ? mt::tensor_device_bytes(e->T) + mt::integ_bytes(e->T, e->B) : need;
   {
     std::lock_guard<std::mutex> lk(S->mu);
-    S->in_use += need;
+    S->in_use += e->bytes;
   }
   g.eng = std::move(e);
   if (st != MT_OK) {
