@@ -695,10 +695,13 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
     mtd::fence_mbar_init();
   }
   __syncthreads();
-  // Before the wait on the previous kernel (which writes the operand, not the
-  // tensor nor the active set): the CTA's first chunks, the ring's into shared
-  // memory (as far as they are the first ones the loop below takes: units of
-  // one live simulation group), the next ones into L2
+  // Before the wait on the previous kernel: the CTA's first chunks, the ring's
+  // into shared memory (as far as they are the first ones the loop below takes:
+  // units of one live simulation group), the next ones into L2.  The kernel
+  // just ahead writes the operand; it must not write the tensor nor the active
+  // set, which is read here and again after the wait (the one ahead is the
+  // operand's, k_begin or stage 2 .. 6; stages 1 and 7, admissions and copies
+  // write the set, and one of those others always comes between)
   const int64_t g0 = u0 / A.CH, pre_end = u1 < (g0 + 1) * A.CH ? u1 : (g0 + 1) * A.CH;
   const int pre = !half_live(A, g0, SB) ? 0 : (int)(pre_end - u0 < S::STAGES ? pre_end - u0 : S::STAGES);
   auto chunk_at = [&](int64_t u) {
@@ -759,9 +762,11 @@ __global__ void __launch_bounds__(HalfShape<PREC, SB>::THREADS, 1) k_matvec_half
           ++it;
         }
       }
-      // drain: every copy issued must have landed before the CTA may exit
-      for (int s = 0; s < S::STAGES && s < it; ++s) {
-        const int last = it - 1 - ((it - 1 - s) % S::STAGES);  // last issue on stage s
+      // drain: every copy issued must have landed before the CTA may exit, the
+      // early ones too should the loop have taken fewer
+      const int issued = it > pre ? it : pre;
+      for (int s = 0; s < S::STAGES && s < issued; ++s) {
+        const int last = issued - 1 - ((issued - 1 - s) % S::STAGES);  // last issue on stage s
         mtd::mbar_wait_bounded(&full[s], (uint32_t)(last / S::STAGES) & 1u, A.status);
       }
     }
