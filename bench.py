@@ -447,8 +447,9 @@ def run_batched(args, quiet=False):
     gemm_ms = e0.elapsed_time(e1) / reps
     Kp = int(math.ceil(n / 128) * 128)
     stored = info["bytes"]
-    # plane products per block: off-diagonal planes are multiplied twice
-    flops = 2.0 * (5 if info["planes"] == 4 else 9) * Kp * Kp * mt_pad(B) * (3 if args.prec == "split" else 1)
+    # plane products per block: off-diagonal planes are multiplied twice; split
+    # precision: N_hi with three operand terms, N_lo with two
+    flops = 2.0 * (5 if info["planes"] == 4 else 9) * Kp * Kp * mt_pad(B) * (5 if args.prec == "split" else 1)
     Td.close()
     I.close()
     # plain FP32 path, one simulation at a time
@@ -580,14 +581,17 @@ def run_serving(args, quiet=False):
 
 
 def mt_tensor_gb(t, prec):
-    """Stored bytes of a geometry's tensor (GB): streaming FP32 16 B (one
-    layer of tiles) or 24 B per block, dense BF16 2 B / split 4 B per entry
-    of the padded 3n x 3n matrix."""
-    n = t.n
+    """Stored bytes of a geometry's tensor (GB), in entry planes: 4 for one
+    layer of tiles, else 6, of 4 (FP32), 2 (dense BF16) or 4 (dense split) bytes
+    a block, the dense ones padded to 128 rows and columns.  FP32 sets of more
+    than 4,096 tiles of one shape are stored half, without zz."""
+    n, layer = t.n, t.shape[2] == 1
     if prec == "f32":
-        return (16.0 if t.shape[2] == 1 else 24.0) * n * n / 1e9
-    kp = math.ceil(3 * n / 128) * 128
-    return (2.0 if prec == "bf16" else 4.0) * kp * kp / 1e9
+        if n > 4096 and np.allclose(t.edge, t.edge[0], rtol=1e-12, atol=0.0):
+            return (3 if layer else 5) * 4 * n * (n + 128) / 2 / 1e9
+        return (4 if layer else 6) * 4.0 * n * n / 1e9
+    kp = math.ceil(n / 128) * 128
+    return (4 if layer else 6) * (2.0 if prec == "bf16" else 4.0) * kp * kp / 1e9
 
 
 def run_threshold(args):
