@@ -1615,6 +1615,23 @@ SmallWords small_words(int64_t n, int B, int G) {
 // stay there (L2: 129 MB)
 constexpr size_t kSmallL2Bytes = 96ull << 20;
 
+// The bound on tile sets and batches of the one-kernel path, in bytes per CTA:
+// the state of all tiles, 28 floats per row and simulation, 17 per row, the
+// rows of the tensor (six planes) and 43 words and a control block per
+// simulation, within 225 KB.  It is a rule of its own, wider than what the
+// kernel takes, so that a tile set's path does not change with the kernel; near
+// it the path has lost its lead (1,800 tiles, per attempt: 4 simulations 98 us
+// against 117 of the step graph, 8 simulations 187 and 170).
+size_t small_bound(int64_t n, int B, int R, bool nsmem) {
+  size_t o = 0;
+  small_take(o, sizeof(SimCtl) * B);
+  for (const int64_t words : {(int64_t)kSmallRed, (int64_t)3 * B * R, (int64_t)21 * B * R, (int64_t)36 * B, (int64_t)6 * B,
+                              (int64_t)B, n, (int64_t)3 * B * n, nsmem ? 6 * R * n : 0, (int64_t)3 * B * R,
+                              (int64_t)B * R, (int64_t)6 * R, (int64_t)6 * R, (int64_t)R, (int64_t)3 * R, (int64_t)R})
+    small_take(o, sizeof(float) * words);
+  return o;
+}
+
 // Does the one-kernel path fit this tile set and batch?  An FP32 streaming
 // tensor; one CTA per SM (or per tile) and a co-resident grid; either at
 // most 8 rows per CTA whose tensor rows and the state of all tiles fit the
@@ -1635,16 +1652,7 @@ bool small_plan(mt_integrator *I) {
     if (R > (nsmem ? 8 : 2 * kSmallWarps)) continue;
     if (!nsmem && (T->bytes > kSmallL2Bytes || T->L.TC % 4 != 0)) continue;
     size_t bytes = small_smem(n, I->B, R, nsmem, 1).total;
-    // (the limit counts one buffer of row sums, unpadded states, and H_d, the torque and the
-    // constants of the CTA's rows, once held in shared memory: the same tile
-    // sets qualify for this path whatever its kernel keeps there)
-    size_t counted = bytes - sizeof(float) * (2 * (nsmem ? kSmallRed : kSmallRedL2) - kSmallRed);
-    size_t state = 0, unpadded = 0;
-    small_take(state, sizeof(float) * ((size_t)I->B * small_stride(n) + 12));
-    small_take(unpadded, sizeof(float) * I->B * 3 * n);
-    counted += unpadded - state;
-    for (const int per_row : {3 * I->B, I->B, 6, 6, 1, 3, 1}) small_take(counted, sizeof(float) * R * per_row);
-    if (counted > kSmallSmemMax) continue;
+    if (small_bound(n, I->B, R, nsmem) > kSmallSmemMax || bytes > (size_t)kSmallSmemLimit) continue;
     // Several simulations: `group` of them (as many as fit) between two CTA
     // barriers, one to a warp, and the threads divided among as many as keep
     // the poll of one a single round of four vectors per thread.  One after
