@@ -260,21 +260,24 @@ MT_API mt_status mt_demag_assemble(mt_tiles *tiles, mt_prec prec, mt_tensor **ou
  * and otherwise stores all 6 planes (mt_tensor_info.planes tells).
  * mt_tensor_info.half tells;
  * MT_LAYOUT_STREAM_FULL stores every block.  Up to four simulations share a
- * read of either storage; the half storage's product is the faster one for
- * every batch (n = 10,000 film, half against full: 0.11 and 0.25 ms for one
- * simulation, 0.14 and 0.25 for two, 0.20 and 0.24 for four, 0.37 and 0.46 for
- * eight).  A pass over two or more simulations forms the row sums in another
- * order than a pass over one (each chunk's warp total first), so a
- * simulation's field from a half-stored tensor in a batch and alone agree to
+ * read of either storage; from 4,096 tiles the half storage's product was the
+ * faster one at every batch measured (1 to 16), by least for three or four
+ * simulations.  Half against full, ms, for 1, 2, 4 and 8: film of 10,000 tiles
+ * 0.11 and 0.24, 0.13 and 0.24, 0.19 and 0.24, 0.37 and 0.45; cube of 8,000
+ * 0.11 and 0.22, 0.11 and 0.22, 0.17 and 0.23, 0.32 and 0.37; cube of 4,096
+ * 0.036 and 0.060, 0.043 and 0.061, 0.059 and 0.062, 0.098 and 0.107.  A pass
+ * over two or more simulations forms the row sums in another order than a pass
+ * over one (each chunk's warp total first), so a simulation's field from a half-stored tensor in a batch and alone agree to
  * rounding, not bit for bit.
  * Thresholding and the allocation-free product need every block stored. */
 /* As mt_demag_assemble, with an explicit storage layout (mt_layout_kind).
  * MT_LAYOUT_DENSE turns every product over a batch of B simulations into a
  * GEMM on the tensor cores (tcgen05, BF16 in, FP32 accumulate); the rows and
  * columns of each entry plane are padded to a multiple of 128 (zeros), an
- * off-diagonal plane serves both entries it stands for, and the blocks of touching tiles are kept apart in FP64 as for the streaming
- * layout.  Errors as mt_demag_assemble, plus MT_EINVAL for a precision the
- * layout does not support. */
+ * off-diagonal plane serves both entries it stands for, and the blocks of
+ * touching tiles are kept apart in FP64 as for the streaming layout.  Errors as
+ * mt_demag_assemble, plus MT_EINVAL for a precision the layout does not
+ * support. */
 MT_API mt_status mt_demag_assemble_ex(mt_tiles *tiles, mt_prec prec, int layout, mt_tensor **out);
 
 /* Thresholded copy of an FP32 streaming-layout tensor (Sec. 4.3.1): the
@@ -544,9 +547,10 @@ MT_API mt_status mt_selftest_grid_barrier_timeout(mt_ctx *ctx);
  * stream); jobs queue per geometry in arrival order and take free slots
  * between graph replays, so work that arrives while other jobs run joins
  * the batch as slots free up.  Engines of different geometries overlap on
- * the device.  Residency is admitted by device footprint (tensor + batch
- * state) against hbm_budget_bytes; idle engines are evicted least recently
- * used.  A relax job integrates its own simulation until
+ * the device.  Residency is admitted by device footprint (tensor, batch state
+ * and the product's work areas) against hbm_budget_bytes; idle engines are
+ * evicted least recently used, and a geometry whose engine exceeds the budget
+ * by itself fails its jobs with MT_ENOMEM.  A relax job integrates its own simulation until
  * max_i |m_i x H_eff,i| / Ms_i < tol (Eq. 2) or its time cap.  A sweep job
  * is the field loop of Sec. 4.1 as one request: its simulation is relaxed
  * at each applied field of its schedule in turn (tolerance tol, time cap

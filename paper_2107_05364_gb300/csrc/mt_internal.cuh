@@ -244,11 +244,15 @@ constexpr double kPlanarTol = 1e-12;
 // distant tiles is absolute: their small entries are differences of O(1)
 // terms); else all 6 planes are stored.
 constexpr double kTraceTol = 1e-9;
-// MT_LAYOUT_STREAM stores a tensor of tiles of one shape half from this many
-// tiles on: measured on single-layer films, one simulation, per attempted
-// integrator step, half against full storage 0.178 / 0.140 ms at 2,500 tiles,
-// 0.255 / 0.253 at 3,600, 0.384 / 0.413 at 4,900, 0.516 / 0.646 at 6,400
-// (the column pass costs a fixed ~15 us that a small tensor does not repay)
+// MT_LAYOUT_STREAM stores a tensor of tiles of one shape half above this many
+// tiles.  The half product gains from about 2,500 tiles on (us per attempted
+// integrator step, half against full storage, 1 and 8 simulations: films of
+// 2,500 tiles 112 / 126 and 226 / 255, of 3,600 150 / 220 and 385 / 451; 3-D
+// sets of 2,548 tiles 119 / 165 and 287 / 324, of 4,096 230 / 380 and 601 / 688;
+// four simulations gain least, 314 / 326 at 3,600), below that it loses (1,500
+// tiles 94 / 81, and 47 in one kernel, which reads full storage only).  The
+// line lies higher because up to it a tensor keeps every block, as thresholding
+// and the allocation-free product need.
 constexpr int64_t kHalfMinTiles = 4096;
 
 // Index of entry e of block (i, j) in the tile-blocked streaming layout.
