@@ -675,6 +675,13 @@ mt_status plan_storage(mt_tensor *T, int layout, size_t *scale_bytes) {
   return MT_OK;
 }
 
+// device bytes of a tensor, the blocks kept apart among them
+size_t tensor_device_bytes(const mt_tensor *T) {
+  return T->bytes + (T->near_count > 0 ? sizeof(int32_t) * (size_t)(T->n + 1 + T->near_count) +
+                                             6 * (sizeof(double) + sizeof(float2)) * (size_t)T->near_count
+                                       : 0);
+}
+
 // Device bytes to reserve for the tensor of cuboid tiles (centre, edge) and an
 // integrator of B simulations on it, before either exists: the tensor with all
 // the planes that its assembly may turn out to need.
@@ -701,15 +708,8 @@ size_t engine_bytes_bound(mt_ctx *ctx, int64_t n, const std::vector<double> &cen
     layout_for(prec, &all);
     T.bytes = (size_t)T.L.CH * (all.chunk_bytes() + all.scale_bytes_per_chunk);
   }
-  return T.bytes + integ_bytes(&T, B);
-}
-
-// device bytes of an assembled tensor, the blocks kept apart among them
-size_t tensor_device_bytes(const mt_tensor *T) {
-  const size_t near = T->d_near_ptr ? sizeof(int32_t) * (T->n + 1 + T->near_count) +
-                                          6 * (sizeof(double) + sizeof(float2)) * (size_t)T->near_count
-                                    : 0;
-  return T->bytes + near;
+  if (prec == MT_BF16_SCALED || prec == MT_BF16_SPLIT) T.near_count = 27 * n;  // a tile and all its neighbours in a grid
+  return tensor_device_bytes(&T) + integ_bytes(&T, B);
 }
 
 }  // namespace mt

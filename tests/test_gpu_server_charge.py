@@ -34,7 +34,8 @@ S = mt.Server(ctx, opts=mt.ode_opts(rtol=1e-5, atol=1e-5), **json.loads(sys.argv
 g = S.add_geometry(t)
 s, r, _ = S.wait(S.submit(g, wl.m_noisy(t.n), alpha=0.5, tol=1e-1, t_max=1e-14), 60.0)
 assert s == 0
-print(json.dumps([S.stats()["bytes_in_use"], before - torch.cuda.mem_get_info()[0]]))
+st = S.stats()
+print(json.dumps([st["bytes_in_use"], before - torch.cuda.mem_get_info()[0], st["budget"]]))
 S.close()
 """
 
@@ -42,8 +43,11 @@ S.close()
 @pytest.mark.parametrize("tiles,opts", [
     ("wl.film(50, 10, 1)", dict(max_batch=128, prec="split", layout="MT_LAYOUT_DENSE")),
     ("wl.film(80, 52, 1)", dict(max_batch=4)),
+    ("solid(16, 16, 12)", dict(max_batch=2, prec="bf16")),
     ("solid(18, 25, 10)", dict(max_batch=8)),
     ("wl.graded_film(60, 50, 1, (300e-9, 200e-9, 3e-9), seed=4)", dict(max_batch=64)),
+    # 18.0 MB without the blocks kept apart, 20.2 with them: does not fit 19.5
+    ("solid(10, 10, 10)", dict(max_batch=1, prec="bf16", hbm_budget_bytes=19500000)),
 ])
 def test_charge_is_what_an_engine_takes(tiles, opts):
     torch = pytest.importorskip("torch")
@@ -57,5 +61,6 @@ def test_charge_is_what_an_engine_takes(tiles, opts):
     out = subprocess.run([sys.executable, "-c", CHILD, tiles, json.dumps(opts)], cwd=root, capture_output=True, text=True,
                          timeout=120)
     assert out.returncode == 0, out.stderr[-2000:]
-    charged, taken = json.loads(out.stdout.strip().splitlines()[-1])
+    charged, taken, budget = json.loads(out.stdout.strip().splitlines()[-1])
+    assert charged <= budget
     assert taken - ROUNDING <= charged <= taken + FLAT, (charged, taken)
